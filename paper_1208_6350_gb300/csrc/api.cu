@@ -432,6 +432,7 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
             fl.mode = mode;
             // the classes the plan can have used, from the longest query
             fl.class_mask = fill_class_mask(mode, maxm, sc, force_s32, force_s32 || may_overflow);
+            fl.half_mask = fill_half_mask(mode, maxm, maxn, sc, fl.class_mask);
             cudaError_t e = launch_fill(fl, ctx->sms, S.max_blocks, st);
             if (e != cudaSuccess) return set_err(GSW_ECUDA, "fill: %s", cudaGetErrorString(e));
             S.launches += __builtin_popcount(fl.class_mask);

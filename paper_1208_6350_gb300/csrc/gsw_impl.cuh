@@ -177,6 +177,27 @@ inline uint32_t fill_class_mask(int mode, int maxm, const Scoring &sc, bool forc
     return m;
 }
 
+// The classes of a launch (`mask`, from fill_class_mask) whose pairs cannot
+// leave the lanes whose clamp is a half-precision multiply-add (fill.cuh, LH):
+// a local score is at most min(rows, columns) x the largest matrix entry, and
+// every lane value at most the score + O + one matrix entry, which must stay
+// within the integers half precision holds exactly (2048); and O >= -wmin
+// keeps the sums of the shifted scores non-negative.
+inline uint32_t fill_half_mask(int mode, int maxm, int maxn, const Scoring &sc, uint32_t mask) {
+    if (sc.O < -sc.wmin) return 0;
+    const long long top = sc.wmax > 0 ? sc.wmax : 0;
+    auto fits = [&](int rows) { return (rows < maxn ? rows : maxn) * top + top + sc.O <= 2047; };
+    int most[kNumFillClasses] = {};
+    const int upto = maxm < GSW_TUNE_BUCKETS * GSW_TUNE_ROWS ? maxm : GSW_TUNE_BUCKETS * GSW_TUNE_ROWS;
+    for (int r = 1; r <= upto; r++)
+        most[mode == kFillForward ? pick_class16(r, sc) : pick_class_reverse(r, false, sc)] = r;
+    if (maxm > upto) most[kVarMaxS16] = maxm;
+    uint32_t m = 0;
+    for (int c = 0; c < kNumVariants; c++)
+        if (((mask >> c) & 1u) && !variant_at(c).s32 && fits(most[c])) m |= 1u << c;
+    return m;
+}
+
 // Work plan of one fill launch: pairs sorted by (variant, cost descending),
 // cut into warp tasks of 32/P pairs of one variant.  Task indices are handed
 // out heaviest variant first (variant index descending).
@@ -204,6 +225,7 @@ struct FillLaunch {
     FillScratch scr;
     int32_t mode;
     uint32_t class_mask;  // classes launched (bit c: class c); the others hold no pair
+    uint32_t half_mask;   // classes whose values stay below 2048: the half-precision clamp lanes
     // nonzero once the batch's letter check found a code >= the alphabet
     // (written by the check, which runs first on the stream): the fill then
     // writes empty records and touches no letter, so its steady steps need
@@ -424,6 +446,11 @@ int fill_max_pairs_per_warp();
 // one persistent launch per class in fl.class_mask, heaviest first; each grid
 // capped at max_blocks and at the slots the scratch holds
 cudaError_t launch_fill(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st);
+// launch_fill and fill_slots of one alphabet kind (fill_dna.cu, fill_general.cu)
+cudaError_t launch_fill_dna(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st);
+cudaError_t launch_fill_general(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st);
+int fill_slots_dna(int A, int sms);
+int fill_slots_general(int A, int sms);
 
 struct PlanBuffers {
     int32_t *keys;       // [npairs]

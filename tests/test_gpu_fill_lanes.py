@@ -1,0 +1,69 @@
+"""The fill's lanes whose clamp is a half-precision multiply-add: taken when no
+value of the batch's class can reach 2048 and O >= -(smallest matrix entry).
+Every output against the oracle at the edges of that rule (all integers, so the
+tolerance is zero)."""
+import numpy as np
+import pytest
+
+from paper_1208_6350_gb300 import gsw
+from paper_1208_6350_gb300 import workloads as wl
+from parity_util import compare, run_gpu_host, run_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = gsw.Context(0, 4 << 30)
+    yield c
+    c.close()
+
+
+def batch(qs, ts, W, O, X, alphabet):
+    ql, tl = np.array([len(x) for x in qs], np.int32), np.array([len(x) for x in ts], np.int32)
+    off = lambda n: np.concatenate([[0], np.cumsum(n.astype(np.int64))[:-1]])
+    return wl.Batch("lanes", np.concatenate(qs), off(ql), ql, np.concatenate(ts), off(tl), tl, W, O, X, alphabet)
+
+
+def edge_batch(seed, rows, cols, W, O, X):
+    """Exact copies (the largest scores), related and unrelated pairs, odd lengths."""
+    rng = np.random.default_rng(seed)
+    A = W.shape[0]
+    top = int(np.argmax(np.diag(W)))
+    qs, ts = [], []
+    for k in range(24):
+        m = rows if k < 4 else int(rng.integers(1, rows + 1))
+        n = cols if k < 4 else int(rng.integers(1, cols + 1))
+        q = np.full(m, top, np.uint8) if k % 4 == 0 else rng.integers(0, A, m).astype(np.uint8)
+        t = rng.integers(0, A, n).astype(np.uint8)
+        w = min(m, n)
+        if k % 3 != 2:
+            at = int(rng.integers(0, n - w + 1))
+            t[at:at + w] = q[:w]
+            if k % 3 == 1:
+                t[rng.integers(0, n, max(1, n // 20))] = rng.integers(0, A)
+        qs.append(q)
+        ts.append(t)
+    return batch(qs, ts, W, O, X, wl.DNA if A == 4 else wl.PROTEIN[:A])
+
+
+# (match, mismatch, open, extend, rows): 7 * 291 + 7 + 3 = 2047 is the last row
+# count whose values fit; O one below -mismatch keeps the biased lanes
+@pytest.mark.parametrize("match,mismatch,O,X,rows", [
+    (7, -3, 3, 1, 291), (7, -3, 3, 1, 292), (7, -3, 2, 1, 250), (1, -4, 4, 4, 256), (2, -2, 3, 0, 257),
+    (127, -127, 127, 20, 14), (127, -127, 127, 20, 15), (1, 0, 0, 0, 120)])
+def test_dna_lanes_at_the_edges_of_the_rule(ctx, match, mismatch, O, X, rows):
+    for table in (None, [9] * 32, [13] * 32, [0] * 32):
+        ctx.set_tune(table)
+        try:
+            b = edge_batch(match * 1000 + rows + O, rows, max(40, 2 * rows + 13), wl.dna_matrix(match, mismatch), O, X)
+            compare(b, run_oracle(b), run_gpu_host(ctx, b))
+        finally:
+            ctx.set_tune(None)
+
+
+@pytest.mark.parametrize("A,O,X,rows", [(20, 11, 1, 182), (20, 11, 1, 200), (5, 6, 2, 300), (20, 3, 1, 100)])
+def test_general_alphabet_lanes(ctx, A, O, X, rows):
+    W = np.ascontiguousarray(wl.synthetic_protein_matrix()[:A, :A])
+    b = edge_batch(A + rows, rows, rows + 41, W, O, X)
+    compare(b, run_oracle(b), run_gpu_host(ctx, b))
