@@ -135,8 +135,10 @@ int gsw_context_destroy(gsw_ctx *ctx);
  * (64..256 query rows per strip; longer queries run several strips), 8 = one
  * pair per CTA (512-row strips pipelined across the warps), 9..13 = one pair
  * per 8-lane group with 8, 10, 12, 14, 16 row words per lane (128..256 rows
- * per strip), -1 = the default rule (the smallest one-strip class of 0..6, the
- * CTA class from 1792 rows).  The choice changes speed only: every class
+ * per strip), -1 = the default rule (by the batch's size: these classes, 4-lane
+ * groups of up to 128 rows and 16-lane groups of up to 512 rows per strip; a
+ * pair whose strips would take a large part of the batch's time, and queries
+ * from 1792 rows, on a CTA).  The choice changes speed only: every class
  * gives the same results.
  * Paper: none for the tuner itself; it chooses among layouts of the one
  * fill the paper describes (Algorithm and implementation, item (1)).
@@ -145,15 +147,16 @@ int gsw_context_destroy(gsw_ctx *ctx);
 #define GSW_TUNE_ROWS 32
 typedef struct gsw_tune {
     int8_t fill_class[GSW_TUNE_BUCKETS]; /* bucket b: queries of 32b+1 .. 32(b+1) rows */
-    float gcups[GSW_TUNE_BUCKETS];       /* measured forward-fill rate of the chosen class */
-    float gcups_default[GSW_TUNE_BUCKETS]; /* ... of the default rule's class */
+    float gcups[GSW_TUNE_BUCKETS];       /* measured forward-fill rate of what was installed */
+    float gcups_default[GSW_TUNE_BUCKETS]; /* ... of the default rule */
 } gsw_tune;
 
 /* Measures every candidate class of every bucket on seeded random pairs
  * (queries of the bucket's largest length against targets of target_len
  * letters, the given scoring, score-only batches of about 2 G cells, best of 3
- * runs), installs the fastest in the context and copies the table to *out (may
- * be NULL).  Takes a few seconds; allocates its own temporary device buffers.
+ * runs), installs the fastest in the context (a bucket where the default rule
+ * is fastest is left to it) and copies the table of the fastest named classes
+ * to *out (may be NULL).  Takes a few seconds; allocates its own temporary device buffers.
  * Errors: GSW_EINVAL, GSW_ENOMEM, GSW_ECUDA. */
 int gsw_autotune(gsw_ctx *ctx, const int8_t *matrix, int32_t alphabet, int32_t gap_open, int32_t gap_extend,
                  int32_t target_len, gsw_tune *out);

@@ -77,8 +77,7 @@ struct DevBuf {
 struct PipeState {
     gsw::PlanBuffers pb;
     gsw::FillLaunch fl;
-    size_t slots = 0, ncap = 0;
-    int max_blocks = 0;
+    size_t ncap = 0;
     long long *ring_prefix = nullptr;
     int *ring_final = nullptr, *ring_group = nullptr;
     long long ring_words = 0, ring_pool = 0;  // wide-band traceback sizes (stats)
@@ -120,7 +119,7 @@ struct gsw_ctx {
     bool capturing = false;         // a segment is being captured: no allocation
     cudaStream_t st = nullptr;     // stream of the call in progress
     DevBuf plan_keys, plan_order, plan_small;
-    DevBuf fill_cm, fill_bnd;
+    DevBuf fill_scr;
     DevBuf trace_dirs, trace_ops, band_scr, ring_meta;
     DevBuf misc;  // counters: trace head, cigar cursor, trace need, max lengths
     DevBuf io_q, io_t, io_qoff, io_toff, io_qlen, io_tlen, io_res, io_cigar, io_colmax, io_cmoff;
@@ -128,7 +127,7 @@ struct gsw_ctx {
     DevBuf prof_qoff, prof_qlen;
     void *host_small = nullptr;  // pinned readback area
     cudaEvent_t ev[GSW_NSTAGES + 1] = {};
-    BandStreams aux = {};  // side streams of the band kernel's classes (created on first use)
+    SideStreams aux = {};  // side streams of the fill and band classes (created on first use)
     bool timing = false;
     int launches = 0;
     int stage_done[GSW_NSTAGES] = {};
@@ -210,26 +209,26 @@ enum MiscSlot {
     kMiscValid = 3,
     kMiscNeed = 4,   // 2 words: anti-diagonal traceback (direction words, op words per pair)
     kMiscRing = 6,   // 3 words: wide-band traceback (total words, max words of a pair, max op words)
-    kMiscStats = 12,   // 5 words: largest lengths, arena extents, bad lengths or offsets
-    kMiscNeed16 = 17,  // 4 words: 16-bit rectangle traceback (direction words per group, per class)
-    kMiscWords = 21
+    kMiscStats = 12,   // 7 words: largest lengths, arena extents, bad lengths or offsets, smallest query, cells
+    kMiscNeed16 = 19,  // 4 words: 16-bit rectangle traceback (direction words per group, per class)
+    kMiscWords = 23
 };
 
-// Side streams and fork/join events of the band classes, created once per
+// Side streams and fork/join events of the fill and band classes, created once per
 // context outside any capture (the first call of a shape is never captured).
-void destroy_aux(BandStreams &a) {
+void destroy_aux(SideStreams &a) {
     for (int k = 0; k < 2; k++) {
         if (a.s[k]) cudaStreamDestroy(a.s[k]);
         if (a.join[k]) cudaEventDestroy(a.join[k]);
     }
     if (a.fork) cudaEventDestroy(a.fork);
-    a = BandStreams{};
+    a = SideStreams{};
 }
 
 int ensure_aux(gsw_ctx *ctx) {
     if (ctx->aux.fork) return GSW_OK;
     if (ctx->capturing) return GSW_ESTATE;
-    BandStreams a{};
+    SideStreams a{};
     cudaError_t e = cudaSuccess;
     for (int k = 0; k < 2 && e == cudaSuccess; k++) {
         e = cudaStreamCreateWithFlags(&a.s[k], cudaStreamNonBlocking);
@@ -238,7 +237,7 @@ int ensure_aux(gsw_ctx *ctx) {
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&a.fork, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         destroy_aux(a);  // all or nothing: a later call tries again
-        return set_err(GSW_ECUDA, "band side streams: %s", cudaGetErrorString(e));
+        return set_err(GSW_ECUDA, "side streams: %s", cudaGetErrorString(e));
     }
     ctx->aux = a;
     return GSW_OK;
@@ -338,7 +337,8 @@ uint64_t bucket_up(uint64_t x) {
     return b;
 }
 
-int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st, int maxm, int maxn) {
+int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st, int minm, int maxm,
+                 int maxn) {
     const int npairs = bv.npairs;
     unsigned long long *misc = reinterpret_cast<unsigned long long *>(ctx->misc.p);
     unsigned long long *hs = reinterpret_cast<unsigned long long *>(ctx->host_small);
@@ -347,6 +347,7 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
     key.reserve(2048);
     key_add(key, bv);
     key_add(key, sc);
+    key_add(key, minm);
     key_add(key, maxm);
     key_add(key, maxn);
     key_add(key, st);
@@ -355,7 +356,7 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
     key_add(key, ctx->used);
     key_add(key, ctx->timing);
     key_add(key, ctx->ev);
-    for (const DevBuf *d : {&ctx->plan_keys, &ctx->plan_order, &ctx->plan_small, &ctx->fill_cm, &ctx->fill_bnd,
+    for (const DevBuf *d : {&ctx->plan_keys, &ctx->plan_order, &ctx->plan_small, &ctx->fill_scr,
                             &ctx->band_scr, &ctx->ring_meta, &ctx->trace_dirs, &ctx->trace_ops, &ctx->misc})
         key_buf(key, *d);
 
@@ -378,33 +379,14 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
         pb.ntasks = pb.task_hi + kNumFillClasses;
         pb.head = pb.ntasks + 1;
 
-        // fill launch geometry and per-slot scratch
-        const int warps_per_block = fill_block_threads() / 32;
         // columns per slot, a multiple of 4: every slot's max array starts on
-        // a 16-byte boundary (the fill stores four 16-bit column maxima at a
+        // an 8-byte boundary (the fill stores four 16-bit column maxima at a
         // time with one 8-byte store)
         S.ncap = ((size_t)std::max(maxn, 1) + 3) & ~(size_t)3;
-        const size_t per_slot = S.ncap * sizeof(int32_t) + 2 * S.ncap * sizeof(int2);
-        S.slots = (size_t)fill_slots(sc, ctx->sms);
-        if (S.slots == 0) return set_err(GSW_ECUDA, "fill kernels cannot be resident");
-        S.max_blocks = INT32_MAX;
-        {
-            // keep the scratch inside half of what the budget has left
-            size_t have = room(ctx, ctx->fill_cm, ctx->fill_bnd);
-            size_t cap_slots = have / 2 / per_slot;
-            if (S.slots > cap_slots) {
-                // a warp holds at most fill_max_pairs_per_warp() pairs
-                const size_t per_warp = (size_t)fill_max_pairs_per_warp();
-                S.max_blocks = (int)std::max<size_t>(1, cap_slots / (per_warp * warps_per_block));
-                S.slots = (size_t)S.max_blocks * warps_per_block * per_warp;
-            }
-        }
-        GSW_TRY(ensure2(ctx, ctx->fill_cm, S.slots * S.ncap * sizeof(int32_t), ctx->fill_bnd,
-                        S.slots * 2 * S.ncap * sizeof(int2)));
-
         FillLaunch &fl = S.fl;
         fl.b = bv;
         fl.sc = sc;
+        fl.maxm = maxm;
         fl.bad_letters = reinterpret_cast<const int32_t *>(misc + kMiscValid);
         fl.plan.order = pb.order;
         fl.plan.var_start = pb.var_start;
@@ -412,10 +394,44 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
         fl.plan.task_hi = pb.task_hi;
         fl.plan.head = pb.head;
         fl.plan.ntasks = pb.ntasks;
-        fl.scr.colmax = ctx->fill_cm.p;
-        fl.scr.boundary = ctx->fill_bnd.p;
+        fl.scr.bnd_off = 0;
         fl.scr.ncap = (int32_t)S.ncap;
-        fl.scr.nslots = (int32_t)S.slots;
+
+        // a local score is at most min(m, n) x the largest matrix entry (gaps
+        // never add), so when that stays within the 16-bit lanes' bound no
+        // pair is flagged for the 32-bit refill
+        const bool force_s32 = (bv.flags & GSW_FORCE_S32) != 0;
+        const bool may_overflow = (long long)std::min(maxm, maxn) * std::max(sc.wmax, 0) > 32767 - sc.wmax;
+        const bool refill = !force_s32 && may_overflow;
+        const bool reverse = (bv.flags & (GSW_BEGIN | GSW_CIGAR)) != 0;
+        auto set_mode = [&](int32_t mode) {
+            fl.mode = mode;
+            // the classes the plan can have used, from the longest query
+            fl.class_mask = fill_class_mask(mode, maxm, sc, force_s32, force_s32 || may_overflow, minm);
+            const ClassRows rows = fill_class_rows(mode, maxm, sc, fl.class_mask);
+            fl.half_mask = fill_half_mask(rows, maxn, sc);
+            fl.multi_mask = fill_multi_mask(rows);
+        };
+        // scratch of the stages' launches: full occupancy within half of what
+        // the budget has left, at least one block of the widest class (4 warps
+        // of 4 pairs, or of one pair in 32-bit lanes, with boundary rows) and
+        // one CTA of the wide-band traceback
+        size_t want = 0;
+        for (int32_t mode : {(int32_t)kFillForward, (int32_t)kFillRerun, (int32_t)kFillReverse}) {
+            if ((mode == kFillRerun && !refill) || (mode == kFillReverse && !reverse)) continue;
+            set_mode(mode);
+            want = std::max(want, fill_scratch_want(fl, ctx->sms));
+        }
+        if (want == 0) return set_err(GSW_ECUDA, "fill kernels cannot be resident");
+        const size_t ring_slot = 2 * S.ncap * sizeof(int2);
+        if ((bv.flags & GSW_CIGAR) && maxn > 512)
+            want = std::max(want, ring_slot * (size_t)ctx->sms * 2 * (size_t)ring_slots_per_cta());
+        const size_t least = 160 * S.ncap + 512;
+        want = std::max(least, std::min(want, room(ctx, ctx->fill_scr, DevBuf()) / 2));
+        if (want > ctx->fill_scr.bytes) release(ctx, ctx->fill_scr);
+        GSW_TRY(ensure(ctx, ctx->fill_scr, want));
+        fl.scr.base = ctx->fill_scr.p;
+        fl.scr.bytes = ctx->fill_scr.bytes;
 
         auto plan = [&](int32_t mode) -> int {
             cudaError_t e = launch_plan(bv, sc, mode, pb, st);
@@ -423,21 +439,16 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
             S.launches += 3;
             return GSW_OK;
         };
-        // a local score is at most min(m, n) x the largest matrix entry (gaps
-        // never add), so when that stays within the 16-bit lanes' bound no
-        // pair is flagged for the 32-bit refill
-        const bool force_s32 = (bv.flags & GSW_FORCE_S32) != 0;
-        const bool may_overflow = (long long)std::min(maxm, maxn) * std::max(sc.wmax, 0) > 32767 - sc.wmax;
+        // (a context limited to some SMs runs its classes one after the other)
+        const bool limited = ctx->sms < ctx->sms_all;
         auto fill = [&](int32_t mode) -> int {
-            fl.mode = mode;
-            // the classes the plan can have used, from the longest query
-            fl.class_mask = fill_class_mask(mode, maxm, sc, force_s32, force_s32 || may_overflow);
-            fl.half_mask = fill_half_mask(mode, maxm, maxn, sc, fl.class_mask);
-            cudaError_t e = launch_fill(fl, ctx->sms, S.max_blocks, st);
+            set_mode(mode);
+            cudaError_t e = launch_fill(fl, ctx->sms, st, limited ? SideStreams{} : ctx->aux);
             if (e != cudaSuccess) return set_err(GSW_ECUDA, "fill: %s", cudaGetErrorString(e));
             S.launches += __builtin_popcount(fl.class_mask);
             return GSW_OK;
         };
+        GSW_TRY(ensure_aux(ctx));
         GSW_TRY(mark(ctx, 0, st));
         GSW_TRY(plan(kFillForward));
         GSW_TRY(mark(ctx, 1, st));
@@ -445,20 +456,20 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
         GSW_TRY(mark(ctx, 2, st));
         S.stage_done[0] = S.stage_done[1] = 1;
         // no pair flagged for the refill: its plan and launches are left out
-        if (!force_s32 && may_overflow) {
+        if (refill) {
             GSW_TRY(plan(kFillRerun));
             GSW_TRY(fill(kFillRerun));
             S.stage_done[2] = 1;
         }
         GSW_TRY(mark(ctx, 3, st));
-        if (bv.flags & (GSW_BEGIN | GSW_CIGAR)) {
+        if (reverse) {
             // reversed fill in the ring kernels for pairs whose reverse band is wide
             GSW_TRY(plan(kFillReverse));
             GSW_TRY(fill(kFillReverse));
             S.stage_done[3] = 1;
         }
         GSW_TRY(mark(ctx, 4, st));
-        if (bv.flags & (GSW_BEGIN | GSW_CIGAR)) {
+        if (reverse) {
             // thread-per-pair banded reverse and traceback for narrow bands
             // (the plan also hands a small batch's pairs to the warp tracebacks)
             GSW_TRY(plan(kPlanBand));
@@ -470,7 +481,6 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
                 const BandGrids bg = band_grids(rows_cap, ctx->sms, have / 4);
                 if (bg.total_bytes > ctx->band_scr.bytes) release(ctx, ctx->band_scr);
                 GSW_TRY(ensure(ctx, ctx->band_scr, bg.total_bytes));
-                GSW_TRY(ensure_aux(ctx));
                 CUDA_TRY(launch_band(bv, sc, pb, ctx->band_scr.p, bg, st, ctx->aux));
                 S.launches += 3;
             }
@@ -501,7 +511,7 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
 
     if (bv.flags & GSW_CIGAR) {
         CUDA_TRY(cudaStreamSynchronize(st));
-        // [0, 1] anti-diagonal, [2, 4] ring, [13, 16] 16-bit rectangle classes (others unused here)
+        // [0, 1] anti-diagonal, [2, 4] ring, kMiscNeed16 - kMiscNeed.. 16-bit rectangle classes (others unused here)
         unsigned long long need[kMiscWords - kMiscNeed];
         std::memcpy(need, hs, sizeof(need));
         for (int k = 5; k < kMiscNeed16 - kMiscNeed; k++) need[k] = 0;
@@ -509,7 +519,7 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
             for (unsigned long long &x : need) x = bucket_up(x);
         std::vector<uint8_t> key2 = key;
         key_add(key2, need);
-        for (const DevBuf *d : {&ctx->fill_bnd, &ctx->trace_dirs, &ctx->trace_ops, &ctx->ring_meta})
+        for (const DevBuf *d : {&ctx->fill_scr, &ctx->trace_dirs, &ctx->trace_ops, &ctx->ring_meta})
             key_buf(key2, *d);
         key_add(key2, ctx->used);
 
@@ -555,7 +565,8 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
             const unsigned long long ring_total = need[2], ring_max = need[3], ring_ops = need[4];
             size_t ring_pool = 0, ring_walk_warps = 0;
             if (ring_total > 0) {
-                ring_walk_warps = (size_t)ctx->sms * 16;
+                // (one warp per pair: no more warps, and op words, than pairs)
+                ring_walk_warps = std::min<size_t>((size_t)ctx->sms * 16, ((size_t)npairs + 1) & ~(size_t)1);
                 const size_t have_all = room(ctx, ctx->trace_dirs, ctx->trace_ops);
                 const size_t ops_bytes = ring_walk_warps * (size_t)ring_ops * sizeof(uint32_t);
                 size_t cap = have_all > ops_bytes ? (have_all - ops_bytes) / 2 / sizeof(uint32_t) : 0;
@@ -600,9 +611,9 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
                     ra.group = S.ring_group;
                     ra.pool = reinterpret_cast<uint32_t *>(ctx->trace_dirs.p);
                     ra.pool_words = (long long)ring_pool;
-                    ra.bnd = reinterpret_cast<int2 *>(ctx->fill_bnd.p);
+                    ra.bnd = reinterpret_cast<int2 *>(ctx->fill_scr.p);
                     ra.bnd_stride = 2 * (long long)S.ncap;
-                    ra.slots = (int)S.slots;
+                    ra.slots = (int)std::min<size_t>(ctx->fill_scr.bytes / (2 * S.ncap * sizeof(int2)), 1 << 20);
                     ra.ops = reinterpret_cast<uint32_t *>(ctx->trace_ops.p);
                     ra.op_words = (long long)ring_ops;
                     ra.walk_warps = (int)ring_walk_warps;
@@ -681,19 +692,25 @@ int batch_impl(gsw_ctx *ctx, int32_t npairs, const uint8_t *q, const int64_t *q_
     bv.mask_len = mask_len;
     bv.cigar_cap = cigar_capacity;
     bv.cigar_cursor = misc + kMiscCursor;
-    int maxm = 0, maxn = 0;
+    int minm = 0, maxm = 0, maxn = 0;
+    double cells = 0;  // of the forward fill
     int64_t cmext = 0;  // host I/O: colmax words from 0 to the end of the last pair's range
     const bool hio = (flags & GSW_HOST_IO) != 0;
     unsigned long long *hstat = reinterpret_cast<unsigned long long *>(ctx->host_small);
     // the batch's sizes and the checks of its lengths and offsets, on the
-    // device in one pass (one 40-byte readback before anything is sized)
+    // device in one pass (one 56-byte readback before anything is sized)
     auto batch_stats = [&](const int64_t *qo, const int32_t *ql, const int64_t *to, const int32_t *tl) -> int {
         CUDA_TRY(launch_batch_stats(qo, ql, to, tl, npairs, misc + kMiscStats, st));
         ctx->launches += 1;
-        CUDA_TRY(cudaMemcpyAsync(hstat, misc + kMiscStats, 5 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+        CUDA_TRY(cudaMemcpyAsync(hstat, misc + kMiscStats, 7 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                                  st));
         CUDA_TRY(cudaStreamSynchronize(st));
         return GSW_OK;
+    };
+    // the smallest query, rounded down to its class bucket's first length, so
+    // that batches of like lengths keep their captured graphs
+    auto smallest = [](unsigned long long x) {
+        return x < 1 ? 0 : (int)((x - 1) / GSW_TUNE_ROWS * GSW_TUNE_ROWS + 1);
     };
     if (hio) {
         // offsets and lengths first; the arenas once their extents are known
@@ -714,6 +731,8 @@ int batch_impl(gsw_ctx *ctx, int32_t npairs, const uint8_t *q, const int64_t *q_
                 if (q_off[p] < 0 || t_off[p] < 0) return set_err(GSW_EINVAL, "pair %d: negative offset", p);
             }
         }
+        minm = smallest(hstat[5]);
+        cells = (double)hstat[6];
         maxm = (int)hstat[0];
         maxn = (int)hstat[1];
         const int64_t qext = (int64_t)hstat[2], text = (int64_t)hstat[3];
@@ -773,6 +792,8 @@ int batch_impl(gsw_ctx *ctx, int32_t npairs, const uint8_t *q, const int64_t *q_
         bv.colmax_off = colmax_off;
         GSW_TRY(batch_stats(q_off, q_len, t_off, t_len));
         if (hstat[4]) return set_err(GSW_EINVAL, "a length is outside [0, 2^24) or an offset is negative");
+        minm = smallest(hstat[5]);
+        cells = (double)hstat[6];
         maxm = (int)hstat[0];
         maxn = (int)hstat[1];
         if (flags & GSW_PACKED2) {
@@ -788,9 +809,12 @@ int batch_impl(gsw_ctx *ctx, int32_t npairs, const uint8_t *q, const int64_t *q_
         }
     }
     if (ctx->graph_buckets) {
+        minm = 0;
+        cells = (double)bucket_up((uint64_t)cells);
         maxm = (int)bucket_up((uint64_t)maxm);
         maxn = (int)bucket_up((uint64_t)maxn);
     }
+    default_classes(sc, npairs, maxn, cells);
     CUDA_TRY(cudaMemsetAsync(misc + kMiscCursor, 0, 2 * sizeof(unsigned long long), st));  // cursor, internal
     if ((flags & GSW_PACKED2) && sc.A >= 4) {
         // 2-bit letters are 0..3: valid under any matrix of 4 or more letters
@@ -799,7 +823,7 @@ int batch_impl(gsw_ctx *ctx, int32_t npairs, const uint8_t *q, const int64_t *q_
         CUDA_TRY(launch_validate(bv, sc, reinterpret_cast<int32_t *>(misc + kMiscValid), st));
         ctx->launches += 1;
     }
-    GSW_TRY(run_pipeline(ctx, bv, sc, st, maxm, maxn));
+    GSW_TRY(run_pipeline(ctx, bv, sc, st, minm, maxm, maxn));
 
     // completion: invalid letters, internal checks, CIGAR space
     CUDA_TRY(launch_count_flag(bv.res, npairs, kResInternal, misc + kMiscInternal, st));
@@ -991,7 +1015,7 @@ int gsw_context_destroy(gsw_ctx *c) {
     if (!c) return GSW_OK;
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
-    DevBuf *all[] = {&c->plan_keys, &c->plan_order, &c->plan_small, &c->fill_cm, &c->fill_bnd, &c->trace_dirs,
+    DevBuf *all[] = {&c->plan_keys, &c->plan_order, &c->plan_small, &c->fill_scr, &c->trace_dirs,
                      &c->trace_ops, &c->band_scr, &c->misc, &c->io_q, &c->io_t, &c->io_qoff, &c->io_toff, &c->io_qlen,
                      &c->io_tlen, &c->io_res, &c->io_cigar, &c->io_colmax, &c->io_cmoff, &c->prof_qoff,
                      &c->prof_qlen, &c->ring_meta, &c->io_qp, &c->io_tp};

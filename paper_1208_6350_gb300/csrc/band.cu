@@ -488,7 +488,7 @@ BandGrids band_grids(int rows_cap, int sms, size_t budget_bytes) {
 }
 
 cudaError_t launch_band(const BatchView &b, const Scoring &sc, const PlanBuffers &pb, void *scratch,
-                        const BandGrids &g, cudaStream_t st, const BandStreams &aux) {
+                        const BandGrids &g, cudaStream_t st, const SideStreams &aux) {
     BandLaunch L;
     L.b = b;
     L.sc = sc;

@@ -5,23 +5,102 @@
 
 namespace gsw {
 
-int fill_block_threads() { return kBlock; }
+namespace {
 
-int fill_max_pairs_per_warp() {
-    int most = 1;
-#define GSW_PER_WARP(id, P_, R_, S_) most = 32 / P_ > most ? 32 / P_ : most;
-    GSW_FILL_VARIANTS(GSW_PER_WARP)
-#undef GSW_PER_WARP
-    return most;
+// Calls f(class, geometry) for every class in fl.class_mask, heaviest first:
+// the CTA kernel for queries of many strips, then the variants by rows per
+// strip.  Stops when f returns false.
+template <class F>
+void each_class(const FillLaunch &fl, int sms, F f) {
+    for (int c = kNumFillClasses - 1; c >= 0; c--) {
+        if (!((fl.class_mask >> c) & 1u)) continue;  // no pair of the class
+        const bool half = ((fl.half_mask >> c) & 1u) != 0;
+        const ClassGeom g = fl.sc.dna4 ? (half ? fill_geom_dna_half(c, fl, sms) : fill_geom_dna(c, fl, sms))
+                                       : (half ? fill_geom_general_half(c, fl, sms) : fill_geom_general(c, fl, sms));
+        if (!f(c, g)) return;
+    }
 }
 
-// Slots (pairs in flight) the largest variant launch can hold, at full
-// occupancy on `sms` SMs; a launch is never given more blocks than
-// max_blocks, so callers can cap the scratch.
-int fill_slots(const Scoring &sc, int sms) { return sc.dna4 ? fill_slots_dna(sc.A, sms) : fill_slots_general(sc.A, sms); }
+// No more blocks than the batch has pairs for (the CTA classes: one pair per
+// block, whose warps share its strips).
+void fit_pairs(const FillLaunch &fl, int c, ClassGeom &g) {
+    const int per = c >= kNumVariants ? 1 : std::max(1, g.slots_per_block);
+    g.grid = std::min(g.grid, std::max(1, (fl.b.npairs + per - 1) / per));
+}
 
-cudaError_t launch_fill(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st) {
-    return fl.sc.dna4 ? launch_fill_dna(fl, sms, max_blocks, st) : launch_fill_general(fl, sms, max_blocks, st);
+// Every pair in flight has a slot: no more blocks than `bytes` hold.
+bool fit_scratch(ClassGeom &g, size_t bytes) {
+    const size_t per = (size_t)g.slots_per_block * (g.cm + g.bnd);
+    if (g.grid > 0 && g.bytes(g.grid) > bytes)
+        g.grid = (int)std::min<size_t>((size_t)g.grid, (bytes - std::min<size_t>(bytes, 256)) / per);
+    return g.grid > 0;
+}
+
+size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+}  // namespace
+
+size_t fill_scratch_want(const FillLaunch &fl, int sms) {
+    size_t sum = 0;
+    each_class(fl, sms, [&](int c, ClassGeom g) {
+        fit_pairs(fl, c, g);
+        sum += align256(g.bytes(g.grid));
+        return true;
+    });
+    return sum;
+}
+
+cudaError_t launch_fill(const FillLaunch &fl, int sms, cudaStream_t st, const SideStreams &aux) {
+    struct Todo {
+        int c;
+        ClassGeom g;
+        size_t at;
+    } todo[kNumFillClasses];
+    int n = 0;
+    size_t sum = 0;
+    each_class(fl, sms, [&](int c, ClassGeom g) {
+        fit_pairs(fl, c, g);
+        todo[n++] = Todo{c, g, sum};
+        sum += align256(g.bytes(g.grid));
+        return true;
+    });
+    // the classes whose pairs take longest first (strips x row words of a step)
+    const ClassRows rows = fill_class_rows(fl.mode, fl.maxm, fl.sc, fl.class_mask);
+    auto longest = [&](int c) {
+        const int strips = (rows.most[c] + variant_rows(c) - 1) / variant_rows(c);
+        return c >= kNumVariants ? INT_MAX : strips * (4 + variant_at(c).R);
+    };
+    std::stable_sort(todo, todo + n, [&](const Todo &a, const Todo &b) { return longest(a.c) > longest(b.c); });
+    // classes side by side: the next one's blocks move in as one drains (a
+    // batch of 20,000 reads of 100 to 250 nt is five launches, none of which
+    // fills the chip)
+    const bool side = n > 1 && aux.fork && sum <= fl.scr.bytes;
+    cudaError_t e = cudaSuccess;
+    if (side) {
+        if ((e = cudaEventRecord(aux.fork, st))) return e;
+        for (int k = 0; k < 2 && k + 1 < n; k++)
+            if ((e = cudaStreamWaitEvent(aux.s[k], aux.fork, 0))) return e;
+    }
+    for (int i = 0; i < n && e == cudaSuccess; i++) {
+        FillLaunch x = fl;
+        ClassGeom &g = todo[i].g;
+        if (side) x.scr.base = static_cast<char *>(fl.scr.base) + todo[i].at;
+        else if (!fit_scratch(g, fl.scr.bytes)) return cudaErrorInvalidConfiguration;
+        if (g.grid < 1) return cudaErrorInvalidConfiguration;
+        x.scr.bnd_off = align256((size_t)g.grid * g.slots_per_block * g.cm);
+        const cudaStream_t on = side && i % 3 ? aux.s[i % 3 - 1] : st;
+        const int c = todo[i].c;
+        const bool half = ((fl.half_mask >> c) & 1u) != 0;
+        e = fl.sc.dna4 ? (half ? fill_launch_dna_half(c, x, g, on) : fill_launch_dna(c, x, g, on))
+                       : (half ? fill_launch_general_half(c, x, g, on) : fill_launch_general(c, x, g, on));
+    }
+    if (side)
+        for (int k = 0; k < 2 && k + 1 < n; k++) {
+            cudaError_t e2 = cudaEventRecord(aux.join[k], aux.s[k]);
+            if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(st, aux.join[k], 0);
+            if (e == cudaSuccess) e = e2;
+        }
+    return e;
 }
 
 // ---------------------------------------------------------------------------
@@ -173,7 +252,9 @@ extern "C" int gsw_fill_static(int32_t npairs, const uint8_t *q, const int64_t *
     if ((flags & GSW_COLMAX) && (!colmax || !colmax_off)) return set_err(GSW_EINVAL, "colmax output missing");
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return set_err(GSW_ECUDA, "no current device");
-    const size_t per_warp = (size_t)prof_words(8, true, sc.dna4 != 0, alphabet) * 32 * sizeof(uint32_t);
+    // (the 32-bit refill's profile may be the larger)
+    const size_t per_warp = (size_t)std::max(prof_words(8, true, sc.dna4 != 0, alphabet),
+                                             prof_words(8, false, sc.dna4 != 0, alphabet)) * 32 * sizeof(uint32_t);
     int wpb = (int)((200u << 10) / per_warp);
     wpb = wpb > 4 ? 4 : (wpb < 1 ? 1 : wpb);
     const size_t smem = per_warp * wpb;

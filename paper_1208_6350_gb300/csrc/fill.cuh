@@ -42,6 +42,7 @@
 #include "gsw_impl.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <climits>
 
 #include <type_traits>
@@ -94,10 +95,6 @@ struct L16 {
     static __device__ __forceinline__ uint32_t halves(int lo, int hi) {
         return ((uint32_t)lo & 0xFFFFu) | (((uint32_t)hi & 0xFFFFu) << 16);
     }
-    // low half of a, high half of b (words made by halves)
-    static __device__ __forceinline__ uint32_t merge(uint32_t a, uint32_t b) {
-        return (a & 0x0000FFFFu) | (b & 0xFFFF0000u);
-    }
 };
 
 // 16-bit lanes for pairs whose every value stays below 2048: non-negative
@@ -136,9 +133,6 @@ struct LH {
     static __device__ __forceinline__ uint32_t halves(int lo, int hi) {
         return ((uint32_t)lo & 0xFFFFu) | (((uint32_t)hi & 0xFFFFu) << 16);
     }
-    static __device__ __forceinline__ uint32_t merge(uint32_t a, uint32_t b) {
-        return (a & 0x0000FFFFu) | (b & 0xFFFF0000u);
-    }
     // gap state of a cell outside (a gap that never pays): E + O = 0
     static __device__ __forceinline__ uint32_t gap1(int) { return 0u; }
     // -O in both halves (sign and magnitude: half-precision integers)
@@ -169,7 +163,6 @@ struct L32 {
     static __device__ __forceinline__ uint32_t addk(int c) { return (uint32_t)c; }
     static __device__ __forceinline__ uint32_t addmax(uint32_t a, uint32_t b, uint32_t c) { return vmax(a + b, c); }
     static __device__ __forceinline__ uint32_t halves(int lo, int hi) { return (uint32_t)lo; }
-    static __device__ __forceinline__ uint32_t merge(uint32_t a, uint32_t b) { return a; }
     static __device__ __forceinline__ uint32_t cm16(uint32_t x) { return x; }
     static __device__ __forceinline__ uint32_t tt_relu(uint32_t d, uint32_t w, uint32_t e) {
         return vmax(addmax(d, w, e), Z2);
@@ -183,9 +176,13 @@ struct L32 {
 // added per step (measured against one word per letter pair, 16 R words,
 // whose larger profile costs occupancy, and one table holding both halves,
 // 4 R words, merged by a logic op that issues at a lower rate than the add:
-// both slower); other alphabets: one table with both halves per letter.
+// both slower).  Other alphabets in 16-bit lanes: one byte per score, both
+// halves' scores of two rows in a word (byte_words); the step's byte permute,
+// which takes the low half from the low letter's word and the high half from
+// the high letter's, also extends the signs.  32-bit lanes: a word per score.
+__host__ __device__ constexpr int byte_words(int R) { return (R + 1) / 2; }
 __host__ __device__ constexpr int prof_words(int R, bool fold, bool dna, int A) {
-    return dna ? (fold ? 8 * R : 4 * R) : A * R;
+    return dna ? (fold ? 8 * R : 4 * R) : A * (fold ? byte_words(R) : R);
 }
 
 // Index of profile word (table c, row r) of lane l inside the warp region:
@@ -238,6 +235,15 @@ __device__ __forceinline__ void load_words(const uint32_t *base, int c, int l, u
     }
 }
 
+// Row 2w + odd of byte-profile words lo (the low letter's) and hi (the high
+// letter's): the low half's score of lo and the high half's of hi, sign-extended
+__device__ __forceinline__ uint32_t merge_bytes(uint32_t lo, uint32_t hi, int odd) {
+    uint32_t r;
+    if (odd) asm("prmt.b32 %0, %1, %2, 0xF7A2;" : "=r"(r) : "r"(lo), "r"(hi));
+    else asm("prmt.b32 %0, %1, %2, 0xD580;" : "=r"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+
 __device__ __forceinline__ int sc_w(const Scoring &sc, int a, int b) { return sc.W[a * sc.A + b]; }
 
 // Builds this lane's profile for strip `st` (padded rows of the strip:
@@ -265,13 +271,16 @@ __device__ __forceinline__ void build_profile(uint32_t *psm, const Job &job, con
                     psm[pidx<R>(A + a, r, lane)] = L::halves(0, (qhi >= 0 ? sc_w(sc, qhi, a) : 0) + add);
             }
         } else {
-            // general alphabets: one table, both halves' scores in one word
-            // (the step takes the low half from the low letter's word and the
-            // high half from the high letter's), half the shared memory of
-            // two tables
-            for (int a = 0; a < A; a++)
-                psm[pidx<R>(a, r, lane)] =
-                    L::halves((qlo >= 0 ? sc_w(sc, qlo, a) : 0) + add, (L::FOLD && qhi >= 0 ? sc_w(sc, qhi, a) : 0) + add);
+            if constexpr (L::FOLD) {
+                uint8_t *bytes = reinterpret_cast<uint8_t *>(psm);
+                for (int a = 0; a < A; a++) {
+                    uint8_t *p = bytes + 4 * pidx<byte_words(R)>(a, r / 2, lane) + 2 * (r & 1);
+                    p[0] = (uint8_t)((qlo >= 0 ? sc_w(sc, qlo, a) : 0) + add);
+                    p[1] = (uint8_t)((qhi >= 0 ? sc_w(sc, qhi, a) : 0) + add);
+                }
+            } else {
+                for (int a = 0; a < A; a++) psm[pidx<R>(a, r, lane)] = (uint32_t)(qlo >= 0 ? sc_w(sc, qlo, a) : 0);
+            }
         }
     }
 }
@@ -459,14 +468,12 @@ struct StripRunner {
                 if constexpr (L::FOLD) nah = min((int)job.t[(long long)(j1 - P) * job.ts], A - 1);
             }
         }
-        uint32_t pw[R], ph[L::FOLD ? R : 1];
-        if constexpr (DNA) {
-            load_words<R>(psm, al, lane, pw);
-            if constexpr (L::FOLD) load_words<R>(psm, A + ah, lane, ph);
-        } else {
-            load_words<R>(psm, al, lane, pw);
-            if constexpr (L::FOLD) load_words<R>(psm, ah, lane, ph);
-        }
+        // the two letters' scores: words to add (DNA), bytes to merge (other
+        // alphabets), or the scores themselves (32-bit lanes)
+        constexpr int PW = (DNA || !L::FOLD) ? R : byte_words(R);
+        uint32_t pw[PW], ph[L::FOLD ? PW : 1];
+        load_words<PW>(psm, al, lane, pw);
+        if constexpr (L::FOLD) load_words<PW>(psm, DNA ? A + ah : ah, lane, ph);
         uint32_t diag = hdiag;
         hdiag = hin;
         uint32_t f = fin, m = cmin;
@@ -476,13 +483,15 @@ struct StripRunner {
             if constexpr (L::HALF) {
                 uint32_t d;
                 if constexpr (DNA) d = diag + pw[r] + ph[r];
-                else d = diag + L::merge(pw[r], ph[r]);
+                else d = diag + merge_bytes(pw[r / 2], ph[r / 2], r & 1);
                 h = L::relu_sub(L::vmax3(d, E[r], f), kO);
                 f = L::addmax(f, kXm, h);
                 E[r] = L::addmax(E[r], kXm, h);
             } else {
-                uint32_t w = pw[r];
-                if constexpr (L::FOLD) w = DNA ? w + ph[r] : L::merge(w, ph[r]);
+                uint32_t w;
+                if constexpr (!L::FOLD) w = pw[r];
+                else if constexpr (DNA) w = pw[r] + ph[r];
+                else w = merge_bytes(pw[r / 2], ph[r / 2], r & 1);
                 const uint32_t tt = L::tt_relu(diag, w, E[r]);
                 h = L::vmax(tt, f);
                 // one H - O for both gap states; the F chain then runs through
@@ -609,9 +618,9 @@ struct StripRunner {
     // MAYBE_FAST the steady steps of a one-strip forward fill take the FAST
     // form (the CTA kernel's strips never do).  With MAYBE_MULTI the strips of
     // a forward fill of several strips take the kModeFwdFirst/Later forms;
-    // the 8-lane variants (one-strip short reads, whose registers the extra
+    // the 8- and 4-lane variants (one-strip short reads, whose registers the extra
     // loops would crowd) keep the general step for them.
-    template <bool MAYBE_FAST = true, bool MAYBE_MULTI = (P != 8)>
+    template <bool MAYBE_FAST = true, bool MAYBE_MULTI = (P > 8)>
     __device__ bool run(int s0, int s1) {
         const int s_steady = L::FOLD ? 2 * P - 1 : P - 1;
         const int s_drain = max(s_steady, n - 1);
@@ -762,13 +771,37 @@ __device__ void secondary(const BatchView &b, int pair, const Job &job, int end_
     const long long lo = (long long)end_t - Lm, hi = (long long)end_t + Lm;
     int bv = 0, bj = INT_MAX;
     int32_t *out = (b.flags & GSW_COLMAX) ? b.colmax + b.colmax_off[pair] : nullptr;
-    for (int j = k; j < n; j += P) {
-        int v;
-        if constexpr (L::FOLD) v = L::value(cms[j]);
-        else v = cms[j];
-        if (out) out[j] = v;
-        if (end_t >= 0 && j >= lo && j <= hi) continue;
-        if (v > bv) { bv = v; bj = j; }
+    // four columns a lane and load (a slot holds a multiple of 4 columns), so
+    // that the narrow groups make few trips to L2
+    const bool wide = out && ((uintptr_t)out & 15) == 0;
+#pragma unroll 2
+    for (int j = 4 * k; j < n; j += 4 * P) {
+        int v[4];
+        if constexpr (L::FOLD) {
+            const uint2 w = *reinterpret_cast<const uint2 *>(cms + j);
+            v[0] = L::value(w.x & 0xFFFFu);
+            v[1] = L::value(w.x >> 16);
+            v[2] = L::value(w.y & 0xFFFFu);
+            v[3] = L::value(w.y >> 16);
+        } else {
+            const int4 w = *reinterpret_cast<const int4 *>(cms + j);
+            v[0] = w.x;
+            v[1] = w.y;
+            v[2] = w.z;
+            v[3] = w.w;
+        }
+        if (wide && j + 4 <= n) {
+            *reinterpret_cast<int4 *>(out + j) = make_int4(v[0], v[1], v[2], v[3]);
+        } else if (out) {
+#pragma unroll
+            for (int e = 0; e < 4; e++)
+                if (j + e < n) out[j + e] = v[e];
+        }
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            if (j + e >= n || (end_t >= 0 && j + e >= lo && j + e <= hi)) continue;
+            if (v[e] > bv) { bv = v[e]; bj = j + e; }
+        }
     }
 #pragma unroll
     for (int d = 1; d < P; d <<= 1) {
@@ -844,12 +877,18 @@ __device__ __forceinline__ void finish_forward(const BatchView &b, const Scoring
     }
 }
 
-// Per-slot scratch of a fill launch: one stride for every variant, so slots
-// never overlap when 16-bit and 32-bit tasks run in the same launch.
+// Per-slot scratch of a fill launch: the column maxima (and, when the class
+// has pairs of several strips, the two boundary rows) of one pair in flight,
+// as wide as the launch's lanes.
+template <class L>
+__host__ __device__ size_t slot_cm_bytes(int ncap) { return (size_t)ncap * sizeof(typename L::cm_t); }
+template <class L>
+__host__ __device__ size_t slot_bnd_bytes(int ncap) { return 2 * (size_t)ncap * sizeof(typename L::bnd_t); }
+
+template <class L>
 __device__ __forceinline__ void slot_scratch(const FillScratch &scr, int slot, Job *job) {
-    const size_t ncap = (size_t)scr.ncap;
-    job->cms = (char *)scr.colmax + slot * ncap * sizeof(int32_t);
-    job->bnd = (char *)scr.boundary + slot * 2 * ncap * sizeof(int2);
+    job->cms = (char *)scr.base + slot * slot_cm_bytes<L>(scr.ncap);
+    job->bnd = (char *)scr.base + scr.bnd_off + slot * slot_bnd_bytes<L>(scr.ncap);
 }
 
 template <int P, int R, class L, bool DNA>
@@ -874,7 +913,7 @@ __device__ void run_task(const FillLaunch &fl, int first, int last, uint32_t *ws
         return;
     }
     Job job;
-    slot_scratch(fl.scr, slot_base + g, &job);
+    slot_scratch<L>(fl.scr, slot_base + g, &job);
     if (fl.mode == kFillReverse) {
         reverse_job(b, sc, pair, &job);
         job.stop_u = L::lane1(rp->score1);
@@ -917,7 +956,7 @@ GSW_FILL_VARIANTS(GSW_VARC)
 // to 14 row words run best capped at 128 registers (4 blocks of 4 warps);
 // the 16-word one keeps its own choice (about 160 registers, 3 blocks).
 __host__ __device__ constexpr int fill_min_blocks(int v) {
-    return v >= kVarP8First && v < kNumVariants - 1 ? 4 : 0;
+    return (is_p8(v) && v != kVarP4First - 1) || (is_p4(v) && v != kVarTallFirst - 1) ? 4 : 0;
 }
 template <bool DNA, int VID, bool HALF>
 __global__ void __launch_bounds__(kBlock, fill_min_blocks(VID)) k_fill(FillLaunch fl, int warp_words) {
@@ -1048,7 +1087,7 @@ __device__ bool long_open(const FillLaunch &fl, int cls, LongSlot &S, int s, int
     if (t >= ntasks) return false;
     const int pair = fl.plan.order[fl.plan.var_start[cls] + t];
     Job job;
-    slot_scratch(fl.scr, blockIdx.x * kLongSlots + s, &job);
+    slot_scratch<L>(fl.scr, blockIdx.x * kLongSlots + s, &job);
     S.band = 0;
     S.G = S.Gn = 0;
     if (fl.mode == kFillReverse) {
@@ -1269,94 +1308,101 @@ size_t long_smem_bytes(int A) {
     return (size_t)prof_words(C::R, C::L::FOLD, DNA, A) * 32 * sizeof(uint32_t) * C::NW;
 }
 
-template <bool DNA, bool S32>
-int long_occupancy(int A) {
-    using C = LongCfg<DNA, S32>;
-    const size_t sm = long_smem_bytes<DNA, S32>(A);
-    cudaFuncSetAttribute(k_fill_long<DNA, S32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    int nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_fill_long<DNA, S32>, C::NW * 32, sm);
-    return nb;
-}
-
-template <bool DNA, bool S32>
-cudaError_t launch_long(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st) {
-    using C = LongCfg<DNA, S32>;
-    if (!((fl.class_mask >> C::CLS) & 1u)) return cudaSuccess;  // no pair of the class
-    const size_t sm = long_smem_bytes<DNA, S32>(fl.sc.A);
-    const int nb = long_occupancy<DNA, S32>(fl.sc.A);
-    if (nb < 1) return cudaErrorInvalidConfiguration;
-    int grid = sms * nb;
-    grid = std::min(grid, max_blocks);
-    grid = std::min(grid, fl.scr.nslots / kLongSlots);
-    if (grid < 1) return cudaErrorInvalidConfiguration;
-    k_fill_long<DNA, S32><<<grid, C::NW * 32, sm, st>>>(fl, (int)(sm / sizeof(uint32_t) / C::NW));
-    return cudaGetLastError();
-}
-
 template <bool DNA, int VID>
 size_t smem_bytes(int A) {
     using V = VarC<VID>;
     return (size_t)prof_words(V::R, V::Lanes::FOLD, DNA, A) * 32 * sizeof(uint32_t) * (kBlock / 32);
 }
 
-template <bool DNA, int VID, bool HALF>
-int occupancy(int A) {
-    const size_t sm = smem_bytes<DNA, VID>(A);
-    cudaFuncSetAttribute(k_fill<DNA, VID, HALF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    int nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_fill<DNA, VID, HALF>, kBlock, sm);
-    return nb;
+// Resident blocks per SM of a kernel with `smem` bytes of dynamic shared
+// memory, asked of the driver once per device and alphabet size (the limit is
+// raised to the largest alphabet's need, so any later launch fits it).
+struct OccupancyCache {
+    std::atomic<int> blocks[16][kMaxAlpha + 1] = {};  // 0: not asked yet, else blocks + 1
+    template <class K>
+    int get(K kernel, int threads, int A, size_t smem, size_t most) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+        std::atomic<int> *slot = dev < 16 ? &blocks[dev][A] : nullptr;
+        if (slot && slot->load(std::memory_order_acquire) > 0) return slot->load(std::memory_order_acquire) - 1;
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+        int nb = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, smem) != cudaSuccess) return 0;
+        if (slot) slot->store(nb + 1, std::memory_order_release);
+        return nb;
+    }
+};
+
+template <bool DNA, bool S32>
+ClassGeom long_geom(const FillLaunch &fl, int sms) {
+    using C = LongCfg<DNA, S32>;
+    static OccupancyCache cache;
+    ClassGeom g;
+    g.smem = long_smem_bytes<DNA, S32>(fl.sc.A);
+    g.grid = sms * cache.get(k_fill_long<DNA, S32>, C::NW * 32, fl.sc.A, g.smem,
+                             long_smem_bytes<DNA, S32>(DNA ? 4 : kMaxAlpha));
+    g.slots_per_block = kLongSlots;
+    g.cm = slot_cm_bytes<typename C::L>(fl.scr.ncap);
+    g.bnd = slot_bnd_bytes<typename C::L>(fl.scr.ncap);
+    return g;
 }
 
-template <bool DNA, int VID, bool HALF>
-cudaError_t launch_one(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st) {
-    const size_t sm = smem_bytes<DNA, VID>(fl.sc.A);
-    int nb = occupancy<DNA, VID, HALF>(fl.sc.A);
-    if (nb < 1) return cudaErrorInvalidConfiguration;
-    int grid = sms * nb;
-    if (grid > max_blocks) grid = max_blocks;
-    // every pair in flight has a slot: never more warps than the slots hold
-    grid = std::min(grid, fl.scr.nslots / ((kBlock / 32) * (32 / VarC<VID>::P)));
-    if (grid < 1) return cudaErrorInvalidConfiguration;
-    k_fill<DNA, VID, HALF><<<grid, kBlock, sm, st>>>(fl, (int)(sm / sizeof(uint32_t) / (kBlock / 32)));
+template <bool DNA, bool S32>
+cudaError_t launch_long(const FillLaunch &fl, const ClassGeom &g, cudaStream_t st) {
+    using C = LongCfg<DNA, S32>;
+    k_fill_long<DNA, S32><<<g.grid, C::NW * 32, g.smem, st>>>(fl, (int)(g.smem / sizeof(uint32_t) / C::NW));
     return cudaGetLastError();
 }
 
-template <bool DNA, int VID>
-cudaError_t launch_class(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st) {
-    if (!((fl.class_mask >> VID) & 1u)) return cudaSuccess;  // no pair of the class
-    if constexpr (VarC<VID>::Lanes::FOLD)
-        if ((fl.half_mask >> VID) & 1u) return launch_one<DNA, VID, true>(fl, sms, max_blocks, st);
-    return launch_one<DNA, VID, false>(fl, sms, max_blocks, st);
+template <bool DNA, int VID, bool HALF>
+ClassGeom class_geom(const FillLaunch &fl, int sms) {
+    using L = typename VarC<VID>::Lanes;
+    static OccupancyCache cache;
+    ClassGeom g;
+    g.smem = smem_bytes<DNA, VID>(fl.sc.A);
+    g.grid = sms * cache.get(k_fill<DNA, VID, HALF>, kBlock, fl.sc.A, g.smem, smem_bytes<DNA, VID>(DNA ? 4 : kMaxAlpha));
+    g.slots_per_block = (kBlock / 32) * (32 / VarC<VID>::P);
+    g.cm = slot_cm_bytes<L>(fl.scr.ncap);
+    g.bnd = ((fl.multi_mask >> VID) & 1u) ? slot_bnd_bytes<L>(fl.scr.ncap) : 0;
+    return g;
 }
 
-template <bool DNA>
-cudaError_t launch_all(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st) {
-    // heaviest classes first: the CTA kernel for queries of many strips, then
-    // the per-group variants by rows per strip
-    cudaError_t e = launch_long<DNA, true>(fl, sms, max_blocks, st);
-    if (e == cudaSuccess) e = launch_long<DNA, false>(fl, sms, max_blocks, st);
+template <bool DNA, int VID, bool HALF>
+cudaError_t launch_one(const FillLaunch &fl, const ClassGeom &g, cudaStream_t st) {
+    k_fill<DNA, VID, HALF><<<g.grid, kBlock, g.smem, st>>>(fl, (int)(g.smem / sizeof(uint32_t) / (kBlock / 32)));
+    return cudaGetLastError();
+}
+
+// Which kernels a translation unit holds: the 4-lane variants only for 4-letter
+// alphabets and only with the half-precision clamp (the host picks them for
+// such batches alone), the 32-bit variant and the CTA kernels only without.
+template <bool DNA, bool HALF, int VID>
+constexpr bool kHeld = is_p4(VID) ? DNA && HALF : (!HALF || VarC<VID>::Lanes::FOLD);
+
+template <bool DNA, bool HALF>
+ClassGeom tu_geom(int c, const FillLaunch &fl, int sms) {
+    if constexpr (!HALF) {
+        if (c == kClassLong32) return long_geom<DNA, true>(fl, sms);
+        if (c == kClassLong16) return long_geom<DNA, false>(fl, sms);
+    }
+#define GSW_GEOM(id, P_, R_, S_) \
+    if constexpr (kHeld<DNA, HALF, id>) if (c == id) return class_geom<DNA, id, HALF>(fl, sms);
+    GSW_FILL_VARIANTS(GSW_GEOM)
+#undef GSW_GEOM
+    return ClassGeom{};
+}
+
+template <bool DNA, bool HALF>
+cudaError_t tu_launch(int c, const FillLaunch &fl, const ClassGeom &g, cudaStream_t st) {
+    if constexpr (!HALF) {
+        if (c == kClassLong32) return launch_long<DNA, true>(fl, g, st);
+        if (c == kClassLong16) return launch_long<DNA, false>(fl, g, st);
+    }
 #define GSW_LAUNCH(id, P_, R_, S_) \
-    if (e == cudaSuccess) e = launch_class<DNA, kNumVariants - 1 - id>(fl, sms, max_blocks, st);
+    if constexpr (kHeld<DNA, HALF, id>) if (c == id) return launch_one<DNA, id, HALF>(fl, g, st);
     GSW_FILL_VARIANTS(GSW_LAUNCH)
 #undef GSW_LAUNCH
-    return e;
-}
-
-template <bool DNA>
-int max_slots(int A, int sms) {
-    int best = 0;
-#define GSW_SLOTS(id, P_, R_, S_)                                                   \
-    {                                                                             \
-        int nb = occupancy<DNA, id, false>(A);                                    \
-        if constexpr (VarC<id>::Lanes::FOLD) nb = std::max(nb, occupancy<DNA, id, true>(A)); \
-        const int slots = sms * nb * (kBlock / 32) * (32 / VarC<id>::P);          \
-        best = slots > best ? slots : best;                                       \
-    }
-    GSW_FILL_VARIANTS(GSW_SLOTS)
-#undef GSW_SLOTS
-    return best;
+    return cudaErrorInvalidConfiguration;
 }
 
 }  // namespace

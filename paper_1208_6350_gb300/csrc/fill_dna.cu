@@ -4,10 +4,10 @@
 
 namespace gsw {
 
-cudaError_t launch_fill_dna(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st) {
-    return launch_all<true>(fl, sms, max_blocks, st);
-}
+ClassGeom fill_geom_dna(int c, const FillLaunch &fl, int sms) { return tu_geom<true, false>(c, fl, sms); }
 
-int fill_slots_dna(int A, int sms) { return max_slots<true>(A, sms); }
+cudaError_t fill_launch_dna(int c, const FillLaunch &fl, const ClassGeom &g, cudaStream_t st) {
+    return tu_launch<true, false>(c, fl, g, st);
+}
 
 }  // namespace gsw

@@ -4,10 +4,10 @@
 
 namespace gsw {
 
-cudaError_t launch_fill_general(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st) {
-    return launch_all<false>(fl, sms, max_blocks, st);
-}
+ClassGeom fill_geom_general(int c, const FillLaunch &fl, int sms) { return tu_geom<false, false>(c, fl, sms); }
 
-int fill_slots_general(int A, int sms) { return max_slots<false>(A, sms); }
+cudaError_t fill_launch_general(int c, const FillLaunch &fl, const ClassGeom &g, cudaStream_t st) {
+    return tu_launch<false, false>(c, fl, g, st);
+}
 
 }  // namespace gsw

@@ -33,7 +33,11 @@ struct Scoring {
     int32_t dna4;   // 1 when A == 4: the fill uses the letter-pair profile
     int32_t one;    // 1, unknown to the compiler: x * one + y issues as an integer multiply-add on the FMA pipe
     int8_t W[kMaxAlpha * kMaxAlpha];  // W[a * A + b]: query letter a vs target letter b
-    int8_t fill_class[GSW_TUNE_BUCKETS];  // tuned 16-bit fill class per query-row bucket, -1: default rule
+    // 16-bit fill class per query-row bucket: the tuned one, or the one
+    // default_classes chose for the batch (-1: the smallest one-strip variant)
+    int8_t fill_class[GSW_TUNE_BUCKETS];
+    int8_t rev_class[GSW_TUNE_BUCKETS];  // of the reversed fill, + 1 (0: as the forward fill)
+    int32_t cta_steps;  // a pair whose strips one after the other take more steps runs on a CTA (0: off)
 };
 
 // Batch view (device pointers) shared by every stage.
@@ -80,11 +84,20 @@ enum FillMode : int32_t {
     X(9, 8, 10, 0)           \
     X(10, 8, 12, 0)          \
     X(11, 8, 14, 0)          \
-    X(12, 8, 16, 0)
+    X(12, 8, 16, 0)          \
+    X(13, 4, 6, 0)           \
+    X(14, 4, 8, 0)           \
+    X(15, 4, 10, 0)          \
+    X(16, 4, 12, 0)          \
+    X(17, 4, 14, 0)          \
+    X(18, 4, 16, 0)          \
+    X(19, 16, 10, 0)         \
+    X(20, 16, 12, 0)         \
+    X(21, 16, 16, 0)
 struct Variant {
     int P, R, s32;
 };
-constexpr int kNumVariants = 13;
+constexpr int kNumVariants = 22;
 constexpr int kVarS32 = 7;
 constexpr int kVarMaxS16 = 6;  // the default rule picks among 0..6
 // 8..12: one pair per 8 lanes with 8..16 row words per lane (128..256 rows per
@@ -92,6 +105,17 @@ constexpr int kVarMaxS16 = 6;  // the default rule picks among 0..6
 // per-step costs (shuffles, letter loads, trackers) weigh half as much; chosen
 // per query length by the autotuner
 constexpr int kVarP8First = 8;
+// 13..18: one pair per 4 lanes with 6..16 row words per lane (48..128 rows per
+// strip): half the wavefront's skew again and strips that fit reads of up to
+// 128 rows closely; 4-letter alphabets only (a general alphabet's profile
+// would leave few warps per SM)
+constexpr int kVarP4First = 13;
+// 19..21: one pair per 16 lanes with 10, 12 or 16 row words per lane (320, 384
+// or 512 rows per strip): queries of 257 to 512 rows in one strip, without the
+// boundary rows and the second pass over the target
+constexpr int kVarTallFirst = 19;
+__host__ __device__ constexpr bool is_p8(int v) { return v >= kVarP8First && v < kVarP4First; }
+__host__ __device__ constexpr bool is_p4(int v) { return v >= kVarP4First && v < kVarTallFirst; }
 // Two more fill classes: pairs whose query spans many strips run on a whole
 // CTA (k_fill_long), one 32-lane warp per strip, strips pipelined across the
 // CTA's warps; 16-bit lanes (2*32*16 = 1,024 rows per strip for DNA, 2*32*8 =
@@ -146,30 +170,114 @@ __host__ __device__ inline int pick_class16(int rows, const Scoring &sc) {
 // the forward rule, or the 32-bit classes for a pair in 32-bit lanes; a DNA
 // query of several strips reverses in the CTA kernel.
 __host__ __device__ inline int pick_class_reverse(int rows, bool s32, const Scoring &sc) {
-    int v = s32 ? (long_pair(rows, true, sc.dna4) ? kClassLong32 : kVarS32) : pick_class16(rows, sc);
+    const int b = (rows - 1) / GSW_TUNE_ROWS;
+    int v;
+    if (s32) v = long_pair(rows, true, sc.dna4) ? kClassLong32 : kVarS32;
+    else if (rows >= 1 && b < GSW_TUNE_BUCKETS && sc.rev_class[b] > 0) v = sc.rev_class[b] - 1;
+    else v = pick_class16(rows, sc);
     if (sc.dna4 && v != kClassLong16 && v != kClassLong32 && rows > variant_rows(v))
         v = v == kVarS32 ? kClassLong32 : kClassLong16;
     return v;
 }
 
-// The fill classes a launch of `mode` can meet when no query has more than
-// maxm rows (a superset; each fill launch leaves the other classes out).
+// A pair of at most rows x cols letters cannot leave the lanes whose clamp is
+// a half-precision multiply-add (fill.cuh, LH): a local score is at most
+// min(rows, cols) x the largest matrix entry, and every lane value at most the
+// score + O + one matrix entry, which must stay within the integers half
+// precision holds exactly (2048); O >= -wmin keeps the sums of the shifted
+// scores non-negative (signed bytes outside the 4-letter alphabets).
+inline bool half_fits(int rows, int cols, const Scoring &sc) {
+    if (sc.O < -sc.wmin || (!sc.dna4 && sc.wmax + sc.O > 127)) return false;
+    const long long top = sc.wmax > 0 ? sc.wmax : 0;
+    return (rows < cols ? rows : cols) * top + top + sc.O <= 2047;
+}
+
+// Whether a pair that class v would run strip after strip goes to the CTA
+// class instead (sc.cta_steps, default_classes).
+__host__ __device__ inline bool cta_pair(int v, int rows, int cols, const Scoring &sc) {
+    if (sc.cta_steps <= 0 || v >= kNumVariants || v == kVarS32) return false;
+    const int strips = (rows + variant_rows(v) - 1) / variant_rows(v);
+    return strips > 1 && (long long)strips * cols > sc.cta_steps;
+}
+
+// Chooses the fill classes of a batch's untuned buckets from its size (pairs,
+// longest target, forward cells).
+//
+// A class costs its strips x the time of a strip's step.  The table holds that
+// time (ps per pair and column on a whole GB300, measured with the chip full:
+// 6 G cells of equal pairs, targets of 650 letters, 360 for 20-letter
+// alphabets); strips of a query that needs several cost kMulti times as much
+// (boundary rows in and out).  Narrower groups pay less skew and fewer per-step
+// instructions per pair but need more pairs to fill the chip: 8 lanes from
+// 8,192 pairs (100 rows, 1,000 columns: 883 GCUPS against 1,155 at 3,000 pairs,
+// 2,503 against 2,307 at 10,000), 4 lanes from 16,384 (1,888 against 2,503 at
+// 10,000 pairs, 3,907 against 3,193 at 92,000).  A pair of several strips that
+// alone would take more than about a quarter of the batch's time (its steps x 0.3 us
+// against the cells at 2.5 T cells/s; 0.46 us and 1.5 T for general alphabets)
+// runs its strips side by side on a CTA (600 x 1,000 DNA: 1,851 GCUPS against
+// 1,513 at 3,000 pairs, 1,961 against 2,321 at 10,000; 350 x 360 protein: 691
+// against 330 at 1,000 pairs, 1,352 against 1,468 at 10,000).
+inline void default_classes(Scoring &sc, int npairs, int maxn, double cells) {
+    constexpr int kWide = 8192, kNarrow = 16384;
+    // (a power of two: batches of like size keep their captured graphs)
+    sc.cta_steps = 256;
+    while (sc.cta_steps < cells * 3.5e-7 && sc.cta_steps < (1 << 28)) sc.cta_steps *= 2;
+    static constexpr float dna[kNumVariants] = {28.3f, 33.4f, 39.2f, 45.8f, 50.1f, 59.6f, 61.2f, 0,
+                                                32.1f, 36.3f, 42.6f, 52.3f, 55.8f, 13.8f, 16.8f, 19.5f,
+                                                21.4f, 24.8f, 29.5f, 72.6f, 85.0f, 112.0f};
+    static constexpr float gen[kNumVariants] = {32.0f, 41.5f, 47.4f, 57.7f, 65.0f, 84.2f, 94.9f, 0,
+                                                39.7f, 48.0f, 59.5f, 73.7f, 97.1f, 0,     0,     0,
+                                                0,     0,     0,     110.0f, 136.0f, 203.0f};
+    for (int b = 0; b < GSW_TUNE_BUCKETS; b++) {
+        if (sc.fill_class[b] >= 0) continue;
+        const int rows = (b + 1) * GSW_TUNE_ROWS;
+        if (long_pair(rows, false, sc.dna4)) continue;
+        const float multi = sc.dna4 ? 1.3f : 1.08f;
+        float best = 0, best16 = 0;
+        int pick = -1, pick16 = -1;
+        for (int v = 0; v < kNumVariants; v++) {
+            const bool p8 = is_p8(v), p4 = is_p4(v);
+            if (v == kVarS32) continue;
+            if (p8 && (npairs < kWide || rows > variant_rows(v))) continue;
+            if (p4 && (npairs < kNarrow || rows > variant_rows(v) || !sc.dna4 || !half_fits(rows, maxn, sc))) continue;
+            const int strips = (rows + variant_rows(v) - 1) / variant_rows(v);
+            const float cost = strips * (sc.dna4 ? dna[v] : gen[v]) * (strips > 1 ? multi : 1.0f);
+            if (pick < 0 || cost < best) {
+                best = cost;
+                pick = v;
+            }
+            if (!p8 && !p4 && (pick16 < 0 || cost < best16)) {
+                best16 = cost;
+                pick16 = v;
+            }
+        }
+        // (codes of the table, pick_class16)
+        sc.fill_class[b] = (int8_t)(pick >= kVarP8First ? 9 + (pick - kVarP8First) : pick);
+        sc.rev_class[b] = (int8_t)(pick16 + 1);
+    }
+}
+
+// The fill classes a launch of `mode` can meet when every query has minm to
+// maxm rows (a superset; each fill launch leaves the other classes out; the
+// reversed fill's queries end anywhere, so have 1 to maxm).
 // force_s32: the batch runs in 32-bit lanes; s32: some pair may have been
 // refilled in 32-bit lanes.  Empty pairs of the forward fill take class 0.
-inline uint32_t fill_class_mask(int mode, int maxm, const Scoring &sc, bool force_s32, bool s32) {
+inline uint32_t fill_class_mask(int mode, int maxm, const Scoring &sc, bool force_s32, bool s32,
+                                int minm = 0) {
     uint32_t m = 0;
     const int upto = maxm < GSW_TUNE_BUCKETS * GSW_TUNE_ROWS ? maxm : GSW_TUNE_BUCKETS * GSW_TUNE_ROWS;
     if (mode == kFillForward && force_s32) return (1u << kVarS32) | (1u << kClassLong32);
     if (mode == kFillRerun) return (1u << kVarS32) | (1u << kClassLong32);
-    if (mode == kFillForward) m |= 1u << 0;
+    if (mode == kFillForward && minm <= 0) m |= 1u << 0;
+    bool strips = maxm > upto;  // some class can hold a pair of several strips
     for (int r = 1; r <= upto; r++) {
-        if (mode == kFillForward) {
-            m |= 1u << pick_class16(r, sc);
-        } else {
-            m |= 1u << pick_class_reverse(r, false, sc);
-            if (s32) m |= 1u << pick_class_reverse(r, true, sc);
-        }
+        if (mode == kFillForward && r < minm) continue;
+        const int c = mode == kFillForward ? pick_class16(r, sc) : pick_class_reverse(r, false, sc);
+        m |= 1u << c;
+        strips |= r > variant_rows(c);
+        if (s32 && mode != kFillForward) m |= 1u << pick_class_reverse(r, true, sc);
     }
+    if (sc.cta_steps > 0 && strips) m |= 1u << kClassLong16;
     if (maxm > upto) {  // past the tuned buckets: the tallest variant or the CTA classes
         m |= (1u << kVarMaxS16) | (1u << kClassLong16);
         if (s32 && mode != kFillForward) m |= (1u << kVarS32) | (1u << kClassLong32);
@@ -177,24 +285,35 @@ inline uint32_t fill_class_mask(int mode, int maxm, const Scoring &sc, bool forc
     return m;
 }
 
-// The classes of a launch (`mask`, from fill_class_mask) whose pairs cannot
-// leave the lanes whose clamp is a half-precision multiply-add (fill.cuh, LH):
-// a local score is at most min(rows, columns) x the largest matrix entry, and
-// every lane value at most the score + O + one matrix entry, which must stay
-// within the integers half precision holds exactly (2048); and O >= -wmin
-// keeps the sums of the shifted scores non-negative.
-inline uint32_t fill_half_mask(int mode, int maxm, int maxn, const Scoring &sc, uint32_t mask) {
-    if (sc.O < -sc.wmin) return 0;
-    const long long top = sc.wmax > 0 ? sc.wmax : 0;
-    auto fits = [&](int rows) { return (rows < maxn ? rows : maxn) * top + top + sc.O <= 2047; };
+// Most rows a class of a launch can hold when no query has more than maxm.
+struct ClassRows {
     int most[kNumFillClasses] = {};
+};
+inline ClassRows fill_class_rows(int mode, int maxm, const Scoring &sc, uint32_t mask) {
+    ClassRows r;
     const int upto = maxm < GSW_TUNE_BUCKETS * GSW_TUNE_ROWS ? maxm : GSW_TUNE_BUCKETS * GSW_TUNE_ROWS;
-    for (int r = 1; r <= upto; r++)
-        most[mode == kFillForward ? pick_class16(r, sc) : pick_class_reverse(r, false, sc)] = r;
-    if (maxm > upto) most[kVarMaxS16] = maxm;
+    for (int x = 1; x <= upto; x++)
+        r.most[mode == kFillForward ? pick_class16(x, sc) : pick_class_reverse(x, false, sc)] = x;
+    if (maxm > upto) r.most[kVarMaxS16] = maxm;
+    for (int c : {kVarS32, kClassLong16, kClassLong32}) r.most[c] = maxm;
+    for (int c = 0; c < kNumFillClasses; c++)
+        if (!((mask >> c) & 1u)) r.most[c] = 0;
+    return r;
+}
+
+// The classes of a launch whose pairs all fit the half-precision clamp lanes.
+inline uint32_t fill_half_mask(const ClassRows &rows, int maxn, const Scoring &sc) {
     uint32_t m = 0;
     for (int c = 0; c < kNumVariants; c++)
-        if (((mask >> c) & 1u) && !variant_at(c).s32 && fits(most[c])) m |= 1u << c;
+        if (!variant_at(c).s32 && half_fits(rows.most[c], maxn, sc)) m |= 1u << c;
+    return m;
+}
+
+// The classes that can hold a pair of several strips (which needs boundary rows).
+inline uint32_t fill_multi_mask(const ClassRows &rows) {
+    uint32_t m = (1u << kClassLong16) | (1u << kClassLong32);
+    for (int c = 0; c < kNumVariants; c++)
+        if (rows.most[c] > variant_rows(c)) m |= 1u << c;
     return m;
 }
 
@@ -210,12 +329,14 @@ struct FillPlan {
     const int32_t *ntasks;     // total tasks
 };
 
-// Per-slot scratch of a persistent fill launch (one slot per pair in flight).
+// Scratch of the fill launches: each launch (they run one after the other)
+// lays out its own slots, one per pair in flight (column maxima, then boundary
+// rows), as wide as its lanes need.
 struct FillScratch {
-    void *colmax;    // slots x ncap elements (uint16 biased for 16-bit, int32 for 32-bit)
-    void *boundary;  // slots x 2 x ncap boundary words (uint32 for 16-bit, int2 for 32-bit)
+    void *base;
+    size_t bytes;
+    size_t bnd_off;  // the launch's boundary rows start here
     int32_t ncap;    // columns per slot (a multiple of 4: 8-byte stores of four 16-bit maxima)
-    int32_t nslots;  // slots allocated
 };
 
 struct FillLaunch {
@@ -224,7 +345,9 @@ struct FillLaunch {
     FillPlan plan;
     FillScratch scr;
     int32_t mode;
+    int32_t maxm;         // longest query
     uint32_t class_mask;  // classes launched (bit c: class c); the others hold no pair
+    uint32_t multi_mask;  // classes that can hold pairs of several strips
     uint32_t half_mask;   // classes whose values stay below 2048: the half-precision clamp lanes
     // nonzero once the batch's letter check found a code >= the alphabet
     // (written by the check, which runs first on the stream): the fill then
@@ -437,20 +560,35 @@ int make_scoring(const int8_t *matrix, int32_t A, int32_t O, int32_t X, Scoring 
 cudaError_t launch_count_flag(const gsw_result *res, int32_t n, int32_t flag, unsigned long long *count,
                               cudaStream_t st);
 
-int fill_block_threads();
-// largest number of slots (pairs in flight) of any variant's launch
-int fill_slots(const Scoring &sc, int sms);
-// Largest number of pairs a warp of a fill variant holds at once (32 / P for
-// the narrowest group): the slots a capped launch needs per warp.
-int fill_max_pairs_per_warp();
-// one persistent launch per class in fl.class_mask, heaviest first; each grid
-// capped at max_blocks and at the slots the scratch holds
-cudaError_t launch_fill(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st);
-// launch_fill and fill_slots of one alphabet kind (fill_dna.cu, fill_general.cu)
-cudaError_t launch_fill_dna(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st);
-cudaError_t launch_fill_general(const FillLaunch &fl, int sms, int max_blocks, cudaStream_t st);
-int fill_slots_dna(int A, int sms);
-int fill_slots_general(int A, int sms);
+// Geometry of one class's launch: blocks resident on the SMs asked for, pairs
+// in flight and scratch per block.
+struct ClassGeom {
+    int grid = 0, slots_per_block = 0;
+    size_t cm = 0, bnd = 0;  // bytes per slot
+    size_t smem = 0;
+    size_t bytes(int blocks) const {
+        return (((size_t)blocks * slots_per_block * cm + 255) & ~(size_t)255) + (size_t)blocks * slots_per_block * bnd;
+    }
+};
+// scratch bytes with which every class of fl.class_mask runs at full occupancy
+size_t fill_scratch_want(const FillLaunch &fl, int sms);
+struct SideStreams {
+    cudaStream_t s[2];
+    cudaEvent_t fork, join[2];
+};
+// one persistent launch per class in fl.class_mask, heaviest first, each with
+// the slots its share of the scratch holds; side by side on `st` and the side
+// streams (forked and joined by events) when the scratch holds all of them
+cudaError_t launch_fill(const FillLaunch &fl, int sms, cudaStream_t st, const SideStreams &aux);
+// Geometry and launch of one class, by kind of alphabet and lanes (one
+// translation unit each, compiled in parallel: fill_dna.cu, fill_dna_half.cu,
+// fill_general.cu, fill_general_half.cu)
+#define GSW_FILL_UNITS(X) X(dna, true, false) X(dna_half, true, true) X(general, false, false) X(general_half, false, true)
+#define GSW_DECLARE_UNIT(name, DNA, HALF)                                          \
+    ClassGeom fill_geom_##name(int c, const FillLaunch &fl, int sms);              \
+    cudaError_t fill_launch_##name(int c, const FillLaunch &fl, const ClassGeom &g, cudaStream_t st);
+GSW_FILL_UNITS(GSW_DECLARE_UNIT)
+#undef GSW_DECLARE_UNIT
 
 struct PlanBuffers {
     int32_t *keys;       // [npairs]
@@ -542,18 +680,15 @@ struct BandGrids {
     size_t total_bytes;
 };
 BandGrids band_grids(int rows_cap, int sms, size_t budget_bytes);
-struct BandStreams {
-    cudaStream_t s[2];
-    cudaEvent_t fork, join[2];
-};
 cudaError_t launch_band(const BatchView &b, const Scoring &sc, const PlanBuffers &pb, void *scratch,
-                        const BandGrids &g, cudaStream_t st, const BandStreams &aux);
+                        const BandGrids &g, cudaStream_t st, const SideStreams &aux);
 
 // small helpers (misc.cu)
 // one pass over the pairs: [0, 1] largest lengths, [2, 3] arena extents,
-// [4] nonzero if a length is outside [0, 2^24) or an offset negative
+// [4] nonzero if a length is outside [0, 2^24) or an offset negative,
+// [5] smallest query length (0 if any query or target is empty), [6] cells
 cudaError_t launch_batch_stats(const int64_t *q_off, const int32_t *q_len, const int64_t *t_off,
-                               const int32_t *t_len, int32_t n, unsigned long long *out5, cudaStream_t st);
+                               const int32_t *t_len, int32_t n, unsigned long long *out7, cudaStream_t st);
 // 2-bit packed DNA letters to one byte per letter
 cudaError_t launch_unpack2(const uint8_t *in, uint8_t *out, long long nletters, cudaStream_t st);
 cudaError_t launch_validate(const BatchView &b, const Scoring &sc, int32_t *bad, cudaStream_t st);

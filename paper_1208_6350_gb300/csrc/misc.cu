@@ -30,16 +30,21 @@ __global__ void k_validate(BatchView b, int32_t A, int32_t *bad) {
 // Checks and sizes of a batch in one pass: [0] largest query length, [1]
 // largest target length, [2] query arena extent, [3] target arena extent
 // (offset + length, letters), [4] nonzero if a length is outside [0, 2^24)
-// or an offset is negative.
+// or an offset is negative, [5] smallest query length (0 if a query or a
+// target is empty), [6] cells (sum of the products of the lengths).
 __global__ void k_batch_stats(const int64_t *q_off, const int32_t *q_len, const int64_t *t_off,
-                              const int32_t *t_len, int32_t n, unsigned long long *out5) {
+                              const int32_t *t_len, int32_t n, unsigned long long *out7) {
     unsigned long long mq = 0, mt = 0, eq = 0, et = 0, bad = 0;
+    unsigned least = 0xFFFFFFFFu;
+    unsigned long long cells = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int32_t ql = q_len[i], tl = t_len[i];
         const int64_t qo = q_off[i], to = t_off[i];
         bad |= ((uint32_t)ql >= (1u << 24)) | ((uint32_t)tl >= (1u << 24)) | (qo < 0) | (to < 0);
         mq = max(mq, (unsigned long long)(uint32_t)ql);
         mt = max(mt, (unsigned long long)(uint32_t)tl);
+        cells += (unsigned long long)(uint32_t)ql * (uint32_t)tl;
+        least = min(least, tl == 0 ? 0u : (unsigned)ql);
         eq = max(eq, (unsigned long long)(qo + ql));
         et = max(et, (unsigned long long)(to + tl));
     }
@@ -49,14 +54,18 @@ __global__ void k_batch_stats(const int64_t *q_off, const int32_t *q_len, const 
     for (int d = 16; d > 0; d >>= 1) {
         eq = max(eq, __shfl_xor_sync(0xFFFFFFFFu, eq, d));
         et = max(et, __shfl_xor_sync(0xFFFFFFFFu, et, d));
+        cells += __shfl_xor_sync(0xFFFFFFFFu, cells, d);
     }
     bad = __reduce_or_sync(0xFFFFFFFFu, (unsigned)bad);
+    least = __reduce_min_sync(0xFFFFFFFFu, least);
     if ((threadIdx.x & 31) == 0) {
-        atomicMax(&out5[0], mq);
-        atomicMax(&out5[1], mt);
-        atomicMax(&out5[2], eq);
-        atomicMax(&out5[3], et);
-        if (bad) atomicOr(&out5[4], 1ull);
+        atomicMax(&out7[0], mq);
+        atomicMax(&out7[1], mt);
+        atomicMax(&out7[2], eq);
+        atomicMax(&out7[3], et);
+        if (bad) atomicOr(&out7[4], 1ull);
+        atomicMin(&out7[5], (unsigned long long)least);
+        atomicAdd(&out7[6], cells);
     }
 }
 
@@ -114,12 +123,14 @@ cudaError_t launch_validate(const BatchView &b, const Scoring &sc, int32_t *bad,
 }
 
 cudaError_t launch_batch_stats(const int64_t *q_off, const int32_t *q_len, const int64_t *t_off,
-                               const int32_t *t_len, int32_t n, unsigned long long *out5, cudaStream_t st) {
-    cudaMemsetAsync(out5, 0, 5 * sizeof(unsigned long long), st);
+                               const int32_t *t_len, int32_t n, unsigned long long *out7, cudaStream_t st) {
+    cudaMemsetAsync(out7, 0, 5 * sizeof(unsigned long long), st);
+    cudaMemsetAsync(out7 + 5, 0xFF, sizeof(unsigned long long), st);
+    cudaMemsetAsync(out7 + 6, 0, sizeof(unsigned long long), st);
     if (n > 0) {
         int blocks = (n + 255) / 256;
         blocks = blocks > 1024 ? 1024 : blocks;
-        k_batch_stats<<<blocks, 256, 0, st>>>(q_off, q_len, t_off, t_len, n, out5);
+        k_batch_stats<<<blocks, 256, 0, st>>>(q_off, q_len, t_off, t_len, n, out7);
     }
     return cudaGetLastError();
 }

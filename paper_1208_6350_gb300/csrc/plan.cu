@@ -32,6 +32,7 @@ __global__ void k_plan_keys(BatchView b, Scoring sc, int32_t mode, int32_t *keys
         cols = b.t_len[p];
         if (b.flags & GSW_FORCE_S32) v = (cols > 0 && long_pair(rows, true, sc.dna4)) ? kClassLong32 : kVarS32;
         else v = (cols > 0 && rows > 0) ? pick_class16(rows, sc) : 0;  // (any class writes an empty pair's record)
+        if (cta_pair(v, rows, cols, sc)) v = kClassLong16;
     } else if (mode == kFillRerun) {
         if (!(b.res[p].flags & kResPendingS32)) { keys[p] = -1; return; }
         rows = b.q_len[p];
@@ -56,6 +57,7 @@ __global__ void k_plan_keys(BatchView b, Scoring sc, int32_t mode, int32_t *keys
         // before the last one starts (4-letter DNA: a general alphabet's CTA
         // holds 4 warps per SM)
         v = pick_class_reverse(rows, (r.flags & GSW_RES_S32) != 0, sc);
+        if (cta_pair(v, rows, cols, sc)) v = kClassLong16;
     } else if (mode == kPlanTrace) {
         const gsw_result r = b.res[p];
         if (r.score1 <= 0 || !(r.flags & kResPendingTrace) || (r.flags & kResInternal) || r.read_begin1 < 0) {

@@ -1,5 +1,9 @@
 // Autotuner of the fill class per query length (gsw_autotune, include/gsw.h).
 //
+// The default rule (default_classes, gsw_impl.cuh) is measured beside the
+// classes a table can name: it also knows narrower and taller groups, and where
+// it is the fastest the bucket is left to it.
+//
 // The classes trade differently against each other with the query length: a
 // 16-lane group with fewer row words per lane wastes no rows on a short query
 // but spends more of each step on the wavefront's fixed costs (shuffles,
@@ -56,7 +60,8 @@ extern "C" int gsw_autotune(gsw_ctx *ctx, const int8_t *matrix, int32_t alphabet
     if (!ctx || !matrix || alphabet < 1 || alphabet > kMaxAlpha || target_len < 1 || target_len > (1 << 20))
         return GSW_EINVAL;
     if (cudaSetDevice(context_device(ctx)) != cudaSuccess) return GSW_ECUDA;
-    gsw_tune tune;
+    gsw_tune tune, use;  // the fastest named classes; the same, with the buckets left to the default rule
+    std::memset(use.fill_class, -1, sizeof(use.fill_class));
     std::memset(tune.fill_class, -1, sizeof(tune.fill_class));
     std::memset(tune.gcups, 0, sizeof(tune.gcups));
     std::memset(tune.gcups_default, 0, sizeof(tune.gcups_default));
@@ -104,13 +109,13 @@ extern "C" int gsw_autotune(gsw_ctx *ctx, const int8_t *matrix, int32_t alphabet
         if (rows <= variant_rows(kVarMaxS16)) {
             cand = {def, std::min(def + 1, (int)kVarMaxS16), kVarMaxS16, 8};
             // 8-lane variants: the smallest holding the query in one strip, and the next
-            for (int i = 0, got = 0; i <= kNumVariants - 1 - kVarP8First && got < 2; i++)
+            for (int i = 0, got = 0; i <= kVarP4First - 1 - kVarP8First && got < 2; i++)
                 if (variant_rows(kVarP8First + i) >= rows) {
                     cand.push_back(9 + i);
                     got++;
                 }
         } else {
-            cand = {4, 5, kVarMaxS16, 8, 9 + (kNumVariants - 1 - kVarP8First)};  // several strips, or the CTA kernel
+            cand = {4, 5, kVarMaxS16, 8, 9 + (kVarP4First - 1 - kVarP8First)};  // several strips, or the CTA kernel
             cand.push_back(def);
         }
         std::sort(cand.begin(), cand.end());
@@ -118,6 +123,7 @@ extern "C" int gsw_autotune(gsw_ctx *ctx, const int8_t *matrix, int32_t alphabet
         const double cells = (double)np * rows * target_len;
         float best_rate = -1.f, def_rate = 0.f;
         int best = def;
+        cand.push_back(-1);  // the default rule
         for (int c : cand) {
             gsw_tune one;
             std::memset(one.fill_class, -1, sizeof(one.fill_class));
@@ -138,14 +144,15 @@ extern "C" int gsw_autotune(gsw_ctx *ctx, const int8_t *matrix, int32_t alphabet
             }
             if (rc != GSW_OK) break;
             const float rate = (float)(cells / (ms_best * 1e-3) / 1e9);
-            if (c == def) def_rate = rate;
-            if (rate > best_rate) {
+            if (c < 0) def_rate = rate;
+            else if (rate > best_rate) {
                 best_rate = rate;
                 best = c;
             }
         }
         tune.fill_class[b] = (int8_t)best;
-        tune.gcups[b] = best_rate;
+        use.fill_class[b] = (int8_t)(def_rate >= best_rate ? -1 : best);
+        tune.gcups[b] = std::max(best_rate, def_rate);
         tune.gcups_default[b] = def_rate;
     }
     d.free_all();
@@ -154,7 +161,7 @@ extern "C" int gsw_autotune(gsw_ctx *ctx, const int8_t *matrix, int32_t alphabet
         gsw_context_set_tune(ctx, nullptr);
         return rc;
     }
-    rc = gsw_context_set_tune(ctx, &tune);
+    rc = gsw_context_set_tune(ctx, &use);
     if (out) *out = tune;
     return rc;
 }

@@ -67,3 +67,35 @@ def test_general_alphabet_lanes(ctx, A, O, X, rows):
     W = np.ascontiguousarray(wl.synthetic_protein_matrix()[:A, :A])
     b = edge_batch(A + rows, rows, rows + 41, W, O, X)
     compare(b, run_oracle(b), run_gpu_host(ctx, b))
+
+
+def _sized(n, rows, cols, seed, A=4):
+    rng = np.random.default_rng(seed)
+    qs = [rng.integers(0, A, int(rng.integers(max(1, rows - 31), rows + 1))).astype(np.uint8) for _ in range(n)]
+    ts = []
+    for q in qs:
+        t = rng.integers(0, A, int(rng.integers(cols // 2, cols + 1))).astype(np.uint8)
+        w = min(len(q), len(t))
+        if rng.random() < 0.7:
+            at = int(rng.integers(0, len(t) - w + 1))
+            t[at:at + w] = q[:w]
+        ts.append(t)
+    W = wl.dna_matrix(2, -3) if A == 4 else np.ascontiguousarray(wl.synthetic_protein_matrix()[:A, :A])
+    return batch(qs, ts, W, 5 if A == 4 else 11, 1, wl.DNA if A == 4 else wl.PROTEIN[:A])
+
+
+# (pairs, longest query, longest target, alphabet): the 4-lane groups from
+# 16,384 pairs, the 8-lane ones from 8,192, the tall 16-lane groups, several
+# strips, and pairs heavy enough for the CTA class
+@pytest.mark.parametrize("n,rows,cols,A", [
+    (16384, 32, 40, 4), (16384, 48, 50, 4), (16400, 80, 90, 4), (16384, 112, 130, 4), (16384, 128, 60, 4),
+    (8192, 129, 70, 4), (8191, 129, 70, 4), (300, 257, 300, 4), (300, 320, 200, 4), (300, 384, 401, 4),
+    (200, 512, 300, 4), (200, 513, 300, 4), (8200, 100, 60, 20), (200, 321, 300, 20), (150, 512, 200, 20),
+    (60, 900, 700, 20), (40, 1500, 900, 4)])
+def test_classes_chosen_by_batch_size(ctx, n, rows, cols, A):
+    b = _sized(n, rows, cols, n + rows, A)
+    got = run_gpu_host(ctx, b)
+    keep = np.random.default_rng(3).permutation(n)[:300]
+    s = b.subset(keep)
+    res, cig, (cm, off) = got
+    compare(s, run_oracle(s), (res[keep], cig, (cm, off[keep])))
