@@ -21,11 +21,14 @@ void each_class(const FillLaunch &fl, int sms, F f) {
     }
 }
 
-// No more blocks than the batch has pairs for (the CTA classes: one pair per
-// block, whose warps share its strips).
+// No more blocks than the batch has pairs for (the CTA classes: a cluster per
+// pair, whose warps share its strips).
 void fit_pairs(const FillLaunch &fl, int c, ClassGeom &g) {
-    const int per = c >= kNumVariants ? 1 : std::max(1, g.slots_per_block);
-    g.grid = std::min(g.grid, std::max(1, (fl.b.npairs + per - 1) / per));
+    const long long blocks = c >= kNumVariants ? (long long)fl.b.npairs * g.cluster
+                                               : (fl.b.npairs + g.slots_per_block - 1) / std::max(1, g.slots_per_block);
+    g.grid = (int)std::min<long long>(g.grid, std::max(1LL, blocks));
+    if (g.grid < g.cluster) g.cluster = 1;
+    g.grid -= g.grid % g.cluster;
 }
 
 // Every pair in flight has a slot: no more blocks than `bytes` hold.
@@ -33,6 +36,8 @@ bool fit_scratch(ClassGeom &g, size_t bytes) {
     const size_t per = (size_t)g.slots_per_block * (g.cm + g.bnd);
     if (g.grid > 0 && g.bytes(g.grid) > bytes)
         g.grid = (int)std::min<size_t>((size_t)g.grid, (bytes - std::min<size_t>(bytes, 256)) / per);
+    if (g.grid < g.cluster) g.cluster = 1;
+    g.grid -= g.grid % g.cluster;
     return g.grid > 0;
 }
 

@@ -46,11 +46,13 @@
 #include <climits>
 
 #include <type_traits>
+#include <cooperative_groups.h>
 #include <cstring>
 #include <mutex>
 
 namespace gsw {
 namespace {
+namespace cg = cooperative_groups;
 
 constexpr int kBlock = 128;
 constexpr int kUnrollFast = 4;  // steady loop of one-strip forward fills
@@ -363,8 +365,13 @@ struct StripRunner {
     // their word by shuffle, so no step waits on global memory.
     __device__ __forceinline__ void prefetch(const int s0) {
         const int jb = s0 + k, jc = s0 + CM_OFF + k;
-        b_nxt = (jb >= 0 && jb < n) ? bin[jb] : bnd_t{};
-        c_nxt = (has_cms && jc >= 0 && jc < n) ? cms[jc] : cm_t{};
+        if constexpr (P == 32) {  // (a strip of the CTA kernel: written on another SM, maybe)
+            b_nxt = (jb >= 0 && jb < n) ? __ldcg(bin + jb) : bnd_t{};
+            c_nxt = (has_cms && jc >= 0 && jc < n) ? __ldcg(cms + jc) : cm_t{};
+        } else {
+            b_nxt = (jb >= 0 && jb < n) ? bin[jb] : bnd_t{};
+            c_nxt = (has_cms && jc >= 0 && jc < n) ? cms[jc] : cm_t{};
+        }
     }
 
     // Starts strip st_ (boundary in from bin_, out to bout_).
@@ -778,13 +785,15 @@ __device__ void secondary(const BatchView &b, int pair, const Job &job, int end_
     for (int j = 4 * k; j < n; j += 4 * P) {
         int v[4];
         if constexpr (L::FOLD) {
-            const uint2 w = *reinterpret_cast<const uint2 *>(cms + j);
+            const uint2 *at = reinterpret_cast<const uint2 *>(cms + j);
+            const uint2 w = P == 32 ? __ldcg(at) : *at;
             v[0] = L::value(w.x & 0xFFFFu);
             v[1] = L::value(w.x >> 16);
             v[2] = L::value(w.y & 0xFFFFu);
             v[3] = L::value(w.y >> 16);
         } else {
-            const int4 w = *reinterpret_cast<const int4 *>(cms + j);
+            const int4 *at = reinterpret_cast<const int4 *>(cms + j);
+            const int4 w = P == 32 ? __ldcg(at) : *at;
             v[0] = w.x;
             v[1] = w.y;
             v[2] = w.z;
@@ -984,23 +993,35 @@ __global__ void __launch_bounds__(kBlock, fill_min_blocks(VID)) k_fill(FillLaunc
 // CTA kernel for pairs whose query spans many strips.  Strip x reads only the
 // bottom row (H, F) and the running column maxima that strip x-1 leaves in
 // global scratch, one column at a time, so several strips of a pair can run
-// at once when each stays far enough behind the one above it.  The warps of
-// the CTA (one 32-lane folded ring each; in 16-bit lanes 1,024 rows per strip
-// for DNA, 512 for general alphabets) advance in phases of kLongChunk steps
-// separated by a CTA barrier, which
-// also makes the previous phases' global writes visible.  Strip x+1 starts
+// at once when each stays far enough behind the one above it.  The warps of a
+// cluster of CTAs (one 32-lane folded ring each; in 16-bit lanes 1,024 rows per
+// strip for DNA, 512 for general alphabets) advance in phases of kLongChunk
+// steps separated by a cluster barrier, which also makes the previous phases'
+// global writes visible (they are read through L2).  Strip x+1 starts
 // long_lag() phases after strip x, so every boundary word and column maximum
 // it reads (one block of 32 columns ahead) was written in a completed phase,
 // and the ping-pong boundary buffer it writes was read a phase earlier.
 //
-// One thread schedules between the two barriers of a phase: it merges the
-// results of strips that ended, hands a finished pair to one warp (secondary
-// score or begins), hands strips to idle warps (oldest pair first, the next
-// strip of a pair no earlier than long_lag() phases after the previous one),
-// and opens the next pair of the class in a free scratch slot, so the end of
-// one pair overlaps the start of the next.
+// One warp of the cluster's first CTA schedules between the two barriers of a
+// phase, a lane per scratch slot: it merges the results of strips that ended,
+// hands finished pairs to idle warps (secondary score or begins), hands strips
+// to idle warps (oldest pair first, the next strip of a pair no earlier than
+// long_lag() phases after the previous one), and opens the next pairs of the
+// class in free slots, so the end of one pair overlaps the start of the next.
+//
+// Clusters: what bounds a batch of a few long reads is its longest pair.  On
+// one CTA a 20 kb read ran its 20 strips 4 at a time; on 8 CTAs all of them run
+// at once (kLongFewPairs).
 constexpr int kLongChunk = 128;
 constexpr int kLongSlots = 4;  // pairs in flight per CTA
+constexpr int kLongMaxCluster = 8;
+// Batches of at most this many pairs run on clusters of as many CTAs as the
+// longest query's strips fill (measured with 8: 300 reads of 1-20 kb 40.3 ->
+// 14.8 ms forward, 40 of 8-16 kb in 32-bit lanes 56.8 -> 11.9 ms, one of 20 kb
+// 34.1 -> 8.8 ms; 1,000 reads 58.5 -> 36.1 ms; 3,000 reads 104.7 -> 94.4 ms
+// forward but 37.7 -> 43.9 ms reversed, where the CTAs are busy anyway; 300
+// reads of 1-3 kb, three strips at most, 1.43 -> 1.97 ms).
+constexpr int kLongFewPairs = 2048;
 
 template <class L>
 __host__ __device__ constexpr int long_lag() {
@@ -1071,23 +1092,24 @@ struct LongRep {
     int v, c, row, stop;
 };
 
+// (in the first CTA of the cluster: one entry per slot and warp of all its CTAs)
 template <int NW>
 struct LongShared {
-    LongSlot slot[kLongSlots];
-    LongCmd cmd[NW];
-    LongRep rep[NW];
+    LongSlot slot[kLongSlots * kLongMaxCluster];
+    LongCmd cmd[NW * kLongMaxCluster];
+    LongRep rep[NW * kLongMaxCluster];
     int seq, exhausted, done;
 };
 
 // Opens the next pair of class CLS in slot s; false when none is left.
 template <class L, int SP>
-__device__ bool long_open(const FillLaunch &fl, int cls, LongSlot &S, int s, int seq) {
+__device__ bool long_open(const FillLaunch &fl, int cls, LongSlot &S, int slot, int seq) {
     const int ntasks = fl.plan.task_hi[cls] - fl.plan.task_lo[cls];
     const int t = atomicAdd(&fl.plan.head[cls], 1);
     if (t >= ntasks) return false;
     const int pair = fl.plan.order[fl.plan.var_start[cls] + t];
     Job job;
-    slot_scratch<L>(fl.scr, blockIdx.x * kLongSlots + s, &job);
+    slot_scratch<L>(fl.scr, slot, &job);
     S.band = 0;
     S.G = S.Gn = 0;
     if (fl.mode == kFillReverse) {
@@ -1122,75 +1144,99 @@ __device__ bool long_open(const FillLaunch &fl, int cls, LongSlot &S, int s, int
     return true;
 }
 
+// The schedule of phase ph, by one warp: lane = slot, and lane = warp of the
+// cluster (nslots, nw <= 32); slot0 is the cluster's first scratch slot.
 template <class L, int NW, int SP>
-__device__ void long_schedule(const FillLaunch &fl, int cls, LongShared<NW> &sh, int ph) {
+__device__ void long_schedule(const FillLaunch &fl, int cls, LongShared<NW> &sh, int ph, int nw, int nslots,
+                              int slot0, int nclusters, int lane) {
+    static_assert(kLongSlots * kLongMaxCluster <= 32 && NW * kLongMaxCluster <= 32, "a lane per slot and warp");
+    constexpr unsigned ALL = 0xFFFFFFFFu;
     // results of strips that ended, finished finalisations
-    for (int w = 0; w < NW; w++) {
-        if (!sh.rep[w].ended) continue;
-        sh.rep[w].ended = 0;
-        LongCmd &c = sh.cmd[w];
-        LongSlot &S = sh.slot[c.slot];
-        if (c.strip < 0) {
-            S.pair = -1;
-        } else {
-            best_merge(sh.rep[w].v, sh.rep[w].c, sh.rep[w].row, &S.bv, &S.bc, &S.br);
-            S.running--;
-            if (sh.rep[w].stop) S.stopped = 1;
+    for (unsigned m = __ballot_sync(ALL, lane < nw && sh.rep[lane].ended); m; m &= m - 1) {
+        if (lane == 0) {
+            const int w = __ffs(m) - 1;
+            sh.rep[w].ended = 0;
+            LongCmd &c = sh.cmd[w];
+            LongSlot &S = sh.slot[c.slot];
+            if (c.strip < 0) {
+                S.pair = -1;
+            } else {
+                best_merge(sh.rep[w].v, sh.rep[w].c, sh.rep[w].row, &S.bv, &S.bc, &S.br);
+                S.running--;
+                if (sh.rep[w].stop) S.stopped = 1;
+            }
+            c.slot = -1;
         }
-        c.slot = -1;
     }
+    __syncwarp();
     // idle warps: finalisations first, then strips of the oldest pair that
-    // may start one, then a new pair
-    for (int w = 0; w < NW; w++) {
-        LongCmd &c = sh.cmd[w];
-        if (c.slot >= 0) continue;
-        int pick = -1;
-        for (int s = 0; s < kLongSlots; s++) {
-            const LongSlot &S = sh.slot[s];
-            if (S.pair >= 0 && !S.fin && S.running == 0 && (S.stopped || S.next == S.nstrips)) {
-                pick = s;
-                break;
-            }
-        }
-        if (pick >= 0) {
-            sh.slot[pick].fin = 1;
+    // may start one
+    unsigned idle = __ballot_sync(ALL, lane < nw && sh.cmd[lane].slot < 0);
+    const bool mine = lane < nslots;
+    while (idle) {
+        const LongSlot &S = sh.slot[mine ? lane : 0];
+        const bool fin = mine && S.pair >= 0 && !S.fin && S.running == 0 && (S.stopped || S.next == S.nstrips);
+        const bool can = mine && S.pair >= 0 && !S.stopped && S.next < S.nstrips &&
+                         (S.next == 0 || ph >= S.last_start + S.lag);
+        const unsigned fins = __ballot_sync(ALL, fin);
+        const int first = __reduce_min_sync(ALL, can ? S.seq : INT_MAX);
+        const unsigned cans = __ballot_sync(ALL, can && S.seq == first);
+        if (!fins && !cans) break;
+        const int pick = __ffs(fins ? fins : cans) - 1;
+        if (lane == 0) {
+            LongSlot &T = sh.slot[pick];
+            LongCmd &c = sh.cmd[__ffs(idle) - 1];
             c.slot = pick;
-            c.strip = -1;
             c.start = ph;
-            continue;
-        }
-        int best_seq = INT_MAX;
-        for (int s = 0; s < kLongSlots; s++) {
-            const LongSlot &S = sh.slot[s];
-            if (S.pair >= 0 && !S.stopped && S.next < S.nstrips && (S.next == 0 || ph >= S.last_start + S.lag) &&
-                S.seq < best_seq) {
-                best_seq = S.seq;
-                pick = s;
+            if (fins) {
+                T.fin = 1;
+                c.strip = -1;
+            } else {
+                c.strip = T.next++;
+                T.last_start = ph;
+                T.running++;
             }
         }
-        if (pick < 0 && !sh.exhausted) {
-            for (int s = 0; s < kLongSlots; s++) {
-                if (sh.slot[s].pair >= 0) continue;
-                if (long_open<L, SP>(fl, cls, sh.slot[s], s, sh.seq)) {
-                    sh.seq++;
-                    pick = s;
-                } else {
-                    sh.exhausted = 1;
-                }
-                break;
-            }
-        }
-        if (pick < 0) break;  // nothing can start in this phase
-        LongSlot &S = sh.slot[pick];
-        c.slot = pick;
-        c.strip = S.next++;
-        c.start = ph;
-        S.last_start = ph;
-        S.running++;
+        idle &= idle - 1;
+        __syncwarp();
     }
-    bool busy = !sh.exhausted;
-    for (int s = 0; s < kLongSlots; s++) busy |= sh.slot[s].pair >= 0;
-    sh.done = busy ? 0 : 1;
+    // new pairs for the warps still idle, opened side by side: one a phase, and
+    // more while the class holds many for every cluster (the heaviest pairs
+    // come first, so a cluster that took several at once would end last: 40
+    // reads of 8-16 kb on 10 CTAs of 4 each, 82 ms against 21)
+    if (idle && !sh.exhausted) {
+        const int left = fl.plan.task_hi[cls] - fl.plan.task_lo[cls] - *(volatile const int32_t *)&fl.plan.head[cls];
+        const int most = 1 + (ph > 0 ? max(left, 0) / (4 * nclusters) : 0);
+        const unsigned free_slots = __ballot_sync(ALL, mine && sh.slot[mine ? lane : 0].pair < 0);
+        const int rank = __popc(free_slots & ((1u << lane) - 1u));
+        const bool try_open = ((free_slots >> lane) & 1u) && rank < min(most, __popc(idle));
+        const int seq = sh.seq + rank;
+        bool ok = false;
+        if (try_open) ok = long_open<L, SP>(fl, cls, sh.slot[lane], slot0 + lane, seq);
+        const unsigned opened = __ballot_sync(ALL, ok);
+        const bool none_left = __any_sync(ALL, try_open && !ok);
+        if (ok) {
+            // the k-th opened slot goes to the k-th idle warp
+            unsigned m = idle;
+            for (int k = __popc(opened & ((1u << lane) - 1u)); k > 0; k--) m &= m - 1;
+            LongCmd &c = sh.cmd[__ffs(m) - 1];
+            c.slot = lane;
+            c.start = ph;
+            c.strip = 0;
+            sh.slot[lane].next = 1;
+            sh.slot[lane].last_start = ph;
+            sh.slot[lane].running = 1;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            sh.seq += __popc(free_slots);
+            if (none_left) sh.exhausted = 1;
+        }
+        __syncwarp();
+    }
+    const bool busy = __any_sync(ALL, mine && sh.slot[mine ? lane : 0].pair >= 0);
+    if (lane == 0) sh.done = (busy || !sh.exhausted) ? 0 : 1;
+    __syncwarp();
 }
 
 template <bool DNA, bool S32>
@@ -1217,26 +1263,39 @@ __global__ void __launch_bounds__(LongCfg<DNA, S32>::NW * 32, LongCfg<DNA, S32>:
     using L = typename C::L;
     constexpr int NW = C::NW, SP = C::SP;
     extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ LongShared<NW> sh;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint32_t *psm = smem + (size_t)warp * warp_words;
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kLongSlots; s++) sh.slot[s].pair = -1;
-        for (int w = 0; w < NW; w++) {
-            sh.cmd[w].slot = -1;
-            sh.rep[w].ended = 0;
+    __shared__ LongShared<NW> sh_own;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int cl = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int cta_warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = rank * NW + cta_warp;  // of the cluster
+    const int nw = cl * NW, nslots = cl * kLongSlots;
+    uint32_t *psm = smem + (size_t)cta_warp * warp_words;
+    if (rank == 0) {
+        if (threadIdx.x < nslots) sh_own.slot[threadIdx.x].pair = -1;
+        if (threadIdx.x < nw) {
+            sh_own.cmd[threadIdx.x].slot = -1;
+            sh_own.rep[threadIdx.x].ended = 0;
         }
-        sh.seq = 0;
-        sh.exhausted = 0;
-        sh.done = 0;
+        if (threadIdx.x == 0) {
+            sh_own.seq = 0;
+            sh_own.exhausted = 0;
+            sh_own.done = 0;
+        }
     }
+    LongShared<NW> &sh = *cluster.map_shared_rank(&sh_own, 0);
+    auto barrier = [&]() {
+        if (cl == 1) __syncthreads();
+        else cluster.sync();
+    };
     StripRunner<C::P, C::R, L, DNA> sr;
     int strip_c0 = 0;  // first window column of the warp's strip
 #pragma unroll 1
     for (int ph = 0;; ph++) {
-        __syncthreads();
-        if (threadIdx.x == 0) long_schedule<L, NW, SP>(fl, C::CLS, sh, ph);
-        __syncthreads();
+        barrier();
+        if (rank == 0 && cta_warp == 0)
+            long_schedule<L, NW, SP>(fl, C::CLS, sh_own, ph, nw, nslots, (blockIdx.x / cl) * nslots,
+                                         gridDim.x / cl, lane);
+        barrier();
         if (sh.done) break;
         const LongCmd cmd = sh.cmd[warp];
         if (cmd.slot < 0) continue;
@@ -1300,6 +1359,7 @@ __global__ void __launch_bounds__(LongCfg<DNA, S32>::NW * 32, LongCfg<DNA, S32>:
             }
         }
     }
+    barrier();  // the first CTA's shared memory stays until every warp has read `done`
 }
 
 template <bool DNA, bool S32>
@@ -1342,6 +1402,9 @@ ClassGeom long_geom(const FillLaunch &fl, int sms) {
     g.grid = sms * cache.get(k_fill_long<DNA, S32>, C::NW * 32, fl.sc.A, g.smem,
                              long_smem_bytes<DNA, S32>(DNA ? 4 : kMaxAlpha));
     g.slots_per_block = kLongSlots;
+    const int ctas = ((fl.maxm + C::SP - 1) / C::SP + C::NW - 1) / C::NW;
+    if (fl.b.npairs <= kLongFewPairs)
+        while (g.cluster < ctas && g.cluster < kLongMaxCluster) g.cluster *= 2;
     g.cm = slot_cm_bytes<typename C::L>(fl.scr.ncap);
     g.bnd = slot_bnd_bytes<typename C::L>(fl.scr.ncap);
     return g;
@@ -1350,8 +1413,18 @@ ClassGeom long_geom(const FillLaunch &fl, int sms) {
 template <bool DNA, bool S32>
 cudaError_t launch_long(const FillLaunch &fl, const ClassGeom &g, cudaStream_t st) {
     using C = LongCfg<DNA, S32>;
-    k_fill_long<DNA, S32><<<g.grid, C::NW * 32, g.smem, st>>>(fl, (int)(g.smem / sizeof(uint32_t) / C::NW));
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(g.grid);
+    cfg.blockDim = dim3(C::NW * 32);
+    cfg.dynamicSmemBytes = g.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = g.cluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_fill_long<DNA, S32>, fl, (int)(g.smem / sizeof(uint32_t) / C::NW));
 }
 
 template <bool DNA, int VID, bool HALF>

@@ -99,3 +99,20 @@ def test_classes_chosen_by_batch_size(ctx, n, rows, cols, A):
     s = b.subset(keep)
     res, cig, (cm, off) = got
     compare(s, run_oracle(s), (res[keep], cig, (cm, off[keep])))
+
+
+# the CTA class on clusters: more strips than warps, several pairs a cluster,
+# 32-bit lanes, banded reversed strips, and a scratch that holds few CTAs
+@pytest.mark.parametrize("n,lo,hi,match,O,X,budget_mb", [
+    (1, 9000, 9000, 2, 4, 2, 4096), (7, 4000, 9000, 5, 10, 1, 4096), (60, 1800, 4200, 2, 4, 2, 4096),
+    (5, 8000, 9000, 2, 4, 2, 256)])
+def test_long_pairs_on_clusters(n, lo, hi, match, O, X, budget_mb):
+    b = wl.dna_long_reads(n, lo, hi, match=match, mismatch=-4, gap_open=O, gap_extend=X, seed=n + lo)
+    c = gsw.Context(0, budget_mb << 20)
+    try:
+        keep = np.arange(n)[:12]
+        got = run_gpu_host(c, b, colmax=False)
+    finally:
+        c.close()
+    s = b.subset(keep)
+    compare(s, run_oracle(s, colmax=False), (got[0][keep], got[1], (None, None)), check_colmax=False)
