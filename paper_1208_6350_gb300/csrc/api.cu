@@ -207,11 +207,10 @@ enum MiscSlot {
     kMiscCursor = 1,
     kMiscInternal = 2,  // records flagged kResInternal (counted after the pipeline)
     kMiscValid = 3,
-    kMiscNeed = 4,   // 2 words: anti-diagonal traceback (direction words, op words per pair)
-    kMiscRing = 6,   // 3 words: wide-band traceback (total words, max words of a pair, max op words)
-    kMiscStats = 12,   // 7 words: largest lengths, arena extents, bad lengths or offsets, smallest query, cells
-    kMiscNeed16 = 19,  // 4 words: 16-bit rectangle traceback (direction words per group, per class)
-    kMiscWords = 23
+    kMiscNeed = 4,   // kNeedWords words: needs of the tracebacks (trace_needs)
+    kMiscStats = kMiscNeed + kNeedWords,  // 7 words: largest lengths, arena extents, bad lengths or offsets,
+                                          // smallest query, cells
+    kMiscWords = kMiscStats + 7
 };
 
 // Side streams and fork/join events of the fill and band classes, created once per
@@ -371,8 +370,8 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
         pb.keys = reinterpret_cast<int32_t *>(ctx->plan_keys.p);
         pb.order = reinterpret_cast<int32_t *>(ctx->plan_order.p);
         pb.hist = ps;
-        pb.binoff = ps + kPlanBins;
-        pb.cursor = ps + 2 * kPlanBins;
+        pb.cursor = ps + kPlanBins;
+        pb.binoff = ps + 2 * kPlanBins;
         pb.var_start = ps + 3 * kPlanBins;
         pb.task_lo = pb.var_start + kNumFillClasses + 1;
         pb.task_hi = pb.task_lo + kNumFillClasses;
@@ -434,9 +433,10 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
         fl.scr.bytes = ctx->fill_scr.bytes;
 
         auto plan = [&](int32_t mode) -> int {
-            cudaError_t e = launch_plan(bv, sc, mode, pb, st);
+            cudaError_t e = launch_plan(bv, sc, mode, pb,
+                                        mode == kPlanTrace ? misc + kMiscNeed : nullptr, st);
             if (e != cudaSuccess) return set_err(GSW_ECUDA, "plan: %s", cudaGetErrorString(e));
-            S.launches += 3;
+            S.launches += plan_launches(npairs);
             return GSW_OK;
         };
         // (a context limited to some SMs runs its classes one after the other)
@@ -471,9 +471,10 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
         GSW_TRY(mark(ctx, 4, st));
         if (reverse) {
             // thread-per-pair banded reverse and traceback for narrow bands
-            // (the plan also hands a small batch's pairs to the warp tracebacks)
-            GSW_TRY(plan(kPlanBand));
-            if (!small_batch(bv)) {  // a small batch's band classes are empty
+            // (a small batch has no such stage: its pairs reverse in the ring
+            // fill and the trace plan hands them to the warp tracebacks)
+            if (!small_batch(bv)) {
+                GSW_TRY(plan(kPlanBand));
                 const int rows_cap = std::min(std::max(maxm, 1), kBandMaxRows);
                 // a quarter of what is left: the band scratch holds every row of
                 // the pairs in flight
@@ -493,16 +494,21 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
             // diagonals, CTA strip kernel beyond; their scratch is sized from
             // the needs read back after this segment
             GSW_TRY(plan(kPlanTrace));
-            CUDA_TRY(launch_trace_need(bv, sc, misc + kMiscNeed, misc + kMiscNeed16, st));
-            const size_t meta_bytes = sizeof(long long) * ((size_t)npairs + 1) + sizeof(int) * ((size_t)npairs + 4);
-            GSW_TRY(ensure(ctx, ctx->ring_meta, meta_bytes));
-            S.ring_prefix = reinterpret_cast<long long *>(ctx->ring_meta.p);
-            S.ring_final = reinterpret_cast<int *>(S.ring_prefix + npairs + 1);
-            S.ring_group = S.ring_final + npairs;
-            CUDA_TRY(launch_ring_needs(bv, sc, pb.order, pb.var_start, S.ring_prefix, misc + kMiscRing, st));
-            CUDA_TRY(cudaMemsetAsync(S.ring_group, 0, 3 * sizeof(int), st));
-            S.launches += 2;
-            CUDA_TRY(cudaMemcpyAsync(hs, misc + kMiscNeed, (kMiscWords - kMiscNeed) * sizeof(unsigned long long),
+            if (!plan_takes_needs(npairs)) {
+                CUDA_TRY(launch_trace_need(bv, sc, misc + kMiscNeed, st));
+                S.launches += 1;
+            }
+            if (ring_possible(maxm, maxn, sc)) {
+                const size_t meta_bytes = sizeof(long long) * ((size_t)npairs + 1) + sizeof(int) * ((size_t)npairs + 4);
+                GSW_TRY(ensure(ctx, ctx->ring_meta, meta_bytes));
+                S.ring_prefix = reinterpret_cast<long long *>(ctx->ring_meta.p);
+                S.ring_final = reinterpret_cast<int *>(S.ring_prefix + npairs + 1);
+                S.ring_group = S.ring_final + npairs;
+                CUDA_TRY(launch_ring_needs(bv, sc, pb.order, pb.var_start, S.ring_prefix, misc + kMiscNeed + 2, st));
+                CUDA_TRY(cudaMemsetAsync(S.ring_group, 0, 3 * sizeof(int), st));
+                S.launches += 1;
+            }
+            CUDA_TRY(cudaMemcpyAsync(hs, misc + kMiscNeed, kNeedWords * sizeof(unsigned long long),
                                      cudaMemcpyDeviceToHost, st));
         }
         return GSW_OK;
@@ -511,12 +517,11 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
 
     if (bv.flags & GSW_CIGAR) {
         CUDA_TRY(cudaStreamSynchronize(st));
-        // [0, 1] anti-diagonal, [2, 4] ring, kMiscNeed16 - kMiscNeed.. 16-bit rectangle classes (others unused here)
-        unsigned long long need[kMiscWords - kMiscNeed];
+        unsigned long long need[kNeedWords];
         std::memcpy(need, hs, sizeof(need));
-        for (int k = 5; k < kMiscNeed16 - kMiscNeed; k++) need[k] = 0;
         if (ctx->graph_buckets)
-            for (unsigned long long &x : need) x = bucket_up(x);
+            for (int k = 0; k < kNeedWords; k++)
+                need[k] = k == kNeedMask ? (need[k] ? 15 : 0) : bucket_up(need[k]);
         std::vector<uint8_t> key2 = key;
         key_add(key2, need);
         for (const DevBuf *d : {&ctx->fill_scr, &ctx->trace_dirs, &ctx->trace_ops, &ctx->ring_meta})
@@ -526,80 +531,88 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
         // ---- segment 2: the tracebacks, sized from the needs
         auto seg2 = [&]() -> int {
             const PlanBuffers &pb = S.pb;
+            const size_t have = room(ctx, ctx->trace_dirs, ctx->trace_ops);
+            // The kernels' launches, each with its own part of the two scratch
+            // buffers (in words) when half of the room holds all of them: then
+            // they run side by side, since few of them fill the chip.
+            // Otherwise one after the other over the same words.
+            struct Part {
+                size_t dirs = 0, ops = 0;        // words
+                size_t dir_at = 0, op_at = 0;
+            } ad, t16[kTraceT16Classes], ring;
+            auto bytes = [](const Part &x) { return (x.dirs + x.ops) * sizeof(uint32_t); };
+            auto words16 = [](size_t x) { return (x + 3) & ~(size_t)3; };  // 16-byte aligned areas
             // anti-diagonal kernel (<= 512 diagonals): direction and op words per warp
             const long long ad_dir = (long long)need[0], ad_ops = std::max<long long>((long long)need[1], 64);
-            int ad_grid = 0;
-            size_t max_dir = 0, max_ops = 0;
             const int wpb = trace_block_threads() / 32;
-            if (ad_dir > 0) {
-                const size_t have = room(ctx, ctx->trace_dirs, ctx->trace_ops) / 2;
+            int ad_warps = 0;
+            auto size_ad = [&](size_t room_bytes) {
                 const size_t per_warp = (size_t)(ad_dir + ad_ops) * sizeof(uint32_t);
-                int warps = (int)std::min<size_t>((size_t)ctx->sms * 16 * wpb, std::max<size_t>(1, have / per_warp));
-                warps = std::max(wpb, warps - warps % wpb);
-                ad_grid = warps / wpb;
-                max_dir = (size_t)warps * (size_t)ad_dir;
-                max_ops = (size_t)warps * (size_t)ad_ops;
-            }
-            // 16-bit rectangle kernel: per class, 4 groups per warp, direction
-            // and op words per group (the classes run one after the other)
-            T16Scratch t16{};
-            bool any16 = false;
-            {
-                const size_t have = room(ctx, ctx->trace_dirs, ctx->trace_ops) / 2;
-                for (int v = 0; v < kTraceT16Classes; v++) {
-                    // 16-byte aligned group areas
-                    const long long dw = ((long long)need[kMiscNeed16 - kMiscNeed + v] + 3) & ~3LL;
-                    if (dw <= 0) continue;
-                    const size_t per_warp = 4 * (size_t)(dw + ad_ops) * sizeof(uint32_t);
-                    const int w = (int)std::min<size_t>((size_t)t16_max_warps(sc, ctx->sms, v),
-                                                        std::max<size_t>(1, have / per_warp));
-                    if (w <= 0) continue;
-                    t16.dir_words[v] = dw;
-                    t16.warps[v] = w;
-                    max_dir = std::max(max_dir, (size_t)w * 4 * (size_t)dw);
-                    max_ops = std::max(max_ops, (size_t)w * 4 * (size_t)ad_ops);
-                    any16 = true;
-                }
-            }
+                size_t warps = std::min<size_t>((size_t)ctx->sms * 16 * wpb, std::max<size_t>(1, room_bytes / per_warp));
+                warps = std::min<size_t>(warps, ((size_t)npairs + wpb - 1) / wpb * wpb);
+                ad_warps = std::max(wpb, (int)(warps - warps % wpb));
+                ad.dirs = words16((size_t)ad_warps * (size_t)ad_dir);
+                ad.ops = words16((size_t)ad_warps * (size_t)ad_ops);
+            };
+            // 16-bit rectangle kernel: per class, 4 groups per warp
+            int t16_warps[kTraceT16Classes] = {};
+            auto t16_dir = [&](int v) { return ((long long)need[kNeed16 + v] + 3) & ~3LL; };
+            auto size_t16 = [&](int v, size_t room_bytes) {
+                const size_t per_warp = 4 * (size_t)(t16_dir(v) + ad_ops) * sizeof(uint32_t);
+                size_t w = std::min<size_t>((size_t)t16_max_warps(sc, ctx->sms, v), std::max<size_t>(1, room_bytes / per_warp));
+                w = std::min<size_t>(w, ((size_t)npairs + 15) / 16 * 4);  // (whole blocks of 4 warps)
+                t16_warps[v] = (int)w;
+                t16[v].dirs = std::max<size_t>(w, 4) * 4 * (size_t)t16_dir(v);
+                t16[v].ops = words16(std::max<size_t>(w, 4) * 4 * (size_t)ad_ops);
+            };
             // wide bands: the pool of direction words, groups of pairs that fit it
             const unsigned long long ring_total = need[2], ring_max = need[3], ring_ops = need[4];
-            size_t ring_pool = 0, ring_walk_warps = 0;
+            // (one warp per pair: no more warps, and op words, than pairs)
+            const size_t ring_walk_warps = std::min<size_t>((size_t)ctx->sms * 16, ((size_t)npairs + 1) & ~(size_t)1);
+            if (ad_dir > 0) size_ad(have / 2);
+            for (int v = 0; v < kTraceT16Classes; v++)
+                if (need[kNeed16 + v] > 0) size_t16(v, have / 2);
             if (ring_total > 0) {
-                // (one warp per pair: no more warps, and op words, than pairs)
-                ring_walk_warps = std::min<size_t>((size_t)ctx->sms * 16, ((size_t)npairs + 1) & ~(size_t)1);
-                const size_t have_all = room(ctx, ctx->trace_dirs, ctx->trace_ops);
+                ring.dirs = words16((size_t)ring_total);
+                ring.ops = words16(ring_walk_warps * (size_t)ring_ops);
+            }
+            size_t all = bytes(ad) + bytes(ring);
+            for (const Part &x : t16) all += bytes(x);
+            const bool side = all <= have / 2 && ctx->aux.fork && ctx->sms == ctx->sms_all;
+            size_t max_dir = 0, max_ops = 0;
+            size_t ring_pool = (size_t)ring_total;
+            auto place = [&](Part &x) {
+                if (side) {
+                    x.dir_at = max_dir;
+                    x.op_at = max_ops;
+                    max_dir += x.dirs;
+                    max_ops += x.ops;
+                } else {
+                    max_dir = std::max(max_dir, x.dirs);
+                    max_ops = std::max(max_ops, x.ops);
+                }
+            };
+            if (!side && ring_total > 0) {
                 const size_t ops_bytes = ring_walk_warps * (size_t)ring_ops * sizeof(uint32_t);
-                size_t cap = have_all > ops_bytes ? (have_all - ops_bytes) / 2 / sizeof(uint32_t) : 0;
+                const size_t cap = have > ops_bytes ? (have - ops_bytes) / 2 / sizeof(uint32_t) : 0;
                 ring_pool = (size_t)std::min<unsigned long long>(ring_total, cap);
                 if (ring_pool < ring_max)
                     return set_err(GSW_ENOMEM, "wide-band traceback of one pair needs %llu words", ring_max);
-                max_dir = std::max(max_dir, ring_pool);
-                max_ops = std::max(max_ops, ring_walk_warps * (size_t)ring_ops);
+                ring.dirs = ring_pool;
             }
+            place(ad);
+            for (Part &x : t16) place(x);
+            place(ring);
             if (max_dir > 0) {
                 GSW_TRY(ensure2(ctx, ctx->trace_dirs, max_dir * sizeof(uint32_t), ctx->trace_ops,
                                 max_ops * sizeof(uint32_t)));
-                if (any16) {
-                    t16.dirs = reinterpret_cast<uint32_t *>(ctx->trace_dirs.p);
-                    t16.ops = reinterpret_cast<uint32_t *>(ctx->trace_ops.p);
-                    t16.op_words = ad_ops;
-                    t16.order = pb.order;
-                    t16.var_start = pb.var_start;
-                    t16.head = pb.head;
-                    CUDA_TRY(launch_trace16(bv, sc, t16, ctx->sms, st));
-                    for (int v = 0; v < kTraceT16Classes; v++) S.launches += t16.warps[v] > 0 ? 1 : 0;
+                uint32_t *dirs = reinterpret_cast<uint32_t *>(ctx->trace_dirs.p);
+                uint32_t *ops = reinterpret_cast<uint32_t *>(ctx->trace_ops.p);
+                if (side) {
+                    CUDA_TRY(cudaEventRecord(ctx->aux.fork, st));
+                    for (int k = 0; k < 2; k++) CUDA_TRY(cudaStreamWaitEvent(ctx->aux.s[k], ctx->aux.fork, 0));
                 }
-                if (ad_grid > 0) {
-                    TraceScratch ts;
-                    ts.dirs = reinterpret_cast<uint32_t *>(ctx->trace_dirs.p);
-                    ts.dir_words = ad_dir;
-                    ts.ops = reinterpret_cast<uint32_t *>(ctx->trace_ops.p);
-                    ts.op_words = ad_ops;
-                    ts.order = pb.order;
-                    ts.var_start = pb.var_start;
-                    CUDA_TRY(launch_trace_ad(bv, sc, ts, ad_grid, st));
-                    S.launches += 4;
-                }
+                const cudaStream_t on[3] = {st, side ? ctx->aux.s[0] : st, side ? ctx->aux.s[1] : st};
                 if (ring_total > 0) {
                     RingLaunchArgs ra;
                     ra.b = bv;
@@ -609,12 +622,12 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
                     ra.prefix = S.ring_prefix;
                     ra.final_h = S.ring_final;
                     ra.group = S.ring_group;
-                    ra.pool = reinterpret_cast<uint32_t *>(ctx->trace_dirs.p);
+                    ra.pool = dirs + ring.dir_at;
                     ra.pool_words = (long long)ring_pool;
                     ra.bnd = reinterpret_cast<int2 *>(ctx->fill_scr.p);
                     ra.bnd_stride = 2 * (long long)S.ncap;
                     ra.slots = (int)std::min<size_t>(ctx->fill_scr.bytes / (2 * S.ncap * sizeof(int2)), 1 << 20);
-                    ra.ops = reinterpret_cast<uint32_t *>(ctx->trace_ops.p);
+                    ra.ops = ops + ring.op_at;
                     ra.op_words = (long long)ring_ops;
                     ra.walk_warps = (int)ring_walk_warps;
                     // every group but the last fills more than pool - max_pair
@@ -622,13 +635,45 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
                     const unsigned long long groups =
                         ring_total <= ring_pool ? 1 : (ring_total + per - 1) / per + 1;
                     for (unsigned long long gi = 0; gi < groups; gi++) {
-                        CUDA_TRY(launch_ring_group(ra, ctx->sms, st));
+                        CUDA_TRY(launch_ring_group(ra, ctx->sms, on[0]));
                         S.launches += 4;
                     }
                     S.ring_words = (long long)ring_total;
                     S.ring_pool = (long long)ring_pool;
                     S.ring_groups = (int)groups;
                 }
+                if (ad_dir > 0) {
+                    TraceScratch ts;
+                    ts.dirs = dirs + ad.dir_at;
+                    ts.dir_words = ad_dir;
+                    ts.ops = ops + ad.op_at;
+                    ts.op_words = ad_ops;
+                    ts.order = pb.order;
+                    ts.var_start = pb.var_start;
+                    CUDA_TRY(launch_trace_ad(bv, sc, ts, ad_warps / wpb, (unsigned)need[kNeedMask], on[1]));
+                    S.launches += __builtin_popcount((unsigned)need[kNeedMask]);
+                }
+                int turn = ring_total > 0 || ad_dir > 0 ? 2 : 0;
+                for (int v = kTraceT16Classes - 1; v >= 0; v--) {
+                    if (t16_warps[v] <= 0) continue;
+                    T16Scratch ts{};
+                    ts.dirs = dirs + t16[v].dir_at;
+                    ts.dir_words = t16_dir(v);
+                    ts.ops = ops + t16[v].op_at;
+                    ts.op_words = ad_ops;
+                    ts.order = pb.order;
+                    ts.var_start = pb.var_start;
+                    ts.head = pb.head;
+                    ts.warps = t16_warps[v];
+                    CUDA_TRY(launch_trace16(bv, sc, ts, ctx->sms, v, on[turn]));
+                    turn = (turn + 1) % 3;
+                    S.launches += 1;
+                }
+                if (side)
+                    for (int k = 0; k < 2; k++) {
+                        CUDA_TRY(cudaEventRecord(ctx->aux.join[k], ctx->aux.s[k]));
+                        CUDA_TRY(cudaStreamWaitEvent(st, ctx->aux.join[k], 0));
+                    }
             }
             S.stage_done[5] = 1;
             GSW_TRY(mark(ctx, 6, st));
@@ -685,6 +730,7 @@ int batch_impl(gsw_ctx *ctx, int32_t npairs, const uint8_t *q, const int64_t *q_
     if (ctx->timing && !ctx->ev[0])
         for (int k = 0; k <= GSW_NSTAGES; k++) CUDA_TRY(cudaEventCreate(&ctx->ev[k]));
     unsigned long long *misc = reinterpret_cast<unsigned long long *>(ctx->misc.p);
+    CUDA_TRY(cudaMemsetAsync(misc, 0, kMiscWords * sizeof(unsigned long long), st));  // every counter of the call
     BatchView bv;
     std::memset(&bv, 0, sizeof(bv));
     bv.npairs = npairs;
@@ -731,7 +777,7 @@ int batch_impl(gsw_ctx *ctx, int32_t npairs, const uint8_t *q, const int64_t *q_
                 if (q_off[p] < 0 || t_off[p] < 0) return set_err(GSW_EINVAL, "pair %d: negative offset", p);
             }
         }
-        minm = smallest(hstat[5]);
+        minm = smallest(0xFFFFFFFFull - hstat[5]);
         cells = (double)hstat[6];
         maxm = (int)hstat[0];
         maxn = (int)hstat[1];
@@ -792,7 +838,7 @@ int batch_impl(gsw_ctx *ctx, int32_t npairs, const uint8_t *q, const int64_t *q_
         bv.colmax_off = colmax_off;
         GSW_TRY(batch_stats(q_off, q_len, t_off, t_len));
         if (hstat[4]) return set_err(GSW_EINVAL, "a length is outside [0, 2^24) or an offset is negative");
-        minm = smallest(hstat[5]);
+        minm = smallest(0xFFFFFFFFull - hstat[5]);
         cells = (double)hstat[6];
         maxm = (int)hstat[0];
         maxn = (int)hstat[1];
@@ -815,11 +861,8 @@ int batch_impl(gsw_ctx *ctx, int32_t npairs, const uint8_t *q, const int64_t *q_
         maxn = (int)bucket_up((uint64_t)maxn);
     }
     default_classes(sc, npairs, maxn, cells);
-    CUDA_TRY(cudaMemsetAsync(misc + kMiscCursor, 0, 2 * sizeof(unsigned long long), st));  // cursor, internal
-    if ((flags & GSW_PACKED2) && sc.A >= 4) {
-        // 2-bit letters are 0..3: valid under any matrix of 4 or more letters
-        CUDA_TRY(cudaMemsetAsync(misc + kMiscValid, 0, sizeof(int32_t), st));
-    } else {
+    // (2-bit letters are 0..3: valid under any matrix of 4 or more letters)
+    if (!((flags & GSW_PACKED2) && sc.A >= 4)) {
         CUDA_TRY(launch_validate(bv, sc, reinterpret_cast<int32_t *>(misc + kMiscValid), st));
         ctx->launches += 1;
     }

@@ -539,6 +539,58 @@ __host__ __device__ inline int trace_class(int la, int lb, int score1, const Sco
     return ad;
 }
 
+// decision words of one pair in the anti-diagonal kernel: 8 anti-diagonals per
+// word row, nch x 32 words a row
+__host__ __device__ inline long long ad_dir_words(int la, int lb, int nch) {
+    return ((long long)(la + lb + 1 + 7) / 8) * nch * 32;
+}
+
+// pairs left to the warp tracebacks
+__host__ __device__ inline bool wants_trace(const gsw_result &r) {
+    return r.score1 > 0 && (r.flags & kResPendingTrace) && !(r.flags & kResInternal) && r.read_begin1 >= 0 &&
+           r.ref_begin1 >= 0;
+}
+
+// Largest needs of the warp tracebacks' pairs: [0] direction words of the
+// anti-diagonal classes, [1] op words (anti-diagonal and 16-bit classes),
+// [2..4] wide bands (launch_ring_needs: total words, largest pair, largest op
+// words), [5] bit c: anti-diagonal class c has pairs, [6 + v] direction words of
+// 16-bit class v (per group of 8 lanes)
+constexpr int kNeedMask = 5, kNeed16 = 6, kNeedWords = kNeed16 + kTraceT16Classes;
+// A pair's share of those (v zeroed by the caller; the ring words are not set).
+__host__ __device__ inline void trace_needs(const gsw_result &r, const Scoring &sc, bool small, unsigned v[kNeedWords]) {
+    if (!wants_trace(r)) return;
+    const int la = r.read_end1 - r.read_begin1 + 1, lb = r.ref_end1 - r.ref_begin1 + 1;
+    const long long top = 0xFFFFFFFFLL;
+    auto capped = [&](long long x) { return (unsigned)(x < top ? x : top); };
+    int dlo, dhi;
+    const int cls = trace_class(la, lb, r.score1, sc, small, &dlo, &dhi);
+    if (cls == kTraceRingClass) return;
+    v[1] = capped((long long)la + lb + 2);
+    if (cls < kTraceRingClass) {
+        v[0] = capped(ad_dir_words(la, lb, 1 << cls));
+        v[kNeedMask] = 1u << cls;
+    } else {
+        v[kNeed16 + cls - kTraceT16First] = capped(t16_need_words(la, lb, cls - kTraceT16First));
+    }
+}
+
+// Whether a pair of a batch with these largest lengths can be of the wide-band
+// class: not when every region the lengths allow fits the anti-diagonal kernel
+// (at most 512 diagonals) or the 16-bit rectangle (trace_class; its needs and
+// value ranges grow with the lengths).
+inline bool ring_possible(int maxm, int maxn, const Scoring &sc) {
+    if (maxm + maxn + 1 <= 512) return false;
+    if (maxn > kT16MaxCols) return true;
+    const long long rows = (long long)maxm + 256, cols = maxn + 2 * kT16P;
+    const long long lo = 3LL * sc.O + (long long)sc.X * (rows + cols + 2) - (sc.wmin < 0 ? sc.wmin : 0);
+    const long long hi = (long long)sc.wmax * ((cols < rows ? cols : rows) + 1);
+    if (lo > 30000 || hi > 30000) return true;
+    const int m = maxm < 1 ? 1 : maxm, n = maxn < 1 ? 1 : maxn;
+    if (sc.dna4) return t16_need_words(m, n, kTraceT16Classes - 1) > kT16MaxWords;
+    return t16_need_words(m, n, 0) > kT16MaxWords && t16_need_words(m, n, 1) > kT16MaxWordsBig;
+}
+
 // stage launchers (host side, enqueue on `st`)
 // Status of a completed batch from what its kernels counted, in order of
 // precedence: letter codes outside the alphabet (GSW_EINVAL), records that
@@ -594,8 +646,8 @@ GSW_FILL_UNITS(GSW_DECLARE_UNIT)
 struct PlanBuffers {
     int32_t *keys;       // [npairs]
     int32_t *hist;       // [kPlanBins]
+    int32_t *cursor;     // [kPlanBins], after hist (cleared together)
     int32_t *binoff;     // [kPlanBins]
-    int32_t *cursor;     // [kPlanBins]
     int32_t *order;      // [npairs]
     int32_t *var_start;  // [kNumFillClasses+1]
     int32_t *task_lo;    // [kNumFillClasses]
@@ -603,8 +655,11 @@ struct PlanBuffers {
     int32_t *ntasks;     // [1]
     int32_t *head;       // [kNumFillClasses]
 };
+int plan_launches(int npairs);  // kernels of one plan
+// (a small batch's kPlanTrace plan also writes `need`, kNeedWords words)
 cudaError_t launch_plan(const BatchView &b, const Scoring &sc, int32_t mode, const PlanBuffers &pb,
-                        cudaStream_t st);
+                        unsigned long long *need, cudaStream_t st);
+bool plan_takes_needs(int npairs);
 
 // Wide-band traceback (trace_ring.cu): banded global fill with direction
 // bits on the CTA strip pipeline, then a warp walk per pair, group by group
@@ -646,30 +701,29 @@ struct TraceScratch {
     const int32_t *var_start;
 };
 int trace_block_threads();
-// largest needs of a pair: [0] direction words of the anti-diagonal classes,
-// [1] op words of the warp classes; need16[v]: direction words of 16-bit class v
-cudaError_t launch_trace_need(const BatchView &b, const Scoring &sc, unsigned long long *max_need,
-                              unsigned long long *need16, cudaStream_t st);
-cudaError_t launch_trace_ad(const BatchView &b, const Scoring &sc, const TraceScratch &ts, int grid,
+// the needs (trace_needs) of a batch whose plan did not take them along, into
+// zeroed words
+cudaError_t launch_trace_need(const BatchView &b, const Scoring &sc, unsigned long long *need, cudaStream_t st);
+// the classes in `mask`, one after the other
+cudaError_t launch_trace_ad(const BatchView &b, const Scoring &sc, const TraceScratch &ts, int grid, unsigned mask,
                             cudaStream_t st);
 
-// 16-bit full-rectangle traceback (trace16.cu): per class v (strips of
-// 64(v+1) rows) and group of 8 lanes, dir_words[v] direction words (0: no
-// pairs) and op_words op words; the classes run one after the other on the
-// stream and share the buffers
+// 16-bit full-rectangle traceback (trace16.cu), class v (strips of 64(v+1)
+// rows): direction and op words per group of 8 lanes, 4 groups a warp
 struct T16Scratch {
     uint32_t *dirs;
-    int64_t dir_words[kTraceT16Classes];  // per group
+    int64_t dir_words;  // per group
     uint32_t *ops;
     int64_t op_words;   // per group
     const int32_t *order;
     const int32_t *var_start;
     int32_t *head;      // per-class task counters (zeroed by the plan)
-    int warps[kTraceT16Classes];  // warps of each class's launch (the scratch holds 4 groups each)
+    int warps;          // of the launch (the scratch holds 4 groups each)
 };
 // warps of class v's launch that can be resident
 int t16_max_warps(const Scoring &sc, int sms, int v);
-cudaError_t launch_trace16(const BatchView &b, const Scoring &sc, const T16Scratch &ts, int sms, cudaStream_t st);
+cudaError_t launch_trace16(const BatchView &b, const Scoring &sc, const T16Scratch &ts, int sms, int v,
+                           cudaStream_t st);
 
 int band_block_threads();
 // Grids and scratch of the three band classes (widths 8, 16, 32), each
@@ -687,11 +741,13 @@ cudaError_t launch_band(const BatchView &b, const Scoring &sc, const PlanBuffers
 // small helpers (misc.cu)
 // one pass over the pairs: [0, 1] largest lengths, [2, 3] arena extents,
 // [4] nonzero if a length is outside [0, 2^24) or an offset negative,
-// [5] smallest query length (0 if any query or target is empty), [6] cells
+// [5] 2^32 - 1 - the smallest query length (0 if any query or target is
+// empty), [6] cells; the words are zero before
 cudaError_t launch_batch_stats(const int64_t *q_off, const int32_t *q_len, const int64_t *t_off,
                                const int32_t *t_len, int32_t n, unsigned long long *out7, cudaStream_t st);
 // 2-bit packed DNA letters to one byte per letter
 cudaError_t launch_unpack2(const uint8_t *in, uint8_t *out, long long nletters, cudaStream_t st);
+// (*bad is zero before)
 cudaError_t launch_validate(const BatchView &b, const Scoring &sc, int32_t *bad, cudaStream_t st);
 cudaError_t launch_fill_const(int32_t *dst, int32_t v, int32_t n, cudaStream_t st);
 cudaError_t launch_fill_const64(int64_t *dst, int64_t v, int32_t n, cudaStream_t st);

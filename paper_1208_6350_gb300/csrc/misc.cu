@@ -30,8 +30,9 @@ __global__ void k_validate(BatchView b, int32_t A, int32_t *bad) {
 // Checks and sizes of a batch in one pass: [0] largest query length, [1]
 // largest target length, [2] query arena extent, [3] target arena extent
 // (offset + length, letters), [4] nonzero if a length is outside [0, 2^24)
-// or an offset is negative, [5] smallest query length (0 if a query or a
-// target is empty), [6] cells (sum of the products of the lengths).
+// or an offset is negative, [5] 2^32 - 1 - the smallest query length (0 if a
+// query or a target is empty), [6] cells (sum of the products of the lengths).
+// The words start at zero.
 __global__ void k_batch_stats(const int64_t *q_off, const int32_t *q_len, const int64_t *t_off,
                               const int32_t *t_len, int32_t n, unsigned long long *out7) {
     unsigned long long mq = 0, mt = 0, eq = 0, et = 0, bad = 0;
@@ -64,7 +65,7 @@ __global__ void k_batch_stats(const int64_t *q_off, const int32_t *q_len, const 
         atomicMax(&out7[2], eq);
         atomicMax(&out7[3], et);
         if (bad) atomicOr(&out7[4], 1ull);
-        atomicMin(&out7[5], (unsigned long long)least);
+        atomicMax(&out7[5], (unsigned long long)(0xFFFFFFFFu - least));
         atomicAdd(&out7[6], cells);
     }
 }
@@ -113,7 +114,6 @@ cudaError_t launch_unpack2(const uint8_t *in, uint8_t *out, long long nletters, 
 }
 
 cudaError_t launch_validate(const BatchView &b, const Scoring &sc, int32_t *bad, cudaStream_t st) {
-    cudaMemsetAsync(bad, 0, sizeof(int32_t), st);
     if (b.npairs > 0) {
         int blocks = (b.npairs * 32 + 255) / 256;
         blocks = blocks > 4096 ? 4096 : blocks;
@@ -124,9 +124,6 @@ cudaError_t launch_validate(const BatchView &b, const Scoring &sc, int32_t *bad,
 
 cudaError_t launch_batch_stats(const int64_t *q_off, const int32_t *q_len, const int64_t *t_off,
                                const int32_t *t_len, int32_t n, unsigned long long *out7, cudaStream_t st) {
-    cudaMemsetAsync(out7, 0, 5 * sizeof(unsigned long long), st);
-    cudaMemsetAsync(out7 + 5, 0xFF, sizeof(unsigned long long), st);
-    cudaMemsetAsync(out7 + 6, 0, sizeof(unsigned long long), st);
     if (n > 0) {
         int blocks = (n + 255) / 256;
         blocks = blocks > 1024 ? 1024 : blocks;

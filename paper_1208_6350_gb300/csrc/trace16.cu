@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(kT16Block) k_trace16(BatchView b, Scoring sc, 
     const int gwarp = blockIdx.x * (kT16Block / 32) + warp;
     const size_t gid = (size_t)gwarp * (32 / kP) + g;
     const int v = cls - kTraceT16First;
-    const int64_t dir_words = ts.dir_words[v];
+    const int64_t dir_words = ts.dir_words;
     uint32_t *dirs = ts.dirs + gid * dir_words;
     uint32_t *ops = ts.ops + gid * ts.op_words;
     const int first = ts.var_start[cls], last = ts.var_start[cls + 1];
@@ -511,14 +511,12 @@ int t16_blocks(const Scoring &sc) {
 }
 
 template <int R, bool DNA>
-cudaError_t t16_launch(const BatchView &b, const Scoring &sc, const T16Scratch &ts, int sms, int cls,
-                       cudaStream_t st) {
-    const int v = cls - kTraceT16First;
-    if (ts.dir_words[v] <= 0 || ts.warps[v] <= 0) return cudaSuccess;  // no pairs of the class
+cudaError_t t16_launch(const BatchView &b, const Scoring &sc, const T16Scratch &ts, int sms, int v, cudaStream_t st) {
     const int per_sm = t16_blocks<R, DNA>(sc);
     if (per_sm <= 0) return cudaErrorInvalidConfiguration;
-    const int grid = std::max(1, std::min(sms * per_sm, ts.warps[v] / (kT16Block / 32)));
-    k_trace16<R, DNA><<<grid, kT16Block, t16_smem_bytes<R, DNA>(sc), st>>>(b, sc, ts, cls);
+    const int wpb = kT16Block / 32;
+    const int grid = std::max(1, std::min(sms * per_sm, ts.warps / wpb));
+    k_trace16<R, DNA><<<grid, kT16Block, t16_smem_bytes<R, DNA>(sc), st>>>(b, sc, ts, kTraceT16First + v);
     return cudaGetLastError();
 }
 
@@ -539,19 +537,17 @@ int t16_max_warps(const Scoring &sc, int sms, int v) {
     return std::max(0, sms * per_sm) * (kT16Block / 32);
 }
 
-cudaError_t launch_trace16(const BatchView &b, const Scoring &sc, const T16Scratch &ts, int sms, cudaStream_t st) {
-    cudaError_t e;
-    const int c0 = kTraceT16First;
+cudaError_t launch_trace16(const BatchView &b, const Scoring &sc, const T16Scratch &ts, int sms, int v,
+                           cudaStream_t st) {
     if (sc.dna4) {
-        if ((e = t16_launch<16, true>(b, sc, ts, sms, c0 + 3, st))) return e;
-        if ((e = t16_launch<12, true>(b, sc, ts, sms, c0 + 2, st))) return e;
-        if ((e = t16_launch<8, true>(b, sc, ts, sms, c0 + 1, st))) return e;
-        if ((e = t16_launch<4, true>(b, sc, ts, sms, c0, st))) return e;
-    } else {
-        if ((e = t16_launch<8, false>(b, sc, ts, sms, c0 + 1, st))) return e;
-        if ((e = t16_launch<4, false>(b, sc, ts, sms, c0, st))) return e;
+        switch (v) {
+        case 0: return t16_launch<4, true>(b, sc, ts, sms, v, st);
+        case 1: return t16_launch<8, true>(b, sc, ts, sms, v, st);
+        case 2: return t16_launch<12, true>(b, sc, ts, sms, v, st);
+        default: return t16_launch<16, true>(b, sc, ts, sms, v, st);
+        }
     }
-    return cudaSuccess;
+    return v == 0 ? t16_launch<4, false>(b, sc, ts, sms, v, st) : t16_launch<8, false>(b, sc, ts, sms, v, st);
 }
 
 }  // namespace gsw

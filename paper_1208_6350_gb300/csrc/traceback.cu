@@ -30,43 +30,17 @@ constexpr int kNegT = -(1 << 28);
 constexpr int kNegHalf = -(1 << 27);
 constexpr int kAdLetters = 2048;  // per warp: query + target letters staged in shared memory
 
-// decision words of one pair: 8 anti-diagonals per word row, NCH x 32 words a row
-__host__ __device__ inline long long ad_dir_words(int la, int lb, int nch) {
-    return ((long long)(la + lb + 1 + 7) / 8) * nch * 32;
-}
-
-// pairs the thread-per-pair band kernel left to the warp tracebacks (band wider than 32)
-__device__ __forceinline__ bool wants_trace(const gsw_result &r) {
-    return r.score1 > 0 && (r.flags & kResPendingTrace) && !(r.flags & kResInternal) && r.read_begin1 >= 0 &&
-           r.ref_begin1 >= 0;
-}
-
-// Largest needs of a pair of the warp classes: [0] direction words of the
-// anti-diagonal classes, [1] op words (anti-diagonal and 16-bit classes);
-// need16[v]: direction words of 16-bit class v (per group of 8 lanes).
-__global__ void k_trace_need(BatchView b, Scoring sc, unsigned long long *max_need, unsigned long long *need16) {
+__global__ void k_trace_need(BatchView b, Scoring sc, unsigned long long *need) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned v[2 + kTraceT16Classes] = {};
-    if (p < b.npairs) {
-        const gsw_result r = b.res[p];
-        if (wants_trace(r)) {
-            const int la = r.read_end1 - r.read_begin1 + 1, lb = r.ref_end1 - r.ref_begin1 + 1;
-            int dlo, dhi;
-            const int cls = trace_class(la, lb, r.score1, sc, small_batch(b), &dlo, &dhi);
-            if (cls < kTraceRingClass) {
-                v[0] = (unsigned)min(ad_dir_words(la, lb, 1 << cls), (long long)UINT_MAX);
-                v[1] = (unsigned)min((long long)la + lb + 2, (long long)UINT_MAX);
-            } else if (cls >= kTraceT16First) {
-                v[2 + cls - kTraceT16First] =
-                    (unsigned)min(t16_need_words(la, lb, cls - kTraceT16First), (long long)UINT_MAX);
-                v[1] = (unsigned)min((long long)la + lb + 2, (long long)UINT_MAX);
-            }
-        }
-    }
+    unsigned v[kNeedWords] = {};
+    if (p < b.npairs) trace_needs(b.res[p], sc, small_batch(b), v);
 #pragma unroll
-    for (int k = 0; k < 2 + kTraceT16Classes; k++) {
-        const unsigned m = __reduce_max_sync(0xFFFFFFFFu, v[k]);
-        if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(k < 2 ? &max_need[k] : &need16[k - 2], (unsigned long long)m);
+    for (int k = 0; k < kNeedWords; k++) {
+        const unsigned m = k == kNeedMask ? __reduce_or_sync(0xFFFFFFFFu, v[k]) : __reduce_max_sync(0xFFFFFFFFu, v[k]);
+        if ((threadIdx.x & 31) == 0 && m > 0) {
+            if (k == kNeedMask) atomicOr(&need[k], (unsigned long long)m);
+            else atomicMax(&need[k], (unsigned long long)m);
+        }
     }
 }
 
@@ -264,24 +238,21 @@ __global__ void __launch_bounds__(kTBlock) k_trace_ad(BatchView b, Scoring sc, T
 }  // namespace
 
 
-cudaError_t launch_trace_ad(const BatchView &b, const Scoring &sc, const TraceScratch &ts, int grid,
+cudaError_t launch_trace_ad(const BatchView &b, const Scoring &sc, const TraceScratch &ts, int grid, unsigned mask,
                             cudaStream_t st) {
-    k_trace_ad<1><<<grid, kTBlock, 0, st>>>(b, sc, ts, 0);
-    k_trace_ad<2><<<grid, kTBlock, 0, st>>>(b, sc, ts, 1);
-    k_trace_ad<4><<<grid, kTBlock, 0, st>>>(b, sc, ts, 2);
-    k_trace_ad<8><<<grid, kTBlock, 0, st>>>(b, sc, ts, 3);
+    // the widest bands (the longest pairs) first
+    if (mask & 8u) k_trace_ad<8><<<grid, kTBlock, 0, st>>>(b, sc, ts, 3);
+    if (mask & 4u) k_trace_ad<4><<<grid, kTBlock, 0, st>>>(b, sc, ts, 2);
+    if (mask & 2u) k_trace_ad<2><<<grid, kTBlock, 0, st>>>(b, sc, ts, 1);
+    if (mask & 1u) k_trace_ad<1><<<grid, kTBlock, 0, st>>>(b, sc, ts, 0);
     return cudaGetLastError();
 }
 
 int trace_block_threads() { return kTBlock; }
 
-// Largest needs of the anti-diagonal classes: [0] direction words, [1] op words.
-cudaError_t launch_trace_need(const BatchView &b, const Scoring &sc, unsigned long long *max_need,
-                              unsigned long long *need16, cudaStream_t st) {
-    cudaMemsetAsync(max_need, 0, 2 * sizeof(unsigned long long), st);
-    cudaMemsetAsync(need16, 0, kTraceT16Classes * sizeof(unsigned long long), st);
+cudaError_t launch_trace_need(const BatchView &b, const Scoring &sc, unsigned long long *need, cudaStream_t st) {
     const int nb = (b.npairs + 255) / 256;
-    if (nb > 0) k_trace_need<<<nb, 256, 0, st>>>(b, sc, max_need, need16);
+    if (nb > 0) k_trace_need<<<nb, 256, 0, st>>>(b, sc, need);
     return cudaGetLastError();
 }
 
