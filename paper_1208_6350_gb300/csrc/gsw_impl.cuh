@@ -186,7 +186,7 @@ __host__ __device__ inline int pick_class_reverse(int rows, bool s32, const Scor
 // score + O + one matrix entry, which must stay within the integers half
 // precision holds exactly (2048); O >= -wmin keeps the sums of the shifted
 // scores non-negative (signed bytes outside the 4-letter alphabets).
-inline bool half_fits(int rows, int cols, const Scoring &sc) {
+__host__ __device__ inline bool half_fits(int rows, int cols, const Scoring &sc) {
     if (sc.O < -sc.wmin || (!sc.dna4 && sc.wmax + sc.O > 127)) return false;
     const long long top = sc.wmax > 0 ? sc.wmax : 0;
     return (rows < cols ? rows : cols) * top + top + sc.O <= 2047;
