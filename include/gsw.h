@@ -171,10 +171,11 @@ int gsw_context_set_tune(gsw_ctx *ctx, const gsw_tune *tune);
  * record gsw_align_batch would give for the pair (read, whole reference):
  * score1, ends, score2 / ref_end2 over the whole reference's max array,
  * begins and CIGAR (flags GSW_BEGIN, GSW_CIGAR), bit-exact.  The reference is
- * cut into windows owning `window` columns (0: the default, at least 65,536)
- * that start earlier by the longest reference span of a positive-scoring
- * local alignment of the longest read, so the work is one batch of
- * reads x windows plus two small passes.  Pointers follow gsw_align_batch's
+ * cut into windows owning `window` columns (0: chosen from the reference's
+ * length and the number of reads, at most 65,536 unless the reads are long)
+ * that start earlier by the longest reference span of a positive-scoring local
+ * alignment of the longest read, so the work is one batch of reads x windows
+ * plus two small passes.  Pointers follow gsw_align_batch's
  * rules (GSW_HOST_IO: all host); ref_len < 2^31; the reads' lengths < 2^24.
  * Work and the read-back of device read lengths are ordered on `stream`, so
  * inputs written by work queued there before the call are seen.

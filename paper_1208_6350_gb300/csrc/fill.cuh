@@ -411,7 +411,7 @@ struct StripRunner {
     // Returns true when the reverse fill found its target column.
     template <bool CHECKED, int MODE = kModeGen, int PK = -1>
     __device__ __forceinline__ bool step(const int s) {
-        constexpr bool FAST = MODE == kModeFast;
+        constexpr bool FAST = MODE == kModeFast, REV = MODE == kModeRev;
         const int jlo = s - k;
         const int jhi = L::FOLD ? jlo - P : jlo;
         uint32_t hin, fin, cmin;
@@ -421,7 +421,6 @@ struct StripRunner {
         hin = xh * mulh + bzh;
         fin = xf * mulh + bzf;
         cmin = xc * mulh + bzc;
-        constexpr bool REV = MODE == kModeRev;
         cm_t cm_prev{};
         if ((MODE == kModeGen || REV) ? st > 0 : MODE == kModeFwdLater) {
             const int bi = s & (P - 1);
@@ -465,14 +464,15 @@ struct StripRunner {
                     const int j2 = j1 - P;
                     nah = (j2 >= 0 && j2 < n) ? min((int)job.t[(long long)j2 * job.ts], A - 1) : 0;
                 }
-            } else if constexpr (FAST) {
-                // letters were checked before the fill (bad_letters, or the
-                // static entry's per-pair check): no clamp
-                nal = job.t[j1];
-                if constexpr (L::FOLD) nah = job.t[j1 - P];
             } else {
-                nal = min((int)job.t[(long long)j1 * job.ts], A - 1);
-                if constexpr (L::FOLD) nah = min((int)job.t[(long long)(j1 - P) * job.ts], A - 1);
+                // letters were checked before the fill (bad_letters, or the
+                // static entry's per-pair check): no clamp.  The direction is
+                // known in the specialised steps: one address and immediates
+                // instead of a 64-bit product per letter.
+                const long long at = MODE == kModeGen ? (long long)j1 * job.ts : REV ? -(long long)j1 : (long long)j1;
+                const long long back = MODE == kModeGen ? (long long)P * job.ts : REV ? -P : P;
+                nal = job.t[at];
+                if constexpr (L::FOLD) nah = job.t[at - back];
             }
         }
         // the two letters' scores: words to add (DNA), bytes to merge (other
@@ -636,8 +636,8 @@ struct StripRunner {
 #pragma unroll 1
         for (; s < s1 && s < s_steady; s++)
             if (step<true>(s)) return true;
-        const bool fwd = !job.stop_u && has_cms;
-        if (MAYBE_FAST && st == 0 && last_strip && fwd && job.ts == 1 && (!L::FOLD || n <= kFastMaxCols)) {
+        const bool fwd = !job.stop_u && has_cms && job.ts == 1;
+        if (MAYBE_FAST && st == 0 && last_strip && fwd && (!L::FOLD || n <= kFastMaxCols)) {
             if constexpr (L::FOLD) {
                 // blocks of 4 steps whose max-array values go out in one
                 // store (the first steady step's column is 0, so the blocks
@@ -667,7 +667,7 @@ struct StripRunner {
                 c_lo = (int)(int16_t)(cpk & 0xFFFFu);
                 c_hi = (int)(int16_t)(cpk >> 16);
             }
-        } else if (MAYBE_MULTI && L::FOLD && job.stop_u && n <= kFastMaxCols) {
+        } else if (MAYBE_MULTI && L::FOLD && job.stop_u && job.ts == -1 && n <= kFastMaxCols) {
             // steady reversed steps: no max array, the tracker's columns packed
             if constexpr (L::FOLD) {
                 cpk = ((uint32_t)c_hi << 16) | ((uint32_t)c_lo & 0xFFFFu);
@@ -900,6 +900,12 @@ __device__ __forceinline__ void slot_scratch(const FillScratch &scr, int slot, J
     job->bnd = (char *)scr.base + scr.bnd_off + slot * slot_bnd_bytes<L>(scr.ncap);
 }
 
+__device__ __forceinline__ void empty_record(gsw_result *rp) {
+    rp->score1 = 0; rp->score2 = 0; rp->ref_begin1 = -1; rp->ref_end1 = -1;
+    rp->read_begin1 = -1; rp->read_end1 = -1; rp->ref_end2 = -1; rp->cigar_len = 0;
+    rp->cigar_off = -1; rp->flags = 0; rp->reserved = 0;
+}
+
 template <int P, int R, class L, bool DNA>
 __device__ void run_task(const FillLaunch &fl, int first, int last, uint32_t *wsm, int lane, int slot_base) {
     const int g = lane / P, k = lane % P, gbase = g * P;
@@ -914,11 +920,7 @@ __device__ void run_task(const FillLaunch &fl, int first, int last, uint32_t *ws
     if (*fl.bad_letters) {
         // a letter outside the alphabet somewhere in the batch: no letter
         // is read (the steady steps index the profile unclamped)
-        if (k == 0 && fl.mode != kFillReverse) {
-            rp->score1 = 0; rp->score2 = 0; rp->ref_begin1 = -1; rp->ref_end1 = -1;
-            rp->read_begin1 = -1; rp->read_end1 = -1; rp->ref_end2 = -1; rp->cigar_len = 0;
-            rp->cigar_off = -1; rp->flags = 0; rp->reserved = 0;
-        }
+        if (k == 0 && fl.mode != kFillReverse) empty_record(rp);
         return;
     }
     Job job;
@@ -995,7 +997,7 @@ __global__ void __launch_bounds__(kBlock, fill_min_blocks(VID)) k_fill(FillLaunc
 // global scratch, one column at a time, so several strips of a pair can run
 // at once when each stays far enough behind the one above it.  The warps of a
 // cluster of CTAs (one 32-lane folded ring each; in 16-bit lanes 1,024 rows per
-// strip for DNA, 512 for general alphabets) advance in phases of kLongChunk
+// strip for DNA, 512 for general alphabets) advance in phases of CH (LongCfg)
 // steps separated by a cluster barrier, which also makes the previous phases'
 // global writes visible (they are read through L2).  Strip x+1 starts
 // long_lag() phases after strip x, so every boundary word and column maximum
@@ -1012,7 +1014,6 @@ __global__ void __launch_bounds__(kBlock, fill_min_blocks(VID)) k_fill(FillLaunc
 // Clusters: what bounds a batch of a few long reads is its longest pair.  On
 // one CTA a 20 kb read ran its 20 strips 4 at a time; on 8 CTAs all of them run
 // at once (kLongFewPairs).
-constexpr int kLongChunk = 128;
 constexpr int kLongSlots = 4;  // pairs in flight per CTA
 constexpr int kLongMaxCluster = 8;
 // Batches of at most this many pairs run on clusters of as many CTAs as the
@@ -1022,13 +1023,14 @@ constexpr int kLongMaxCluster = 8;
 // forward but 37.7 -> 43.9 ms reversed, where the CTAs are busy anyway; 300
 // reads of 1-3 kb, three strips at most, 1.43 -> 1.97 ms).
 constexpr int kLongFewPairs = 2048;
+constexpr int kLongNarrowPairs = 512;  // ... and reverse in narrow strips (LongCfg)
 
-template <class L>
+template <class L, int CH>
 __host__ __device__ constexpr int long_lag() {
     // strip x-1 writes column j at its step j + dw; strip x reads columns up
     // to s + 2P - 1 at step s: (lag - 1) * C >= 2P - 1 + dw
     constexpr int P = 32, dw = L::FOLD ? 2 * P - 1 : P - 1;
-    return 1 + (2 * P - 1 + dw + kLongChunk - 1) / kLongChunk;
+    return 1 + (2 * P - 1 + dw + CH - 1) / CH;
 }
 
 // Lag of a banded reversed fill, whose strip x+1 starts up to SP columns
@@ -1037,10 +1039,10 @@ __host__ __device__ constexpr int long_lag() {
 // + dw, so (lag - 1) * C >= SP + 2P - 1 + dw (16-bit DNA lanes: 10 phases).  The
 // same lag keeps strip x+2's writes after strip x+1's reads of the ping-pong
 // buffer (lag * C + dw > SP).
-template <class L, int SP>
+template <class L, int SP, int CH>
 __host__ __device__ constexpr int long_lag_band() {
     constexpr int P = 32, dw = L::FOLD ? 2 * P - 1 : P - 1;
-    return 1 + (SP + 2 * P - 1 + dw + kLongChunk - 1) / kLongChunk;
+    return 1 + (SP + 2 * P - 1 + dw + CH - 1) / CH;
 }
 
 struct LongSlot {
@@ -1102,7 +1104,7 @@ struct LongShared {
 };
 
 // Opens the next pair of class CLS in slot s; false when none is left.
-template <class L, int SP>
+template <class L, int SP, int CH>
 __device__ bool long_open(const FillLaunch &fl, int cls, LongSlot &S, int slot, int seq) {
     const int ntasks = fl.plan.task_hi[cls] - fl.plan.task_lo[cls];
     const int t = atomicAdd(&fl.plan.head[cls], 1);
@@ -1127,7 +1129,7 @@ __device__ bool long_open(const FillLaunch &fl, int cls, LongSlot &S, int slot, 
     } else {
         forward_job(fl.b, pair, &job);
     }
-    S.lag = S.band ? long_lag_band<L, SP>() : long_lag<L>();
+    S.lag = S.band ? long_lag_band<L, SP, CH>() : long_lag<L, CH>();
     S.job = job;
     S.pair = pair;
     S.seq = seq;
@@ -1146,7 +1148,7 @@ __device__ bool long_open(const FillLaunch &fl, int cls, LongSlot &S, int slot, 
 
 // The schedule of phase ph, by one warp: lane = slot, and lane = warp of the
 // cluster (nslots, nw <= 32); slot0 is the cluster's first scratch slot.
-template <class L, int NW, int SP>
+template <class L, int NW, int SP, int CH>
 __device__ void long_schedule(const FillLaunch &fl, int cls, LongShared<NW> &sh, int ph, int nw, int nslots,
                               int slot0, int nclusters, int lane) {
     static_assert(kLongSlots * kLongMaxCluster <= 32 && NW * kLongMaxCluster <= 32, "a lane per slot and warp");
@@ -1212,7 +1214,7 @@ __device__ void long_schedule(const FillLaunch &fl, int cls, LongShared<NW> &sh,
         const bool try_open = ((free_slots >> lane) & 1u) && rank < min(most, __popc(idle));
         const int seq = sh.seq + rank;
         bool ok = false;
-        if (try_open) ok = long_open<L, SP>(fl, cls, sh.slot[lane], slot0 + lane, seq);
+        if (try_open) ok = long_open<L, SP, CH>(fl, cls, sh.slot[lane], slot0 + lane, seq);
         const unsigned opened = __ballot_sync(ALL, ok);
         const bool none_left = __any_sync(ALL, try_open && !ok);
         if (ok) {
@@ -1239,7 +1241,7 @@ __device__ void long_schedule(const FillLaunch &fl, int cls, LongShared<NW> &sh,
     __syncwarp();
 }
 
-template <bool DNA, bool S32>
+template <bool DNA, bool S32, bool NARROW>
 struct LongCfg {
     using L = std::conditional_t<S32, L32, L16>;
     // DNA in 16-bit lanes: 16 row words per lane (1,024 rows per strip), so
@@ -1249,17 +1251,23 @@ struct LongCfg {
     // profile per CTA).  Measured on 10,000 long reads against 8 row words and
     // 8 warps (2 CTAs per SM): forward fill 265 -> 218 ms, reverse 105 -> 91
     // ms; 12 or 20-24 row words, 2 or 8 warps per CTA were slower.
-    static constexpr int P = 32, R = (DNA && !S32) ? 16 : 8;
+    // NARROW: the banded reversed fill of few pairs, whose time is the chain of
+    // strips along the band, each of which waits until the one above is a
+    // strip's rows and a phase ahead.  512-row strips and 64-step phases make
+    // the chain's steps half as long for a tenth more of them (300 reads of
+    // 1-20 kb: reverse 14.1 -> 12.7 ms; 1,000, which fill the chip: 18.1 -> 19.2).
+    static constexpr int P = 32, R = (DNA && !S32 && !NARROW) ? 16 : 8;
     static constexpr int NW = 4;
-    static constexpr int MINB = DNA ? 3 : 4;
+    static constexpr int MINB = DNA && !NARROW ? 3 : 4;
     static constexpr int SP = S32 ? P * R : 2 * P * R;
+        static constexpr int CH = NARROW ? 64 : 128;  // steps of a phase
     static constexpr int CLS = S32 ? kClassLong32 : kClassLong16;
 };
 
-template <bool DNA, bool S32>
-__global__ void __launch_bounds__(LongCfg<DNA, S32>::NW * 32, LongCfg<DNA, S32>::MINB)
+template <bool DNA, bool S32, bool NARROW>
+__global__ void __launch_bounds__(LongCfg<DNA, S32, NARROW>::NW * 32, LongCfg<DNA, S32, NARROW>::MINB)
     k_fill_long(FillLaunch fl, int warp_words) {
-    using C = LongCfg<DNA, S32>;
+    using C = LongCfg<DNA, S32, NARROW>;
     using L = typename C::L;
     constexpr int NW = C::NW, SP = C::SP;
     extern __shared__ __align__(16) uint32_t smem[];
@@ -1269,6 +1277,13 @@ __global__ void __launch_bounds__(LongCfg<DNA, S32>::NW * 32, LongCfg<DNA, S32>:
     const int cta_warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int warp = rank * NW + cta_warp;  // of the cluster
     const int nw = cl * NW, nslots = cl * kLongSlots;
+    if (*fl.bad_letters) {  // (as in run_task: no letter is read)
+        if (fl.mode != kFillReverse)
+            for (int x = fl.plan.var_start[C::CLS] + blockIdx.x * blockDim.x + threadIdx.x;
+                 x < fl.plan.var_start[C::CLS + 1]; x += gridDim.x * blockDim.x)
+                empty_record(fl.b.res + fl.plan.order[x]);
+        return;
+    }
     uint32_t *psm = smem + (size_t)cta_warp * warp_words;
     if (rank == 0) {
         if (threadIdx.x < nslots) sh_own.slot[threadIdx.x].pair = -1;
@@ -1293,7 +1308,7 @@ __global__ void __launch_bounds__(LongCfg<DNA, S32>::NW * 32, LongCfg<DNA, S32>:
     for (int ph = 0;; ph++) {
         barrier();
         if (rank == 0 && cta_warp == 0)
-            long_schedule<L, NW, SP>(fl, C::CLS, sh_own, ph, nw, nslots, (blockIdx.x / cl) * nslots,
+            long_schedule<L, NW, SP, C::CH>(fl, C::CLS, sh_own, ph, nw, nslots, (blockIdx.x / cl) * nslots,
                                          gridDim.x / cl, lane);
         barrier();
         if (sh.done) break;
@@ -1343,8 +1358,8 @@ __global__ void __launch_bounds__(LongCfg<DNA, S32>::NW * 32, LongCfg<DNA, S32>:
         bool stop = false, fin = S.stopped != 0;
         if (!fin) {
             const int q = ph - cmd.start;
-            stop = sr.template run<false>(q * kLongChunk, (q + 1) * kLongChunk);
-            fin = stop || (q + 1) * kLongChunk >= sr.nsteps;
+            stop = sr.template run<false>(q * C::CH, (q + 1) * C::CH);
+            fin = stop || (q + 1) * C::CH >= sr.nsteps;
         }
         if (fin) {
             int v, c, row;
@@ -1362,9 +1377,9 @@ __global__ void __launch_bounds__(LongCfg<DNA, S32>::NW * 32, LongCfg<DNA, S32>:
     barrier();  // the first CTA's shared memory stays until every warp has read `done`
 }
 
-template <bool DNA, bool S32>
+template <bool DNA, bool S32, bool NARROW>
 size_t long_smem_bytes(int A) {
-    using C = LongCfg<DNA, S32>;
+    using C = LongCfg<DNA, S32, NARROW>;
     return (size_t)prof_words(C::R, C::L::FOLD, DNA, A) * 32 * sizeof(uint32_t) * C::NW;
 }
 
@@ -1393,26 +1408,33 @@ struct OccupancyCache {
     }
 };
 
-template <bool DNA, bool S32>
+template <bool DNA, bool S32, bool NARROW = false>
 ClassGeom long_geom(const FillLaunch &fl, int sms) {
-    using C = LongCfg<DNA, S32>;
+    using C = LongCfg<DNA, S32, NARROW>;
     static OccupancyCache cache;
     ClassGeom g;
-    g.smem = long_smem_bytes<DNA, S32>(fl.sc.A);
-    g.grid = sms * cache.get(k_fill_long<DNA, S32>, C::NW * 32, fl.sc.A, g.smem,
-                             long_smem_bytes<DNA, S32>(DNA ? 4 : kMaxAlpha));
-    g.slots_per_block = kLongSlots;
+    // (DNA, so in the reversed fill a pair's band is what its strips run)
     const int ctas = ((fl.maxm + C::SP - 1) / C::SP + C::NW - 1) / C::NW;
     if (fl.b.npairs <= kLongFewPairs)
         while (g.cluster < ctas && g.cluster < kLongMaxCluster) g.cluster *= 2;
+    if constexpr (DNA && !S32 && !NARROW)
+        if (fl.mode == kFillReverse && g.cluster > 1 && fl.b.npairs <= kLongNarrowPairs)
+            return long_geom<DNA, S32, true>(fl, sms);
+    g.narrow = NARROW;
+    g.smem = long_smem_bytes<DNA, S32, NARROW>(fl.sc.A);
+    g.grid = sms * cache.get(k_fill_long<DNA, S32, NARROW>, C::NW * 32, fl.sc.A, g.smem,
+                             long_smem_bytes<DNA, S32, NARROW>(DNA ? 4 : kMaxAlpha));
+    g.slots_per_block = kLongSlots;
     g.cm = slot_cm_bytes<typename C::L>(fl.scr.ncap);
     g.bnd = slot_bnd_bytes<typename C::L>(fl.scr.ncap);
     return g;
 }
 
-template <bool DNA, bool S32>
+template <bool DNA, bool S32, bool NARROW = false>
 cudaError_t launch_long(const FillLaunch &fl, const ClassGeom &g, cudaStream_t st) {
-    using C = LongCfg<DNA, S32>;
+    using C = LongCfg<DNA, S32, NARROW>;
+    if constexpr (DNA && !S32 && !NARROW)
+        if (g.narrow) return launch_long<DNA, S32, true>(fl, g, st);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(g.grid);
     cfg.blockDim = dim3(C::NW * 32);
@@ -1424,7 +1446,7 @@ cudaError_t launch_long(const FillLaunch &fl, const ClassGeom &g, cudaStream_t s
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_fill_long<DNA, S32>, fl, (int)(g.smem / sizeof(uint32_t) / C::NW));
+    return cudaLaunchKernelEx(&cfg, k_fill_long<DNA, S32, NARROW>, fl, (int)(g.smem / sizeof(uint32_t) / C::NW));
 }
 
 template <bool DNA, int VID, bool HALF>

@@ -617,6 +617,7 @@ cudaError_t launch_count_flag(const gsw_result *res, int32_t n, int32_t flag, un
 struct ClassGeom {
     int grid = 0, slots_per_block = 0;
     int cluster = 1;  // CTAs that share their pairs (the CTA classes)
+    bool narrow = false;  // the CTA kernel of narrow strips
     size_t cm = 0, bnd = 0;  // bytes per slot
     size_t smem = 0;
     size_t bytes(int blocks) const {

