@@ -216,7 +216,7 @@ enum MiscSlot {
 // Side streams and fork/join events of the fill and band classes, created once per
 // context outside any capture (the first call of a shape is never captured).
 void destroy_aux(SideStreams &a) {
-    for (int k = 0; k < 2; k++) {
+    for (int k = 0; k < kSideStreams; k++) {
         if (a.s[k]) cudaStreamDestroy(a.s[k]);
         if (a.join[k]) cudaEventDestroy(a.join[k]);
     }
@@ -229,7 +229,7 @@ int ensure_aux(gsw_ctx *ctx) {
     if (ctx->capturing) return GSW_ESTATE;
     SideStreams a{};
     cudaError_t e = cudaSuccess;
-    for (int k = 0; k < 2 && e == cudaSuccess; k++) {
+    for (int k = 0; k < kSideStreams && e == cudaSuccess; k++) {
         e = cudaStreamCreateWithFlags(&a.s[k], cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&a.join[k], cudaEventDisableTiming);
     }
@@ -558,12 +558,13 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
             int t16_warps[kTraceT16Classes] = {};
             auto t16_dir = [&](int v) { return ((long long)need[kNeed16 + v] + 3) & ~3LL; };
             auto size_t16 = [&](int v, size_t room_bytes) {
-                const size_t per_warp = 4 * (size_t)(t16_dir(v) + ad_ops) * sizeof(uint32_t);
+                const size_t groups = 32 / (size_t)t16_shape(v, sc.dna4 != 0).P;  // of a warp
+                const size_t per_warp = groups * (size_t)(t16_dir(v) + ad_ops) * sizeof(uint32_t);
                 size_t w = std::min<size_t>((size_t)t16_max_warps(sc, ctx->sms, v), std::max<size_t>(1, room_bytes / per_warp));
-                w = std::min<size_t>(w, ((size_t)npairs + 15) / 16 * 4);  // (whole blocks of 4 warps)
+                w = std::min<size_t>(w, ((size_t)npairs + groups * 4 - 1) / (groups * 4) * 4);  // (whole blocks of 4 warps)
                 t16_warps[v] = (int)w;
-                t16[v].dirs = std::max<size_t>(w, 4) * 4 * (size_t)t16_dir(v);
-                t16[v].ops = words16(std::max<size_t>(w, 4) * 4 * (size_t)ad_ops);
+                t16[v].dirs = std::max<size_t>(w, 4) * groups * (size_t)t16_dir(v);
+                t16[v].ops = words16(std::max<size_t>(w, 4) * groups * (size_t)ad_ops);
             };
             // wide bands: the pool of direction words, groups of pairs that fit it
             const unsigned long long ring_total = need[2], ring_max = need[3], ring_ops = need[4];
@@ -579,6 +580,9 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
             size_t all = bytes(ad) + bytes(ring);
             for (const Part &x : t16) all += bytes(x);
             const bool side = all <= have / 2 && ctx->aux.fork && ctx->sms == ctx->sms_all;
+            int nside = (ring_total > 0) + (ad_dir > 0) - 1;
+            for (int v = 0; v < kTraceT16Classes; v++) nside += t16_warps[v] > 0;
+            static_assert(kTraceT16Classes + 2 <= kSideStreams + 1, "a stream per traceback kernel");
             size_t max_dir = 0, max_ops = 0;
             size_t ring_pool = (size_t)ring_total;
             auto place = [&](Part &x) {
@@ -608,11 +612,16 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
                                 max_ops * sizeof(uint32_t)));
                 uint32_t *dirs = reinterpret_cast<uint32_t *>(ctx->trace_dirs.p);
                 uint32_t *ops = reinterpret_cast<uint32_t *>(ctx->trace_ops.p);
-                if (side) {
+                if (side && nside > 0) {
                     CUDA_TRY(cudaEventRecord(ctx->aux.fork, st));
-                    for (int k = 0; k < 2; k++) CUDA_TRY(cudaStreamWaitEvent(ctx->aux.s[k], ctx->aux.fork, 0));
+                    for (int k = 0; k < nside; k++) CUDA_TRY(cudaStreamWaitEvent(ctx->aux.s[k], ctx->aux.fork, 0));
                 }
-                const cudaStream_t on[3] = {st, side ? ctx->aux.s[0] : st, side ? ctx->aux.s[1] : st};
+                // a stream per kernel (nside streams beside the caller's)
+                int turn = 0;
+                auto next_stream = [&]() {
+                    const int k = turn++;
+                    return side && k > 0 ? ctx->aux.s[k - 1] : st;
+                };
                 if (ring_total > 0) {
                     RingLaunchArgs ra;
                     ra.b = bv;
@@ -634,8 +643,9 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
                     const unsigned long long per = ring_pool > ring_max ? ring_pool - ring_max : 1;
                     const unsigned long long groups =
                         ring_total <= ring_pool ? 1 : (ring_total + per - 1) / per + 1;
+                    const cudaStream_t on = next_stream();
                     for (unsigned long long gi = 0; gi < groups; gi++) {
-                        CUDA_TRY(launch_ring_group(ra, ctx->sms, on[0]));
+                        CUDA_TRY(launch_ring_group(ra, ctx->sms, on));
                         S.launches += 4;
                     }
                     S.ring_words = (long long)ring_total;
@@ -650,10 +660,9 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
                     ts.op_words = ad_ops;
                     ts.order = pb.order;
                     ts.var_start = pb.var_start;
-                    CUDA_TRY(launch_trace_ad(bv, sc, ts, ad_warps / wpb, (unsigned)need[kNeedMask], on[1]));
+                    CUDA_TRY(launch_trace_ad(bv, sc, ts, ad_warps / wpb, (unsigned)need[kNeedMask], next_stream()));
                     S.launches += __builtin_popcount((unsigned)need[kNeedMask]);
                 }
-                int turn = ring_total > 0 || ad_dir > 0 ? 2 : 0;
                 for (int v = kTraceT16Classes - 1; v >= 0; v--) {
                     if (t16_warps[v] <= 0) continue;
                     T16Scratch ts{};
@@ -665,12 +674,11 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
                     ts.var_start = pb.var_start;
                     ts.head = pb.head;
                     ts.warps = t16_warps[v];
-                    CUDA_TRY(launch_trace16(bv, sc, ts, ctx->sms, v, on[turn]));
-                    turn = (turn + 1) % 3;
+                    CUDA_TRY(launch_trace16(bv, sc, ts, ctx->sms, v, next_stream()));
                     S.launches += 1;
                 }
                 if (side)
-                    for (int k = 0; k < 2; k++) {
+                    for (int k = 0; k < nside; k++) {
                         CUDA_TRY(cudaEventRecord(ctx->aux.join[k], ctx->aux.s[k]));
                         CUDA_TRY(cudaStreamWaitEvent(st, ctx->aux.join[k], 0));
                     }
@@ -860,7 +868,7 @@ int batch_impl(gsw_ctx *ctx, int32_t npairs, const uint8_t *q, const int64_t *q_
         maxm = (int)bucket_up((uint64_t)maxm);
         maxn = (int)bucket_up((uint64_t)maxn);
     }
-    default_classes(sc, npairs, maxn, cells);
+    default_classes(sc, npairs, maxm, maxn, cells);
     // (2-bit letters are 0..3: valid under any matrix of 4 or more letters)
     if (!((flags & GSW_PACKED2) && sc.A >= 4)) {
         CUDA_TRY(launch_validate(bv, sc, reinterpret_cast<int32_t *>(misc + kMiscValid), st));

@@ -83,7 +83,7 @@ cudaError_t launch_fill(const FillLaunch &fl, int sms, cudaStream_t st, const Si
     cudaError_t e = cudaSuccess;
     if (side) {
         if ((e = cudaEventRecord(aux.fork, st))) return e;
-        for (int k = 0; k < 2 && k + 1 < n; k++)
+        for (int k = 0; k < kSideStreams && k + 1 < n; k++)
             if ((e = cudaStreamWaitEvent(aux.s[k], aux.fork, 0))) return e;
     }
     for (int i = 0; i < n && e == cudaSuccess; i++) {
@@ -93,14 +93,15 @@ cudaError_t launch_fill(const FillLaunch &fl, int sms, cudaStream_t st, const Si
         else if (!fit_scratch(g, fl.scr.bytes)) return cudaErrorInvalidConfiguration;
         if (g.grid < 1) return cudaErrorInvalidConfiguration;
         x.scr.bnd_off = align256((size_t)g.grid * g.slots_per_block * g.cm);
-        const cudaStream_t on = side && i % 3 ? aux.s[i % 3 - 1] : st;
+        const int turn = i % (kSideStreams + 1);
+        const cudaStream_t on = side && turn ? aux.s[turn - 1] : st;
         const int c = todo[i].c;
         const bool half = ((fl.half_mask >> c) & 1u) != 0;
         e = fl.sc.dna4 ? (half ? fill_launch_dna_half(c, x, g, on) : fill_launch_dna(c, x, g, on))
                        : (half ? fill_launch_general_half(c, x, g, on) : fill_launch_general(c, x, g, on));
     }
     if (side)
-        for (int k = 0; k < 2 && k + 1 < n; k++) {
+        for (int k = 0; k < kSideStreams && k + 1 < n; k++) {
             cudaError_t e2 = cudaEventRecord(aux.join[k], aux.s[k]);
             if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(st, aux.join[k], 0);
             if (e == cudaSuccess) e = e2;

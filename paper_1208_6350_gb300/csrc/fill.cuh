@@ -237,15 +237,6 @@ __device__ __forceinline__ void load_words(const uint32_t *base, int c, int l, u
     }
 }
 
-// Row 2w + odd of byte-profile words lo (the low letter's) and hi (the high
-// letter's): the low half's score of lo and the high half's of hi, sign-extended
-__device__ __forceinline__ uint32_t merge_bytes(uint32_t lo, uint32_t hi, int odd) {
-    uint32_t r;
-    if (odd) asm("prmt.b32 %0, %1, %2, 0xF7A2;" : "=r"(r) : "r"(lo), "r"(hi));
-    else asm("prmt.b32 %0, %1, %2, 0xD580;" : "=r"(r) : "r"(lo), "r"(hi));
-    return r;
-}
-
 __device__ __forceinline__ int sc_w(const Scoring &sc, int a, int b) { return sc.W[a * sc.A + b]; }
 
 // Builds this lane's profile for strip `st` (padded rows of the strip:

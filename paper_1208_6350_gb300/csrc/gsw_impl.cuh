@@ -197,7 +197,8 @@ __host__ __device__ inline bool half_fits(int rows, int cols, const Scoring &sc)
 __host__ __device__ inline bool cta_pair(int v, int rows, int cols, const Scoring &sc) {
     if (sc.cta_steps <= 0 || v >= kNumVariants || v == kVarS32) return false;
     const int strips = (rows + variant_rows(v) - 1) / variant_rows(v);
-    return strips > 1 && (long long)strips * cols > sc.cta_steps;
+    // (a step's time grows with its row words; 0.3 us is that of 8)
+    return strips > 1 && (long long)strips * cols * (4 + variant_at(v).R) > 12LL * sc.cta_steps;
 }
 
 // Chooses the fill classes of a batch's untuned buckets from its size (pairs,
@@ -217,8 +218,8 @@ __host__ __device__ inline bool cta_pair(int v, int rows, int cols, const Scorin
 // runs its strips side by side on a CTA (600 x 1,000 DNA: 1,851 GCUPS against
 // 1,513 at 3,000 pairs, 1,961 against 2,321 at 10,000; 350 x 360 protein: 691
 // against 330 at 1,000 pairs, 1,352 against 1,468 at 10,000).
-inline void default_classes(Scoring &sc, int npairs, int maxn, double cells) {
-    constexpr int kWide = 8192, kNarrow = 16384;
+inline void default_classes(Scoring &sc, int npairs, int maxm, int maxn, double cells) {
+    constexpr int kWide = 8192, kNarrow = 16384, kFewPairs = 2048;
     // (a power of two: batches of like size keep their captured graphs)
     sc.cta_steps = 256;
     while (sc.cta_steps < cells * 3.5e-7 && sc.cta_steps < (1 << 28)) sc.cta_steps *= 2;
@@ -255,6 +256,13 @@ inline void default_classes(Scoring &sc, int npairs, int maxn, double cells) {
         sc.fill_class[b] = (int8_t)(pick >= kVarP8First ? 9 + (pick - kVarP8First) : pick);
         sc.rev_class[b] = (int8_t)(pick16 + 1);
     }
+    // a batch that leaves the chip half empty reverses every query (of one strip)
+    // in the longest one's class: one launch instead of one per class below it,
+    // and its time is the longest pair's anyway
+    const int top = maxm < 1 ? 0 : (maxm - 1) / GSW_TUNE_ROWS;
+    if (npairs < kFewPairs && top < GSW_TUNE_BUCKETS && sc.rev_class[top] > 0 && variant_rows(sc.rev_class[top] - 1) >= maxm)
+        for (int b = 0; b < top; b++)
+            if (sc.rev_class[b] > 0) sc.rev_class[b] = sc.rev_class[top];
 }
 
 // The fill classes a launch of `mode` can meet when every query has minm to
@@ -486,6 +494,7 @@ constexpr long long kT16MaxWords = 1 << 17;  // scratch words of one pair (512 K
 // 128-row class with this allowance (its own launch and scratch, so the few
 // large pairs do not shrink the groups of the others)
 constexpr long long kT16MaxWordsBig = 1 << 20;
+// Class v as trace_class names and sizes it: 8 lanes, strips of 64(v+1) rows.
 __host__ __device__ inline int t16_R(int v) { return 4 * (v + 1); }
 __host__ __device__ inline int t16_strip_rows(int v) { return 2 * kT16P * t16_R(v); }
 __host__ __device__ inline int t16_strips(int la, int v) { return (la + t16_strip_rows(v) - 1) / t16_strip_rows(v); }
@@ -499,6 +508,31 @@ __host__ __device__ inline long long t16_dir_words(int la, int lb, int v) {
 __host__ __device__ inline long long t16_need_words(int la, int lb, int v) {
     const long long d = t16_dir_words(la, lb, v);
     return t16_strips(la, v) > 1 ? d + 2LL * ((lb + 3) & ~3) : d;
+}
+// How launch class v runs: P lanes a pair and R row words a lane, so strips of
+// 2PR rows.  DNA: as its name says.  Other alphabets have three launches: v = 0
+// (64-row strips), and whole warps with 256-row strips for v = 1 (regions whose
+// decisions are too many for v = 0's scratch) and v = 2 (regions of v = 0 taller
+// than kT16Tall rows): a group of 8 lanes runs the 16 strips of a 1,000-row
+// region one after the other, and beside the bulk of the pairs those few
+// regions then ended last (40 x 1,000 protein pairs: traceback 9.0 -> 5.9 ms).
+struct T16Shape {
+    int P, R;
+    __host__ __device__ int rows() const { return 2 * P * R; }
+    __host__ __device__ int strips(int la) const { return (la + rows() - 1) / rows(); }
+    __host__ __device__ int steps(int lb) const { return lb + 2 * P - 1; }
+    __host__ __device__ long long need_words(int la, int lb) const {
+        const long long d = (long long)strips(la) * steps(lb) * (R / 4) * P;
+        return strips(la) > 1 ? d + 2LL * ((lb + 3) & ~3) : d;
+    }
+};
+constexpr int kT16Tall = 256;
+__host__ __device__ inline T16Shape t16_shape(int v, bool dna) {
+    return dna ? T16Shape{kT16P, t16_R(v)} : (v == 0 ? T16Shape{kT16P, 4} : T16Shape{32, 4});
+}
+// launch class of a region trace_class gave class c
+__host__ __device__ inline int t16_launch_class(int c, int la, bool dna) {
+    return !dna && c == kTraceT16First && la > kT16Tall ? kTraceT16First + 2 : c;
 }
 // small: a batch of fewer than 2^14 pairs (the rectangle needs a wider margin
 // there, where the anti-diagonal kernel's one pair per warp keeps more pairs
@@ -523,8 +557,11 @@ __host__ __device__ inline int trace_class(int la, int lb, int score1, const Sco
         // every value of the DP over the padded rectangle lies in
         // [-(3O + X(rows + cols) + |wmin|), wmax * min(rows, cols) + wmax]:
         // it must fit a biased 16-bit lane
-        const long long lo = 3LL * sc.O + (long long)sc.X * (rows + cols + 2) - (sc.wmin < 0 ? sc.wmin : 0);
-        const long long hi = (long long)sc.wmax * ((cols < rows ? cols : rows) + 1);
+        const T16Shape shape = t16_shape(t16_launch_class(kTraceT16First + v, la, sc.dna4 != 0) - kTraceT16First,
+                                         sc.dna4 != 0);
+        const long long padded = (long long)shape.strips(la) * shape.rows();
+        const long long lo = 3LL * sc.O + (long long)sc.X * (padded + cols + 2) - (sc.wmin < 0 ? sc.wmin : 0);
+        const long long hi = (long long)sc.wmax * ((cols < padded ? cols : padded) + 1);
         if (lo <= 30000 && hi <= 30000 && t16_need_words(la, lb, v) <= cap) {
             // cell updates: the padded rectangle against the band's
             // anti-diagonal slots; a 16-bit pair of cells costs about the
@@ -555,7 +592,7 @@ __host__ __device__ inline bool wants_trace(const gsw_result &r) {
 // anti-diagonal classes, [1] op words (anti-diagonal and 16-bit classes),
 // [2..4] wide bands (launch_ring_needs: total words, largest pair, largest op
 // words), [5] bit c: anti-diagonal class c has pairs, [6 + v] direction words of
-// 16-bit class v (per group of 8 lanes)
+// 16-bit launch class v (per group)
 constexpr int kNeedMask = 5, kNeed16 = 6, kNeedWords = kNeed16 + kTraceT16Classes;
 // A pair's share of those (v zeroed by the caller; the ring words are not set).
 __host__ __device__ inline void trace_needs(const gsw_result &r, const Scoring &sc, bool small, unsigned v[kNeedWords]) {
@@ -571,7 +608,8 @@ __host__ __device__ inline void trace_needs(const gsw_result &r, const Scoring &
         v[0] = capped(ad_dir_words(la, lb, 1 << cls));
         v[kNeedMask] = 1u << cls;
     } else {
-        v[kNeed16 + cls - kTraceT16First] = capped(t16_need_words(la, lb, cls - kTraceT16First));
+        const int c = t16_launch_class(cls, la, sc.dna4 != 0) - kTraceT16First;
+        v[kNeed16 + c] = capped(t16_shape(c, sc.dna4 != 0).need_words(la, lb));
     }
 }
 
@@ -590,6 +628,17 @@ inline bool ring_possible(int maxm, int maxn, const Scoring &sc) {
     if (sc.dna4) return t16_need_words(m, n, kTraceT16Classes - 1) > kT16MaxWords;
     return t16_need_words(m, n, 0) > kT16MaxWords && t16_need_words(m, n, 1) > kT16MaxWordsBig;
 }
+
+#ifdef __CUDACC__
+// Row 2w + odd of byte-profile words lo (the low letter's) and hi (the high
+// letter's): the low half's score of lo and the high half's of hi, sign-extended
+__device__ __forceinline__ uint32_t merge_bytes(uint32_t lo, uint32_t hi, int odd) {
+    uint32_t r;
+    if (odd) asm("prmt.b32 %0, %1, %2, 0xF7A2;" : "=r"(r) : "r"(lo), "r"(hi));
+    else asm("prmt.b32 %0, %1, %2, 0xD580;" : "=r"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+#endif
 
 // stage launchers (host side, enqueue on `st`)
 // Status of a completed batch from what its kernels counted, in order of
@@ -626,9 +675,12 @@ struct ClassGeom {
 };
 // scratch bytes with which every class of fl.class_mask runs at full occupancy
 size_t fill_scratch_want(const FillLaunch &fl, int sms);
+// (a stream per kernel, as far as they go: kernels that share one wait for each
+// other's longest pair)
+constexpr int kSideStreams = 7;
 struct SideStreams {
-    cudaStream_t s[2];
-    cudaEvent_t fork, join[2];
+    cudaStream_t s[kSideStreams];
+    cudaEvent_t fork, join[kSideStreams];
 };
 // one persistent launch per class in fl.class_mask, heaviest first, each with
 // the slots its share of the scratch holds; side by side on `st` and the side
@@ -709,8 +761,8 @@ cudaError_t launch_trace_need(const BatchView &b, const Scoring &sc, unsigned lo
 cudaError_t launch_trace_ad(const BatchView &b, const Scoring &sc, const TraceScratch &ts, int grid, unsigned mask,
                             cudaStream_t st);
 
-// 16-bit full-rectangle traceback (trace16.cu), class v (strips of 64(v+1)
-// rows): direction and op words per group of 8 lanes, 4 groups a warp
+// 16-bit full-rectangle traceback (trace16.cu), launch class v (t16_shape):
+// direction and op words per group of P lanes, 32/P groups a warp
 struct T16Scratch {
     uint32_t *dirs;
     int64_t dir_words;  // per group
@@ -719,7 +771,7 @@ struct T16Scratch {
     const int32_t *order;
     const int32_t *var_start;
     int32_t *head;      // per-class task counters (zeroed by the plan)
-    int warps;          // of the launch (the scratch holds 4 groups each)
+    int warps;          // of the launch (the scratch holds 32/P groups each)
 };
 // warps of class v's launch that can be resident
 int t16_max_warps(const Scoring &sc, int sms, int v);

@@ -72,10 +72,13 @@ __device__ int plan_key(const BatchView &b, const Scoring &sc, int32_t mode, int
         int dlo, dhi;
         // 0-3: anti-diagonal warp kernel (<= 64/128/256/512 diagonals); 4:
         // wider bands, the CTA strip kernel; 5-8: the 16-bit rectangle
-        const int cls = trace_class(la, lb, r.score1, sc, small_batch(b), &dlo, &dhi);
+        const int cls = t16_launch_class(trace_class(la, lb, r.score1, sc, small_batch(b), &dlo, &dhi), la, sc.dna4 != 0);
         const int width = dhi - dlo + 1;
-        const long long cost = cls >= kTraceT16First ? (long long)t16_strips(la, cls - kTraceT16First) * t16_steps(lb)
-                                                     : (long long)(la + lb + 1) * ((width + 31) / 32);
+        long long cost = (long long)(la + lb + 1) * ((width + 31) / 32);
+        if (cls >= kTraceT16First) {
+            const T16Shape shape = t16_shape(cls - kTraceT16First, sc.dna4 != 0);
+            cost = (long long)shape.strips(la) * shape.steps(lb);
+        }
         return cls * kPlanBinsPerVariant + cost_bin(cost);
     } else {
         // kPlanBand: classes 0/1/2 = band width <= 8/16/32 diagonals

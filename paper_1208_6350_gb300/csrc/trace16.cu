@@ -11,7 +11,8 @@
 // rectangle in the folded ring of the fill (fill.cu) costs about a quarter of
 // the instructions per cell of the 32-bit anti-diagonal kernel.
 //
-// Layout: a group of 8 lanes per pair; lane k holds R 32-bit words, word r
+// Layout: a group of P lanes per pair (8, or 32 for tall regions of general
+// alphabets; the text below says 8); lane k holds R 32-bit words, word r
 // packing row k*R + r (bits 0-15) and row S + k*R + r (bits 16-31), S = 8R,
 // each as value + 0x8000.  Step s computes target column s - k of the low
 // half and column s - k - 8 of the high half; the bottom row (H, F) goes down
@@ -39,35 +40,44 @@
 
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 namespace gsw {
 namespace {
 
 constexpr int kT16Block = 128;
-constexpr int kP = kT16P;
 
 // per-lane profile words: DNA a low-letter and a high-letter table (4 + 4
 // letters x R words, plain integers w and w * 65536: H(i-1,j-1) + W is one
-// 3-input add); other alphabets one table of A letters x R words with both
-// halves' scores (16-bit two's-complement halves)
-__host__ __device__ inline int t16_prof_words(int R, bool dna, int A) { return dna ? 8 * R : A * R; }
+// 3-input add); other alphabets one byte per score, both halves' scores of two
+// rows in a word, merged by the step's byte permute (as in the fill)
+__host__ __device__ inline int t16_prof_words(int R, bool dna, int A) { return dna ? 8 * R : A * R / 2; }
 
-// word (table entry c, row r) of lane l inside a warp's region: lane-minor
-// 16-byte vectors, so the 8 lanes of a quarter warp cover all 32 banks
-template <int R>
+// word (table entry c, word r of PW) of lane l inside a warp's region:
+// lane-minor 16-byte vectors (8-byte ones when a lane has two words), so the
+// lanes of a quarter (or half) warp cover all 32 banks
+template <int PW>
 __device__ __forceinline__ int t16_pidx(int c, int r, int l) {
-    return ((c * (R / 4) + r / 4) * 32 + l) * 4 + (r & 3);
+    constexpr int V = PW % 4 == 0 ? 4 : 2;
+    return ((c * (PW / V) + r / V) * 32 + l) * V + (r & (V - 1));
 }
 
-template <int R>
-__device__ __forceinline__ void t16_load(const uint32_t *base, int c, int l, uint32_t (&w)[R]) {
+template <int PW>
+__device__ __forceinline__ void t16_load(const uint32_t *base, int c, int l, uint32_t (&w)[PW]) {
+    if constexpr (PW % 4 == 0) {
 #pragma unroll
-    for (int r = 0; r < R; r += 4) {
-        const uint4 v = *reinterpret_cast<const uint4 *>(base + t16_pidx<R>(c, r, l));
-        w[r] = v.x;
-        w[r + 1] = v.y;
-        w[r + 2] = v.z;
-        w[r + 3] = v.w;
+        for (int r = 0; r < PW; r += 4) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(base + t16_pidx<PW>(c, r, l));
+            w[r] = v.x;
+            w[r + 1] = v.y;
+            w[r + 2] = v.z;
+            w[r + 3] = v.w;
+        }
+    } else {
+        static_assert(PW == 2, "two words or vectors of four");
+        const uint2 v = *reinterpret_cast<const uint2 *>(base + t16_pidx<PW>(c, 0, l));
+        w[0] = v.x;
+        w[1] = v.y;
     }
 }
 
@@ -76,8 +86,12 @@ __device__ __forceinline__ uint32_t t16_edge(int i, int O, int X) {
     return (uint32_t)(0x8000 - (i == 0 ? 0 : O + (i - 1) * X)) & 0xFFFFu;
 }
 
-template <int R, bool DNA>
+// SHIFT (other alphabets whose scores span at most 127): the bytes hold
+// W - wmin >= 0, so H(i-1,j-1) + W is a plain 3-input add; else a saturation-free
+// add-max of signed halves.
+template <int kP, int R, bool DNA, bool SHIFT>
 struct T16Runner {
+    static constexpr int PW = DNA ? R : R / 2;  // profile words per letter
     static constexpr int S = kP * R;
     static constexpr int SS = 2 * S;  // rows of a strip
     static constexpr int Q = R / 4;
@@ -90,7 +104,7 @@ struct T16Runner {
     const uint32_t *bin;  // previous strip's last row: H | F(next row) << 16 per column
     uint32_t *bout;
     int lane;
-    uint32_t kO, kXm, hb0, stepX;
+    uint32_t kO, kXm, hb0, stepX, kW;
     uint32_t H[R], E[R];
     uint32_t xh, xf, hdiag, b_cur, b_nxt;
     int nal, nah;
@@ -116,6 +130,7 @@ struct T16Runner {
         psm = psm_;
         fin_words = fin_words_;
         kO = (uint32_t)(-O * 65537);
+        kW = SHIFT ? (uint32_t)(sc.wmin * 65537) : 0u;
         kXm = ((uint32_t)(-X) & 0xFFFFu) * 0x10001u;
         stepX = (uint32_t)X * 0x10001u;
         st_fin = (la - 1) / SS;
@@ -155,10 +170,12 @@ struct T16Runner {
                     psm[t16_pidx<R>(4 + a, r, lane)] = (uint32_t)(wh * 65536);
                 }
             } else {
+                uint8_t *bytes = reinterpret_cast<uint8_t *>(psm);
+                const int add = SHIFT ? -sc.wmin : 0;
                 for (int a = 0; a < A; a++) {
-                    const int wl = qlo >= 0 ? sc.W[qlo * A + a] : 0;
-                    const int wh = qhi >= 0 ? sc.W[qhi * A + a] : 0;
-                    psm[t16_pidx<R>(a, r, lane)] = ((uint32_t)wl & 0xFFFFu) | (((uint32_t)wh & 0xFFFFu) << 16);
+                    uint8_t *p = bytes + 4 * t16_pidx<PW>(a, r / 2, lane) + 2 * (r & 1);
+                    p[0] = (uint8_t)((qlo >= 0 ? sc.W[qlo * A + a] : 0) + add);
+                    p[1] = (uint8_t)((qhi >= 0 ? sc.W[qhi * A + a] : 0) + add);
                 }
             }
         }
@@ -181,7 +198,7 @@ struct T16Runner {
         if (st > 0) prefetch(0);
     }
 
-    // The previous strip's row for columns [s0, s0 + 8): lane k loads column
+    // The previous strip's row for columns [s0, s0 + kP): lane k loads column
     // s0 + k, lane 0 takes each by a shuffle in its step
     __device__ __forceinline__ void prefetch(int s0) {
         const int j = s0 + k;
@@ -221,14 +238,9 @@ struct T16Runner {
                 nah = min((int)ts[j1 - kP], A - 1);
             }
         }
-        uint32_t pw[R], ph[R];
-        if constexpr (DNA) {
-            t16_load<R>(psm, al, lane, pw);
-            t16_load<R>(psm, 4 + ah, lane, ph);
-        } else {
-            t16_load<R>(psm, al, lane, pw);
-            t16_load<R>(psm, ah, lane, ph);
-        }
+        uint32_t pw[PW], ph[PW];
+        t16_load<PW>(psm, al, lane, pw);
+        t16_load<PW>(psm, DNA ? 4 + ah : ah, lane, ph);
         uint32_t diag = hdiag;
         hdiag = hin;
         uint32_t f = fin;
@@ -240,7 +252,8 @@ struct T16Runner {
         for (int r = 0; r < R; r++) {
             uint32_t hdg;
             if constexpr (DNA) hdg = diag + pw[r] + ph[r];
-            else hdg = __viaddmax_u16x2(diag, (pw[r] & 0x0000FFFFu) | (ph[r] & 0xFFFF0000u), 0u);
+            else if constexpr (SHIFT) hdg = diag + merge_bytes(pw[r / 2], ph[r / 2], r & 1) + kW;
+            else hdg = __viaddmax_u16x2(diag, merge_bytes(pw[r / 2], ph[r / 2], r & 1), 0u);
             const uint32_t e = E[r];
             const uint32_t h = __vmaxu2(hdg, __vmaxu2(e, f));
             const uint32_t ho = h + kO;
@@ -285,7 +298,7 @@ struct T16Runner {
     // the strip over every column: start-up (some half before its first
     // column), steady (every column in range), drain (columns past lb)
     __device__ __forceinline__ void run() {
-        const int nsteps = t16_steps(lb);
+        const int nsteps = lb + 2 * kP - 1;
         const int s_steady = 2 * kP - 1;
         const int s_drain = max(s_steady, lb - 1);
         int s = 0;
@@ -319,16 +332,16 @@ __device__ __forceinline__ void t16_emit(int op, int n, int &cur, int &len, int 
     len = n;
 }
 
-// Walk of one pair from (la, lb) over the group's direction words; all 8
+// Walk of one pair from (la, lb) over the group's direction words; all its
 // lanes take the same path, lane 0 writes the runs.  Returns the run count,
 // or -1 if the walk left the rectangle (never for consistent words).
-template <int R>
+template <int kP, int R>
 __device__ __forceinline__ int t16_walk(const uint32_t *dirs, uint32_t *stage, int tile_steps, int la, int lb, int k,
                                         unsigned gmask, uint32_t *ops) {
     constexpr int S = kP * R;
     constexpr int SS = 2 * S;
     constexpr int Q = R / 4;
-    const int nsteps = t16_steps(lb);
+    const int nsteps = lb + 2 * kP - 1;
     int i = la, j = lb, mode = 0, cur = -1, len = 0, runs = 0;
     int tile_lo = INT_MAX;
     const bool writer = k == 0;
@@ -397,12 +410,12 @@ __device__ __forceinline__ int t16_walk(const uint32_t *dirs, uint32_t *stage, i
     return runs;
 }
 
-template <int R, bool DNA>
+template <int kP, int R, bool DNA, bool SHIFT>
 __global__ void __launch_bounds__(kT16Block) k_trace16(BatchView b, Scoring sc, T16Scratch ts, int cls) {
     extern __shared__ __align__(16) uint32_t t16_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane / kP, k = lane & (kP - 1), gbase = lane & ~(kP - 1);
-    const unsigned gmask = ((1u << kP) - 1u) << gbase;
+    const unsigned gmask = kP == 32 ? 0xFFFFFFFFu : ((1u << (kP & 31)) - 1u) << gbase;
     const int pwords = t16_prof_words(R, DNA, sc.A);
     uint32_t *psm = t16_smem + (size_t)warp * 32 * pwords;
     // after the fills, group g stages its walk tiles in quarter g of the region
@@ -410,7 +423,7 @@ __global__ void __launch_bounds__(kT16Block) k_trace16(BatchView b, Scoring sc, 
     const int tile_steps = pwords / (R / 4);
     const int gwarp = blockIdx.x * (kT16Block / 32) + warp;
     const size_t gid = (size_t)gwarp * (32 / kP) + g;
-    const int v = cls - kTraceT16First;
+    constexpr T16Shape shape{kP, R};
     const int64_t dir_words = ts.dir_words;
     uint32_t *dirs = ts.dirs + gid * dir_words;
     uint32_t *ops = ts.ops + gid * ts.op_words;
@@ -432,7 +445,7 @@ __global__ void __launch_bounds__(kT16Block) k_trace16(BatchView b, Scoring sc, 
             lb = rr.ref_end1 - tb + 1;
             const bool fits = score1 > 0 && (flags & kResPendingTrace) && !(flags & kResInternal) && qb >= 0 &&
                               tb >= 0 && la >= 1 && lb >= 1 && lb <= kT16MaxCols &&
-                              t16_need_words(la, lb, v) <= dir_words && (long long)la + lb + 2 <= ts.op_words;
+                              shape.need_words(la, lb) <= dir_words && (long long)la + lb + 2 <= ts.op_words;
             if (!fits) {
                 if (k == 0 && score1 > 0 && (flags & kResPendingTrace)) b.res[p].flags |= kResInternal;
                 p = -1;
@@ -441,11 +454,11 @@ __global__ void __launch_bounds__(kT16Block) k_trace16(BatchView b, Scoring sc, 
         int fh = INT_MIN;
         if (p >= 0) {
             // each lane builds and reads only its own profile words
-            T16Runner<R, DNA> run;
+            T16Runner<kP, R, DNA, SHIFT> run;
             run.init(b.q + b.q_off[p] + b.res[p].read_begin1, la, b.t + b.t_off[p] + b.res[p].ref_begin1, lb, sc,
                      psm, ops, k, lane, gmask, gbase);
-            const int nst = t16_strips(la, v);
-            const size_t strip_words = (size_t)t16_steps(lb) * (R / 4) * kP;
+            const int nst = shape.strips(la);
+            const size_t strip_words = (size_t)shape.steps(lb) * (R / 4) * kP;
             uint32_t *bnd0 = dirs + strip_words * nst, *bnd1 = bnd0 + ((lb + 3) & ~3);
 #pragma unroll 1
             for (int st = 0; st < nst; st++) {
@@ -460,7 +473,7 @@ __global__ void __launch_bounds__(kT16Block) k_trace16(BatchView b, Scoring sc, 
         int nr = -1;
         if (p >= 0 && fh == score1) {
             // the dirs the group wrote are visible to its lanes after the warp barrier
-            nr = t16_walk<R>(dirs, stage, tile_steps, la, lb, k, gmask, ops);
+            nr = t16_walk<kP, R>(dirs, stage, tile_steps, la, lb, k, gmask, ops);
         }
         if (p >= 0) {
             __syncwarp(gmask);
@@ -498,56 +511,65 @@ size_t t16_smem_bytes(const Scoring &sc) {
 }
 
 // resident blocks per SM of one variant (0 when it cannot launch)
-template <int R, bool DNA>
+template <int P, int R, bool DNA, bool SHIFT>
 int t16_blocks(const Scoring &sc) {
     const size_t smem = t16_smem_bytes<R, DNA>(sc);
-    if (cudaFuncSetAttribute(k_trace16<R, DNA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+    if (cudaFuncSetAttribute(k_trace16<P, R, DNA, SHIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
         return 0;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_trace16<R, DNA>, kT16Block, smem) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_trace16<P, R, DNA, SHIFT>, kT16Block, smem) != cudaSuccess)
         return 0;
     return n;
 }
 
-template <int R, bool DNA>
+template <int P, int R, bool DNA, bool SHIFT>
 cudaError_t t16_launch(const BatchView &b, const Scoring &sc, const T16Scratch &ts, int sms, int v, cudaStream_t st) {
-    const int per_sm = t16_blocks<R, DNA>(sc);
+    const int per_sm = t16_blocks<P, R, DNA, SHIFT>(sc);
     if (per_sm <= 0) return cudaErrorInvalidConfiguration;
     const int wpb = kT16Block / 32;
     const int grid = std::max(1, std::min(sms * per_sm, ts.warps / wpb));
-    k_trace16<R, DNA><<<grid, kT16Block, t16_smem_bytes<R, DNA>(sc), st>>>(b, sc, ts, kTraceT16First + v);
+    k_trace16<P, R, DNA, SHIFT><<<grid, kT16Block, t16_smem_bytes<R, DNA>(sc), st>>>(b, sc, ts, kTraceT16First + v);
     return cudaGetLastError();
+}
+
+// f(kernel's P, R, DNA, SHIFT as constants) of launch class v (t16_shape)
+template <class F>
+auto t16_dispatch(const Scoring &sc, int v, F f) {
+    using std::integral_constant;
+    using False = std::false_type;
+    using True = std::true_type;
+    if (sc.dna4) {
+        switch (v) {
+        case 0: return f(integral_constant<int, 8>{}, integral_constant<int, 4>{}, True{}, False{});
+        case 1: return f(integral_constant<int, 8>{}, integral_constant<int, 8>{}, True{}, False{});
+        case 2: return f(integral_constant<int, 8>{}, integral_constant<int, 12>{}, True{}, False{});
+        default: return f(integral_constant<int, 8>{}, integral_constant<int, 16>{}, True{}, False{});
+        }
+    }
+    const bool shift = sc.wmax - sc.wmin <= 127 && sc.wmin <= 0;
+    if (v == 0)
+        return shift ? f(integral_constant<int, 8>{}, integral_constant<int, 4>{}, False{}, True{})
+                     : f(integral_constant<int, 8>{}, integral_constant<int, 4>{}, False{}, False{});
+    return shift ? f(integral_constant<int, 32>{}, integral_constant<int, 4>{}, False{}, True{})
+                 : f(integral_constant<int, 32>{}, integral_constant<int, 4>{}, False{}, False{});
 }
 
 }  // namespace
 
 int t16_max_warps(const Scoring &sc, int sms, int v) {
-    int per_sm = 0;
-    if (sc.dna4) {
-        switch (v) {
-        case 0: per_sm = t16_blocks<4, true>(sc); break;
-        case 1: per_sm = t16_blocks<8, true>(sc); break;
-        case 2: per_sm = t16_blocks<12, true>(sc); break;
-        default: per_sm = t16_blocks<16, true>(sc); break;
-        }
-    } else if (v <= 1) {
-        per_sm = v == 0 ? t16_blocks<4, false>(sc) : t16_blocks<8, false>(sc);
-    }
+    const int per_sm = t16_dispatch(sc, v, [&](auto P, auto R, auto DNA, auto SHIFT) {
+        return t16_blocks<decltype(P)::value, decltype(R)::value, decltype(DNA)::value, decltype(SHIFT)::value>(sc);
+    });
     return std::max(0, sms * per_sm) * (kT16Block / 32);
 }
 
 cudaError_t launch_trace16(const BatchView &b, const Scoring &sc, const T16Scratch &ts, int sms, int v,
                            cudaStream_t st) {
-    if (sc.dna4) {
-        switch (v) {
-        case 0: return t16_launch<4, true>(b, sc, ts, sms, v, st);
-        case 1: return t16_launch<8, true>(b, sc, ts, sms, v, st);
-        case 2: return t16_launch<12, true>(b, sc, ts, sms, v, st);
-        default: return t16_launch<16, true>(b, sc, ts, sms, v, st);
-        }
-    }
-    return v == 0 ? t16_launch<4, false>(b, sc, ts, sms, v, st) : t16_launch<8, false>(b, sc, ts, sms, v, st);
+    return t16_dispatch(sc, v, [&](auto P, auto R, auto DNA, auto SHIFT) {
+        return t16_launch<decltype(P)::value, decltype(R)::value, decltype(DNA)::value, decltype(SHIFT)::value>(
+            b, sc, ts, sms, v, st);
+    });
 }
 
 }  // namespace gsw

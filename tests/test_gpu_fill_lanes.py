@@ -116,3 +116,24 @@ def test_long_pairs_on_clusters(n, lo, hi, match, O, X, budget_mb):
         c.close()
     s = b.subset(keep)
     compare(s, run_oracle(s, colmax=False), (got[0][keep], got[1], (None, None)), check_colmax=False)
+
+
+# the 16-bit rectangle traceback's byte profiles: scores spanning at most 127
+# (shifted bytes) and more (signed bytes), regions at the edges of its strips
+@pytest.mark.parametrize("A,scale,O,X", [(20, 1, 11, 1), (20, 9, 40, 3), (3, 1, 4, 2), (32, 1, 9, 1)])
+def test_general_alphabet_rectangle_traceback(ctx, A, scale, O, X):
+    rng = np.random.default_rng(A * 100 + scale)
+    W = rng.integers(-4, 2, (A, A))
+    W = np.triu(W, 1) + np.triu(W, 1).T
+    np.fill_diagonal(W, rng.integers(4, 9, A))
+    W = np.ascontiguousarray((W * scale).astype(np.int8))
+    qs, ts = [], []
+    for m in (1, 63, 64, 65, 127, 128, 129, 255, 257, 300):
+        q = rng.integers(0, A, m).astype(np.uint8)
+        t = np.concatenate([q[: m // 2], rng.integers(0, A, 9 + m // 7), q[m // 2:]]).astype(np.uint8)
+        mut = rng.random(len(t)) < 0.25
+        t[mut] = rng.integers(0, A, int(mut.sum()))
+        qs.append(q)
+        ts.append(t)
+    b = batch(qs, ts, W, O, X, "ABCDEFGHIJKLMNOPQRSTUVWXYZabcdef"[:A])
+    compare(b, run_oracle(b), run_gpu_host(ctx, b))
