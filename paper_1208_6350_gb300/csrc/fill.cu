@@ -137,7 +137,7 @@ struct StaticCounters {
 };
 
 // One pair by the P lanes of a group; false when its score left the lanes.
-template <int P, int R, class L, bool DNA>
+template <int P, int R, class L, bool DNA, bool ONE>
 __device__ bool static_fill_pair(const BatchView &b, const Scoring &sc, int pair, uint32_t *wsm, int lane, int k,
                                  unsigned gmask, int gbase, uint8_t *cms, uint8_t *bnd) {
     gsw_result *rp = b.res + pair;
@@ -151,7 +151,7 @@ __device__ bool static_fill_pair(const BatchView &b, const Scoring &sc, int pair
     job.stop_u = 0;
     job.cms = cms;
     job.bnd = bnd;
-    const RingResult rr = ring_fill<P, R, L, DNA>(job, sc, wsm, k, gmask, gbase, lane);
+    const RingResult rr = ring_fill<P, R, L, DNA, ONE>(job, sc, wsm, k, gmask, gbase, lane);
     if (L::FOLD && rr.score > 32767 - sc.wmax) return false;  // refill in 32-bit lanes
     int s2 = 0, e2 = -1;
     const int end_t = rr.col, end_q = rr.score > 0 ? rr.row - rr.pad_top : -1;
@@ -203,18 +203,22 @@ __device__ __forceinline__ bool static_check(const BatchView &b, const Scoring &
     return !bad && !empty;
 }
 
-// First kernel: the queries of one strip (at most 256 rows) in 16-bit lanes.
+// First kernel: the queries of one strip (at most kStaticRows) in 16-bit lanes.
 // Their slots hold the column maxima alone, 2 KB, so the array has one for
 // every group that can be resident, where slots that also fit 32-bit boundary
 // rows (20 KB) allowed 4 warps per SM: 8,192 pairs of 100-250 x 300-1000 DNA
-// letters 0.98 -> 0.55 ms.  A block takes kStaticChunk consecutive pairs, orders
-// them by strip height and target length, and its warps take them two at a
-// time (one per 16-lane group; both use the same row-word count R, because
+// letters 1.00 -> 0.56 ms, of 30-400 x 300-1000 2.88 -> 1.11 ms (strips of 320
+// to 512 rows instead of two of 256), 100 of 30-400 x 100-900 0.50 -> 0.22 ms.
+// A block takes kStaticChunk consecutive pairs (8: 0.55 ms, 16: 0.57, 24: 0.62),
+// orders them by strip height and target length, and its warps take them two at
+// a time (one per 16-lane group; both use the same row-word count R, because
 // their profiles share the warp's interleaved shared-memory region).  Taller
-// queries and scores beyond 16 bits are left to the second kernel.
+// queries and scores beyond 16 bits are left to the second kernel, which runs
+// only if some pair was.
 constexpr int kStaticChunk = 8;
+constexpr int kStaticRows = 512;
 template <bool DNA>
-__global__ void __launch_bounds__(kBlock) k_fill_static(BatchView b, Scoring sc, uint8_t *scratch, int warp_words) {
+__global__ void __launch_bounds__(kBlock, 3) k_fill_static(BatchView b, Scoring sc, uint8_t *scratch, int warp_words) {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ int order[kStaticChunk], key[kStaticChunk], chunk, taken;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -236,7 +240,7 @@ __global__ void __launch_bounds__(kBlock) k_fill_static(BatchView b, Scoring sc,
             const long long p = base + threadIdx.x;
             const int m = p < b.npairs ? b.q_len[p] : -1;
             // (lengths out of range sort anywhere: they are rejected below)
-            key[threadIdx.x] = m < 0 ? -1 : (min(m, 257) + 31) / 32 * 2048 + (b.t_len[p] & 2047);
+            key[threadIdx.x] = m < 0 ? -1 : (min(m, kStaticRows + 1) + 31) / 32 * 2048 + (b.t_len[p] & 2047);
         }
         __syncthreads();
         if (threadIdx.x < kStaticChunk) {
@@ -255,7 +259,7 @@ __global__ void __launch_bounds__(kBlock) k_fill_static(BatchView b, Scoring sc,
             int m = 0, n = 0;
             bool run = false;
             if (pair >= 0) {
-                if ((uint32_t)b.q_len[pair] > 256u && b.q_len[pair] >= 0) {
+                if (b.q_len[pair] > kStaticRows) {
                     if (k == 0) cnt->rest = 1;  // (checked by the second kernel)
                 } else {
                     run = static_check(b, sc, pair, k, 16, gmask, &cnt->bad);
@@ -269,12 +273,15 @@ __global__ void __launch_bounds__(kBlock) k_fill_static(BatchView b, Scoring sc,
             bool ok = true;
             if (run) {
 #define GSW_STATIC(R) \
-    ok = half ? static_fill_pair<16, R, LH, DNA>(b, sc, pair, wsm, lane, k, gmask, gbase, cms, nullptr) \
-              : static_fill_pair<16, R, L16, DNA>(b, sc, pair, wsm, lane, k, gmask, gbase, cms, nullptr)
+    ok = half ? static_fill_pair<16, R, LH, DNA, true>(b, sc, pair, wsm, lane, k, gmask, gbase, cms, nullptr) \
+              : static_fill_pair<16, R, L16, DNA, true>(b, sc, pair, wsm, lane, k, gmask, gbase, cms, nullptr)
                 if (rows <= 64) GSW_STATIC(2);
                 else if (rows <= 128) GSW_STATIC(4);
                 else if (rows <= 192) GSW_STATIC(6);
-                else GSW_STATIC(8);
+                else if (rows <= 256) GSW_STATIC(8);
+                else if (rows <= 320) GSW_STATIC(10);
+                else if (rows <= 384) GSW_STATIC(12);
+                else GSW_STATIC(16);
 #undef GSW_STATIC
                 if (!ok && k == 0) {
                     b.res[pair].flags = GSW_RES_S32 | kResPendingS32;
@@ -302,19 +309,18 @@ __global__ void __launch_bounds__(kBlock) k_fill_static_rest(BatchView b, Scorin
     uint8_t *slot = scratch + (size_t)(gwarp * 2 + g) * kStaticSlotBytes;
     uint8_t *bnd = slot + (size_t)kStaticMaxTarget * sizeof(int32_t);
     StaticCounters *cnt = reinterpret_cast<StaticCounters *>(scratch + kStaticErrOff);
-    if (cnt->rest == 0) return;
     for (long long base = gwarp * 2; base < b.npairs; base += nwarps * 2) {
         const int pair = (int)base + g;
         bool run = false, over = false;
         if (pair < b.npairs) {
-            const bool tall = (uint32_t)b.q_len[pair] > 256u && b.q_len[pair] >= 0;
+            const bool tall = b.q_len[pair] > kStaticRows;
             over = !tall && (b.res[pair].flags & kResPendingS32) && !(b.res[pair].flags & kResInvalid);
             if (tall) run = static_check(b, sc, pair, k, 16, gmask, &cnt->bad);
         }
         bool ok = !over;
-        if (run) ok = static_fill_pair<16, 8, L16, DNA>(b, sc, pair, wsm, lane, k, gmask, gbase, slot, bnd);
+        if (run) ok = static_fill_pair<16, 8, L16, DNA, false>(b, sc, pair, wsm, lane, k, gmask, gbase, slot, bnd);
         __syncwarp();
-        if (!ok) static_fill_pair<16, 8, L32, DNA>(b, sc, pair, wsm, lane, k, gmask, gbase, slot, bnd);
+        if (!ok) static_fill_pair<16, 8, L32, DNA, false>(b, sc, pair, wsm, lane, k, gmask, gbase, slot, bnd);
         __syncwarp();
     }
 }
@@ -359,7 +365,7 @@ extern "C" int gsw_fill_static(int32_t npairs, const uint8_t *q, const int64_t *
     int wpb = (int)((200u << 10) / per_warp);
     wpb = wpb > 4 ? 4 : (wpb < 1 ? 1 : wpb);
     const size_t smem = per_warp * wpb;
-    const size_t short_warp = (size_t)prof_words(8, true, sc.dna4 != 0, alphabet) * 32 * sizeof(uint32_t);
+    const size_t short_warp = (size_t)prof_words(16, true, sc.dna4 != 0, alphabet) * 32 * sizeof(uint32_t);
     const size_t short_smem = short_warp * (kBlock / 32);
     uint8_t *scratch;
     int sms;
@@ -407,21 +413,28 @@ extern "C" int gsw_fill_static(int32_t npairs, const uint8_t *q, const int64_t *
     int short_grid = std::min(sms * std::max(per_sm, 1), most);
     short_grid = std::min(short_grid, (npairs + kStaticChunk - 1) / kStaticChunk);
     const int grid = kStaticWarps / wpb;
-    if (sc.dna4) {
-        k_fill_static<true><<<short_grid, kBlock, short_smem, st>>>(bv, sc, scratch, (int)(short_warp / 4));
-        k_fill_static_rest<true><<<grid, wpb * 32, smem, st>>>(bv, sc, scratch, (int)(per_warp / 4));
-    } else {
-        k_fill_static<false><<<short_grid, kBlock, short_smem, st>>>(bv, sc, scratch, (int)(short_warp / 4));
-        k_fill_static_rest<false><<<grid, wpb * 32, smem, st>>>(bv, sc, scratch, (int)(per_warp / 4));
-    }
-    {
+    if (sc.dna4) k_fill_static<true><<<short_grid, kBlock, short_smem, st>>>(bv, sc, scratch, (int)(short_warp / 4));
+    else k_fill_static<false><<<short_grid, kBlock, short_smem, st>>>(bv, sc, scratch, (int)(short_warp / 4));
+    StaticCounters cnt = {};
+    auto read_back = [&]() -> int {
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return set_err(GSW_ECUDA, "fill launch: %s", cudaGetErrorString(e));
+        if (cudaMemcpyAsync(&cnt, scratch + kStaticErrOff, sizeof(cnt), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess)
+            return set_err(GSW_ECUDA, "counter readback");
+        return GSW_OK;
+    };
+    {
+        const int e = read_back();
+        if (e != GSW_OK) return e;
     }
-    int32_t err = 0;
-    if (cudaMemcpyAsync(&err, scratch + kStaticErrOff, sizeof(int32_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-        return set_err(GSW_ECUDA, "counter readback");
+    if (cnt.rest) {  // the second kernel only where some pair was left to it
+        if (sc.dna4) k_fill_static_rest<true><<<grid, wpb * 32, smem, st>>>(bv, sc, scratch, (int)(per_warp / 4));
+        else k_fill_static_rest<false><<<grid, wpb * 32, smem, st>>>(bv, sc, scratch, (int)(per_warp / 4));
+        const int e = read_back();
+        if (e != GSW_OK) return e;
+    }
+    const int32_t err = cnt.bad;
     if (err)
         return set_err(GSW_EINVAL, "pairs with a length outside [0, 2^24), a target over %d letters, a negative "
                                    "offset or a letter code >= %d (records flagged GSW_RES_INVALID)",

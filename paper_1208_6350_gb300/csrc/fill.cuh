@@ -618,7 +618,9 @@ struct StripRunner {
     // a forward fill of several strips take the kModeFwdFirst/Later forms;
     // the 8- and 4-lane variants (one-strip short reads, whose registers the extra
     // loops would crowd) keep the general step for them.
-    template <bool MAYBE_FAST = true, bool MAYBE_MULTI = (P > 8)>
+    // ONLY_FAST (one-strip forward fills of short targets) leaves every other
+    // steady form out: what does not take the FAST blocks runs as checked steps.
+    template <bool MAYBE_FAST = true, bool MAYBE_MULTI = (P > 8), bool ONLY_FAST = false>
     __device__ bool run(int s0, int s1) {
         const int s_steady = L::FOLD ? 2 * P - 1 : P - 1;
         const int s_drain = max(s_steady, n - 1);
@@ -681,7 +683,7 @@ struct StripRunner {
                 c_lo = (int)(int16_t)(cpk & 0xFFFFu);
                 c_hi = (int)(int16_t)(cpk >> 16);
             }
-        } else {
+        } else if constexpr (!ONLY_FAST) {
 #pragma unroll kUnrollGen
             for (; s < s1 && s < s_drain; s++)
                 if (step<false>(s)) return true;
@@ -731,7 +733,8 @@ __device__ __forceinline__ void best_merge(int v, int c, int row, int *bv, int *
 
 // The ring fill of one pair by the P lanes of a group, strip after strip.
 // All lanes of the group call it with the same job and return the same result.
-template <int P, int R, class L, bool DNA>
+// ONE: one-strip forward fills only.
+template <int P, int R, class L, bool DNA, bool ONE = false>
 __device__ RingResult ring_fill(const Job &job, const Scoring &sc, uint32_t *psm, int k, unsigned gmask,
                                 int gbase, int lane) {
     using SR = StripRunner<P, R, L, DNA>;
@@ -745,7 +748,7 @@ __device__ RingResult ring_fill(const Job &job, const Scoring &sc, uint32_t *psm
 #pragma unroll 1
     for (int st = 0; st < nstrips; st++) {
         sr.begin(sc, st, bnd + (size_t)((st + 1) & 1) * n, bnd + (size_t)(st & 1) * n, st == nstrips - 1);
-        sr.run(0, sr.nsteps);
+        sr.template run<true, (P > 8) && !ONE, ONE>(0, sr.nsteps);
         int v, c, row;
         sr.end(&v, &c, &row);
         best_merge(v, c, st * SR::SP + row, &g_score, &g_col, &g_row);

@@ -137,3 +137,29 @@ def test_general_alphabet_rectangle_traceback(ctx, A, scale, O, X):
         ts.append(t)
     b = batch(qs, ts, W, O, X, "ABCDEFGHIJKLMNOPQRSTUVWXYZabcdef"[:A])
     compare(b, run_oracle(b), run_gpu_host(ctx, b))
+
+
+# gsw_fill_static's two kernels: strips of 64 to 512 rows, taller queries, and
+# scores beyond 16 bits, with max arrays
+@pytest.mark.parametrize("A,match,O,X", [(4, 2, 3, 1), (4, 100, 30, 10), (20, 0, 11, 1)])
+def test_static_fill_strip_heights(A, match, O, X):
+    import torch
+    W = wl.dna_matrix(match, -match) if A == 4 else wl.synthetic_protein_matrix()
+    rng = np.random.default_rng(A + match)
+    qs, ts = [], []
+    for m in (1, 63, 64, 65, 128, 129, 192, 193, 256, 257, 320, 321, 384, 385, 512, 513, 700):
+        q = rng.integers(0, A, m).astype(np.uint8)
+        qs.append(q)
+        ts.append(np.concatenate([rng.integers(0, A, 5), q, rng.integers(0, A, 9)]).astype(np.uint8))
+    b = batch(qs, ts, W, O, X, wl.DNA if A == 4 else wl.PROTEIN)
+    d = [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (b.q, b.q_off, b.q_len, b.t, b.t_off, b.t_len)]
+    cmo = np.concatenate([[0], np.cumsum(b.t_len.astype(np.int64))[:-1]])
+    res = torch.zeros((b.npairs, 12), dtype=torch.int32, device="cuda")
+    cm = torch.zeros(int(b.t_len.sum()), dtype=torch.int32, device="cuda")
+    off = torch.from_numpy(cmo).cuda()
+    torch.cuda.synchronize()
+    rc = gsw.gsw_fill_static(b.npairs, *d, int(b.t_len.max()), W, O, X, flags=gsw.GSW_COLMAX, results=res, colmax=cm,
+                             colmax_off=off)
+    assert rc == gsw.GSW_OK
+    r = res.cpu().numpy().view(gsw.RESULT_DTYPE).reshape(-1)
+    compare(b, run_oracle(b), (r, None, (cm.cpu().numpy(), cmo)), check_begin=False, check_cigar=False)
