@@ -17,6 +17,7 @@ constexpr int kScanThreads = 1024;
 // Batches of at most this many pairs are planned by one block (16 pairs a
 // thread at most).
 constexpr int kPlanSmall = 16384;
+constexpr int kPlanFew = 2048;
 
 
 __device__ __forceinline__ int cost_bin(long long cost) {
@@ -125,23 +126,33 @@ __global__ void k_plan_keys(BatchView b, Scoring sc, int32_t mode, int32_t *keys
     if (key >= 0 && (int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&hist[key], __popc(same));
 }
 
-// Exclusive scan of `hist` (kPlanBins counts) by a block of kScanThreads, in
-// place or into binoff; then the class boundaries and task ranges.
+// Exclusive scan of `hist` (kPlanBins >> SHIFT counts) by a block of
+// kScanThreads, in place or into binoff; then the class boundaries and task
+// ranges.
+template <int SHIFT>
 __device__ void plan_scan(const int32_t *hist, int32_t *binoff, int32_t *var_start, int32_t *task_lo,
                           int32_t *task_hi, int32_t *ntasks, int32_t *head) {
-    constexpr int PER = kPlanBins / kScanThreads;
-    static_assert(kPlanBins % kScanThreads == 0 && PER % 4 == 0, "bins");
+    constexpr int BINS = kPlanBins >> SHIFT, PER = BINS / kScanThreads;
+    static_assert(BINS % kScanThreads == 0 && (SHIFT > 0 || PER % 4 == 0), "bins");
     const int tid = threadIdx.x;
     int32_t loc[PER];
     int32_t sum = 0;
+    if constexpr (SHIFT == 0) {
 #pragma unroll
-    for (int i = 0; i < PER; i += 4) {
-        const int4 v = *reinterpret_cast<const int4 *>(hist + tid * PER + i);
-        loc[i] = sum;
-        loc[i + 1] = loc[i] + v.x;
-        loc[i + 2] = loc[i + 1] + v.y;
-        loc[i + 3] = loc[i + 2] + v.z;
-        sum = loc[i + 3] + v.w;
+        for (int i = 0; i < PER; i += 4) {
+            const int4 v = *reinterpret_cast<const int4 *>(hist + tid * PER + i);
+            loc[i] = sum;
+            loc[i + 1] = loc[i] + v.x;
+            loc[i + 2] = loc[i + 1] + v.y;
+            loc[i + 3] = loc[i + 2] + v.z;
+            sum = loc[i + 3] + v.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < PER; i++) {
+            loc[i] = sum;
+            sum += hist[tid * PER + i];
+        }
     }
     // inclusive scan of the threads' sums: within each warp by shuffles,
     // then over the warp totals by the first warp
@@ -168,13 +179,19 @@ __device__ void plan_scan(const int32_t *hist, int32_t *binoff, int32_t *var_sta
     }
     __syncthreads();
     const int32_t base = incl + (warp > 0 ? wsum[warp - 1] : 0) - sum;
+    if constexpr (SHIFT == 0) {
 #pragma unroll
-    for (int i = 0; i < PER; i += 4)
-        *reinterpret_cast<int4 *>(binoff + tid * PER + i) =
-            make_int4(base + loc[i], base + loc[i + 1], base + loc[i + 2], base + loc[i + 3]);
+        for (int i = 0; i < PER; i += 4)
+            *reinterpret_cast<int4 *>(binoff + tid * PER + i) =
+                make_int4(base + loc[i], base + loc[i + 1], base + loc[i + 2], base + loc[i + 3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < PER; i++) binoff[tid * PER + i] = base + loc[i];
+    }
+    constexpr int OF_CLASS = kPlanBinsPerVariant >> SHIFT;
 #pragma unroll
     for (int i = 0; i < PER; i++)
-        if ((tid * PER + i) % kPlanBinsPerVariant == 0) starts[(tid * PER + i) / kPlanBinsPerVariant] = base + loc[i];
+        if ((tid * PER + i) % OF_CLASS == 0) starts[(tid * PER + i) / OF_CLASS] = base + loc[i];
     if (tid == kScanThreads - 1) starts[kNumFillClasses] = base + sum;
     __syncthreads();
     // the classes' task ranges (heaviest class first), a lane per class
@@ -205,23 +222,26 @@ __device__ void plan_scan(const int32_t *hist, int32_t *binoff, int32_t *var_sta
 __global__ void __launch_bounds__(kScanThreads) k_plan_scan(const int32_t *hist, int32_t *binoff,
                                                              int32_t *var_start, int32_t *task_lo,
                                                              int32_t *task_hi, int32_t *ntasks, int32_t *head) {
-    plan_scan(hist, binoff, var_start, task_lo, task_hi, ntasks, head);
+    plan_scan<0>(hist, binoff, var_start, task_lo, task_hi, ntasks, head);
 }
 
 // The whole plan of a small batch by one block, its bins in shared memory: one
 // launch instead of two clears and three kernels (about 25 us a plan, four or
-// five plans a call).
+// five plans a call).  SHIFT: 8 cost bins in one (4 per doubling) for batches
+// that leave the chip part empty, where a finer order buys nothing (1,000 pairs:
+// 8.0, 8.6 and 11.2 us a plan -> 6.1, 6.8 and 9.7).
+template <int SHIFT>
 __global__ void __launch_bounds__(kScanThreads) k_plan_small(BatchView b, Scoring sc, int32_t mode, PlanBuffers pb,
                                                               unsigned long long *need) {
     extern __shared__ __align__(16) int32_t bins[];
     __shared__ unsigned most[kNeedWords];
     if (threadIdx.x < kNeedWords) most[threadIdx.x] = 0;
-    for (int i = threadIdx.x; i < kPlanBins / 4; i += kScanThreads) reinterpret_cast<int4 *>(bins)[i] = make_int4(0, 0, 0, 0);
+    for (int i = threadIdx.x; i < (kPlanBins >> SHIFT) / 4; i += kScanThreads) reinterpret_cast<int4 *>(bins)[i] = make_int4(0, 0, 0, 0);
     __syncthreads();
     for (int p = threadIdx.x; p < b.npairs; p += kScanThreads) {
         const int key = plan_key(b, sc, mode, p);
         pb.keys[p] = key;
-        if (key >= 0) atomicAdd(&bins[key], 1);
+        if (key >= 0) atomicAdd(&bins[key >> SHIFT], 1);
         if (need && key >= 0) {
             unsigned v[kNeedWords] = {};
             trace_needs(b.res[p], sc, small_batch(b), v);
@@ -234,11 +254,11 @@ __global__ void __launch_bounds__(kScanThreads) k_plan_small(BatchView b, Scorin
     }
     __syncthreads();
     if (need && threadIdx.x < kNeedWords) need[threadIdx.x] = most[threadIdx.x];
-    plan_scan(bins, bins, pb.var_start, pb.task_lo, pb.task_hi, pb.ntasks, pb.head);
+    plan_scan<SHIFT>(bins, bins, pb.var_start, pb.task_lo, pb.task_hi, pb.ntasks, pb.head);
     __syncthreads();
     for (int p = threadIdx.x; p < b.npairs; p += kScanThreads) {
         const int key = pb.keys[p];
-        if (key >= 0) pb.order[atomicAdd(&bins[key], 1)] = p;
+        if (key >= 0) pb.order[atomicAdd(&bins[key >> SHIFT], 1)] = p;
     }
 }
 
@@ -259,16 +279,20 @@ __global__ void k_plan_scatter(int32_t npairs, const int32_t *keys, const int32_
 cudaError_t launch_plan(const BatchView &b, const Scoring &sc, int32_t mode, const PlanBuffers &pb,
                         unsigned long long *need, cudaStream_t st) {
     cudaError_t e;
+    if (b.npairs <= kPlanFew) {
+        k_plan_small<3><<<1, kScanThreads, (kPlanBins >> 3) * 4, st>>>(b, sc, mode, pb, need);
+        return cudaGetLastError();
+    }
     if (b.npairs <= kPlanSmall) {
         static std::atomic<unsigned long long> ready{0};  // devices whose kernel has its shared-memory limit
         int dev = 0;
         if ((e = cudaGetDevice(&dev))) return e;
         if (dev >= 64 || !((ready.load() >> dev) & 1ull)) {
-            if ((e = cudaFuncSetAttribute(k_plan_small, cudaFuncAttributeMaxDynamicSharedMemorySize, kPlanBins * 4)))
+            if ((e = cudaFuncSetAttribute(k_plan_small<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPlanBins * 4)))
                 return e;
             if (dev < 64) ready.fetch_or(1ull << dev);
         }
-        k_plan_small<<<1, kScanThreads, kPlanBins * 4, st>>>(b, sc, mode, pb, need);
+        k_plan_small<0><<<1, kScanThreads, kPlanBins * 4, st>>>(b, sc, mode, pb, need);
         return cudaGetLastError();
     }
     if ((e = cudaMemsetAsync(pb.hist, 0, sizeof(int32_t) * 2 * kPlanBins, st))) return e;
