@@ -1,0 +1,63 @@
+// C entry points over the rules that choose a batch's kernels (gsw_impl.cuh),
+// compiled by g++ for the CPU tests of those rules.
+#include "gsw_impl.cuh"
+
+namespace {
+gsw::Scoring scoring(int A, const signed char *W, int O, int X) {
+    gsw::Scoring sc{};
+    sc.A = A;
+    sc.O = O;
+    sc.X = X;
+    int mx = W[0], mn = W[0];
+    for (int k = 0; k < A * A; ++k) {
+        mx = W[k] > mx ? W[k] : mx;
+        mn = W[k] < mn ? W[k] : mn;
+        sc.W[k] = W[k];
+    }
+    sc.wmax = mx;
+    sc.wmin = mn;
+    sc.dna4 = A == 4;
+    for (signed char &c : sc.fill_class) c = -1;
+    return sc;
+}
+}  // namespace
+
+extern "C" {
+
+// What a batch of these sizes launches and where a pair of it goes: out[0] the
+// launch mask, [1] the half-precision classes, [2] the classes with boundary
+// rows, [3] the pair's class, [4] rows of that class's strip.
+void cr_route(int A, const signed char *W, int O, int X, int npairs, int minm, int maxm, int maxn, double cells, int mode,
+              int rows, int cols, unsigned *out) {
+    gsw::Scoring sc = scoring(A, W, O, X);
+    gsw::default_classes(sc, npairs, maxm, maxn, cells);
+    out[0] = gsw::fill_class_mask(mode, maxm, sc, false, false, minm);
+    const gsw::ClassRows r = gsw::fill_class_rows(mode, maxm, sc, out[0]);
+    out[1] = gsw::fill_half_mask(r, maxn, sc);
+    out[2] = gsw::fill_multi_mask(r);
+    int v = mode == gsw::kFillForward ? gsw::pick_class16(rows, sc) : gsw::pick_class_reverse(rows, false, sc);
+    if (gsw::cta_pair(v, rows, cols, sc)) v = gsw::kClassLong16;
+    out[3] = (unsigned)v;
+    out[4] = (unsigned)gsw::variant_rows(v);
+}
+
+int cr_half_fits(int A, const signed char *W, int O, int X, int rows, int cols) {
+    return gsw::half_fits(rows, cols, scoring(A, W, O, X));
+}
+
+// trace class of a region, and whether a batch whose lengths reach maxm x maxn
+// launches the wide-band kernel
+int cr_trace(int A, const signed char *W, int O, int X, int maxm, int maxn, int la, int lb, int score1, int small,
+             int *ring) {
+    const gsw::Scoring sc = scoring(A, W, O, X);
+    int dlo, dhi;
+    *ring = gsw::ring_possible(maxm, maxn, sc);
+    return gsw::trace_class(la, lb, score1, sc, small != 0, &dlo, &dhi);
+}
+
+int cr_consts(int which) {
+    const int c[] = {gsw::kNumVariants, gsw::kVarP4First, gsw::kVarTallFirst, gsw::kTraceRingClass, gsw::kClassLong16};
+    return c[which];
+}
+
+}  // extern "C"

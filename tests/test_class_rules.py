@@ -1,0 +1,107 @@
+"""The rules that choose a batch's kernels by its size, compiled from the
+library's own header with g++ (tests/class_rules_shim.cpp): whatever class a
+pair takes is one its batch launches, with the lanes and the boundary rows that
+the pair needs, and a pair of the wide-band traceback is never left out.
+"""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+HERE = os.path.dirname(os.path.abspath(__file__))
+FORWARD, REVERSE = 0, 2
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    gxx = shutil.which("g++")
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    if gxx is None or not os.path.exists(os.path.join(inc, "cuda_runtime.h")):
+        pytest.skip("g++ or cuda_runtime.h not found")
+    out = str(tmp_path_factory.mktemp("class_rules") / "libclassrules.so")
+    subprocess.run([gxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-w", "-I", os.path.join(ROOT, "include"),
+                    "-I", os.path.join(ROOT, "paper_1208_6350_gb300", "csrc"), "-I", inc,
+                    os.path.join(HERE, "class_rules_shim.cpp"), "-o", out], check=True)
+    L = ctypes.CDLL(out)
+    P, i32 = ctypes.c_void_p, ctypes.c_int
+    L.cr_route.argtypes = [i32, P, i32, i32, i32, i32, i32, i32, ctypes.c_double, i32, i32, i32, P]
+    L.cr_route.restype = None
+    L.cr_half_fits.argtypes = [i32, P, i32, i32, i32, i32]
+    L.cr_trace.argtypes = [i32, P, i32, i32, i32, i32, i32, i32, i32, i32, ctypes.POINTER(i32)]
+    return L
+
+
+def schemes():
+    rng = np.random.default_rng(5)
+    for match, mismatch, O, X in ((2, -3, 5, 2), (1, -1, 1, 1), (5, -4, 10, 1), (100, -100, 120, 10), (2, -6, 3, 1)):
+        W = np.full((4, 4), mismatch, dtype=np.int8)
+        np.fill_diagonal(W, match)
+        yield W, O, X
+    for A, O, X in ((20, 11, 1), (5, 4, 2), (24, 120, 3)):
+        W = rng.integers(-4, 4, (A, A)).astype(np.int8)
+        np.fill_diagonal(W, 9)
+        yield W, O, X
+
+
+def edge_lengths(rng, top):
+    """Lengths at the edges of strips and buckets as well as in between."""
+    edges = [x + d for x in (16, 48, 64, 96, 128, 256, 320, 384, 512, 1024, 1792, 4096) for d in (-1, 0, 1)]
+    edges = [x for x in edges if x <= top] + [1, top]
+    return int(rng.choice(edges)) if rng.random() < 0.5 else int(rng.integers(1, top + 1))
+
+
+@pytest.mark.parametrize("mode", [FORWARD, REVERSE])
+def test_every_pair_takes_a_launched_class_that_holds_it(lib, mode):
+    rng = np.random.default_rng(17 + mode)
+    nvar, p4, tall, _, long16 = (lib.cr_consts(k) for k in range(5))
+    out = (ctypes.c_uint * 5)()
+    seen = set()
+    for W, O, X in schemes():
+        p, A = W.ctypes.data_as(ctypes.c_void_p), len(W)
+        for _ in range(400):
+            npairs = int(rng.choice([1, 40, 2047, 2048, 8191, 8192, 16383, 16384, 300000]))
+            maxm, maxn = edge_lengths(rng, 6000), edge_lengths(rng, 40000)
+            minm = int(rng.integers(1, maxm + 1))
+            rows = int(rng.choice([minm, maxm, rng.integers(minm, maxm + 1)])) if mode == FORWARD \
+                else edge_lengths(rng, maxm)
+            cols = int(rng.choice([1, maxn, rng.integers(1, maxn + 1)]))
+            cells = float(npairs) * rng.random() * maxm * maxn
+            lib.cr_route(A, p, O, X, npairs, minm, maxm, maxn, cells, mode, rows, cols, out)
+            mask, half, multi, v, strip = out
+            what = (A, npairs, minm, maxm, maxn, rows, cols, v)
+            assert (mask >> v) & 1, what
+            if (half >> v) & 1:
+                assert lib.cr_half_fits(A, p, O, X, rows, cols), what
+            if rows > strip:
+                assert (multi >> v) & 1, what
+            if p4 <= v < tall:  # four lanes: DNA, one strip, half-precision lanes only
+                assert A == 4 and rows <= strip and (half >> v) & 1 and npairs >= 16384, what
+            seen.add(v)
+    # (the classes the default rule can choose: 4 and 8 lanes go forward only)
+    assert long16 in seen and any(tall <= v < nvar for v in seen)
+    assert any(p4 <= v < tall for v in seen) == (mode == FORWARD)
+
+
+def test_wide_bands_are_never_left_out(lib):
+    rng = np.random.default_rng(23)
+    ring_class = lib.cr_consts(3)
+    ring = ctypes.c_int()
+    wide = without = 0
+    for W, O, X in schemes():
+        p, A = W.ctypes.data_as(ctypes.c_void_p), len(W)
+        for _ in range(6000):
+            top = int(rng.choice([300, 600, 2000, 9000, 40000]))
+            maxm, maxn = edge_lengths(rng, top), edge_lengths(rng, top)
+            la = int(rng.choice([1, maxm, edge_lengths(rng, maxm)]))
+            lb = int(rng.choice([1, maxn, edge_lengths(rng, maxn)]))
+            score = int(rng.integers(1, max(2, min(la, lb) * int(W.max()) + 1)))
+            cls = lib.cr_trace(A, p, O, X, maxm, maxn, la, lb, score, int(rng.integers(0, 2)), ctypes.byref(ring))
+            assert cls != ring_class or ring.value, (A, O, X, maxm, maxn, la, lb, score)
+            wide += cls == ring_class
+            without += not ring.value
+    assert wide and without
