@@ -192,10 +192,18 @@ __host__ __device__ inline bool half_fits(int rows, int cols, const Scoring &sc)
     return (rows < cols ? rows : cols) * top + top + sc.O <= 2047;
 }
 
+// Whether a tune table names the class of queries of `rows` (the default rule
+// marks the buckets it fills in by their rev_class).
+__host__ __device__ inline bool tuned_rows(int rows, const Scoring &sc) {
+    const int b = (rows - 1) / GSW_TUNE_ROWS;
+    return rows >= 1 && b < GSW_TUNE_BUCKETS && sc.fill_class[b] >= 0 && sc.rev_class[b] == 0;
+}
+
 // Whether a pair that class v would run strip after strip goes to the CTA
-// class instead (sc.cta_steps, default_classes).
+// class instead (sc.cta_steps, default_classes).  Not where a tune table names
+// the class: there its strips run one after the other as the table says.
 __host__ __device__ inline bool cta_pair(int v, int rows, int cols, const Scoring &sc) {
-    if (sc.cta_steps <= 0 || v >= kNumVariants || v == kVarS32) return false;
+    if (sc.cta_steps <= 0 || v >= kNumVariants || v == kVarS32 || tuned_rows(rows, sc)) return false;
     const int strips = (rows + variant_rows(v) - 1) / variant_rows(v);
     // (a step's time grows with its row words; 0.3 us is that of 8)
     return strips > 1 && (long long)strips * cols * (4 + variant_at(v).R) > 12LL * sc.cta_steps;
@@ -277,12 +285,12 @@ inline uint32_t fill_class_mask(int mode, int maxm, const Scoring &sc, bool forc
     if (mode == kFillForward && force_s32) return (1u << kVarS32) | (1u << kClassLong32);
     if (mode == kFillRerun) return (1u << kVarS32) | (1u << kClassLong32);
     if (mode == kFillForward && minm <= 0) m |= 1u << 0;
-    bool strips = maxm > upto;  // some class can hold a pair of several strips
+    bool strips = maxm > upto;  // some class of the default rule can hold a pair of several strips
     for (int r = 1; r <= upto; r++) {
         if (mode == kFillForward && r < minm) continue;
         const int c = mode == kFillForward ? pick_class16(r, sc) : pick_class_reverse(r, false, sc);
         m |= 1u << c;
-        strips |= r > variant_rows(c);
+        strips |= r > variant_rows(c) && !tuned_rows(r, sc);
         if (s32 && mode != kFillForward) m |= 1u << pick_class_reverse(r, true, sc);
     }
     if (sc.cta_steps > 0 && strips) m |= 1u << kClassLong16;

@@ -24,12 +24,12 @@ gsw::Scoring scoring(int A, const signed char *W, int O, int X) {
 
 extern "C" {
 
-// What a batch of these sizes launches and where a pair of it goes: out[0] the
-// launch mask, [1] the half-precision classes, [2] the classes with boundary
-// rows, [3] the pair's class, [4] rows of that class's strip.
-void cr_route(int A, const signed char *W, int O, int X, int npairs, int minm, int maxm, int maxn, double cells, int mode,
-              int rows, int cols, unsigned *out) {
+// (table: a tune table's classes, or null)
+void cr_route_tuned(int A, const signed char *W, int O, int X, const signed char *table, int npairs, int minm, int maxm,
+                    int maxn, double cells, int mode, int rows, int cols, unsigned *out) {
     gsw::Scoring sc = scoring(A, W, O, X);
+    if (table)
+        for (int b = 0; b < GSW_TUNE_BUCKETS; b++) sc.fill_class[b] = table[b];
     gsw::default_classes(sc, npairs, maxm, maxn, cells);
     out[0] = gsw::fill_class_mask(mode, maxm, sc, false, false, minm);
     const gsw::ClassRows r = gsw::fill_class_rows(mode, maxm, sc, out[0]);
@@ -39,6 +39,14 @@ void cr_route(int A, const signed char *W, int O, int X, int npairs, int minm, i
     if (gsw::cta_pair(v, rows, cols, sc)) v = gsw::kClassLong16;
     out[3] = (unsigned)v;
     out[4] = (unsigned)gsw::variant_rows(v);
+}
+
+// What a batch of these sizes launches and where a pair of it goes: out[0] the
+// launch mask, [1] the half-precision classes, [2] the classes with boundary
+// rows, [3] the pair's class, [4] rows of that class's strip.
+void cr_route(int A, const signed char *W, int O, int X, int npairs, int minm, int maxm, int maxn, double cells, int mode,
+              int rows, int cols, unsigned *out) {
+    cr_route_tuned(A, W, O, X, nullptr, npairs, minm, maxm, maxn, cells, mode, rows, cols, out);
 }
 
 int cr_half_fits(int A, const signed char *W, int O, int X, int rows, int cols) {

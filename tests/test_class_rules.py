@@ -31,6 +31,8 @@ def lib(tmp_path_factory):
     P, i32 = ctypes.c_void_p, ctypes.c_int
     L.cr_route.argtypes = [i32, P, i32, i32, i32, i32, i32, i32, ctypes.c_double, i32, i32, i32, P]
     L.cr_route.restype = None
+    L.cr_route_tuned.argtypes = [i32, P, i32, i32, P, i32, i32, i32, i32, ctypes.c_double, i32, i32, i32, P]
+    L.cr_route_tuned.restype = None
     L.cr_half_fits.argtypes = [i32, P, i32, i32, i32, i32]
     L.cr_trace.argtypes = [i32, P, i32, i32, i32, i32, i32, i32, i32, i32, ctypes.POINTER(i32)]
     return L
@@ -85,6 +87,38 @@ def test_every_pair_takes_a_launched_class_that_holds_it(lib, mode):
     # (the classes the default rule can choose: 4 and 8 lanes go forward only)
     assert long16 in seen and any(tall <= v < nvar for v in seen)
     assert any(p4 <= v < tall for v in seen) == (mode == FORWARD)
+
+
+def test_a_tune_table_keeps_the_classes_it_names(lib):
+    # classes 0..6 and 9..13 run a longer query strip after strip, whatever the
+    # batch's size; a 4-letter query of several strips reverses on a CTA
+    rng = np.random.default_rng(29)
+    p8, long16, buckets = 8, lib.cr_consts(4), 32
+    out = (ctypes.c_uint * 5)()
+    several = 0
+    for W, O, X in schemes():
+        p, A = W.ctypes.data_as(ctypes.c_void_p), len(W)
+        for _ in range(300):
+            table = rng.choice([-1, 0, 1, 2, 3, 4, 5, 6, 8, 9, 10, 11, 12, 13], buckets).astype(np.int8)
+            t = table.ctypes.data_as(ctypes.c_void_p)
+            npairs = int(rng.choice([1, 160, 8192, 300000]))
+            maxm, maxn = edge_lengths(rng, 1024), edge_lengths(rng, 40000)
+            rows, cols = edge_lengths(rng, maxm), int(rng.choice([1, maxn]))
+            code = int(table[(rows - 1) // 32])
+            if code < 0:
+                continue
+            named = long16 if code == 8 else (p8 + code - 9 if code >= 9 else code)
+            for mode in (FORWARD, REVERSE):
+                lib.cr_route_tuned(A, p, O, X, t, npairs, 1, maxm, maxn, float(npairs) * maxm * maxn, mode, rows, cols, out)
+                mask, half, multi, v, strip = out
+                what = (A, npairs, maxm, maxn, rows, cols, code, mode, v)
+                assert (mask >> v) & 1, what
+                if v != named:
+                    assert mode == REVERSE and A == 4 and v == long16, what
+                elif rows > strip:
+                    several += named != long16
+                    assert (multi >> v) & 1, what
+    assert several > 100
 
 
 def test_wide_bands_are_never_left_out(lib):
