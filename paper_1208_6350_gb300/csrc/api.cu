@@ -877,7 +877,7 @@ int batch_impl(gsw_ctx *ctx, int32_t npairs, const uint8_t *q, const int64_t *q_
     GSW_TRY(run_pipeline(ctx, bv, sc, st, minm, maxm, maxn));
 
     // completion: invalid letters, internal checks, CIGAR space
-    CUDA_TRY(launch_count_flag(bv.res, npairs, kResInternal, misc + kMiscInternal, st));
+    CUDA_TRY(launch_count_internal(bv, misc + kMiscInternal, st));
     ctx->launches += 1;
     unsigned long long *hs = reinterpret_cast<unsigned long long *>(ctx->host_small);
     CUDA_TRY(cudaMemcpyAsync(hs, misc + kMiscCursor, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));

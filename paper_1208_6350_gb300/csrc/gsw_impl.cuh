@@ -669,6 +669,17 @@ int make_scoring(const int8_t *matrix, int32_t A, int32_t O, int32_t X, Scoring 
 cudaError_t launch_count_flag(const gsw_result *res, int32_t n, int32_t flag, unsigned long long *count,
                               cudaStream_t st);
 
+// A record whose begins were asked for (flags of the batch) and never found:
+// every positive score ends its reversed fill somewhere, so some launch left
+// the pair out.
+__host__ __device__ inline bool lost_begin(int score1, int read_begin1, uint32_t flags) {
+    return (flags & (GSW_BEGIN | GSW_CIGAR)) && score1 > 0 && read_begin1 < 0;
+}
+// Counts a finished batch's records flagged kResInternal and flags those that
+// lost their begins (small batches without CIGARs have no later stage that
+// would see them).
+cudaError_t launch_count_internal(const BatchView &b, unsigned long long *count, cudaStream_t st);
+
 // Geometry of one class's launch: blocks resident on the SMs asked for, pairs
 // in flight and scratch per block.
 struct ClassGeom {

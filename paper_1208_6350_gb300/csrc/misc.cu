@@ -79,6 +79,19 @@ __global__ void k_count_flag(const gsw_result *res, int32_t n, int32_t flag, uns
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, (unsigned long long)c);
 }
 
+// number of records flagged kResInternal, those that lost their begins (which
+// it flags) among them
+__global__ void k_count_internal(BatchView b, unsigned long long *count) {
+    unsigned c = 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < b.npairs; i += gridDim.x * blockDim.x) {
+        const bool lost = lost_begin(b.res[i].score1, b.res[i].read_begin1, b.flags);
+        if (lost) b.res[i].flags |= kResInternal;
+        c += (lost || (b.res[i].flags & kResInternal)) ? 1u : 0u;
+    }
+    c = __reduce_add_sync(0xFFFFFFFFu, c);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, (unsigned long long)c);
+}
+
 __global__ void k_unpack2(const uint8_t *in, uint8_t *out, long long nletters) {
     const long long groups = (nletters + 15) / 16;
     for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < groups;
@@ -138,6 +151,15 @@ cudaError_t launch_count_flag(const gsw_result *res, int32_t n, int32_t flag, un
         int blocks = (n + 255) / 256;
         blocks = blocks > 1024 ? 1024 : blocks;
         k_count_flag<<<blocks, 256, 0, st>>>(res, n, flag, count);
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_count_internal(const BatchView &b, unsigned long long *count, cudaStream_t st) {
+    if (b.npairs > 0) {
+        int blocks = (b.npairs + 255) / 256;
+        blocks = blocks > 1024 ? 1024 : blocks;
+        k_count_internal<<<blocks, 256, 0, st>>>(b, count);
     }
     return cudaGetLastError();
 }

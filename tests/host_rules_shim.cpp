@@ -63,6 +63,8 @@ int hr_trace_class(int A, const signed char *W, int O, int X, int la, int lb, in
 
 long long hr_t16_need_words(int la, int lb, int v) { return gsw::t16_need_words(la, lb, v); }
 
+int hr_lost_begin(int score1, int read_begin1, unsigned flags) { return gsw::lost_begin(score1, read_begin1, flags); }
+
 int hr_batch_status(int bad_letters, unsigned long long internal, int cigar, unsigned long long words,
                     long long capacity) {
     return gsw::batch_status(bad_letters, internal, cigar != 0, words, capacity);

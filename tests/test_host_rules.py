@@ -67,6 +67,7 @@ def lib(tmp_path_factory):
     L.hr_fill_class_mask.restype = ctypes.c_uint
     L.hr_batch_status.argtypes = [i32, ctypes.c_ulonglong, i32, ctypes.c_ulonglong, ctypes.c_longlong]
     L.hr_batch_status.restype = i32
+    L.hr_lost_begin.argtypes = [i32, i32, ctypes.c_uint]
     return L
 
 
@@ -516,6 +517,18 @@ def test_batch_status_precedence(lib):
     assert st(0, 5, 0, 0, 0) == gsw.GSW_EINTERNAL
     assert st(1, 5, 1, 11, 10) == gsw.GSW_EINVAL      # bad input first
     assert st(1, 0, 0, 0, 0) == gsw.GSW_EINVAL
+
+
+def test_a_record_without_its_begins_is_flagged(lib):
+    """Also a small batch that asked for begins alone, whose reversed fill no
+    later stage looks at."""
+    from paper_1208_6350_gb300 import gsw
+    lost = lib.hr_lost_begin
+    for flags in (gsw.GSW_BEGIN, gsw.GSW_CIGAR, gsw.GSW_BEGIN | gsw.GSW_CIGAR | gsw.GSW_COLMAX):
+        assert lost(7, -1, flags) and lost(1, -1, flags)
+        assert not lost(7, 0, flags) and not lost(7, 12, flags)  # found
+        assert not lost(0, -1, flags)                            # no alignment
+    assert not lost(7, -1, 0) and not lost(7, -1, gsw.GSW_COLMAX)  # not asked for
 
 
 def test_fill_launch_mask_holds_every_class_the_plan_can_pick(lib):
