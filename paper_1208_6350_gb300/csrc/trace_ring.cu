@@ -426,8 +426,14 @@ __device__ void ring_schedule(const RingLaunch &rl, RingShared<C> &sh, int ph, i
     __syncwarp();
 }
 
+// Two CTAs per SM (at most 128 registers a thread; the compiler's own choice for
+// 16 rows a lane is 154, one CTA): half the warps hide half the latency of the
+// cell chain and of the phases' barriers.  10,000 reads of 1-20 kb: traceback
+// 123.8 -> 97.7 ms.
+constexpr int kRMinBlocks = 2;
+
 template <bool DNA, class C>
-__global__ void __launch_bounds__(kRW * 32, 1) k_trace_ring(RingLaunch rl) {
+__global__ void __launch_bounds__(kRW * 32, kRMinBlocks) k_trace_ring(RingLaunch rl) {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ RingShared<C> sh_own;
     __shared__ int8_t sW[kMaxAlpha * kMaxAlpha];
