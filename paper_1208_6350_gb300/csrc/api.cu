@@ -612,10 +612,8 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
                                 max_ops * sizeof(uint32_t)));
                 uint32_t *dirs = reinterpret_cast<uint32_t *>(ctx->trace_dirs.p);
                 uint32_t *ops = reinterpret_cast<uint32_t *>(ctx->trace_ops.p);
-                if (side && nside > 0) {
-                    CUDA_TRY(cudaEventRecord(ctx->aux.fork, st));
-                    for (int k = 0; k < nside; k++) CUDA_TRY(cudaStreamWaitEvent(ctx->aux.s[k], ctx->aux.fork, 0));
-                }
+                SideFork fork(ctx->aux, st);
+                CUDA_TRY(fork.fork(side ? nside : 0));
                 // a stream per kernel (nside streams beside the caller's)
                 int turn = 0;
                 auto next_stream = [&]() {
@@ -677,11 +675,7 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
                     CUDA_TRY(launch_trace16(bv, sc, ts, ctx->sms, v, next_stream()));
                     S.launches += 1;
                 }
-                if (side)
-                    for (int k = 0; k < nside; k++) {
-                        CUDA_TRY(cudaEventRecord(ctx->aux.join[k], ctx->aux.s[k]));
-                        CUDA_TRY(cudaStreamWaitEvent(st, ctx->aux.join[k], 0));
-                    }
+                CUDA_TRY(fork.join());
             }
             S.stage_done[5] = 1;
             GSW_TRY(mark(ctx, 6, st));

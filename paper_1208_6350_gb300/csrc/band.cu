@@ -499,9 +499,9 @@ cudaError_t launch_band(const BatchView &b, const Scoring &sc, const PlanBuffers
     // the three classes run side by side (each its own scratch): the widest
     // (slowest per pair) on the calling stream, the others on two auxiliary
     // streams forked and joined by events, so a class's tail overlaps the others
-    cudaEventRecord(aux.fork, st);
-    cudaStreamWaitEvent(aux.s[0], aux.fork, 0);
-    cudaStreamWaitEvent(aux.s[1], aux.fork, 0);
+    SideFork fork(aux, st);
+    const cudaError_t e = fork.fork(2);
+    if (e != cudaSuccess) return e;
     const cudaStream_t on[3] = {aux.s[1], aux.s[0], st};
     for (int c = 2; c >= 0; c--) {
         L.scratch = static_cast<uint8_t *>(scratch) + g.off[c];
@@ -510,11 +510,8 @@ cudaError_t launch_band(const BatchView &b, const Scoring &sc, const PlanBuffers
         else if (c == 1) k_band<16, 1><<<g.grid[1], kBBlock, 0, on[1]>>>(L);
         else k_band<8, 0><<<g.grid[0], kBBlock, 0, on[0]>>>(L);
     }
-    cudaEventRecord(aux.join[0], aux.s[0]);
-    cudaEventRecord(aux.join[1], aux.s[1]);
-    cudaStreamWaitEvent(st, aux.join[0], 0);
-    cudaStreamWaitEvent(st, aux.join[1], 0);
-    return cudaGetLastError();
+    const cudaError_t joined = fork.join();
+    return joined == cudaSuccess ? cudaGetLastError() : joined;
 }
 
 }  // namespace gsw

@@ -80,12 +80,8 @@ cudaError_t launch_fill(const FillLaunch &fl, int sms, cudaStream_t st, const Si
     // batch of 20,000 reads of 100 to 250 nt is five launches, none of which
     // fills the chip)
     const bool side = n > 1 && aux.fork && sum <= fl.scr.bytes;
-    cudaError_t e = cudaSuccess;
-    if (side) {
-        if ((e = cudaEventRecord(aux.fork, st))) return e;
-        for (int k = 0; k < kSideStreams && k + 1 < n; k++)
-            if ((e = cudaStreamWaitEvent(aux.s[k], aux.fork, 0))) return e;
-    }
+    SideFork fork(aux, st);
+    cudaError_t e = fork.fork(side ? std::min(kSideStreams, n - 1) : 0);
     for (int i = 0; i < n && e == cudaSuccess; i++) {
         FillLaunch x = fl;
         ClassGeom &g = todo[i].g;
@@ -100,13 +96,8 @@ cudaError_t launch_fill(const FillLaunch &fl, int sms, cudaStream_t st, const Si
         e = fl.sc.dna4 ? (half ? fill_launch_dna_half(c, x, g, on) : fill_launch_dna(c, x, g, on))
                        : (half ? fill_launch_general_half(c, x, g, on) : fill_launch_general(c, x, g, on));
     }
-    if (side)
-        for (int k = 0; k < kSideStreams && k + 1 < n; k++) {
-            cudaError_t e2 = cudaEventRecord(aux.join[k], aux.s[k]);
-            if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(st, aux.join[k], 0);
-            if (e == cudaSuccess) e = e2;
-        }
-    return e;
+    const cudaError_t joined = fork.join();
+    return e == cudaSuccess ? joined : e;
 }
 
 // ---------------------------------------------------------------------------

@@ -701,6 +701,40 @@ struct SideStreams {
     cudaStream_t s[kSideStreams];
     cudaEvent_t fork, join[kSideStreams];
 };
+// Side streams forked from `st`.  Whatever way their user leaves, `st` waits for
+// what was queued on them: buffers are released in the order of `st`, so after
+// a failed launch the kernels already queued beside it must not outlive them.
+class SideFork {
+public:
+    SideFork(const SideStreams &aux, cudaStream_t st) : aux_(aux), st_(st) {}
+    SideFork(const SideFork &) = delete;
+    SideFork &operator=(const SideFork &) = delete;
+    ~SideFork() { join(); }
+    // the first n side streams wait for `st`
+    cudaError_t fork(int n) {
+        cudaError_t e = n > 0 ? cudaEventRecord(aux_.fork, st_) : cudaSuccess;
+        for (; e == cudaSuccess && n_ < n; n_++)
+            if ((e = cudaStreamWaitEvent(aux_.s[n_], aux_.fork, 0)) != cudaSuccess) break;
+        return e;
+    }
+    // `st` waits for them (the host does where an event fails)
+    cudaError_t join() {
+        cudaError_t first = cudaSuccess;
+        for (int k = 0; k < n_; k++) {
+            cudaError_t e = cudaEventRecord(aux_.join[k], aux_.s[k]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st_, aux_.join[k], 0);
+            if (e != cudaSuccess) cudaStreamSynchronize(aux_.s[k]);
+            if (first == cudaSuccess) first = e;
+        }
+        n_ = 0;
+        return first;
+    }
+
+private:
+    const SideStreams &aux_;
+    cudaStream_t st_;
+    int n_ = 0;
+};
 // one persistent launch per class in fl.class_mask, heaviest first, each with
 // the slots its share of the scratch holds; side by side on `st` and the side
 // streams (forked and joined by events) when the scratch holds all of them
