@@ -484,25 +484,22 @@ __host__ __device__ inline int band_range(int la, int lb, int score1, const Scor
 // Traceback classes of the pairs the band kernel leaves (bands wider than 32
 // diagonals, or small batches): 0-3 anti-diagonal warp kernel (bands of at
 // most 64/128/256/512 diagonals), 4 the CTA strip kernel (wider bands), 5-8
-// the 16-bit full-rectangle kernel with strips of 64/128/192/256 query rows
-// (8 lanes x R = 4/8/12/16 words x 2 halves; regions taller than the class's
-// strip run several strips: 256-row strips for DNA; other alphabets 64-row
-// strips, and 128-row ones with a larger scratch allowance for regions whose
-// decisions exceed kT16MaxWords in 64-row strips).
-#ifndef GSW_T16_GEN_VMAX
-#define GSW_T16_GEN_VMAX 0
-#endif
+// the 16-bit full-rectangle kernel.  DNA: 5-8, strips of 64/128/192/256 query
+// rows (8 lanes x R = 4/8/12/16 words x 2 halves; taller regions run several
+// 256-row strips).  Other alphabets: 5, and 6 with a larger scratch allowance
+// for regions whose scratch would exceed kT16MaxWords (strips by t16_shape).
 constexpr int kTraceRingClass = 4;
 constexpr int kTraceT16First = 5;
 constexpr int kTraceT16Classes = 4;
 constexpr int kT16P = 8;                   // lanes per pair
 constexpr int kT16MaxCols = 4096;          // longest target region of the 16-bit kernel
 constexpr long long kT16MaxWords = 1 << 17;  // scratch words of one pair (512 KB)
-// general alphabets: regions over kT16MaxWords in 64-row strips take the
-// 128-row class with this allowance (its own launch and scratch, so the few
-// large pairs do not shrink the groups of the others)
+// general alphabets: regions over kT16MaxWords take class 6 with this
+// allowance (its own launch and scratch, so the few large pairs do not shrink
+// the groups of the others)
 constexpr long long kT16MaxWordsBig = 1 << 20;
-// Class v as trace_class names and sizes it: 8 lanes, strips of 64(v+1) rows.
+// 8 lanes and strips of 64(v+1) rows: the shapes of DNA's classes v, and of
+// v = 0 for other alphabets
 __host__ __device__ inline int t16_R(int v) { return 4 * (v + 1); }
 __host__ __device__ inline int t16_strip_rows(int v) { return 2 * kT16P * t16_R(v); }
 __host__ __device__ inline int t16_strips(int la, int v) { return (la + t16_strip_rows(v) - 1) / t16_strip_rows(v); }
@@ -518,10 +515,10 @@ __host__ __device__ inline long long t16_need_words(int la, int lb, int v) {
     return t16_strips(la, v) > 1 ? d + 2LL * ((lb + 3) & ~3) : d;
 }
 // How launch class v runs: P lanes a pair and R row words a lane, so strips of
-// 2PR rows.  DNA: as its name says.  Other alphabets have three launches: v = 0
-// (64-row strips), and whole warps with 256-row strips for v = 1 (regions whose
-// decisions are too many for v = 0's scratch) and v = 2 (regions of v = 0 taller
-// than kT16Tall rows): a group of 8 lanes runs the 16 strips of a 1,000-row
+// 2PR rows.  DNA: the trace class's.  Other alphabets have three launches: v = 0
+// (64-row strips), and whole warps with 256-row strips for v = 1 (regions over
+// kT16MaxWords) and v = 2 (regions of trace class 5 taller than kT16Tall
+// rows): a group of 8 lanes runs the 16 strips of a 1,000-row
 // region one after the other, and beside the bulk of the pairs those few
 // regions then ended last (40 x 1,000 protein pairs: traceback 9.0 -> 5.9 ms).
 struct T16Shape {
@@ -550,32 +547,32 @@ __host__ __device__ inline int trace_class(int la, int lb, int score1, const Sco
     const int width = band_range(la, lb, score1, sc, dlo, dhi);
     const int ad = width <= 64 ? 0 : width <= 128 ? 1 : width <= 256 ? 2 : width <= 512 ? 3 : kTraceRingClass;
     if (la >= 1 && lb >= 1 && lb <= kT16MaxCols) {
-        // general alphabets keep A x R profile words per lane: 64-row strips
-        // (128 measured 2.5 % slower on protein search: a third of the warps per SM)
-        const int vmax = sc.dna4 ? kTraceT16Classes - 1 : GSW_T16_GEN_VMAX;
-        const int v0 = (la - 1) / 64;
-        int v = v0 < vmax ? v0 : vmax;
+        // the shape of the launch the region would take; general alphabets keep
+        // A x R profile words per lane, so their 8-lane strips have 64 rows (128
+        // measured 2.5 % slower on protein search: a third of the warps per SM)
+        const bool dna = sc.dna4 != 0;
+        int v = dna ? (la - 1) / 64 : 0;
+        v = v < kTraceT16Classes ? v : kTraceT16Classes - 1;
+        T16Shape shape = t16_shape(t16_launch_class(kTraceT16First + v, la, dna) - kTraceT16First, dna);
         long long cap = kT16MaxWords;
-        if (!sc.dna4 && v == 0 && t16_need_words(la, lb, 0) > kT16MaxWords) {
+        if (!dna && shape.need_words(la, lb) > kT16MaxWords) {
             v = 1;
+            shape = t16_shape(v, dna);
             cap = kT16MaxWordsBig;
         }
-        const long long rows = (long long)t16_strips(la, v) * t16_strip_rows(v);
-        const long long cols = lb + 2 * kT16P;
+        const long long rows = (long long)shape.strips(la) * shape.rows();
+        const long long cols = lb + 2 * shape.P;
         // every value of the DP over the padded rectangle lies in
         // [-(3O + X(rows + cols) + |wmin|), wmax * min(rows, cols) + wmax]:
         // it must fit a biased 16-bit lane
-        const T16Shape shape = t16_shape(t16_launch_class(kTraceT16First + v, la, sc.dna4 != 0) - kTraceT16First,
-                                         sc.dna4 != 0);
-        const long long padded = (long long)shape.strips(la) * shape.rows();
-        const long long lo = 3LL * sc.O + (long long)sc.X * (padded + cols + 2) - (sc.wmin < 0 ? sc.wmin : 0);
-        const long long hi = (long long)sc.wmax * ((cols < padded ? cols : padded) + 1);
-        if (lo <= 30000 && hi <= 30000 && t16_need_words(la, lb, v) <= cap) {
+        const long long lo = 3LL * sc.O + (long long)sc.X * (rows + cols + 2) - (sc.wmin < 0 ? sc.wmin : 0);
+        const long long hi = (long long)sc.wmax * ((cols < rows ? cols : rows) + 1);
+        if (lo <= 30000 && hi <= 30000 && shape.need_words(la, lb) <= cap) {
             // cell updates: the padded rectangle against the band's
             // anti-diagonal slots; a 16-bit pair of cells costs about the
             // instructions of one 32-bit anti-diagonal cell
             // (bands wider than 512 diagonals: the rectangle always)
-            const long long rect = rows * t16_steps(lb);
+            const long long rect = rows * shape.steps(lb);
             if (ad == kTraceRingClass) return kTraceT16First + v;
             const long long band = (32LL << ad) * (la + lb + 1);
             if (rect <= (small ? 2 : 3) * band) return kTraceT16First + v;
@@ -628,13 +625,13 @@ __host__ __device__ inline void trace_needs(const gsw_result &r, const Scoring &
 inline bool ring_possible(int maxm, int maxn, const Scoring &sc) {
     if (maxm + maxn + 1 <= 512) return false;
     if (maxn > kT16MaxCols) return true;
-    const long long rows = (long long)maxm + 256, cols = maxn + 2 * kT16P;
+    const long long rows = (long long)maxm + 256, cols = maxn + 2 * (sc.dna4 ? kT16P : 32);
     const long long lo = 3LL * sc.O + (long long)sc.X * (rows + cols + 2) - (sc.wmin < 0 ? sc.wmin : 0);
     const long long hi = (long long)sc.wmax * ((cols < rows ? cols : rows) + 1);
     if (lo > 30000 || hi > 30000) return true;
     const int m = maxm < 1 ? 1 : maxm, n = maxn < 1 ? 1 : maxn;
     if (sc.dna4) return t16_need_words(m, n, kTraceT16Classes - 1) > kT16MaxWords;
-    return t16_need_words(m, n, 0) > kT16MaxWords && t16_need_words(m, n, 1) > kT16MaxWordsBig;
+    return t16_shape(1, false).need_words(m, n) > kT16MaxWordsBig;
 }
 
 #ifdef __CUDACC__

@@ -63,6 +63,16 @@ int cr_trace(int A, const signed char *W, int O, int X, int maxm, int maxn, int 
     return gsw::trace_class(la, lb, score1, sc, small != 0, &dlo, &dhi);
 }
 
+// the 16-bit rectangle as a region of trace class `cls` launches it: scratch
+// words, and the rows and columns it computes
+void cr_rectangle(int A, int cls, int la, int lb, long long *out) {
+    const int v = gsw::t16_launch_class(cls, la, A == 4) - gsw::kTraceT16First;
+    const gsw::T16Shape s = gsw::t16_shape(v, A == 4);
+    out[0] = s.need_words(la, lb);
+    out[1] = (long long)s.strips(la) * s.rows();
+    out[2] = lb + 2 * s.P;
+}
+
 int cr_consts(int which) {
     const int c[] = {gsw::kNumVariants, gsw::kVarP4First, gsw::kVarTallFirst, gsw::kTraceRingClass, gsw::kClassLong16};
     return c[which];

@@ -34,6 +34,8 @@ def lib(tmp_path_factory):
     L.cr_route_tuned.argtypes = [i32, P, i32, i32, P, i32, i32, i32, i32, ctypes.c_double, i32, i32, i32, P]
     L.cr_route_tuned.restype = None
     L.cr_half_fits.argtypes = [i32, P, i32, i32, i32, i32]
+    L.cr_rectangle.argtypes = [i32, i32, i32, i32, P]
+    L.cr_rectangle.restype = None
     L.cr_trace.argtypes = [i32, P, i32, i32, i32, i32, i32, i32, i32, i32, ctypes.POINTER(i32)]
     return L
 
@@ -121,6 +123,26 @@ def test_a_tune_table_keeps_the_classes_it_names(lib):
     assert several > 100
 
 
+def test_large_batches_run_several_strips_in_groups(lib):
+    # 20,000 pairs of 540 to 1,400 x 600 to 1,000 (compared with the oracle in
+    # tests/test_gpu_large_batches.py): no query goes to a CTA, and the classes
+    # of 320 to 512 rows are among those of several strips
+    tall, nvar = lib.cr_consts(2), lib.cr_consts(0)
+    out = (ctypes.c_uint * 5)()
+    seen = {}
+    for A, match, mismatch, O, X in ((4, 1, -3, 5, 2), (4, 5, -4, 10, 1), (20, 6, -2, 11, 1)):
+        W = np.full((A, A), mismatch, np.int8)
+        np.fill_diagonal(W, match)
+        for rows in range(540, 1401):
+            lib.cr_route(A, W.ctypes.data_as(ctypes.c_void_p), O, X, 20_000, 540, 1400, 1000, 20_000 * 970.0 * 800.0,
+                         FORWARD, rows, 1000, out)
+            _, half, _, v, strip = out
+            assert v < nvar and rows > strip, (A, rows, v)
+            seen.setdefault((A, match, bool((half >> v) & 1)), set()).add(v)
+    assert (4, 1, True) in seen and (4, 5, False) in seen and (20, 6, False) in seen
+    assert all(any(v >= tall for v in s) and any(v < tall for v in s) for s in seen.values()), seen
+
+
 def test_wide_bands_are_never_left_out(lib):
     rng = np.random.default_rng(23)
     ring_class = lib.cr_consts(3)
@@ -139,3 +161,29 @@ def test_wide_bands_are_never_left_out(lib):
             wide += cls == ring_class
             without += not ring.value
     assert wide and without
+
+
+def test_rectangles_fit_the_shape_that_runs_them(lib):
+    # scratch of a class within its allowance, and every value of the padded
+    # rectangle within a biased 16-bit lane, in the strips and groups launched
+    rng = np.random.default_rng(31)
+    out = (ctypes.c_longlong * 3)()
+    ring = ctypes.c_int()
+    tall = large = 0
+    for W, O, X in list(schemes()) + [(np.full((20, 20), 2, np.int8), 11, 10), (np.full((24, 24), 40, np.int8), 5, 2)]:
+        p, A = W.ctypes.data_as(ctypes.c_void_p), len(W)
+        for _ in range(4000):
+            la, lb = edge_lengths(rng, 4096), edge_lengths(rng, 4096)
+            score = int(rng.integers(1, max(2, min(la, lb) * max(int(W.max()), 1) + 1)))
+            cls = lib.cr_trace(A, p, O, X, la, lb, la, lb, score, int(rng.integers(0, 2)), ctypes.byref(ring))
+            if cls < 5:
+                continue
+            lib.cr_rectangle(A, cls, la, lb, out)
+            words, rows, cols = out
+            what = (A, O, X, la, lb, cls, words, rows, cols)
+            assert words <= (1 << 17 if A == 4 or cls == 5 else 1 << 20), what
+            assert 3 * O + X * (rows + cols + 2) - min(0, int(W.min())) <= 30000, what
+            assert int(W.max()) * (min(rows, cols) + 1) <= 30000, what
+            tall += A != 4 and la > 256
+            large += cls == 6 and A != 4
+    assert tall and large
