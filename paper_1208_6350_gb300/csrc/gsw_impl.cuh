@@ -789,6 +789,7 @@ int context_device(const gsw_ctx *ctx);
 // Rounds a call's shapes (largest lengths, traceback scratch) up to powers of
 // two, so that calls of similar shape repeat a captured pipeline (serving).
 void context_set_graph_buckets(gsw_ctx *ctx, bool on);
+void context_set_shared(gsw_ctx *ctx, bool on);  // other contexts' batches run beside this one's
 int ring_slots_per_cta();
 // prefix sums of the class's direction words; out[0] total, [1] max words of a pair, [2] max op words
 cudaError_t launch_ring_needs(const BatchView &b, const Scoring &sc, const int32_t *order, const int32_t *var_start,
