@@ -117,6 +117,7 @@ struct gsw_ctx {
     GraphCache seg[2];              // before and after the traceback readback
     bool graph_buckets = false;     // round shapes up to buckets so graphs repeat (serving)
     bool shared = false;            // other contexts' batches run beside this one's (serving)
+    bool one_cta = false;           // ... and this one's long reads run without clusters
     bool capturing = false;         // a segment is being captured: no allocation
     cudaStream_t st = nullptr;     // stream of the call in progress
     DevBuf plan_keys, plan_order, plan_small;
@@ -361,6 +362,7 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
     key_add(key, st);
     key_add(key, ctx->sms);
     key_add(key, ctx->shared);
+    key_add(key, ctx->one_cta);
     key_add(key, ctx->budget);
     key_add(key, ctx->used);
     key_add(key, ctx->timing);
@@ -396,6 +398,7 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
         fl.b = bv;
         fl.sc = sc;
         fl.maxm = maxm;
+        fl.one_cta = ctx->one_cta;
         fl.bad_letters = reinterpret_cast<const int32_t *>(misc + kMiscValid);
         fl.plan.order = pb.order;
         fl.plan.var_start = pb.var_start;
@@ -646,6 +649,7 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
                     ra.ops = ops + ring.op_at;
                     ra.op_words = (long long)ring_ops;
                     ra.walk_warps = (int)ring_walk_warps;
+                    ra.one_cta = ctx->one_cta;
                     // every group but the last fills more than pool - max_pair
                     const unsigned long long per = ring_pool > ring_max ? ring_pool - ring_max : 1;
                     const unsigned long long groups =
@@ -1042,7 +1046,10 @@ int gsw_context_create(int device, size_t mem_budget_bytes, gsw_ctx **out) {
 namespace gsw {
 int context_device(const gsw_ctx *ctx) { return ctx->device; }
 void context_set_graph_buckets(gsw_ctx *ctx, bool on) { ctx->graph_buckets = on; }
-void context_set_shared(gsw_ctx *ctx, bool on) { ctx->shared = on; }
+void context_set_shared(gsw_ctx *ctx, bool on, bool one_cta) {
+    ctx->shared = on;
+    ctx->one_cta = on && one_cta;
+}
 }  // namespace gsw
 
 extern "C" {

@@ -1409,8 +1409,7 @@ ClassGeom long_geom(const FillLaunch &fl, int sms) {
     ClassGeom g;
     // (DNA, so in the reversed fill a pair's band is what its strips run)
     const int ctas = ((fl.maxm + C::SP - 1) / C::SP + C::NW - 1) / C::NW;
-    if (fl.b.npairs <= kLongFewPairs)
-        while (g.cluster < ctas && g.cluster < kLongMaxCluster) g.cluster *= 2;
+    g.cluster = cluster_ctas(fl.b.npairs, kLongFewPairs, ctas, kLongMaxCluster, fl.one_cta);
     if constexpr (DNA && !S32 && !NARROW)
         if (fl.mode == kFillReverse && g.cluster > 1 && fl.b.npairs <= kLongNarrowPairs)
             return long_geom<DNA, S32, true>(fl, sms);

@@ -355,6 +355,19 @@ struct FillScratch {
     int32_t ncap;    // columns per slot (a multiple of 4: 8-byte stores of four 16-bit maxima)
 };
 
+// CTAs that share the pairs of a launch of the CTA kernels: as many as a pair's
+// strips fill (`want`, a power of two up to `most`) where the batch's few pairs
+// leave the chip to the longest one, else one.  One also where other batches
+// need the chip meanwhile (one_cta: a server's heavy worker): a cluster's CTAs hold
+// their SMs until its longest pair ends, most of them waiting at its barriers
+// (mixed stream at 10,000 requests/s: 1,193 GCUPS with clusters, 1,254 without).
+inline int cluster_ctas(int npairs, int few, int want, int most, bool one_cta) {
+    int c = 1;
+    if (npairs <= few && !one_cta)
+        while (c < want && c < most) c *= 2;
+    return c;
+}
+
 struct FillLaunch {
     BatchView b;
     Scoring sc;
@@ -362,6 +375,7 @@ struct FillLaunch {
     FillScratch scr;
     int32_t mode;
     int32_t maxm;         // longest query
+    bool one_cta;         // no clusters (cluster_ctas)
     uint32_t class_mask;  // classes launched (bit c: class c); the others hold no pair
     uint32_t multi_mask;  // classes that can hold pairs of several strips
     uint32_t half_mask;   // classes whose values stay below 2048: the half-precision clamp lanes
@@ -783,13 +797,16 @@ struct RingLaunchArgs {
     uint32_t *ops;            // walk: walk_warps x op_words
     long long op_words;
     int walk_warps;
+    bool one_cta;             // no clusters (cluster_ctas)
 };
 int ring_trace_class();
 int context_device(const gsw_ctx *ctx);
 // Rounds a call's shapes (largest lengths, traceback scratch) up to powers of
 // two, so that calls of similar shape repeat a captured pipeline (serving).
 void context_set_graph_buckets(gsw_ctx *ctx, bool on);
-void context_set_shared(gsw_ctx *ctx, bool on);  // other contexts' batches run beside this one's
+// Other contexts' batches run beside this one's: its kernels keep to the
+// caller's stream, and with one_cta to one CTA per pair (cluster_ctas).
+void context_set_shared(gsw_ctx *ctx, bool on, bool one_cta);
 int ring_slots_per_cta();
 // prefix sums of the class's direction words; out[0] total, [1] max words of a pair, [2] max op words
 cudaError_t launch_ring_needs(const BatchView &b, const Scoring &sc, const int32_t *order, const int32_t *var_start,

@@ -113,7 +113,7 @@ int alloc_worker(Worker *w, const gsw_serve_config &c, size_t budget) {
     const size_t staging = 2 * L + P * (16 + 8 + sizeof(gsw_result)) + G * 4;
     if (budget <= staging) return GSW_ENOMEM;
     const int rc = gsw_context_create(c.device, budget - staging, &w->ctx);
-    if (rc == GSW_OK) gsw::context_set_shared(w->ctx, c.workers > 1);
+    if (rc == GSW_OK) gsw::context_set_shared(w->ctx, c.workers > 1, w->heavy);
     if (rc == GSW_OK && !w->heavy && c.light_graphs >= 0) {
         w->graphs = true;
         gsw::context_set_graph_buckets(w->ctx, true);

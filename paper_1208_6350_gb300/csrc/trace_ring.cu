@@ -746,7 +746,7 @@ cudaError_t launch_ring_fill(const RingLaunch &rl, const RingLaunchArgs &a, int 
     cudaFuncSetAttribute(k_trace_ring<DNA, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_trace_ring<DNA, C>, nw * 32, smem);
     if (nb < 1) return cudaErrorInvalidConfiguration;
-    int cl = C::RR == 8 ? kRMaxCluster : 1;
+    int cl = cluster_ctas(a.b.npairs, kRingFewPairs, kRMaxCluster, kRMaxCluster, a.one_cta);
     long long grid = std::min<long long>((long long)sms * nb, a.slots / kRSlots);
     grid = std::min<long long>(grid, (long long)a.b.npairs * cl);
     if (grid < cl) cl = 1;

@@ -73,6 +73,10 @@ void cr_rectangle(int A, int cls, int la, int lb, long long *out) {
     out[2] = lb + 2 * s.P;
 }
 
+int cr_cluster(int npairs, int few, int want, int most, int one_cta) {
+    return gsw::cluster_ctas(npairs, few, want, most, one_cta != 0);
+}
+
 int cr_consts(int which) {
     const int c[] = {gsw::kNumVariants, gsw::kVarP4First, gsw::kVarTallFirst, gsw::kTraceRingClass, gsw::kClassLong16};
     return c[which];

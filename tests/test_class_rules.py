@@ -187,3 +187,15 @@ def test_rectangles_fit_the_shape_that_runs_them(lib):
             tall += A != 4 and la > 256
             large += cls == 6 and A != 4
     assert tall and large
+
+
+def test_clusters_only_where_a_batch_has_the_chip_to_itself(lib):
+    for npairs in (1, 40, 2048, 2049, 10_000):
+        for want in (0, 1, 2, 3, 5, 8, 40):
+            c = lib.cr_cluster(npairs, 2048, want, 8, 0)
+            if npairs > 2048 or want <= 1:
+                assert c == 1
+            else:
+                assert c == min(8, 1 << (want - 1).bit_length()), (npairs, want, c)
+            assert lib.cr_cluster(npairs, 2048, want, 8, 1) == 1  # a server's heavy worker
+    assert lib.cr_cluster(300, 2048, 4, 4, 0) == 4
