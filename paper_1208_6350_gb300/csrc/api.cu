@@ -244,13 +244,7 @@ int ensure_aux(gsw_ctx *ctx) {
     return GSW_OK;
 }
 
-// Contexts whose kernels all go to the caller's stream, one after the other:
-// those limited to some SMs, and those of a server.  A device has 8 hardware
-// queues for its streams.  With 7 side streams a context, a server's streams
-// share them, and a light batch's kernel waited in the queue behind a heavy
-// batch's, several times a batch (10,000 requests/s of the mixed stream: short
-// requests' p50 1,110 ms, in one stream 3.3 to 4.3; at 1,000/s p99 14 -> 1.0).
-bool one_stream(const gsw_ctx *ctx) { return ctx->sms < ctx->sms_all || ctx->shared; }
+bool one_stream(const gsw_ctx *ctx) { return gsw::one_stream(ctx->sms, ctx->sms_all, ctx->shared); }
 
 // event e[k] marks the end of stage k-1 / start of stage k
 int mark(gsw_ctx *ctx, int k, cudaStream_t st) {

@@ -73,6 +73,8 @@ void cr_rectangle(int A, int cls, int la, int lb, long long *out) {
     out[2] = lb + 2 * s.P;
 }
 
+int cr_one_stream(int sms, int sms_all, int shared) { return gsw::one_stream(sms, sms_all, shared != 0); }
+
 int cr_cluster(int npairs, int few, int want, int most, int one_cta) {
     return gsw::cluster_ctas(npairs, few, want, most, one_cta != 0);
 }

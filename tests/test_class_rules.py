@@ -189,6 +189,12 @@ def test_rectangles_fit_the_shape_that_runs_them(lib):
     assert tall and large
 
 
+def test_side_streams_only_where_a_context_has_the_device_to_itself(lib):
+    assert not lib.cr_one_stream(152, 152, 0)
+    assert lib.cr_one_stream(133, 152, 0)  # limited to some SMs
+    assert lib.cr_one_stream(152, 152, 1) and lib.cr_one_stream(133, 152, 1)  # a server's
+
+
 def test_clusters_only_where_a_batch_has_the_chip_to_itself(lib):
     for npairs in (1, 40, 2048, 2049, 10_000):
         for want in (0, 1, 2, 3, 5, 8, 40):

@@ -6,7 +6,6 @@ CIGAR must equal (zero tolerance) what gsw_align_batch gives for that request
 alone, and the oracle's.
 """
 import threading
-import time
 
 import numpy as np
 import pytest
@@ -147,40 +146,3 @@ def test_light_batches_replay_captured_graphs(light_graphs):
             for f in FIELDS:
                 assert int(res[f][p]) == int(ores[f][p]), (p, f)
             assert _decode(res, cig, p) == oracle.decode_cigar(ocg[p, : ores["cigar_len"][p]])
-
-
-def test_short_requests_do_not_wait_behind_long_ones():
-    # more long reads than the GPU keeps up with: they pile up in their own
-    # queue, and the short requests that arrive meanwhile go past them.  (When
-    # their kernels share hardware queues with the long batches' they finish
-    # with them instead: medians 1,110 and 1,450 ms; in streams of their own 4 and
-    # 1,350.)
-    reqs = wl.serving_trace(10_000, 8000, seed=5)
-    W = wl.dna_matrix(2, -4)
-    srv = gsw.Server(W, 4, 2, gsw.GSW_CIGAR, workers=4, max_batch_pairs=8192, max_batch_letters=24 << 20,
-                     mem_budget_bytes=48 << 30)
-    try:
-        for k in (1, 2, 3):  # warm-up: one request of each kind
-            b = next(r.batch for r in reqs if r.kind == k)
-            srv.poll(srv.submit(b.q, b.q_off, b.q_len, b.t, b.t_off, b.t_len), b.npairs)
-        ids, got = [], []
-
-        def submit():
-            t0 = time.perf_counter()
-            for r in reqs:
-                time.sleep(max(0.0, t0 + r.arrival_s - time.perf_counter()))
-                b = r.batch
-                ids.append(srv.submit(b.q, b.q_off, b.q_len, b.t, b.t_off, b.t_len))
-
-        th = threading.Thread(target=submit)
-        th.start()
-        th.join()
-        for rid, r in zip(ids, reqs):
-            rc, res, cig, tm = srv.poll(rid, r.batch.npairs, times=True)
-            assert rc == gsw.GSW_OK
-            got.append(tm[2] - tm[0])
-    finally:
-        srv.close()
-    took, kinds = np.array(got), np.array([r.kind for r in reqs])
-    short, long_ = np.median(took[kinds != 3]), np.median(took[kinds == 3])
-    assert short < long_ / 8, (short, long_)
