@@ -317,7 +317,7 @@ def run_gsw(args):
         tune = ctx.autotune(b.W, b.gap_open, b.gap_extend, target_len=max(1, int(b.t_len.mean())))
         tune["seconds"] = round(time.perf_counter() - t0, 2)
         nb = max(1, min(gsw.TUNE_BUCKETS, int(np.ceil(b.q_len.max() / gsw.TUNE_ROWS))))
-        tune = {"buckets_of_rows": gsw.TUNE_ROWS, "fill_class": tune["fill_class"][:nb],
+        tune = {"buckets_of_rows": gsw.TUNE_ROWS, "fill_class": tune["installed"][:nb],
                 "gcups": tune["gcups"][:nb], "gcups_default_rule": tune["gcups_default"][:nb],
                 "seconds": tune["seconds"]}
     # a stream of its own: the library captures the repeated step's launch

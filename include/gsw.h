@@ -147,22 +147,25 @@ int gsw_context_destroy(gsw_ctx *ctx);
 #define GSW_TUNE_ROWS 32
 typedef struct gsw_tune {
     int8_t fill_class[GSW_TUNE_BUCKETS]; /* bucket b: queries of 32b+1 .. 32(b+1) rows */
-    float gcups[GSW_TUNE_BUCKETS];       /* measured forward-fill rate of what was installed */
-    float gcups_default[GSW_TUNE_BUCKETS]; /* ... of the default rule */
+    float gcups[GSW_TUNE_BUCKETS];       /* measured forward-fill rate of what the table installs */
+    float gcups_default[GSW_TUNE_BUCKETS]; /* ... of the default rule.  Where it is positive and not below
+                                              gcups the bucket is left to the default rule, and fill_class
+                                              holds the fastest class that can be named.  A table made by
+                                              hand has zeros here. */
 } gsw_tune;
 
 /* Measures every candidate class of every bucket on seeded random pairs
  * (queries of the bucket's largest length against targets of target_len
  * letters, the given scoring, score-only batches of about 2 G cells, best of 3
  * runs), installs the fastest in the context (a bucket where the default rule
- * is fastest is left to it) and copies the table of the fastest named classes
- * to *out (may be NULL).  Takes a few seconds; allocates its own temporary device buffers.
+ * is fastest is left to it) and copies the installed table to *out (may be
+ * NULL).  Takes a few seconds; allocates its own temporary device buffers.
  * Errors: GSW_EINVAL, GSW_ENOMEM, GSW_ECUDA. */
 int gsw_autotune(gsw_ctx *ctx, const int8_t *matrix, int32_t alphabet, int32_t gap_open, int32_t gap_extend,
                  int32_t target_len, gsw_tune *out);
 
-/* Installs a table (e.g. one saved from gsw_autotune); NULL restores the
- * default rule.  Errors: GSW_EINVAL (a class outside -1..6, 8..13). */
+/* Installs a table (one saved from gsw_autotune gives what that call
+ * installed); NULL restores the default rule.  Errors: GSW_EINVAL (a class outside -1..6, 8..13). */
 int gsw_context_set_tune(gsw_ctx *ctx, const gsw_tune *tune);
 
 /*

@@ -1057,7 +1057,7 @@ int gsw_context_set_tune(gsw_ctx *c, const gsw_tune *t) {
     for (int b = 0; b < GSW_TUNE_BUCKETS; b++)
         if (t->fill_class[b] < -1 || t->fill_class[b] > 13 || t->fill_class[b] == 7)
             return set_err(GSW_EINVAL, "fill class %d of bucket %d", t->fill_class[b], b);
-    std::memcpy(c->tune, t->fill_class, sizeof(c->tune));
+    for (int b = 0; b < GSW_TUNE_BUCKETS; b++) c->tune[b] = (int8_t)gsw::tuned_class(*t, b);
     return GSW_OK;
 }
 

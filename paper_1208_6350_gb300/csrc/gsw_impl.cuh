@@ -154,6 +154,12 @@ __host__ __device__ inline int pick_s16(int rows) {
     return kVarMaxS16;
 }
 
+// What a tune table gives bucket b: the class it names, or the default rule (-1)
+// where it holds rates (gsw_autotune's do) and the default rule's is no lower.
+inline int tuned_class(const gsw_tune &t, int b) {
+    return t.gcups_default[b] > 0 && t.gcups_default[b] >= t.gcups[b] ? -1 : t.fill_class[b];
+}
+
 // 16-bit fill class of a query of `rows` (>= 1): the tuned class of its
 // bucket, else the smallest one-strip variant, or the CTA class for queries
 // of many strips.

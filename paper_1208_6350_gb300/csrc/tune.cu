@@ -60,8 +60,7 @@ extern "C" int gsw_autotune(gsw_ctx *ctx, const int8_t *matrix, int32_t alphabet
     if (!ctx || !matrix || alphabet < 1 || alphabet > kMaxAlpha || target_len < 1 || target_len > (1 << 20))
         return GSW_EINVAL;
     if (cudaSetDevice(context_device(ctx)) != cudaSuccess) return GSW_ECUDA;
-    gsw_tune tune, use;  // the fastest named classes; the same, with the buckets left to the default rule
-    std::memset(use.fill_class, -1, sizeof(use.fill_class));
+    gsw_tune tune;
     std::memset(tune.fill_class, -1, sizeof(tune.fill_class));
     std::memset(tune.gcups, 0, sizeof(tune.gcups));
     std::memset(tune.gcups_default, 0, sizeof(tune.gcups_default));
@@ -125,7 +124,7 @@ extern "C" int gsw_autotune(gsw_ctx *ctx, const int8_t *matrix, int32_t alphabet
         int best = def;
         cand.push_back(-1);  // the default rule
         for (int c : cand) {
-            gsw_tune one;
+            gsw_tune one = {};
             std::memset(one.fill_class, -1, sizeof(one.fill_class));
             one.fill_class[b] = (int8_t)c;
             if ((rc = gsw_context_set_tune(ctx, &one)) != GSW_OK) break;
@@ -150,8 +149,8 @@ extern "C" int gsw_autotune(gsw_ctx *ctx, const int8_t *matrix, int32_t alphabet
                 best = c;
             }
         }
+        // (equal rates leave the bucket to the default rule, tuned_class)
         tune.fill_class[b] = (int8_t)best;
-        use.fill_class[b] = (int8_t)(def_rate >= best_rate ? -1 : best);
         tune.gcups[b] = std::max(best_rate, def_rate);
         tune.gcups_default[b] = def_rate;
     }
@@ -161,7 +160,7 @@ extern "C" int gsw_autotune(gsw_ctx *ctx, const int8_t *matrix, int32_t alphabet
         gsw_context_set_tune(ctx, nullptr);
         return rc;
     }
-    rc = gsw_context_set_tune(ctx, &use);
+    rc = gsw_context_set_tune(ctx, &tune);
     if (out) *out = tune;
     return rc;
 }

@@ -385,20 +385,27 @@ class Context:
 
     def autotune(self, matrix, gap_open, gap_extend, target_len=1000) -> dict:
         """Measures the fill class per query-length bucket (gsw_autotune) and
-        installs the fastest; returns {"fill_class", "gcups", "gcups_default"}."""
+        installs the fastest; returns {"fill_class", "gcups", "gcups_default",
+        "installed"}: per bucket the fastest class that can be named, the rates
+        (GCUPS) of what was installed and of the default rule, and the class
+        installed (-1 where the default rule is the fastest)."""
         m = np.ascontiguousarray(matrix, dtype=np.int8)
         t = GswTune()
         _check(load().gsw_autotune(self.handle, m.ctypes.data, m.shape[0], gap_open, gap_extend, target_len,
                                    ctypes.byref(t)), "gsw_autotune")
-        return {"fill_class": list(t.fill_class), "gcups": [round(x, 1) for x in t.gcups],
+        installed = [-1 if 0 < d >= g else c for c, g, d in zip(t.fill_class, t.gcups, t.gcups_default)]
+        return {"fill_class": list(t.fill_class), "installed": installed, "gcups": [round(x, 1) for x in t.gcups],
                 "gcups_default": [round(x, 1) for x in t.gcups_default]}
 
     def set_tune(self, fill_class=None):
-        """Installs a class per bucket (-1 default rule, 0..6 group variants, 8
-        the CTA kernel); None restores the default rule."""
+        """Installs a class per bucket (-1 default rule, 0..6 and 9..13 group
+        variants, 8 the CTA kernel), or what an autotune() returned installed;
+        None restores the default rule."""
         if fill_class is None:
             _check(load().gsw_context_set_tune(self.handle, None), "gsw_context_set_tune")
             return
+        if isinstance(fill_class, dict):
+            fill_class = fill_class["installed"]
         t = GswTune()
         for b, c in enumerate(fill_class):
             t.fill_class[b] = int(c)

@@ -79,6 +79,15 @@ int cr_cluster(int npairs, int few, int want, int most, int one_cta) {
     return gsw::cluster_ctas(npairs, few, want, most, one_cta != 0);
 }
 
+// class that a table of these values gives its bucket
+int cr_tuned_class(int fill_class, float gcups, float gcups_default) {
+    gsw_tune t = {};
+    t.fill_class[7] = (signed char)fill_class;
+    t.gcups[7] = gcups;
+    t.gcups_default[7] = gcups_default;
+    return gsw::tuned_class(t, 7);
+}
+
 int cr_consts(int which) {
     const int c[] = {gsw::kNumVariants, gsw::kVarP4First, gsw::kVarTallFirst, gsw::kTraceRingClass, gsw::kClassLong16};
     return c[which];

@@ -205,3 +205,41 @@ def test_clusters_only_where_a_batch_has_the_chip_to_itself(lib):
                 assert c == min(8, 1 << (want - 1).bit_length()), (npairs, want, c)
             assert lib.cr_cluster(npairs, 2048, want, 8, 1) == 1  # a server's heavy worker
     assert lib.cr_cluster(300, 2048, 4, 4, 0) == 4
+
+
+def test_a_saved_tune_table_installs_what_was_tuned(lib, monkeypatch):
+    from paper_1208_6350_gb300 import gsw
+    lib.cr_tuned_class.argtypes = [ctypes.c_int, ctypes.c_float, ctypes.c_float]
+    rng = np.random.default_rng(37)
+    named = rng.choice([0, 1, 2, 3, 4, 5, 6, 8, 9, 10, 11, 12, 13], gsw.TUNE_BUCKETS).astype(int)
+    rule = rng.uniform(1000, 4000, gsw.TUNE_BUCKETS).astype(np.float32)
+    own = np.where(np.arange(gsw.TUNE_BUCKETS) % 3 == 0, rule, rule + np.float32(0.01))  # the rule wins every third
+    want = [-1 if b % 3 == 0 else int(named[b]) for b in range(gsw.TUNE_BUCKETS)]
+    assert [lib.cr_tuned_class(int(named[b]), own[b], rule[b]) for b in range(gsw.TUNE_BUCKETS)] == want
+    # a table without rates (made by hand), or one that names the default rule
+    assert lib.cr_tuned_class(9, 0.0, 0.0) == 9 and lib.cr_tuned_class(-1, 0.0, 0.0) == -1
+
+    class Lib:  # stands in for the library: a tuned table, and what is installed
+        def gsw_autotune(self, ctx, m, a, o, x, n, out):
+            t = out._obj
+            for b in range(gsw.TUNE_BUCKETS):
+                t.fill_class[b], t.gcups[b], t.gcups_default[b] = int(named[b]), own[b], rule[b]
+            return gsw.GSW_OK
+
+        def gsw_context_set_tune(self, ctx, table):
+            t = table._obj
+            self.table = [lib.cr_tuned_class(t.fill_class[b], t.gcups[b], t.gcups_default[b])
+                          for b in range(gsw.TUNE_BUCKETS)]
+            return gsw.GSW_OK
+
+    fake = Lib()
+    monkeypatch.setattr(gsw, "load", lambda: fake)
+    ctx = gsw.Context.__new__(gsw.Context)
+    ctx.handle = None
+    t = ctx.autotune(np.eye(4, dtype=np.int8), 1, 1)
+    for saved in (t, t["installed"]):
+        ctx.set_tune(saved)
+        assert fake.table == want
+    assert t["fill_class"] == named.tolist()
+    ctx.set_tune(t["fill_class"])  # the classes alone: as named
+    assert fake.table == named.tolist()
