@@ -14,9 +14,12 @@ namespace gsw {
 namespace {
 
 constexpr int kScanThreads = 1024;
-// Batches of at most this many pairs are planned by one block (16 pairs a
-// thread at most).
-constexpr int kPlanSmall = 16384;
+// Batches of at most this many pairs are planned by one block.  Beyond, the
+// block's turns over the pairs cost more than the two clears and three kernels of
+// the chip-wide plan (whole calls of 30 x 60 DNA pairs with CIGARs, one block
+// against the chip: 3,000 pairs 0.177 against 0.174 ms, 8,000 0.266 against
+// 0.219, 16,000 0.411 against 0.304).
+constexpr int kPlanSmall = 4096;
 constexpr int kPlanFew = 2048;
 
 

@@ -107,6 +107,20 @@ def test_cta_fill_opens_several_pairs_in_a_phase():
         c.close()
 
 
+@pytest.mark.parametrize("n", [2048, 2049, 4096, 4097, 16383, 16384])
+def test_plans_by_one_block_or_the_chip(n):
+    rng = np.random.default_rng(83 + n)
+    pairs = list(short_pairs(rng, n))
+    pairs[0] = (pairs[0][0][:0], pairs[0][1])  # an empty query and an empty target
+    pairs[n - 1] = (pairs[n - 1][0], pairs[n - 1][1][:0])
+    b = make([p[0] for p in pairs], [p[1] for p in pairs], wl.dna_matrix(2, -3), 5, 2)
+    c = gsw.Context(0, 2 << 30)
+    try:
+        check(b, run_gpu_device(c, b), np.unique(np.concatenate([[0, n - 1], rng.choice(n, 600)])))
+    finally:
+        c.close()
+
+
 @pytest.mark.parametrize("A,match,mismatch,O,X", [(4, 1, -3, 5, 2), (4, 5, -4, 10, 1), (20, 0, 0, 11, 1)])
 def test_group_fills_of_several_strips(A, match, mismatch, O, X):
     # 20,000 pairs of 540 to 1,400 rows (tests/test_class_rules.py: what such a
