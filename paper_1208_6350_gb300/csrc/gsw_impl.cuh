@@ -230,13 +230,30 @@ __host__ __device__ inline bool cta_pair(int v, int rows, int cols, const Scorin
 // alone would take more than about a quarter of the batch's time (its steps x 0.3 us
 // against the cells at 2.5 T cells/s; 0.46 us and 1.5 T for general alphabets)
 // runs its strips side by side on a CTA (600 x 1,000 DNA: 1,851 GCUPS against
-// 1,513 at 3,000 pairs, 1,961 against 2,321 at 10,000; 350 x 360 protein: 691
-// against 330 at 1,000 pairs, 1,352 against 1,468 at 10,000).
+// 1,513 at 3,000 pairs; 350 x 360 protein: 691 against 330 at 1,000 pairs).
+//
+// Not in an even batch (on average at least a quarter of the largest pair's
+// cells) of more pairs than the 16-lane groups that can be resident, kWave:
+// there no pair outlives the others, and a part of them on CTAs, where strips
+// wait for each other, only takes SMs from the groups (750-1,500 x 600-1,200
+// DNA: 4,000 pairs 2.53 ms with CTAs, 3.05 without; 6,000 pairs 3.52 and 3.09;
+// 10,000 pairs 5.07 and 4.28).  For general alphabets from half as many pairs on
+// where queries have at most 1,024 rows, two CTA strips, which leave half of a
+// CTA's warps idle (450-900 x 400-800 protein: 1,000 pairs 0.57 ms with CTAs,
+// 1.42 without; 4,000 pairs 1.55 and 1.22).
+//
+// General alphabets in less than kWave pairs: a class costs its pairs' latency,
+// strips x the row words of a step, not its share of a full chip (225-450 x
+// 200-400: 2,500 pairs 0.490 -> 0.355 ms, 300-600 x 200-400: 4,000 pairs 0.768
+// -> 0.583 ms, with the rule above).
 inline void default_classes(Scoring &sc, int npairs, int maxm, int maxn, double cells) {
     constexpr int kWide = 8192, kNarrow = 16384, kFewPairs = 2048;
+    constexpr int kWave = 152 * 4 * 8;  // SMs x blocks of 4 warps x pairs of a block
     // (a power of two: batches of like size keep their captured graphs)
     sc.cta_steps = 256;
     while (sc.cta_steps < cells * 3.5e-7 && sc.cta_steps < (1 << 28)) sc.cta_steps *= 2;
+    const bool even = cells >= 0.25 * npairs * (double)maxm * maxn;
+    if (even && (npairs > kWave || (!sc.dna4 && npairs > kWave / 2 && maxm <= 1024))) sc.cta_steps = 0;
     static constexpr float dna[kNumVariants] = {28.3f, 33.4f, 39.2f, 45.8f, 50.1f, 59.6f, 61.2f, 0,
                                                 32.1f, 36.3f, 42.6f, 52.3f, 55.8f, 13.8f, 16.8f, 19.5f,
                                                 21.4f, 24.8f, 29.5f, 72.6f, 85.0f, 112.0f};
@@ -256,7 +273,8 @@ inline void default_classes(Scoring &sc, int npairs, int maxm, int maxn, double 
             if (p8 && (npairs < kWide || rows > variant_rows(v))) continue;
             if (p4 && (npairs < kNarrow || rows > variant_rows(v) || !sc.dna4 || !half_fits(rows, maxn, sc))) continue;
             const int strips = (rows + variant_rows(v) - 1) / variant_rows(v);
-            const float cost = strips * (sc.dna4 ? dna[v] : gen[v]) * (strips > 1 ? multi : 1.0f);
+            float cost = strips * (sc.dna4 ? dna[v] : gen[v]) * (strips > 1 ? multi : 1.0f);
+            if (!sc.dna4 && npairs < kWave) cost = (float)strips * (4 + variant_at(v).R);
             if (pick < 0 || cost < best) {
                 best = cost;
                 pick = v;

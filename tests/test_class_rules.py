@@ -143,6 +143,30 @@ def test_large_batches_run_several_strips_in_groups(lib):
     assert all(any(v >= tall for v in s) and any(v < tall for v in s) for s in seen.values()), seen
 
 
+def test_even_batches_of_many_pairs_stay_in_groups(lib):
+    long16 = lib.cr_consts(4)
+    out = (ctypes.c_uint * 5)()
+
+    def route(A, npairs, rows, cols, share):
+        # a pair of the batch's largest lengths; share: mean cells over its cells
+        W = np.full((A, A), -2, np.int8)
+        np.fill_diagonal(W, 3)
+        lib.cr_route(A, W.ctypes.data_as(ctypes.c_void_p), 5, 2, npairs, 1, rows, cols, share * npairs * rows * cols,
+                     FORWARD, rows, cols, out)
+        assert (out[0] >> out[3]) & 1
+        return out[3]
+
+    for rows, cols in ((1000, 1000), (1500, 1200)):
+        assert route(4, 4000, rows, cols, 0.5) == long16   # the chip part empty
+        assert route(4, 4864, rows, cols, 0.5) == long16
+        assert route(4, 4865, rows, cols, 0.5) != long16   # a group for every pair, and more pairs
+        assert route(4, 4865, rows, cols, 0.05) == long16  # a few pairs far above the others
+    assert route(20, 2432, 900, 800, 0.5) == long16
+    assert route(20, 2433, 900, 800, 0.5) != long16
+    assert route(20, 2433, 1025, 800, 0.5) == long16
+    assert route(20, 4865, 1025, 800, 0.5) != long16
+
+
 def test_wide_bands_are_never_left_out(lib):
     rng = np.random.default_rng(23)
     ring_class = lib.cr_consts(3)
