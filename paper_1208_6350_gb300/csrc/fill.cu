@@ -1,7 +1,7 @@
-// Entry points of the fills (fill.cuh holds the kernels; fill_dna.cu and
-// fill_general.cu instantiate the persistent ones for 4-letter and other
-// alphabets) and the allocation-free forward fill.
-#include "fill.cuh"
+// Entry points of the fills (fill.cuh holds the persistent kernels, which
+// fill_dna.cu, fill_dna_half.cu, fill_general.cu and fill_general_half.cu
+// instantiate; fill_static.cuh those of the allocation-free forward fill).
+#include "fill_static.cuh"
 
 namespace gsw {
 
@@ -106,215 +106,7 @@ cudaError_t launch_fill(const FillLaunch &fl, int sms, cudaStream_t st, const Si
 // file-scope device array instead of context memory.
 namespace {
 
-constexpr int kStaticMaxTarget = GSW_STATIC_MAX_TARGET;
-constexpr size_t kStaticSlotBytes = (size_t)kStaticMaxTarget * sizeof(int32_t) + 2 * (size_t)kStaticMaxTarget * sizeof(int2);
-static_assert(kStaticMaxTarget % 4 == 0 && kStaticSlotBytes % 16 == 0,
-              "slots start on 16-byte boundaries (the fill's 8-byte max-array stores)");
-constexpr int kStaticWarps = 152 * 4;                 // warps of one launch
-constexpr int kStaticSlots = kStaticWarps * 2;        // two pairs in flight per warp
-// slots of the first kernel: the column maxima of one strip in 16-bit lanes
-constexpr size_t kStaticShortBytes = (size_t)kStaticMaxTarget * sizeof(uint16_t);
-constexpr size_t kStaticErrOff = kStaticSlotBytes * kStaticSlots;
-constexpr size_t kStaticBytes = kStaticErrOff + 256;  // + the per-call counters
-static_assert(kStaticBytes == GSW_STATIC_SCRATCH_BYTES, "header states the scratch size");
-
 static __device__ __align__(256) uint8_t g_static_scratch[kStaticBytes];
-
-// counters of a call, zeroed before its kernels
-struct StaticCounters {
-    int32_t bad;   // pairs rejected
-    int32_t next;  // chunks handed out
-    int32_t rest;  // pairs left to the second kernel
-};
-
-// One pair by the P lanes of a group; false when its score left the lanes.
-template <int P, int R, class L, bool DNA, bool ONE>
-__device__ bool static_fill_pair(const BatchView &b, const Scoring &sc, int pair, uint32_t *wsm, int lane, int k,
-                                 unsigned gmask, int gbase, uint8_t *cms, uint8_t *bnd) {
-    gsw_result *rp = b.res + pair;
-    Job job;
-    job.q = b.q + b.q_off[pair];
-    job.qs = 1;
-    job.mrows = b.q_len[pair];
-    job.t = b.t + b.t_off[pair];
-    job.ts = 1;
-    job.ncols = b.t_len[pair];
-    job.stop_u = 0;
-    job.cms = cms;
-    job.bnd = bnd;
-    const RingResult rr = ring_fill<P, R, L, DNA, ONE>(job, sc, wsm, k, gmask, gbase, lane);
-    if (L::FOLD && rr.score > 32767 - sc.wmax) return false;  // refill in 32-bit lanes
-    int s2 = 0, e2 = -1;
-    const int end_t = rr.col, end_q = rr.score > 0 ? rr.row - rr.pad_top : -1;
-    __syncwarp(gmask);
-    secondary<P, L>(b, pair, job, end_t, job.mrows, k, gmask, &s2, &e2);
-    if (k == 0) {
-        rp->score1 = rr.score;
-        rp->score2 = s2;
-        rp->ref_end1 = end_t;
-        rp->read_end1 = end_q;
-        rp->ref_begin1 = -1;
-        rp->read_begin1 = -1;
-        rp->ref_end2 = e2;
-        rp->cigar_len = 0;
-        rp->cigar_off = -1;
-        rp->flags = L::FOLD ? 0 : GSW_RES_S32;
-        rp->reserved = 0;
-    }
-    return true;
-}
-
-// The checks gsw_align_batch makes before any fill, made here by each group
-// before its pair's first access: lengths in [0, 2^24), offsets >= 0 and
-// targets within the slot; then the letter codes.  Writes the record of a
-// rejected or empty pair; true when the pair is to be filled.
-__device__ __forceinline__ bool static_check(const BatchView &b, const Scoring &sc, int pair, int k, int P,
-                                             unsigned gmask, int32_t *bad_count) {
-    const int m = b.q_len[pair], n = b.t_len[pair];
-    bool bad = (uint32_t)m >= (1u << 24) || (uint32_t)n >= (1u << 24) || b.q_off[pair] < 0 || b.t_off[pair] < 0 ||
-               ((b.flags & GSW_COLMAX) && b.colmax_off[pair] < 0) || n > kStaticMaxTarget;
-    if (!bad) {
-        const uint8_t *qp = b.q + b.q_off[pair], *tp = b.t + b.t_off[pair];
-        int found = 0;
-        for (int i = k; i < m; i += P) found |= qp[i] >= sc.A;
-        for (int j = k; j < n; j += P) found |= tp[j] >= sc.A;
-        bad = __any_sync(gmask, found) != 0;
-    }
-    const bool empty = !bad && (m == 0 || n == 0);
-    if (k == 0 && (bad || empty)) {
-        gsw_result *rp = b.res + pair;
-        rp->score1 = 0; rp->score2 = 0; rp->ref_begin1 = -1; rp->ref_end1 = -1; rp->read_begin1 = -1;
-        rp->read_end1 = -1; rp->ref_end2 = -1; rp->cigar_len = 0; rp->cigar_off = -1;
-        rp->flags = bad ? kResInvalid : 0;
-        rp->reserved = 0;
-        if (bad) atomicOr(bad_count, 1);
-    }
-    if (empty && (b.flags & GSW_COLMAX))
-        for (int j = k; j < n; j += P) b.colmax[b.colmax_off[pair] + j] = 0;
-    return !bad && !empty;
-}
-
-// First kernel: the queries of one strip (at most kStaticRows) in 16-bit lanes.
-// Their slots hold the column maxima alone, 2 KB, so the array has one for
-// every group that can be resident, where slots that also fit 32-bit boundary
-// rows (20 KB) allowed 4 warps per SM: 8,192 pairs of 100-250 x 300-1000 DNA
-// letters 1.00 -> 0.56 ms, of 30-400 x 300-1000 2.88 -> 1.11 ms (strips of 320
-// to 512 rows instead of two of 256), 100 of 30-400 x 100-900 0.50 -> 0.22 ms.
-// A block takes kStaticChunk consecutive pairs (8: 0.55 ms, 16: 0.57, 24: 0.62),
-// orders them by strip height and target length, and its warps take them two at
-// a time (one per 16-lane group; both use the same row-word count R, because
-// their profiles share the warp's interleaved shared-memory region).  Taller
-// queries and scores beyond 16 bits are left to the second kernel, which runs
-// only if some pair was.
-constexpr int kStaticChunk = 8;
-constexpr int kStaticRows = 512;
-template <bool DNA>
-__global__ void __launch_bounds__(kBlock, 3) k_fill_static(BatchView b, Scoring sc, uint8_t *scratch, int warp_words) {
-    extern __shared__ __align__(16) uint32_t smem[];
-    __shared__ int order[kStaticChunk], key[kStaticChunk], chunk, taken;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = lane >> 4, k = lane & 15, gbase = g * 16;
-    const unsigned gmask = 0xFFFFu << gbase;
-    uint32_t *wsm = smem + (size_t)warp * warp_words;
-    uint8_t *cms = scratch + (size_t)((blockIdx.x * (kBlock / 32) + warp) * 2 + g) * kStaticShortBytes;
-    StaticCounters *cnt = reinterpret_cast<StaticCounters *>(scratch + kStaticErrOff);
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            chunk = atomicAdd(&cnt->next, 1);
-            taken = 0;
-        }
-        __syncthreads();
-        const long long base = (long long)chunk * kStaticChunk;
-        if (base >= b.npairs) break;
-        if (threadIdx.x < kStaticChunk) {
-            const long long p = base + threadIdx.x;
-            const int m = p < b.npairs ? b.q_len[p] : -1;
-            // (lengths out of range sort anywhere: they are rejected below)
-            key[threadIdx.x] = m < 0 ? -1 : (min(m, kStaticRows + 1) + 31) / 32 * 2048 + (b.t_len[p] & 2047);
-        }
-        __syncthreads();
-        if (threadIdx.x < kStaticChunk) {
-            int rank = 0;
-            for (int x = 0; x < kStaticChunk; x++)
-                rank += key[x] > key[threadIdx.x] || (key[x] == key[threadIdx.x] && x < (int)threadIdx.x);
-            order[rank] = base + threadIdx.x < b.npairs ? (int)(base + threadIdx.x) : -1;
-        }
-        __syncthreads();
-        for (;;) {
-            int t = 0;
-            if (lane == 0) t = atomicAdd(&taken, 2);
-            t = __shfl_sync(0xFFFFFFFFu, t, 0);
-            if (t >= kStaticChunk) break;
-            const int pair = order[t + g];
-            int m = 0, n = 0;
-            bool run = false;
-            if (pair >= 0) {
-                if (b.q_len[pair] > kStaticRows) {
-                    if (k == 0) cnt->rest = 1;  // (checked by the second kernel)
-                } else {
-                    run = static_check(b, sc, pair, k, 16, gmask, &cnt->bad);
-                    m = b.q_len[pair];
-                    n = b.t_len[pair];
-                }
-            }
-            const int rows = __reduce_max_sync(0xFFFFFFFFu, run ? m : 0);
-            const int most = __reduce_max_sync(0xFFFFFFFFu, run ? min(m, n) : 0);
-            const bool half = half_fits(most, most, sc);
-            bool ok = true;
-            if (run) {
-#define GSW_STATIC(R) \
-    ok = half ? static_fill_pair<16, R, LH, DNA, true>(b, sc, pair, wsm, lane, k, gmask, gbase, cms, nullptr) \
-              : static_fill_pair<16, R, L16, DNA, true>(b, sc, pair, wsm, lane, k, gmask, gbase, cms, nullptr)
-                if (rows <= 64) GSW_STATIC(2);
-                else if (rows <= 128) GSW_STATIC(4);
-                else if (rows <= 192) GSW_STATIC(6);
-                else if (rows <= 256) GSW_STATIC(8);
-                else if (rows <= 320) GSW_STATIC(10);
-                else if (rows <= 384) GSW_STATIC(12);
-                else GSW_STATIC(16);
-#undef GSW_STATIC
-                if (!ok && k == 0) {
-                    b.res[pair].flags = GSW_RES_S32 | kResPendingS32;
-                    cnt->rest = 1;
-                }
-            }
-            __syncwarp();
-        }
-    }
-}
-
-// Second kernel: queries of several strips, and pairs whose score left the
-// 16-bit lanes, in slots that hold the boundary rows of 32-bit lanes.  Warps
-// take two pairs at a time (one per 16-lane group), grid-stride.
-template <bool DNA>
-__global__ void __launch_bounds__(kBlock) k_fill_static_rest(BatchView b, Scoring sc, uint8_t *scratch,
-                                                             int warp_words) {
-    extern __shared__ __align__(16) uint32_t smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = lane >> 4, k = lane & 15, gbase = g * 16;
-    const unsigned gmask = 0xFFFFu << gbase;
-    const int gwarp = blockIdx.x * (blockDim.x / 32) + warp;
-    const int nwarps = gridDim.x * (blockDim.x / 32);
-    uint32_t *wsm = smem + (size_t)warp * warp_words;
-    uint8_t *slot = scratch + (size_t)(gwarp * 2 + g) * kStaticSlotBytes;
-    uint8_t *bnd = slot + (size_t)kStaticMaxTarget * sizeof(int32_t);
-    StaticCounters *cnt = reinterpret_cast<StaticCounters *>(scratch + kStaticErrOff);
-    for (long long base = gwarp * 2; base < b.npairs; base += nwarps * 2) {
-        const int pair = (int)base + g;
-        bool run = false, over = false;
-        if (pair < b.npairs) {
-            const bool tall = b.q_len[pair] > kStaticRows;
-            over = !tall && (b.res[pair].flags & kResPendingS32) && !(b.res[pair].flags & kResInvalid);
-            if (tall) run = static_check(b, sc, pair, k, 16, gmask, &cnt->bad);
-        }
-        bool ok = !over;
-        if (run) ok = static_fill_pair<16, 8, L16, DNA, false>(b, sc, pair, wsm, lane, k, gmask, gbase, slot, bnd);
-        __syncwarp();
-        if (!ok) static_fill_pair<16, 8, L32, DNA, false>(b, sc, pair, wsm, lane, k, gmask, gbase, slot, bnd);
-        __syncwarp();
-    }
-}
 
 struct StaticSetup {
     bool done = false;
@@ -350,14 +142,6 @@ extern "C" int gsw_fill_static(int32_t npairs, const uint8_t *q, const int64_t *
     if ((flags & GSW_COLMAX) && (!colmax || !colmax_off)) return set_err(GSW_EINVAL, "colmax output missing");
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return set_err(GSW_ECUDA, "no current device");
-    // the second kernel's 16- or 32-bit profile, whichever is larger
-    const size_t per_warp = (size_t)std::max(prof_words(8, true, sc.dna4 != 0, alphabet),
-                                             prof_words(8, false, sc.dna4 != 0, alphabet)) * 32 * sizeof(uint32_t);
-    int wpb = (int)((200u << 10) / per_warp);
-    wpb = wpb > 4 ? 4 : (wpb < 1 ? 1 : wpb);
-    const size_t smem = per_warp * wpb;
-    const size_t short_warp = (size_t)prof_words(16, true, sc.dna4 != 0, alphabet) * 32 * sizeof(uint32_t);
-    const size_t short_smem = short_warp * (kBlock / 32);
     uint8_t *scratch;
     int sms;
     {
@@ -369,10 +153,8 @@ extern "C" int gsw_fill_static(int32_t npairs, const uint8_t *q, const int64_t *
             void *ptr = nullptr;
             const cudaError_t e = cudaGetSymbolAddress(&ptr, g_static_scratch);
             if (e != cudaSuccess) return set_err(GSW_ECUDA, "scratch address: %s", cudaGetErrorString(e));
-            for (const void *fn : {(const void *)k_fill_static<true>, (const void *)k_fill_static<false>,
-                                   (const void *)k_fill_static_rest<true>, (const void *)k_fill_static_rest<false>})
-                if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 << 10) != cudaSuccess)
-                    return set_err(GSW_ECUDA, "kernel shared-memory limit");
+            if (static_setup_dna() != cudaSuccess || static_setup_general() != cudaSuccess)
+                return set_err(GSW_ECUDA, "kernel shared-memory limit");
             if (cudaDeviceGetAttribute(&su.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
                 return set_err(GSW_ECUDA, "SM count");
             su.ptr = static_cast<uint8_t *>(ptr);
@@ -395,17 +177,17 @@ extern "C" int gsw_fill_static(int32_t npairs, const uint8_t *q, const int64_t *
     // the counters must start at zero; the slots need no clearing
     if (cudaMemsetAsync(scratch + kStaticErrOff, 0, sizeof(StaticCounters), st) != cudaSuccess)
         return set_err(GSW_ECUDA, "clearing the counters");
+    const StaticGeom g = sc.dna4 ? static_geom_dna(alphabet) : static_geom_general(alphabet);
+    auto launch = [&](bool rest, int grid) {
+        if (sc.dna4) static_launch_dna(rest, bv, sc, scratch, g, grid, st);
+        else static_launch_general(rest, bv, sc, scratch, g, grid, st);
+    };
     // as many blocks as can be resident, as the array has slots for and as
     // there are chunks
-    static OccupancyCache occ[2];
-    int per_sm = sc.dna4 ? occ[0].get(k_fill_static<true>, kBlock, alphabet, short_smem, 200 << 10)
-                         : occ[1].get(k_fill_static<false>, kBlock, alphabet, short_smem, 200 << 10);
     const int most = (int)(kStaticErrOff / (kStaticShortBytes * 2 * (kBlock / 32)));
-    int short_grid = std::min(sms * std::max(per_sm, 1), most);
-    short_grid = std::min(short_grid, (npairs + kStaticChunk - 1) / kStaticChunk);
-    const int grid = kStaticWarps / wpb;
-    if (sc.dna4) k_fill_static<true><<<short_grid, kBlock, short_smem, st>>>(bv, sc, scratch, (int)(short_warp / 4));
-    else k_fill_static<false><<<short_grid, kBlock, short_smem, st>>>(bv, sc, scratch, (int)(short_warp / 4));
+    int first_grid = std::min(sms * std::max(g.first_per_sm, 1), most);
+    first_grid = std::min(first_grid, (npairs - 1) / kStaticChunk + 1);
+    launch(false, first_grid);
     StaticCounters cnt = {};
     auto read_back = [&]() -> int {
         const cudaError_t e = cudaGetLastError();
@@ -420,8 +202,7 @@ extern "C" int gsw_fill_static(int32_t npairs, const uint8_t *q, const int64_t *
         if (e != GSW_OK) return e;
     }
     if (cnt.rest) {  // the second kernel only where some pair was left to it
-        if (sc.dna4) k_fill_static_rest<true><<<grid, wpb * 32, smem, st>>>(bv, sc, scratch, (int)(per_warp / 4));
-        else k_fill_static_rest<false><<<grid, wpb * 32, smem, st>>>(bv, sc, scratch, (int)(per_warp / 4));
+        launch(true, std::min(kStaticSlots / g.rest_warps, (npairs - 1) / g.rest_warps + 1));
         const int e = read_back();
         if (e != GSW_OK) return e;
     }

@@ -1,0 +1,269 @@
+// Kernels of the allocation-free forward fill (gsw_fill_static; fill.cu holds the
+// entry point and the scratch, fill_static_dna.cu and fill_static_general.cu
+// instantiate the kernels for 4-letter and other alphabets).
+#pragma once
+#include "fill.cuh"
+
+namespace gsw {
+namespace {
+
+constexpr int kStaticMaxTarget = GSW_STATIC_MAX_TARGET;
+constexpr size_t kStaticSlotBytes = (size_t)kStaticMaxTarget * sizeof(int32_t) + 2 * (size_t)kStaticMaxTarget * sizeof(int2);
+static_assert(kStaticMaxTarget % 4 == 0 && kStaticSlotBytes % 16 == 0,
+              "slots start on 16-byte boundaries (the fill's 8-byte max-array stores)");
+constexpr int kStaticSlots = 152 * 4 * 2;  // pairs in flight of the second kernel, a warp each
+// slots of the first kernel: the column maxima of one strip in 16-bit lanes
+constexpr size_t kStaticShortBytes = (size_t)kStaticMaxTarget * sizeof(uint16_t);
+constexpr size_t kStaticErrOff = kStaticSlotBytes * kStaticSlots;
+constexpr size_t kStaticBytes = kStaticErrOff + 256;  // + the per-call counters
+static_assert(kStaticBytes == GSW_STATIC_SCRATCH_BYTES, "header states the scratch size");
+
+// counters of a call, zeroed before its kernels
+struct StaticCounters {
+    int32_t bad;   // pairs rejected
+    int32_t next;  // chunks handed out
+    int32_t rest;  // pairs left to the second kernel
+};
+
+// One pair by the P lanes of a group; false when its score left the lanes.
+template <int P, int R, class L, bool DNA, bool ONE>
+__device__ bool static_fill_pair(const BatchView &b, const Scoring &sc, int pair, uint32_t *wsm, int lane, int k,
+                                 unsigned gmask, int gbase, uint8_t *cms, uint8_t *bnd) {
+    gsw_result *rp = b.res + pair;
+    Job job;
+    job.q = b.q + b.q_off[pair];
+    job.qs = 1;
+    job.mrows = b.q_len[pair];
+    job.t = b.t + b.t_off[pair];
+    job.ts = 1;
+    job.ncols = b.t_len[pair];
+    job.stop_u = 0;
+    job.cms = cms;
+    job.bnd = bnd;
+    const RingResult rr = ring_fill<P, R, L, DNA, ONE>(job, sc, wsm, k, gmask, gbase, lane);
+    if (L::FOLD && rr.score > 32767 - sc.wmax) return false;  // refill in 32-bit lanes
+    int s2 = 0, e2 = -1;
+    const int end_t = rr.col, end_q = rr.score > 0 ? rr.row - rr.pad_top : -1;
+    __syncwarp(gmask);
+    secondary<P, L>(b, pair, job, end_t, job.mrows, k, gmask, &s2, &e2);
+    if (k == 0) {
+        rp->score1 = rr.score;
+        rp->score2 = s2;
+        rp->ref_end1 = end_t;
+        rp->read_end1 = end_q;
+        rp->ref_begin1 = -1;
+        rp->read_begin1 = -1;
+        rp->ref_end2 = e2;
+        rp->cigar_len = 0;
+        rp->cigar_off = -1;
+        rp->flags = L::FOLD ? 0 : GSW_RES_S32;
+        rp->reserved = 0;
+    }
+    return true;
+}
+
+// The checks gsw_align_batch makes before any fill, made here by each group
+// before its pair's first access: lengths in [0, 2^24), offsets >= 0 and
+// targets within the slot; then the letter codes.  Writes the record of a
+// rejected or empty pair; true when the pair is to be filled.
+__device__ __forceinline__ bool static_check(const BatchView &b, const Scoring &sc, int pair, int k, int P,
+                                             unsigned gmask, int32_t *bad_count) {
+    const int m = b.q_len[pair], n = b.t_len[pair];
+    bool bad = (uint32_t)m >= (1u << 24) || (uint32_t)n >= (1u << 24) || b.q_off[pair] < 0 || b.t_off[pair] < 0 ||
+               ((b.flags & GSW_COLMAX) && b.colmax_off[pair] < 0) || n > kStaticMaxTarget;
+    if (!bad) {
+        const uint8_t *qp = b.q + b.q_off[pair], *tp = b.t + b.t_off[pair];
+        int found = 0;
+        for (int i = k; i < m; i += P) found |= qp[i] >= sc.A;
+        for (int j = k; j < n; j += P) found |= tp[j] >= sc.A;
+        bad = __any_sync(gmask, found) != 0;
+    }
+    const bool empty = !bad && (m == 0 || n == 0);
+    if (k == 0 && (bad || empty)) {
+        gsw_result *rp = b.res + pair;
+        rp->score1 = 0; rp->score2 = 0; rp->ref_begin1 = -1; rp->ref_end1 = -1; rp->read_begin1 = -1;
+        rp->read_end1 = -1; rp->ref_end2 = -1; rp->cigar_len = 0; rp->cigar_off = -1;
+        rp->flags = bad ? kResInvalid : 0;
+        rp->reserved = 0;
+        if (bad) atomicOr(bad_count, 1);
+    }
+    if (empty && (b.flags & GSW_COLMAX))
+        for (int j = k; j < n; j += P) b.colmax[b.colmax_off[pair] + j] = 0;
+    return !bad && !empty;
+}
+
+// First kernel: the queries of one strip (at most kStaticRows) in 16-bit lanes.
+// Their slots hold the column maxima alone, 2 KB, so the array has one for
+// every group that can be resident, where slots that also fit 32-bit boundary
+// rows (20 KB) allowed 4 warps per SM: 8,192 pairs of 100-250 x 300-1000 DNA
+// letters 1.00 -> 0.56 ms.  A block takes kStaticChunk consecutive pairs (8:
+// 0.55 ms, 16: 0.57, 24: 0.62) and orders them by strip height and target length.
+// Its warps take those of up to kStaticHalf rows two at a time (one per 16-lane
+// group; both use the same row-word count R, because their profiles share the
+// warp's interleaved shared-memory region), and taller ones alone, a whole warp
+// over a strip of 640 or 1,024 rows.  (In strips of 256 rows by the second kernel,
+// after the first had ended, 100 pairs of 500-1,000 x 1,000 took 1.11 ms, now
+// 0.48; 8,192 of 300-600 x 900 4.13 ms, now 1.32.)
+// Taller queries and scores beyond 16 bits are left to the second kernel, which
+// runs only if some pair was.
+constexpr int kStaticChunk = 8;
+constexpr int kStaticHalf = 512;
+constexpr int kStaticRows = 1024;
+template <bool DNA>
+__global__ void __launch_bounds__(kBlock, 3) k_fill_static(BatchView b, Scoring sc, uint8_t *scratch, int warp_words) {
+    extern __shared__ __align__(16) uint32_t smem[];
+    constexpr int kNone = -1, kWhole = -2;  // no pair; the pair before takes the whole warp
+    __shared__ int order[2 * kStaticChunk], key[kStaticChunk], chunk, taken, places;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = lane >> 4, k = lane & 15, gbase = g * 16;
+    const unsigned gmask = 0xFFFFu << gbase;
+    uint32_t *wsm = smem + (size_t)warp * warp_words;
+    uint8_t *slots = scratch + (size_t)(blockIdx.x * (kBlock / 32) + warp) * 2 * kStaticShortBytes;
+    StaticCounters *cnt = reinterpret_cast<StaticCounters *>(scratch + kStaticErrOff);
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            chunk = atomicAdd(&cnt->next, 1);
+            taken = 0;
+        }
+        if (threadIdx.x < 2 * kStaticChunk) order[threadIdx.x] = kNone;
+        __syncthreads();
+        const long long base = (long long)chunk * kStaticChunk;
+        if (base >= b.npairs) break;
+        int rows_key = -1;
+        if (threadIdx.x < kStaticChunk) {
+            const long long p = base + threadIdx.x;
+            const int m = p < b.npairs ? b.q_len[p] : -1;
+            // (lengths out of range sort anywhere: they are rejected below; the
+            // second kernel's last, so that whole warps start at even places)
+            rows_key = m < 0 ? -1 : m > kStaticRows ? 0 : (m + 31) / 32 * 2048 + (b.t_len[p] & 2047);
+            key[threadIdx.x] = rows_key;
+        }
+        __syncthreads();
+        if (threadIdx.x < kStaticChunk) {
+            constexpr int above = kStaticHalf / 32 * 2048 + 2047;  // keys of more rows than a half warp's
+            int rank = 0, whole = 0;
+            for (int x = 0; x < kStaticChunk; x++) {
+                rank += key[x] > rows_key || (key[x] == rows_key && x < (int)threadIdx.x);
+                whole += key[x] > above;
+            }
+            const int at = rows_key > above ? 2 * rank : rank + whole;
+            if (base + threadIdx.x < b.npairs) order[at] = (int)(base + threadIdx.x);
+            if (rows_key > above) order[at + 1] = kWhole;
+            if (threadIdx.x == 0) places = kStaticChunk + whole;
+        }
+        __syncthreads();
+        for (;;) {
+            int t = 0;
+            if (lane == 0) t = atomicAdd(&taken, 2);
+            t = __shfl_sync(0xFFFFFFFFu, t, 0);
+            if (t >= places) break;
+            const bool whole = order[t + 1] == kWhole;
+            const int pair = whole ? order[t] : order[t + g];
+            const int P = whole ? 32 : 16;
+            const unsigned mask = whole ? 0xFFFFFFFFu : gmask;
+            int m = 0, n = 0;
+            bool run = false;
+            if (pair >= 0) {
+                if (b.q_len[pair] > kStaticRows) {
+                    if (k == 0) cnt->rest = 1;  // (checked by the second kernel)
+                } else {
+                    run = static_check(b, sc, pair, whole ? lane : k, P, mask, &cnt->bad);
+                    m = b.q_len[pair];
+                    n = b.t_len[pair];
+                }
+            }
+            const int rows = __reduce_max_sync(0xFFFFFFFFu, run ? m : 0);
+            const int most = __reduce_max_sync(0xFFFFFFFFu, run ? min(m, n) : 0);
+            const bool half = half_fits(most, most, sc);
+            bool ok = true;
+#define GSW_STATIC(P, R, k, mask, gbase, cms) \
+    ok = half ? static_fill_pair<P, R, LH, DNA, true>(b, sc, pair, wsm, lane, k, mask, gbase, cms, nullptr) \
+              : static_fill_pair<P, R, L16, DNA, true>(b, sc, pair, wsm, lane, k, mask, gbase, cms, nullptr)
+#define GSW_STATIC_GROUP(R) GSW_STATIC(16, R, k, gmask, gbase, slots + g * kStaticShortBytes)
+#define GSW_STATIC_WARP(R) GSW_STATIC(32, R, lane, 0xFFFFFFFFu, 0, slots)
+            if (run && whole) {
+                if (rows <= 640) GSW_STATIC_WARP(10);
+                else GSW_STATIC_WARP(16);
+            } else if (run) {
+                if (rows <= 64) GSW_STATIC_GROUP(2);
+                else if (rows <= 128) GSW_STATIC_GROUP(4);
+                else if (rows <= 192) GSW_STATIC_GROUP(6);
+                else if (rows <= 256) GSW_STATIC_GROUP(8);
+                else if (rows <= 320) GSW_STATIC_GROUP(10);
+                else if (rows <= 384) GSW_STATIC_GROUP(12);
+                else GSW_STATIC_GROUP(16);
+            }
+#undef GSW_STATIC_WARP
+#undef GSW_STATIC_GROUP
+#undef GSW_STATIC
+            if (!ok && (whole ? lane : k) == 0) {
+                b.res[pair].flags = GSW_RES_S32 | kResPendingS32;
+                cnt->rest = 1;
+            }
+            __syncwarp();
+        }
+    }
+}
+
+// Second kernel: queries of several strips, and pairs whose score left the
+// 16-bit lanes, a whole warp per pair (strips of 1,024 rows, 256 in 32-bit
+// lanes) in slots that hold the boundary rows of 32-bit lanes (400 pairs of
+// 2,000-3,000 x 1,000: 2.94 ms two pairs a warp in 256-row strips, now 0.89).
+template <bool DNA>
+__global__ void __launch_bounds__(kBlock) k_fill_static_rest(BatchView b, Scoring sc, uint8_t *scratch,
+                                                             int warp_words) {
+    extern __shared__ __align__(16) uint32_t smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int gwarp = blockIdx.x * (blockDim.x / 32) + warp;
+    const int nwarps = gridDim.x * (blockDim.x / 32);
+    uint32_t *wsm = smem + (size_t)warp * warp_words;
+    uint8_t *slot = scratch + (size_t)gwarp * kStaticSlotBytes;
+    uint8_t *bnd = slot + (size_t)kStaticMaxTarget * sizeof(int32_t);
+    StaticCounters *cnt = reinterpret_cast<StaticCounters *>(scratch + kStaticErrOff);
+    for (long long at = gwarp; at < b.npairs; at += nwarps) {
+        const int pair = (int)at;
+        const bool tall = b.q_len[pair] > kStaticRows;
+        bool ok = tall || !(b.res[pair].flags & kResPendingS32) || (b.res[pair].flags & kResInvalid);
+        if (tall && static_check(b, sc, pair, lane, 32, 0xFFFFFFFFu, &cnt->bad))
+            ok = static_fill_pair<32, 16, L16, DNA, false>(b, sc, pair, wsm, lane, lane, 0xFFFFFFFFu, 0, slot, bnd);
+        __syncwarp();
+        if (!ok) static_fill_pair<32, 8, L32, DNA, false>(b, sc, pair, wsm, lane, lane, 0xFFFFFFFFu, 0, slot, bnd);
+        __syncwarp();
+    }
+}
+
+template <bool DNA>
+StaticGeom static_geom(int alphabet) {
+    StaticGeom g;
+    g.first_warp = (size_t)prof_words(16, true, DNA, alphabet) * 32 * sizeof(uint32_t);
+    g.first_smem = g.first_warp * (kBlock / 32);
+    static OccupancyCache occ;
+    g.first_per_sm = occ.get(k_fill_static<DNA>, kBlock, alphabet, g.first_smem, kStaticMaxSmem);
+    // the second kernel's 16- or 32-bit profile, whichever is larger
+    g.rest_warp = (size_t)std::max(prof_words(16, true, DNA, alphabet), prof_words(8, false, DNA, alphabet)) * 32 *
+                  sizeof(uint32_t);
+    g.rest_warps = std::max(1, std::min(4, (int)(kStaticMaxSmem / g.rest_warp)));
+    return g;
+}
+
+template <bool DNA>
+cudaError_t static_setup() {
+    cudaError_t e = cudaFuncSetAttribute(k_fill_static<DNA>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStaticMaxSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_fill_static_rest<DNA>, cudaFuncAttributeMaxDynamicSharedMemorySize, kStaticMaxSmem);
+    return e;
+}
+
+template <bool DNA>
+void static_launch(bool rest, const BatchView &b, const Scoring &sc, uint8_t *scratch, const StaticGeom &g, int grid,
+                   cudaStream_t st) {
+    if (rest)
+        k_fill_static_rest<DNA><<<grid, g.rest_warps * 32, g.rest_warp * g.rest_warps, st>>>(b, sc, scratch,
+                                                                                            (int)(g.rest_warp / 4));
+    else
+        k_fill_static<DNA><<<grid, kBlock, g.first_smem, st>>>(b, sc, scratch, (int)(g.first_warp / 4));
+}
+
+}  // namespace
+}  // namespace gsw

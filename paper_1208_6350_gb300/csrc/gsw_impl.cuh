@@ -791,6 +791,23 @@ cudaError_t launch_fill(const FillLaunch &fl, int sms, cudaStream_t st, const Si
 GSW_FILL_UNITS(GSW_DECLARE_UNIT)
 #undef GSW_DECLARE_UNIT
 
+// Geometry and launches of the allocation-free fill's two kernels (fill_static.cuh)
+constexpr int kStaticMaxSmem = 200 << 10;
+struct StaticGeom {
+    size_t first_warp, first_smem;  // profile bytes of a warp and of a block of the first kernel
+    int first_per_sm;               // its resident blocks per SM
+    size_t rest_warp;               // profile bytes of a warp of the second kernel
+    int rest_warps;                 // its warps per block
+};
+#define GSW_DECLARE_STATIC(name)                                                                            \
+    StaticGeom static_geom_##name(int alphabet);                                                            \
+    cudaError_t static_setup_##name();                                                                      \
+    void static_launch_##name(bool rest, const BatchView &b, const Scoring &sc, uint8_t *scratch,           \
+                              const StaticGeom &g, int grid, cudaStream_t st);
+GSW_DECLARE_STATIC(dna)
+GSW_DECLARE_STATIC(general)
+#undef GSW_DECLARE_STATIC
+
 struct PlanBuffers {
     int32_t *keys;       // [npairs]
     int32_t *hist;       // [kPlanBins]
