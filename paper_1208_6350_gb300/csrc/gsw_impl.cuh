@@ -37,7 +37,9 @@ struct Scoring {
     // default_classes chose for the batch (-1: the smallest one-strip variant)
     int8_t fill_class[GSW_TUNE_BUCKETS];
     int8_t rev_class[GSW_TUNE_BUCKETS];  // of the reversed fill, + 1 (0: as the forward fill)
-    int32_t cta_steps;  // a pair whose strips one after the other take more steps runs on a CTA (0: off)
+    // a pair whose strips one after the other take more steps runs on a CTA (0:
+    // off), in the forward and in the reversed fill
+    int32_t cta_steps, cta_steps_rev;
 };
 
 // Batch view (device pointers) shared by every stage.
@@ -208,11 +210,12 @@ __host__ __device__ inline bool tuned_rows(int rows, const Scoring &sc) {
 // Whether a pair that class v would run strip after strip goes to the CTA
 // class instead (sc.cta_steps, default_classes).  Not where a tune table names
 // the class: there its strips run one after the other as the table says.
-__host__ __device__ inline bool cta_pair(int v, int rows, int cols, const Scoring &sc) {
-    if (sc.cta_steps <= 0 || v >= kNumVariants || v == kVarS32 || tuned_rows(rows, sc)) return false;
+__host__ __device__ inline bool cta_pair(int v, int rows, int cols, const Scoring &sc, bool reverse) {
+    const int32_t most = reverse ? sc.cta_steps_rev : sc.cta_steps;
+    if (most <= 0 || v >= kNumVariants || v == kVarS32 || tuned_rows(rows, sc)) return false;
     const int strips = (rows + variant_rows(v) - 1) / variant_rows(v);
     // (a step's time grows with its row words; 0.3 us is that of 8)
-    return strips > 1 && (long long)strips * cols * (4 + variant_at(v).R) > 12LL * sc.cta_steps;
+    return strips > 1 && (long long)strips * cols * (4 + variant_at(v).R) > 12LL * most;
 }
 
 // Chooses the fill classes of a batch's untuned buckets from its size (pairs,
@@ -246,12 +249,17 @@ __host__ __device__ inline bool cta_pair(int v, int rows, int cols, const Scorin
 // strips x the row words of a step, not its share of a full chip (225-450 x
 // 200-400: 2,500 pairs 0.490 -> 0.355 ms, 300-600 x 200-400: 4,000 pairs 0.768
 // -> 0.583 ms, with the rule above).
+//
+// Both forward only: reversed pairs end at their begins, unlike each other (3,000
+// pairs of 350-700 x 200-400 protein with CIGARs 2.06 ms, with both rules in the
+// reversed fill too 2.59).
 inline void default_classes(Scoring &sc, int npairs, int maxm, int maxn, double cells) {
     constexpr int kWide = 8192, kNarrow = 16384, kFewPairs = 2048;
     constexpr int kWave = 152 * 4 * 8;  // SMs x blocks of 4 warps x pairs of a block
     // (a power of two: batches of like size keep their captured graphs)
     sc.cta_steps = 256;
     while (sc.cta_steps < cells * 3.5e-7 && sc.cta_steps < (1 << 28)) sc.cta_steps *= 2;
+    sc.cta_steps_rev = sc.cta_steps;
     const bool even = cells >= 0.25 * npairs * (double)maxm * maxn;
     if (even && (npairs > kWave || (!sc.dna4 && npairs > kWave / 2 && maxm <= 1024))) sc.cta_steps = 0;
     static constexpr float dna[kNumVariants] = {28.3f, 33.4f, 39.2f, 45.8f, 50.1f, 59.6f, 61.2f, 0,
@@ -273,14 +281,14 @@ inline void default_classes(Scoring &sc, int npairs, int maxm, int maxn, double 
             if (p8 && (npairs < kWide || rows > variant_rows(v))) continue;
             if (p4 && (npairs < kNarrow || rows > variant_rows(v) || !sc.dna4 || !half_fits(rows, maxn, sc))) continue;
             const int strips = (rows + variant_rows(v) - 1) / variant_rows(v);
-            float cost = strips * (sc.dna4 ? dna[v] : gen[v]) * (strips > 1 ? multi : 1.0f);
-            if (!sc.dna4 && npairs < kWave) cost = (float)strips * (4 + variant_at(v).R);
+            const float full = strips * (sc.dna4 ? dna[v] : gen[v]) * (strips > 1 ? multi : 1.0f);
+            const float cost = !sc.dna4 && npairs < kWave ? (float)strips * (4 + variant_at(v).R) : full;
             if (pick < 0 || cost < best) {
                 best = cost;
                 pick = v;
             }
-            if (!p8 && !p4 && (pick16 < 0 || cost < best16)) {
-                best16 = cost;
+            if (!p8 && !p4 && (pick16 < 0 || full < best16)) {
+                best16 = full;
                 pick16 = v;
             }
         }
@@ -317,7 +325,7 @@ inline uint32_t fill_class_mask(int mode, int maxm, const Scoring &sc, bool forc
         strips |= r > variant_rows(c) && !tuned_rows(r, sc);
         if (s32 && mode != kFillForward) m |= 1u << pick_class_reverse(r, true, sc);
     }
-    if (sc.cta_steps > 0 && strips) m |= 1u << kClassLong16;
+    if ((mode == kFillForward ? sc.cta_steps : sc.cta_steps_rev) > 0 && strips) m |= 1u << kClassLong16;
     if (maxm > upto) {  // past the tuned buckets: the tallest variant or the CTA classes
         m |= (1u << kVarMaxS16) | (1u << kClassLong16);
         if (s32 && mode != kFillForward) m |= (1u << kVarS32) | (1u << kClassLong32);

@@ -39,7 +39,7 @@ __device__ int plan_key(const BatchView &b, const Scoring &sc, int32_t mode, int
         cols = b.t_len[p];
         if (b.flags & GSW_FORCE_S32) v = (cols > 0 && long_pair(rows, true, sc.dna4)) ? kClassLong32 : kVarS32;
         else v = (cols > 0 && rows > 0) ? pick_class16(rows, sc) : 0;  // (any class writes an empty pair's record)
-        if (cta_pair(v, rows, cols, sc)) v = kClassLong16;
+        if (cta_pair(v, rows, cols, sc, false)) v = kClassLong16;
     } else if (mode == kFillRerun) {
         if (!(b.res[p].flags & kResPendingS32)) return -1;
         rows = b.q_len[p];
@@ -63,7 +63,7 @@ __device__ int plan_key(const BatchView &b, const Scoring &sc, int32_t mode, int
         // before the last one starts (4-letter DNA: a general alphabet's CTA
         // holds 4 warps per SM)
         v = pick_class_reverse(rows, (r.flags & GSW_RES_S32) != 0, sc);
-        if (cta_pair(v, rows, cols, sc)) v = kClassLong16;
+        if (cta_pair(v, rows, cols, sc, true)) v = kClassLong16;
     } else if (mode == kPlanTrace) {
         gsw_result r = b.res[p];
         if (small_batch(b) && r.score1 > 0 && !(r.flags & kResInternal)) {

@@ -36,7 +36,7 @@ void cr_route_tuned(int A, const signed char *W, int O, int X, const signed char
     out[1] = gsw::fill_half_mask(r, maxn, sc);
     out[2] = gsw::fill_multi_mask(r);
     int v = mode == gsw::kFillForward ? gsw::pick_class16(rows, sc) : gsw::pick_class_reverse(rows, false, sc);
-    if (gsw::cta_pair(v, rows, cols, sc)) v = gsw::kClassLong16;
+    if (gsw::cta_pair(v, rows, cols, sc, mode != gsw::kFillForward)) v = gsw::kClassLong16;
     out[3] = (unsigned)v;
     out[4] = (unsigned)gsw::variant_rows(v);
 }
