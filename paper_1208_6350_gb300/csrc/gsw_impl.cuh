@@ -614,11 +614,14 @@ __host__ __device__ inline int trace_class(int la, int lb, int score1, const Sco
         const long long lo = 3LL * sc.O + (long long)sc.X * (rows + cols + 2) - (sc.wmin < 0 ? sc.wmin : 0);
         const long long hi = (long long)sc.wmax * ((cols < rows ? cols : rows) + 1);
         if (lo <= 30000 && hi <= 30000 && shape.need_words(la, lb) <= cap) {
-            // cell updates: the padded rectangle against the band's
-            // anti-diagonal slots; a 16-bit pair of cells costs about the
-            // instructions of one 32-bit anti-diagonal cell
+            // cell updates: the rectangle, in 8-lane strips whatever shape runs
+            // it, against the band's anti-diagonal slots; a 16-bit pair of cells
+            // costs about the instructions of one 32-bit anti-diagonal cell (whole
+            // warps' own padding counts for less: costed by it, too many regions of
+            // general alphabets took the anti-diagonals, 1,000 calls' pairs of
+            // 750-1,500 x 750-1,500 with CIGARs 5.1 -> 7.1 ms)
             // (bands wider than 512 diagonals: the rectangle always)
-            const long long rect = rows * shape.steps(lb);
+            const long long rect = (long long)t16_strips(la, v) * t16_strip_rows(v) * t16_steps(lb);
             if (ad == kTraceRingClass) return kTraceT16First + v;
             const long long band = (32LL << ad) * (la + lb + 1);
             if (rect <= (small ? 2 : 3) * band) return kTraceT16First + v;
