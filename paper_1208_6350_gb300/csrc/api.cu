@@ -341,7 +341,7 @@ uint64_t bucket_up(uint64_t x) {
 }
 
 int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st, int minm, int maxm,
-                 int maxn) {
+                 int maxn, bool equal) {
     const int npairs = bv.npairs;
     unsigned long long *misc = reinterpret_cast<unsigned long long *>(ctx->misc.p);
     unsigned long long *hs = reinterpret_cast<unsigned long long *>(ctx->host_small);
@@ -353,6 +353,7 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
     key_add(key, minm);
     key_add(key, maxm);
     key_add(key, maxn);
+    key_add(key, equal);
     key_add(key, st);
     key_add(key, ctx->sms);
     key_add(key, ctx->shared);
@@ -393,6 +394,7 @@ int run_pipeline(gsw_ctx *ctx, BatchView bv, const Scoring &sc, cudaStream_t st,
         fl.sc = sc;
         fl.maxm = maxm;
         fl.one_cta = ctx->one_cta;
+        fl.equal = equal;
         fl.bad_letters = reinterpret_cast<const int32_t *>(misc + kMiscValid);
         fl.plan.order = pb.order;
         fl.plan.var_start = pb.var_start;
@@ -875,7 +877,9 @@ int batch_impl(gsw_ctx *ctx, int32_t npairs, const uint8_t *q, const int64_t *q_
         CUDA_TRY(launch_validate(bv, sc, reinterpret_cast<int32_t *>(misc + kMiscValid), st));
         ctx->launches += 1;
     }
-    GSW_TRY(run_pipeline(ctx, bv, sc, st, minm, maxm, maxn));
+    // (sizes rounded up to buckets say nothing of it)
+    const bool equal = !ctx->graph_buckets && equal_batch(npairs, maxm, maxn, cells);
+    GSW_TRY(run_pipeline(ctx, bv, sc, st, minm, maxm, maxn, equal));
 
     // completion: invalid letters, internal checks, CIGAR space
     CUDA_TRY(launch_count_internal(bv, misc + kMiscInternal, st));

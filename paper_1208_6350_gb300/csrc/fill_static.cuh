@@ -66,8 +66,9 @@ __device__ bool static_fill_pair(const BatchView &b, const Scoring &sc, int pair
 // before its pair's first access: lengths in [0, 2^24), offsets >= 0 and
 // targets within the slot; then the letter codes.  Writes the record of a
 // rejected or empty pair; true when the pair is to be filled.
-__device__ __forceinline__ bool static_check(const BatchView &b, const Scoring &sc, int pair, int k, int P,
-                                             unsigned gmask, int32_t *bad_count) {
+template <int P>
+__device__ __forceinline__ bool static_check(const BatchView &b, const Scoring &sc, int pair, int k, unsigned gmask,
+                                             int32_t *bad_count) {
     const int m = b.q_len[pair], n = b.t_len[pair];
     bool bad = (uint32_t)m >= (1u << 24) || (uint32_t)n >= (1u << 24) || b.q_off[pair] < 0 || b.t_off[pair] < 0 ||
                ((b.flags & GSW_COLMAX) && b.colmax_off[pair] < 0) || n > kStaticMaxTarget;
@@ -160,15 +161,14 @@ __global__ void __launch_bounds__(kBlock, 3) k_fill_static(BatchView b, Scoring 
             if (t >= places) break;
             const bool whole = order[t + 1] == kWhole;
             const int pair = whole ? order[t] : order[t + g];
-            const int P = whole ? 32 : 16;
-            const unsigned mask = whole ? 0xFFFFFFFFu : gmask;
             int m = 0, n = 0;
             bool run = false;
             if (pair >= 0) {
                 if (b.q_len[pair] > kStaticRows) {
                     if (k == 0) cnt->rest = 1;  // (checked by the second kernel)
                 } else {
-                    run = static_check(b, sc, pair, whole ? lane : k, P, mask, &cnt->bad);
+                    run = whole ? static_check<32>(b, sc, pair, lane, 0xFFFFFFFFu, &cnt->bad)
+                                : static_check<16>(b, sc, pair, k, gmask, &cnt->bad);
                     m = b.q_len[pair];
                     n = b.t_len[pair];
                 }
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kBlock) k_fill_static_rest(BatchView b, Scorin
         const int pair = (int)at;
         const bool tall = b.q_len[pair] > kStaticRows;
         bool ok = tall || !(b.res[pair].flags & kResPendingS32) || (b.res[pair].flags & kResInvalid);
-        if (tall && static_check(b, sc, pair, lane, 32, 0xFFFFFFFFu, &cnt->bad))
+        if (tall && static_check<32>(b, sc, pair, lane, 0xFFFFFFFFu, &cnt->bad))
             ok = static_fill_pair<32, 16, L16, DNA, false>(b, sc, pair, wsm, lane, lane, 0xFFFFFFFFu, 0, slot, bnd);
         __syncwarp();
         if (!ok) static_fill_pair<32, 8, L32, DNA, false>(b, sc, pair, wsm, lane, lane, 0xFFFFFFFFu, 0, slot, bnd);

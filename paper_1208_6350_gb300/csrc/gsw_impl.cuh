@@ -218,6 +218,16 @@ __host__ __device__ inline bool cta_pair(int v, int rows, int cols, const Scorin
     return strips > 1 && (long long)strips * cols * (4 + variant_at(v).R) > 12LL * most;
 }
 
+// A batch whose pairs have on average at least a quarter of the largest one's
+// cells.
+inline bool even_batch(int npairs, int maxm, int maxn, double cells) {
+    return cells >= 0.25 * npairs * (double)maxm * maxn;
+}
+// ... of pairs that are nearly alike: at least three quarters
+inline bool equal_batch(int npairs, int maxm, int maxn, double cells) {
+    return cells >= 0.75 * npairs * (double)maxm * maxn;
+}
+
 // Chooses the fill classes of a batch's untuned buckets from its size (pairs,
 // longest target, forward cells).
 //
@@ -235,20 +245,20 @@ __host__ __device__ inline bool cta_pair(int v, int rows, int cols, const Scorin
 // runs its strips side by side on a CTA (600 x 1,000 DNA: 1,851 GCUPS against
 // 1,513 at 3,000 pairs; 350 x 360 protein: 691 against 330 at 1,000 pairs).
 //
-// Not in an even batch (on average at least a quarter of the largest pair's
-// cells) of more pairs than the 16-lane groups that can be resident, kWave:
-// there no pair outlives the others, and a part of them on CTAs, where strips
-// wait for each other, only takes SMs from the groups (750-1,500 x 600-1,200
-// DNA: 4,000 pairs 2.53 ms with CTAs, 3.05 without; 6,000 pairs 3.52 and 3.09;
-// 10,000 pairs 5.07 and 4.28).  For general alphabets from half as many pairs on
-// where queries have at most 1,024 rows, two CTA strips, which leave half of a
+// Not in an even batch (even_batch) of more pairs than the 16-lane groups that
+// can be resident, kWave: there no pair outlives the others, and a part of them
+// on CTAs, where strips wait for each other, only takes SMs from the groups
+// (750-1,500 x 600-1,200 DNA: 4,000 pairs 2.53 ms with CTAs, 3.05 without; 6,000 pairs 3.52 and 3.09;
+// 10,000 pairs 5.07 and 4.28).  For general alphabets from half as many pairs on,
+// where queries have at most 1,024 rows: two CTA strips, which leave half of a
 // CTA's warps idle (450-900 x 400-800 protein: 1,000 pairs 0.57 ms with CTAs,
-// 1.42 without; 4,000 pairs 1.55 and 1.22).
+// 1.42 without; 4,000 pairs 1.55 and 1.22; 10,000 pairs 2.68 and 3.03, so from
+// kWide pairs on only up to 768 rows: 300-600 x 200-400 1.45 and 0.93).
 //
 // General alphabets in less than kWave pairs: a class costs its pairs' latency,
 // strips x the row words of a step, not its share of a full chip (225-450 x
 // 200-400: 2,500 pairs 0.490 -> 0.355 ms, 300-600 x 200-400: 4,000 pairs 0.768
-// -> 0.583 ms, with the rule above).
+// -> 0.583 ms, with the rule above), where CTAs do not take the tall ones.
 //
 // Both forward only: reversed pairs end at their begins, unlike each other (3,000
 // pairs of 350-700 x 200-400 protein with CIGARs 2.06 ms, with both rules in the
@@ -260,8 +270,8 @@ inline void default_classes(Scoring &sc, int npairs, int maxm, int maxn, double 
     sc.cta_steps = 256;
     while (sc.cta_steps < cells * 3.5e-7 && sc.cta_steps < (1 << 28)) sc.cta_steps *= 2;
     sc.cta_steps_rev = sc.cta_steps;
-    const bool even = cells >= 0.25 * npairs * (double)maxm * maxn;
-    if (even && (npairs > kWave || (!sc.dna4 && npairs > kWave / 2 && maxm <= 1024))) sc.cta_steps = 0;
+    const bool even = even_batch(npairs, maxm, maxn, cells);
+    if (even && (sc.dna4 ? npairs > kWave : npairs > kWave / 2 && maxm <= (npairs > kWide ? 768 : 1024))) sc.cta_steps = 0;
     static constexpr float dna[kNumVariants] = {28.3f, 33.4f, 39.2f, 45.8f, 50.1f, 59.6f, 61.2f, 0,
                                                 32.1f, 36.3f, 42.6f, 52.3f, 55.8f, 13.8f, 16.8f, 19.5f,
                                                 21.4f, 24.8f, 29.5f, 72.6f, 85.0f, 112.0f};
@@ -273,6 +283,7 @@ inline void default_classes(Scoring &sc, int npairs, int maxm, int maxn, double 
         const int rows = (b + 1) * GSW_TUNE_ROWS;
         if (long_pair(rows, false, sc.dna4)) continue;
         const float multi = sc.dna4 ? 1.3f : 1.08f;
+        const bool latency = !sc.dna4 && npairs < kWave && (sc.cta_steps == 0 || rows <= 512);
         float best = 0, best16 = 0;
         int pick = -1, pick16 = -1;
         for (int v = 0; v < kNumVariants; v++) {
@@ -282,7 +293,7 @@ inline void default_classes(Scoring &sc, int npairs, int maxm, int maxn, double 
             if (p4 && (npairs < kNarrow || rows > variant_rows(v) || !sc.dna4 || !half_fits(rows, maxn, sc))) continue;
             const int strips = (rows + variant_rows(v) - 1) / variant_rows(v);
             const float full = strips * (sc.dna4 ? dna[v] : gen[v]) * (strips > 1 ? multi : 1.0f);
-            const float cost = !sc.dna4 && npairs < kWave ? (float)strips * (4 + variant_at(v).R) : full;
+            const float cost = latency ? (float)strips * (4 + variant_at(v).R) : full;
             if (pick < 0 || cost < best) {
                 best = cost;
                 pick = v;
@@ -408,6 +419,7 @@ struct FillLaunch {
     int32_t mode;
     int32_t maxm;         // longest query
     bool one_cta;         // no clusters (cluster_ctas)
+    bool equal;           // equal_batch
     uint32_t class_mask;  // classes launched (bit c: class c); the others hold no pair
     uint32_t multi_mask;  // classes that can hold pairs of several strips
     uint32_t half_mask;   // classes whose values stay below 2048: the half-precision clamp lanes

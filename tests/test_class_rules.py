@@ -164,7 +164,9 @@ def test_even_batches_of_many_pairs_stay_in_groups(lib):
     assert route(20, 2432, 900, 800, 0.5) == long16
     assert route(20, 2433, 900, 800, 0.5) != long16
     assert route(20, 2433, 1025, 800, 0.5) == long16
-    assert route(20, 4865, 1025, 800, 0.5) != long16
+    assert route(20, 9000, 1025, 800, 0.5) == long16
+    assert route(20, 8192, 1000, 800, 0.5) != long16 and route(20, 8193, 1000, 800, 0.5) == long16
+    assert route(20, 8193, 700, 800, 0.5) != long16
 
 
 def test_wide_bands_are_never_left_out(lib):
