@@ -426,14 +426,16 @@ __device__ void ring_schedule(const RingLaunch &rl, RingShared<C> &sh, int ph, i
     __syncwarp();
 }
 
-// Two CTAs per SM (at most 128 registers a thread; the compiler's own choice for
-// 16 rows a lane is 154, one CTA): half the warps hide half the latency of the
-// cell chain and of the phases' barriers.  10,000 reads of 1-20 kb: traceback
-// 123.8 -> 97.7 ms.
-constexpr int kRMinBlocks = 2;
+// MINB CTAs per SM.  In the 16-row form the compiler's own choice is 154
+// registers, one CTA, whose steps are the shorter ones: it wins while the longest
+// pairs' chains of strips bound the batch.  Two CTAs (at most 128 registers) win
+// where all SMs are busy to the end.  Reads of 1-20 kb, traceback with one and with
+// two: 3,000 pairs 37.3 and 59.5 ms, 4,500 56.0 and 61.3, 6,000 73.7 and 65.7,
+// 10,000 123.8 and 97.6.
+constexpr int kRingOnePairs = 5000;  // one CTA up to here
 
-template <bool DNA, class C>
-__global__ void __launch_bounds__(kRW * 32, kRMinBlocks) k_trace_ring(RingLaunch rl) {
+template <bool DNA, class C, int MINB>
+__global__ void __launch_bounds__(kRW * 32, MINB) k_trace_ring(RingLaunch rl) {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ RingShared<C> sh_own;
     __shared__ int8_t sW[kMaxAlpha * kMaxAlpha];
@@ -736,15 +738,15 @@ using RingFlat = RingCfg<8>;
 constexpr int kRingFewPairs = 2048;
 bool ring_few(int npairs) { return npairs <= kRingFewPairs; }
 
-template <bool DNA, class C>
+template <bool DNA, class C, int MINB>
 cudaError_t launch_ring_fill(const RingLaunch &rl, const RingLaunchArgs &a, int sms, cudaStream_t st) {
     const int A = DNA ? 4 : a.sc.A;
     const size_t per_warp = (size_t)A * C::RR * 32 * sizeof(uint32_t);
     const int nw = per_warp * kRW <= 200 * 1024 ? kRW : kRW / 2;
     const size_t smem = per_warp * nw;
     int nb = 0;
-    cudaFuncSetAttribute(k_trace_ring<DNA, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_trace_ring<DNA, C>, nw * 32, smem);
+    cudaFuncSetAttribute(k_trace_ring<DNA, C, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_trace_ring<DNA, C, MINB>, nw * 32, smem);
     if (nb < 1) return cudaErrorInvalidConfiguration;
     int cl = cluster_ctas(a.b.npairs, kRingFewPairs, kRMaxCluster, kRMaxCluster, a.one_cta);
     long long grid = std::min<long long>((long long)sms * nb, a.slots / kRSlots);
@@ -763,13 +765,17 @@ cudaError_t launch_ring_fill(const RingLaunch &rl, const RingLaunchArgs &a, int 
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_trace_ring<DNA, C>, rl);
+    return cudaLaunchKernelEx(&cfg, k_trace_ring<DNA, C, MINB>, rl);
 }
 
 template <class C>
 cudaError_t launch_group(const RingLaunch &rl, const RingLaunchArgs &a, int sms, cudaStream_t st) {
     k_ring_group<<<1, 1, 0, st>>>(a.prefix, a.var_start, rl.cls, a.pool_words, a.group);
-    const cudaError_t e = a.sc.dna4 ? launch_ring_fill<true, C>(rl, a, sms, st) : launch_ring_fill<false, C>(rl, a, sms, st);
+    // (8 rows a lane fit two CTAs without a bound)
+    const bool two = C::RR == 16 && a.b.npairs > kRingOnePairs;
+    constexpr int TWO = C::RR == 16 ? 2 : 1;
+    const cudaError_t e = a.sc.dna4 ? (two ? launch_ring_fill<true, C, TWO>(rl, a, sms, st) : launch_ring_fill<true, C, 1>(rl, a, sms, st))
+                                    : (two ? launch_ring_fill<false, C, TWO>(rl, a, sms, st) : launch_ring_fill<false, C, 1>(rl, a, sms, st));
     if (e != cudaSuccess) return e;
     const int wgrid = std::max(1, a.walk_warps / kWalkWarps);
     k_ring_walk<C><<<wgrid, kWalkWarps * 32, 0, st>>>(rl);

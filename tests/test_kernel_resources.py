@@ -26,8 +26,10 @@ def usage(source, tmp_path):
 
 
 def test_wide_band_traceback_leaves_room_for_two_ctas(tmp_path):
-    # 256 threads a CTA and 65,536 registers an SM
+    # 256 threads a CTA and 65,536 registers an SM: the 16-row form of batches of
+    # more than 5,000 pairs, and the 8-row form
     kernels = {k: v for k, v in usage("trace_ring.cu", tmp_path).items() if "k_trace_ring" in k}
-    assert len(kernels) == 4  # 4-letter or general alphabets, 16 or 8 rows a lane
-    for name, (registers, spilled) in kernels.items():
+    two = {k: v for k, v in kernels.items() if "RingCfgILi8E" in k or "RingCfgILi16EEELi2E" in k}
+    assert len(kernels) == 6 and len(two) == 4, kernels  # 4-letter or general alphabets
+    for name, (registers, spilled) in two.items():
         assert registers <= 128 and spilled == 0, (name, registers, spilled)
