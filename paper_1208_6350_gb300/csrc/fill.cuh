@@ -1196,17 +1196,16 @@ __device__ void long_schedule(const FillLaunch &fl, int cls, LongShared<NW> &sh,
         idle &= idle - 1;
         __syncwarp();
     }
-    // new pairs for the warps still idle, opened side by side: one a phase, and
-    // more while the class holds many for every cluster (the heaviest pairs come
-    // first, so a cluster that took several at once would end last: 40 reads of
-    // 8-16 kb on 10 CTAs of 4 each, 82 ms against 21).  Where the pairs are alike
-    // a CTA alone opens its share at once: one a phase let some CTAs take more
-    // pairs than others (1,800 pairs of 2,000 x 2,000 2.65 -> 2.02 ms, 4,950 6.35 ->
-    // 6.07; of unlike pairs, 2,000 of 1,500-3,000 x 1,500-3,000, 4.06 -> 4.36 ms)
+    // a new pair for the warps still idle, one a phase: the heaviest pairs come
+    // first, and a cluster that took several at once would end last (40 reads of
+    // 8-16 kb on 10 CTAs of 4 each, 82 ms against 21; with up to 1 + left / (4 x
+    // clusters) a phase: 1,000 reads of 1-20 kb 35.0 -> 27.7 ms, 2,000 66.2 -> 47.5,
+    // 3,000 104 -> 87, 6,000 161 -> 125).  Where the pairs are alike a CTA alone
+    // opens its share at once, so that all CTAs have the same number (1,800 pairs
+    // of 2,000 x 2,000 2.65 -> 2.02 ms, 4,950 6.35 -> 6.01)
     if (idle && !sh.exhausted) {
         const int left = fl.plan.task_hi[cls] - fl.plan.task_lo[cls] - *(volatile const int32_t *)&fl.plan.head[cls];
-        const int most = fl.equal && nw == NW ? 1 + max(left - 1, 0) / nclusters
-                                             : 1 + (ph > 0 ? max(left, 0) / (4 * nclusters) : 0);
+        const int most = fl.equal && nw == NW ? 1 + max(left - 1, 0) / nclusters : 1;
         const unsigned free_slots = __ballot_sync(ALL, mine && sh.slot[mine ? lane : 0].pair < 0);
         const int rank = __popc(free_slots & ((1u << lane) - 1u));
         const bool try_open = ((free_slots >> lane) & 1u) && rank < min(most, __popc(idle));

@@ -356,10 +356,10 @@ __device__ int ring_open(const RingLaunch &rl, RingSlot<C> &S, int at, int seq) 
 
 // The schedule of phase ph, by one warp: lane = slot, and lane = warp of the
 // cluster (as the fill's CTA kernel): strips to idle warps, oldest pair first,
-// then new pairs, one a phase and more while the group holds many per cluster.
+// then a new pair.
 template <class C>
 __device__ void ring_schedule(const RingLaunch &rl, RingShared<C> &sh, int ph, int nw, int nslots, int slot0,
-                              int nclusters, int lane) {
+                              int lane) {
     constexpr unsigned ALL = 0xFFFFFFFFu;
     for (unsigned m = __ballot_sync(ALL, lane < nw && sh.ended[lane]); m; m &= m - 1) {
         if (lane == 0) {
@@ -394,19 +394,13 @@ __device__ void ring_schedule(const RingLaunch &rl, RingShared<C> &sh, int ph, i
         __syncwarp();
     }
     if (idle && !sh.exhausted) {
-        const int left = rl.group[1] - rl.group[0] - *(volatile int *)&rl.group[2];
-        const int most = 1 + (ph > 0 ? max(left, 0) / (4 * nclusters) : 0);
+        // one a phase (as the fill's CTA kernel)
         const unsigned free_slots = __ballot_sync(ALL, mine && sh.slot[mine ? lane : 0].pair < 0);
-        const int rank = __popc(free_slots & ((1u << lane) - 1u));
-        const bool try_open = ((free_slots >> lane) & 1u) && rank < min(most, __popc(idle));
+        const bool try_open = free_slots && lane == __ffs(free_slots) - 1;
         int got = -1;
-        if (try_open) got = ring_open(rl, sh.slot[lane], slot0 + lane, sh.seq + rank);
-        const unsigned opened = __ballot_sync(ALL, try_open && got == 1);
-        const bool none_left = __any_sync(ALL, try_open && got == 0);
+        if (try_open) got = ring_open(rl, sh.slot[lane], slot0 + lane, sh.seq);
         if (try_open && got == 1) {
-            unsigned m = idle;  // the k-th opened slot goes to the k-th idle warp
-            for (int k = __popc(opened & ((1u << lane) - 1u)); k > 0; k--) m &= m - 1;
-            RingCmd &c = sh.cmd[__ffs(m) - 1];
+            RingCmd &c = sh.cmd[__ffs(idle) - 1];
             c.slot = lane;
             c.strip = 0;
             c.start = ph;
@@ -414,10 +408,9 @@ __device__ void ring_schedule(const RingLaunch &rl, RingShared<C> &sh, int ph, i
             sh.slot[lane].last_start = ph;
             sh.slot[lane].running = 1;
         }
-        __syncwarp();
-        if (lane == 0) {
-            sh.seq += __popc(free_slots);
-            if (none_left) sh.exhausted = 1;
+        if (try_open) {
+            sh.seq++;
+            if (got == 0) sh.exhausted = 1;
         }
         __syncwarp();
     }
@@ -468,7 +461,7 @@ __global__ void __launch_bounds__(kRW * 32, MINB) k_trace_ring(RingLaunch rl) {
     for (int ph = 0;; ph++) {
         barrier();
         if (rank == 0 && cta_warp == 0)
-            ring_schedule<C>(rl, sh_own, ph, nw, nslots, (blockIdx.x / cl) * nslots, gridDim.x / cl, lane);
+            ring_schedule<C>(rl, sh_own, ph, nw, nslots, (blockIdx.x / cl) * nslots, lane);
         barrier();
         if (sh.done) break;
         const RingCmd cmd = sh.cmd[warp];

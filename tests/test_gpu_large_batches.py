@@ -86,7 +86,7 @@ def test_wide_bands_of_a_large_batch_in_one_pool_group(wide):
         c.close()
 
 
-def test_cta_fill_opens_several_pairs_in_a_phase():
+def test_cta_fill_without_clusters():
     # 8 SMs hold 24 CTAs of the DNA fill: 300 pairs of several strips are more
     # than 4 per CTA, and with them 2,049 short ones, so no clusters
     rng = np.random.default_rng(73)
@@ -103,6 +103,27 @@ def test_cta_fill_opens_several_pairs_in_a_phase():
     try:
         assert gsw.load().gsw_context_set_sm_limit(c.handle, 8) == gsw.GSW_OK
         compare(b, run_oracle(b), run_gpu_device(c, b))
+    finally:
+        c.close()
+
+
+def test_cta_fill_opens_its_share_of_like_pairs():
+    # 2,100 pairs of two strips, nearly alike, on the 24 CTAs of 8 SMs: as many
+    # at once as a CTA has slots
+    rng = np.random.default_rng(77)
+    pairs = []
+    for _ in range(2100):
+        t = rng.integers(0, 4, int(rng.integers(290, 321))).astype(np.uint8)
+        q = rng.integers(0, 4, int(rng.integers(1800, 1851))).astype(np.uint8)
+        at = int(rng.integers(0, len(q) - len(t)))
+        q[at:at + len(t)] = t
+        q[rng.integers(0, len(q), len(q) // 20)] = rng.integers(0, 4)
+        pairs.append((q, t))
+    b = make([p[0] for p in pairs], [p[1] for p in pairs], wl.dna_matrix(2, -3), 5, 2)
+    c = gsw.Context(0, 4 << 30)
+    try:
+        assert gsw.load().gsw_context_set_sm_limit(c.handle, 8) == gsw.GSW_OK
+        check(b, run_gpu_device(c, b), np.sort(rng.choice(2100, 300, replace=False)))
     finally:
         c.close()
 
