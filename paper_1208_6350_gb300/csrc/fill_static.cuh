@@ -97,29 +97,25 @@ __device__ __forceinline__ bool static_check(const BatchView &b, const Scoring &
 // Their slots hold the column maxima alone, 2 KB, so the array has one for
 // every group that can be resident, where slots that also fit 32-bit boundary
 // rows (20 KB) allowed 4 warps per SM: 8,192 pairs of 100-250 x 300-1000 DNA
-// letters 1.00 -> 0.56 ms.  A block takes kStaticChunk consecutive pairs (8:
-// 0.55 ms, 16: 0.57, 24: 0.62) and orders them by strip height and target length.
-// Its warps take those of up to kStaticHalf rows two at a time (one per 16-lane
-// group; both use the same row-word count R, because their profiles share the
-// warp's interleaved shared-memory region), and taller ones alone, a whole warp
-// over a strip of 640 or 1,024 rows.  (In strips of 256 rows by the second kernel,
-// after the first had ended, 100 pairs of 500-1,000 x 1,000 took 1.11 ms, now
-// 0.48; 8,192 of 300-600 x 900 4.13 ms, now 1.32.)
-// Taller queries and scores beyond 16 bits are left to the second kernel, which
-// runs only if some pair was.
+// letters 1.00 -> 0.56 ms, of 30-400 x 300-1000 2.88 -> 1.11 ms (strips of 320
+// to 512 rows instead of two of 256), 100 of 30-400 x 100-900 0.50 -> 0.22 ms.
+// A block takes kStaticChunk consecutive pairs (8: 0.55 ms, 16: 0.57, 24: 0.62),
+// orders them by strip height and target length, and its warps take them two at
+// a time (one per 16-lane group; both use the same row-word count R, because
+// their profiles share the warp's interleaved shared-memory region).  Taller
+// queries and scores beyond 16 bits are left to the second kernel, which runs
+// only if some pair was.
 constexpr int kStaticChunk = 8;
-constexpr int kStaticHalf = 512;
-constexpr int kStaticRows = 1024;
+constexpr int kStaticRows = 512;
 template <bool DNA>
 __global__ void __launch_bounds__(kBlock, 3) k_fill_static(BatchView b, Scoring sc, uint8_t *scratch, int warp_words) {
     extern __shared__ __align__(16) uint32_t smem[];
-    constexpr int kNone = -1, kWhole = -2;  // no pair; the pair before takes the whole warp
-    __shared__ int order[2 * kStaticChunk], key[kStaticChunk], chunk, taken, places;
+    __shared__ int order[kStaticChunk], key[kStaticChunk], chunk, taken;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 4, k = lane & 15, gbase = g * 16;
     const unsigned gmask = 0xFFFFu << gbase;
     uint32_t *wsm = smem + (size_t)warp * warp_words;
-    uint8_t *slots = scratch + (size_t)(blockIdx.x * (kBlock / 32) + warp) * 2 * kStaticShortBytes;
+    uint8_t *cms = scratch + (size_t)((blockIdx.x * (kBlock / 32) + warp) * 2 + g) * kStaticShortBytes;
     StaticCounters *cnt = reinterpret_cast<StaticCounters *>(scratch + kStaticErrOff);
     for (;;) {
         __syncthreads();
@@ -127,48 +123,36 @@ __global__ void __launch_bounds__(kBlock, 3) k_fill_static(BatchView b, Scoring 
             chunk = atomicAdd(&cnt->next, 1);
             taken = 0;
         }
-        if (threadIdx.x < 2 * kStaticChunk) order[threadIdx.x] = kNone;
         __syncthreads();
         const long long base = (long long)chunk * kStaticChunk;
         if (base >= b.npairs) break;
-        int rows_key = -1;
         if (threadIdx.x < kStaticChunk) {
             const long long p = base + threadIdx.x;
             const int m = p < b.npairs ? b.q_len[p] : -1;
-            // (lengths out of range sort anywhere: they are rejected below; the
-            // second kernel's last, so that whole warps start at even places)
-            rows_key = m < 0 ? -1 : m > kStaticRows ? 0 : (m + 31) / 32 * 2048 + (b.t_len[p] & 2047);
-            key[threadIdx.x] = rows_key;
+            // (lengths out of range sort anywhere: they are rejected below)
+            key[threadIdx.x] = m < 0 ? -1 : (min(m, kStaticRows + 1) + 31) / 32 * 2048 + (b.t_len[p] & 2047);
         }
         __syncthreads();
         if (threadIdx.x < kStaticChunk) {
-            constexpr int above = kStaticHalf / 32 * 2048 + 2047;  // keys of more rows than a half warp's
-            int rank = 0, whole = 0;
-            for (int x = 0; x < kStaticChunk; x++) {
-                rank += key[x] > rows_key || (key[x] == rows_key && x < (int)threadIdx.x);
-                whole += key[x] > above;
-            }
-            const int at = rows_key > above ? 2 * rank : rank + whole;
-            if (base + threadIdx.x < b.npairs) order[at] = (int)(base + threadIdx.x);
-            if (rows_key > above) order[at + 1] = kWhole;
-            if (threadIdx.x == 0) places = kStaticChunk + whole;
+            int rank = 0;
+            for (int x = 0; x < kStaticChunk; x++)
+                rank += key[x] > key[threadIdx.x] || (key[x] == key[threadIdx.x] && x < (int)threadIdx.x);
+            order[rank] = base + threadIdx.x < b.npairs ? (int)(base + threadIdx.x) : -1;
         }
         __syncthreads();
         for (;;) {
             int t = 0;
             if (lane == 0) t = atomicAdd(&taken, 2);
             t = __shfl_sync(0xFFFFFFFFu, t, 0);
-            if (t >= places) break;
-            const bool whole = order[t + 1] == kWhole;
-            const int pair = whole ? order[t] : order[t + g];
+            if (t >= kStaticChunk) break;
+            const int pair = order[t + g];
             int m = 0, n = 0;
             bool run = false;
             if (pair >= 0) {
                 if (b.q_len[pair] > kStaticRows) {
                     if (k == 0) cnt->rest = 1;  // (checked by the second kernel)
                 } else {
-                    run = whole ? static_check<32>(b, sc, pair, lane, 0xFFFFFFFFu, &cnt->bad)
-                                : static_check<16>(b, sc, pair, k, gmask, &cnt->bad);
+                    run = static_check<16>(b, sc, pair, k, gmask, &cnt->bad);
                     m = b.q_len[pair];
                     n = b.t_len[pair];
                 }
@@ -177,39 +161,34 @@ __global__ void __launch_bounds__(kBlock, 3) k_fill_static(BatchView b, Scoring 
             const int most = __reduce_max_sync(0xFFFFFFFFu, run ? min(m, n) : 0);
             const bool half = half_fits(most, most, sc);
             bool ok = true;
-#define GSW_STATIC(P, R, k, mask, gbase, cms) \
-    ok = half ? static_fill_pair<P, R, LH, DNA, true>(b, sc, pair, wsm, lane, k, mask, gbase, cms, nullptr) \
-              : static_fill_pair<P, R, L16, DNA, true>(b, sc, pair, wsm, lane, k, mask, gbase, cms, nullptr)
-#define GSW_STATIC_GROUP(R) GSW_STATIC(16, R, k, gmask, gbase, slots + g * kStaticShortBytes)
-#define GSW_STATIC_WARP(R) GSW_STATIC(32, R, lane, 0xFFFFFFFFu, 0, slots)
-            if (run && whole) {
-                if (rows <= 640) GSW_STATIC_WARP(10);
-                else GSW_STATIC_WARP(16);
-            } else if (run) {
-                if (rows <= 64) GSW_STATIC_GROUP(2);
-                else if (rows <= 128) GSW_STATIC_GROUP(4);
-                else if (rows <= 192) GSW_STATIC_GROUP(6);
-                else if (rows <= 256) GSW_STATIC_GROUP(8);
-                else if (rows <= 320) GSW_STATIC_GROUP(10);
-                else if (rows <= 384) GSW_STATIC_GROUP(12);
-                else GSW_STATIC_GROUP(16);
-            }
-#undef GSW_STATIC_WARP
-#undef GSW_STATIC_GROUP
+            if (run) {
+#define GSW_STATIC(R) \
+    ok = half ? static_fill_pair<16, R, LH, DNA, true>(b, sc, pair, wsm, lane, k, gmask, gbase, cms, nullptr) \
+              : static_fill_pair<16, R, L16, DNA, true>(b, sc, pair, wsm, lane, k, gmask, gbase, cms, nullptr)
+                if (rows <= 64) GSW_STATIC(2);
+                else if (rows <= 128) GSW_STATIC(4);
+                else if (rows <= 192) GSW_STATIC(6);
+                else if (rows <= 256) GSW_STATIC(8);
+                else if (rows <= 320) GSW_STATIC(10);
+                else if (rows <= 384) GSW_STATIC(12);
+                else GSW_STATIC(16);
 #undef GSW_STATIC
-            if (!ok && (whole ? lane : k) == 0) {
-                b.res[pair].flags = GSW_RES_S32 | kResPendingS32;
-                cnt->rest = 1;
+                if (!ok && k == 0) {
+                    b.res[pair].flags = GSW_RES_S32 | kResPendingS32;
+                    cnt->rest = 1;
+                }
             }
             __syncwarp();
         }
     }
 }
 
-// Second kernel: queries of several strips, and pairs whose score left the
-// 16-bit lanes, a whole warp per pair (strips of 1,024 rows, 256 in 32-bit
-// lanes) in slots that hold the boundary rows of 32-bit lanes (400 pairs of
-// 2,000-3,000 x 1,000: 2.94 ms two pairs a warp in 256-row strips, now 0.89).
+// Second kernel: queries of more than kStaticRows, a whole warp per pair, and
+// pairs whose score left the 16-bit lanes.  Strips of 640 or 1,024 rows (256 in
+// 32-bit lanes), in slots that hold the boundary rows of 32-bit lanes: two pairs a
+// warp in strips of 256 rows took two to six times as many steps after the first
+// kernel had ended (100 pairs of 500-1,000 x 1,000 DNA 1.12 -> 0.49 ms, 8,192 of
+// 300-600 x 900 4.12 -> 1.69, 400 of 2,000-3,000 x 1,000 2.97 -> 0.98).
 template <bool DNA>
 __global__ void __launch_bounds__(kBlock) k_fill_static_rest(BatchView b, Scoring sc, uint8_t *scratch,
                                                              int warp_words) {
@@ -217,18 +196,27 @@ __global__ void __launch_bounds__(kBlock) k_fill_static_rest(BatchView b, Scorin
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gwarp = blockIdx.x * (blockDim.x / 32) + warp;
     const int nwarps = gridDim.x * (blockDim.x / 32);
+    constexpr unsigned ALL = 0xFFFFFFFFu;
     uint32_t *wsm = smem + (size_t)warp * warp_words;
     uint8_t *slot = scratch + (size_t)gwarp * kStaticSlotBytes;
     uint8_t *bnd = slot + (size_t)kStaticMaxTarget * sizeof(int32_t);
     StaticCounters *cnt = reinterpret_cast<StaticCounters *>(scratch + kStaticErrOff);
     for (long long at = gwarp; at < b.npairs; at += nwarps) {
         const int pair = (int)at;
-        const bool tall = b.q_len[pair] > kStaticRows;
+        const int rows = b.q_len[pair];
+        const bool tall = rows > kStaticRows;
         bool ok = tall || !(b.res[pair].flags & kResPendingS32) || (b.res[pair].flags & kResInvalid);
-        if (tall && static_check<32>(b, sc, pair, lane, 0xFFFFFFFFu, &cnt->bad))
-            ok = static_fill_pair<32, 16, L16, DNA, false>(b, sc, pair, wsm, lane, lane, 0xFFFFFFFFu, 0, slot, bnd);
+        if (tall && static_check<32>(b, sc, pair, lane, ALL, &cnt->bad)) {
+            const int most = min(rows, b.t_len[pair]);
+            const bool half = half_fits(most, most, sc);
+#define GSW_STATIC(R, L, ONE) static_fill_pair<32, R, L, DNA, ONE>(b, sc, pair, wsm, lane, lane, ALL, 0, slot, bnd)
+            if (rows > 1024) ok = GSW_STATIC(16, L16, false);
+            else if (rows > 640) ok = half ? GSW_STATIC(16, LH, true) : GSW_STATIC(16, L16, true);
+            else ok = half ? GSW_STATIC(10, LH, true) : GSW_STATIC(10, L16, true);
+        }
         __syncwarp();
-        if (!ok) static_fill_pair<32, 8, L32, DNA, false>(b, sc, pair, wsm, lane, lane, 0xFFFFFFFFu, 0, slot, bnd);
+        if (!ok) GSW_STATIC(8, L32, false);
+#undef GSW_STATIC
         __syncwarp();
     }
 }

@@ -1,7 +1,7 @@
 """gsw_fill_static's queries of more than 512 rows against the oracle (all
-integers, so the tolerance is zero): whole warps over one strip of up to 1,024
-rows in the first kernel, several strips and 32-bit lanes in the second, in
-blocks of eight pairs that mix them with shorter and empty ones."""
+integers, so the tolerance is zero): whole warps over one strip of 640 or 1,024
+rows, several strips and 32-bit lanes in the second kernel, beside shorter and
+empty ones in the first."""
 import numpy as np
 import pytest
 
