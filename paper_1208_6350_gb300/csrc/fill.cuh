@@ -1412,14 +1412,17 @@ ClassGeom long_geom(const FillLaunch &fl, int sms) {
     ClassGeom g;
     // (DNA, so in the reversed fill a pair's band is what its strips run)
     const int ctas = ((fl.maxm + C::SP - 1) / C::SP + C::NW - 1) / C::NW;
+    g.smem = long_smem_bytes<DNA, S32, NARROW>(fl.sc.A);
+    const int resident = sms * cache.get(k_fill_long<DNA, S32, NARROW>, C::NW * 32, fl.sc.A, g.smem,
+                                         long_smem_bytes<DNA, S32, NARROW>(DNA ? 4 : kMaxAlpha));
     g.cluster = cluster_ctas(fl.b.npairs, kLongFewPairs, ctas, kLongMaxCluster, fl.one_cta);
+    if (fl.equal && fl.mode != kFillReverse)
+        g.cluster = cluster_ctas_alike(fl.b.npairs, (fl.maxm + C::SP - 1) / C::SP, C::NW, resident, g.cluster);
     if constexpr (DNA && !S32 && !NARROW)
         if (fl.mode == kFillReverse && g.cluster > 1 && fl.b.npairs <= kLongNarrowPairs)
             return long_geom<DNA, S32, true>(fl, sms);
     g.narrow = NARROW;
-    g.smem = long_smem_bytes<DNA, S32, NARROW>(fl.sc.A);
-    g.grid = sms * cache.get(k_fill_long<DNA, S32, NARROW>, C::NW * 32, fl.sc.A, g.smem,
-                             long_smem_bytes<DNA, S32, NARROW>(DNA ? 4 : kMaxAlpha));
+    g.grid = resident;
     g.slots_per_block = kLongSlots;
     g.cm = slot_cm_bytes<typename C::L>(fl.scr.ncap);
     g.bnd = slot_bnd_bytes<typename C::L>(fl.scr.ncap);

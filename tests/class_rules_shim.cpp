@@ -73,6 +73,10 @@ void cr_rectangle(int A, int cls, int la, int lb, long long *out) {
     out[2] = lb + 2 * s.P;
 }
 
+int cr_cluster_alike(int npairs, int strips, int warps, int resident, int c) {
+    return gsw::cluster_ctas_alike(npairs, strips, warps, resident, c);
+}
+
 int cr_one_stream(int sms, int sms_all, int shared) { return gsw::one_stream(sms, sms_all, shared != 0); }
 
 int cr_cluster(int npairs, int few, int want, int most, int one_cta) {

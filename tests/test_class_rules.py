@@ -269,3 +269,17 @@ def test_a_saved_tune_table_installs_what_was_tuned(lib, monkeypatch):
     assert t["fill_class"] == named.tolist()
     ctx.set_tune(t["fill_class"])  # the classes alone: as named
     assert fake.table == named.tolist()
+
+
+def test_clusters_of_like_pairs_run_the_fewest_rounds(lib):
+    alike = lib.cr_cluster_alike
+    # 456 CTAs of 4 warps; 5 strips: two rounds either way, then three against two
+    assert alike(300, 5, 4, 456, 2) == 1 and alike(500, 5, 4, 456, 2) == 2 and alike(800, 5, 4, 456, 2) == 1
+    assert alike(40, 20, 4, 456, 8) == 8 and alike(1, 20, 4, 456, 8) == 8 and alike(1, 4, 4, 456, 1) == 1
+    rng = np.random.default_rng(41)
+    for _ in range(2000):
+        n, s, r, c = (int(rng.integers(1, x)) for x in (2100, 40, 500, 9))
+        x = alike(n, s, 4, r, c)
+        assert 1 <= x <= c and x & (x - 1) == 0
+        rounds = lambda y: -(-(-(-n // max(r // y, 1)) * s) // (4 * y))
+        assert all(rounds(x) < rounds(y) or (rounds(x) == rounds(y) and x <= y) for y in (1, 2, 4, 8) if y <= c)
