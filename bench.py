@@ -170,11 +170,11 @@ def fill_traffic_bytes(cells, workload):
     if workload != WORKLOAD:
         return None
     path = os.path.join(ROOT, "profiles", "fill_fwd_traffic.txt")
-    src = os.path.join(ROOT, "paper_1208_6350_gb300", "csrc", "fill.cu")
+    src = os.path.join(ROOT, "paper_1208_6350_gb300", "csrc", "fill.cuh")
     try:
         kv = dict(ln.strip().split("=", 1) for ln in open(path) if "=" in ln and not ln.startswith("#"))
         sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
-        if kv.get("fill_cu_sha256_16") != sha:
+        if kv.get("fill_cuh_sha256_16") != sha:
             return None
         return float(kv["dram_bytes_per_cell"]) * cells
     except (OSError, KeyError, ValueError):

@@ -101,11 +101,11 @@ struct Variant {
 };
 constexpr int kNumVariants = 22;
 constexpr int kVarS32 = 7;
-constexpr int kVarMaxS16 = 6;  // the default rule picks among 0..6
+constexpr int kVarMaxS16 = 6;  // the tallest of 0..6, 16 lanes and 2..8 row words
 // 8..12: one pair per 8 lanes with 8..16 row words per lane (128..256 rows per
 // strip): twice the cells per lane and step of the 16-lane variants, so the
-// per-step costs (shuffles, letter loads, trackers) weigh half as much; chosen
-// per query length by the autotuner
+// per-step costs (shuffles, letter loads, trackers) weigh half as much; taken
+// by large batches (default_classes) and by tune tables
 constexpr int kVarP8First = 8;
 // 13..18: one pair per 4 lanes with 6..16 row words per lane (48..128 rows per
 // strip): half the wavefront's skew again and strips that fit reads of up to
@@ -569,7 +569,7 @@ constexpr int kTraceT16First = 5;
 constexpr int kTraceT16Classes = 4;
 constexpr int kT16P = 8;                   // lanes per pair
 constexpr int kT16MaxCols = 4096;          // longest target region of the 16-bit kernel
-constexpr long long kT16MaxWords = 1 << 17;  // scratch words of one pair (512 KB)
+constexpr long long kT16MaxWords = 1 << 17;  // scratch words of one pair (512 KB), as launched
 // general alphabets: regions over kT16MaxWords take class 6 with this
 // allowance (its own launch and scratch, so the few large pairs do not shrink
 // the groups of the others)
